@@ -349,16 +349,17 @@ int geoflood_counters(geoflood_ctx* ctx, int scenario, long long* cell_updates,
  * returns its number in *variant and the times (ms per launch) in
  * ms_per_variant (one entry per variant, at most 16: eight for 32 x 32
  * patches in FP32, four in FP64, one for 16 x 16; either pointer may be
- * NULL).  Variants of
- * 32 x 32 patches: 0 = one 512-thread CTA per patch staging the whole tile
- * by TMA bulk copies, 1 = four CTAs per patch, each staging a 16 x 16
- * sub-tile with its two-cell halo, 2 = the FP32 shape of 0 or the FP64 shape
- * of 1 with the register budget of one CTA per SM, 3 = FP32: one 1024-thread
- * CTA per patch; FP64: adaptive (four sub-tile CTAs for each patch that held
+ * NULL).  Variants of 32 x 32 patches, FP64 (CTAs of sub-tiles with their
+ * two-cell halo): 0 = 8 x 8 or, from 39 patches on, 16 x 16 sub-tiles (192
+ * threads), 1 = 16 x 16 (256 threads), 2 = 8 x 8 (128 threads), 3 = 16 x 16
+ * (352 threads).  FP32: 0 = one 512-thread CTA per patch staging the whole
+ * tile by TMA bulk copies, 1 = four CTAs per patch, each staging a 16 x 16
+ * sub-tile with its two-cell halo, 2 = the shape of 0 with the register
+ * budget of one CTA per SM, 3 = one 1024-thread CTA per patch, 4 = the
+ * sub-tiles of 1 with three 352-thread CTAs per SM, 5 = with four 320-thread
+ * CTAs per SM, 6 = adaptive (four sub-tile CTAs for each patch that held
  * water in the previous step, one CTA that checks the whole tile for every
- * other patch); FP32 only: 4 = the sub-tiles of 1 with three 352-thread CTAs
- * per SM, 5 = with four 320-thread CTAs per SM, 6 = adaptive as FP64's 3,
- * 7 = one 608-thread CTA per patch, two per SM.  Results do not depend on
+ * other patch), 7 = one 608-thread CTA per patch, two per SM.  Results do not depend on
  * the variant. */
 int geoflood_autotune(geoflood_ctx* ctx, int reps, int* variant,
                       double* ms_per_variant);

@@ -31,7 +31,7 @@ SOURCES = [
     # test): no contraction into fused multiply-adds
     ("gf_api.cpp", ["-Xcompiler", "-ffp-contract=off"]),
 ]
-HEADERS = ["gf_internal.h", "gf_solver.cuh", "gf_forest.h", "gf_step_kernel.cuh"]
+HEADERS = ["gf_internal.h", "gf_solver.cuh", "gf_fp64.cuh", "gf_forest.h", "gf_step_kernel.cuh"]
 
 
 def nvcc() -> str:

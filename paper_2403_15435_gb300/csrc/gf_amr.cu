@@ -549,7 +549,7 @@ __global__ void k_inflow(const __grid_constant__ GfGeom G, const __grid_constant
   const int M = G.M, TT = G.T * G.T;
   // a patch on the inflow side runs in every launch
   if (threadIdx.x == 0 && V.runf != nullptr && V.sched != nullptr)
-    V.runf[(size_t)(V.sched[0] & 1u) * V.runf_stride + p] = 1;
+    V.runf[(size_t)(V.sched[0] % 3u) * V.runf_stride + p] = 1;
   const int l = (int)threadIdx.x - GF_NG;
   if (l >= M + GF_NG) return;
   const GfPatch P = V.patch[p];
@@ -660,9 +660,9 @@ __device__ void mark_and_mirror(const Geo<T>& e, const GfView& V, T* q, const Gf
   const int M = G.M, TT = G.T * G.T;
   const int c = e.tix(i, j);
   // water written into this patch's ghost cells: it runs in the next launch
-  // (the patch step has flipped the parity, so sched[0] selects it)
+  // (the patch step has advanced the counter, so sched[0] selects it)
   if (water && V.runf != nullptr && V.sched != nullptr)
-    V.runf[(size_t)(V.sched[0] & 1u) * V.runf_stride + p] = 1;
+    V.runf[(size_t)(V.sched[0] % 3u) * V.runf_stride + p] = 1;
   const int nxp = G.mi << P.level, nyp = G.mj << P.level;
   int xm[2], ym[2], nx = 0, ny = 0;
   T fx = T(1), fy = T(1);

@@ -89,7 +89,7 @@ struct geoflood_ctx {
   unsigned* d_sched = nullptr;        // launch-order parity and counters
   int* d_ord[2] = {nullptr, nullptr}; // launch orders of the patch step
   unsigned char* d_same = nullptr;    // per work unit: buffers agree
-  unsigned char* d_runf = nullptr;    // [2][cap] run flags (see GfView::runf)
+  unsigned char* d_runf = nullptr;    // [3][cap] run flags (see GfView::runf)
   unsigned char* d_gflag = nullptr;   // per patch: holds a gauge
   unsigned* d_pwet = nullptr;         // adaptive variant: per-patch flags
   unsigned* d_pcnt = nullptr;
@@ -161,6 +161,8 @@ struct geoflood_ctx {
 namespace {
 
 // Device memory the bed cache may take (all scenarios, all levels).
+// work units (sub-tile CTAs) a patch can have: 8 x 8 sub-tiles of 32 x 32
+constexpr size_t kUnits = 16;
 constexpr size_t kBedCacheBudget = size_t(16) << 30;
 
 int fail(geoflood_ctx* c, int code, const std::string& msg) {
@@ -460,8 +462,8 @@ int upload_tables(geoflood_ctx* ctx, int t,
   CK(cudaMemcpyAsync(ctx->d_ord[1], ctx->d_ord[0], sizeof(int) * total,
                      cudaMemcpyDeviceToDevice, ctx->st));
   CK(cudaMemsetAsync(ctx->d_sched, 0, 8 * sizeof(unsigned), ctx->st));
-  CK(cudaMemsetAsync(ctx->d_same, 0, (size_t)ctx->cap * 4, ctx->st));
-  CK(cudaMemsetAsync(ctx->d_runf, 1, (size_t)ctx->cap * 2, ctx->st));
+  CK(cudaMemsetAsync(ctx->d_same, 0, (size_t)ctx->cap * kUnits, ctx->st));
+  CK(cudaMemsetAsync(ctx->d_runf, 1, (size_t)ctx->cap * 3, ctx->st));
   CK(cudaMemsetAsync(ctx->d_pwet, 0, (size_t)ctx->cap * sizeof(unsigned), ctx->st));
   CK(cudaMemsetAsync(ctx->d_gflag, 0, (size_t)ctx->cap, ctx->st));
   CK(cudaMemsetAsync(ctx->d_pcnt, 0, (size_t)ctx->cap * sizeof(unsigned), ctx->st));
@@ -496,7 +498,7 @@ int check_errflag(geoflood_ctx* ctx) {
 int ghost_fill_all(geoflood_ctx* ctx) {
   gf::set_errflag(ctx->d_err);
   // ghost cells rewritten from scratch: every patch runs next
-  CK(cudaMemsetAsync(ctx->d_runf, 1, (size_t)ctx->cap * 2, ctx->st));
+  CK(cudaMemsetAsync(ctx->d_runf, 1, (size_t)ctx->cap * 3, ctx->st));
   ProfRec r;
   prof_begin(ctx, "ghost_fill", &r);
   CKL(gf::launch_ghost_fill(ctx->G, view(ctx), 0, ctx->st), "ghost_fill");
@@ -514,9 +516,9 @@ int ghost_fill_all(geoflood_ctx* ctx) {
 // After the host writes state or beds, no tile is known to agree between
 // the two state buffers.
 int forget_same(geoflood_ctx* ctx) {
-  CK(cudaMemsetAsync(ctx->d_same, 0, (size_t)ctx->cap * 4, ctx->st));
+  CK(cudaMemsetAsync(ctx->d_same, 0, (size_t)ctx->cap * kUnits, ctx->st));
   // every patch runs until the marks of two launches have built up again
-  CK(cudaMemsetAsync(ctx->d_runf, 1, (size_t)ctx->cap * 2, ctx->st));
+  CK(cudaMemsetAsync(ctx->d_runf, 1, (size_t)ctx->cap * 3, ctx->st));
   return 0;
 }
 
@@ -819,8 +821,8 @@ int geoflood_init_forest(const geoflood_config* cfg, void* stream,
   okk &= alloc((void**)&ctx->d_sched, 8 * sizeof(unsigned));
   okk &= alloc((void**)&ctx->d_ord[0], cap * sizeof(int));
   okk &= alloc((void**)&ctx->d_ord[1], cap * sizeof(int));
-  okk &= alloc((void**)&ctx->d_same, cap * 4);
-  okk &= alloc((void**)&ctx->d_runf, cap * 2);
+  okk &= alloc((void**)&ctx->d_same, cap * kUnits);
+  okk &= alloc((void**)&ctx->d_runf, cap * 3);
   okk &= alloc((void**)&ctx->d_pwet, cap * sizeof(unsigned));
   okk &= alloc((void**)&ctx->d_gflag, cap);
   okk &= alloc((void**)&ctx->d_pcnt, cap * sizeof(unsigned));

@@ -1,0 +1,175 @@
+// FP64 building blocks for a part whose FP64 pipe takes about two operations
+// per SM and clock (1/64 of its FP32 rate): quotients, square roots,
+// comparisons and scalings by two done in the integer and FP32 pipes, which
+// the FP64 kernels leave idle.  Every function returns exactly the value of
+// the IEEE operation it replaces (round to nearest even), so results do not
+// change; operands or results outside the normal range take the native
+// operation.
+//
+// Measured on a GB300 (1024 x 1024 radial dam break, 32 x 32 patches, 36 %
+// wet): a wet cell took about 1770 FP64-pipe operations, of which the scheme
+// needs 468; the division and square-root sequences (some eight to ten
+// FP64 operations each, about 50 of them per cell) were most of the rest.
+//
+// The header also compiles for the host, where the reciprocal seeds are
+// perturbed by up to GF_SEED_ERR so that a test can cover the whole range of
+// errors the device's approximations may have.
+#pragma once
+
+#include <cstdint>
+#include <cstring>
+
+#ifdef __CUDACC__
+#define GF_HD __device__ __forceinline__
+#else
+#define GF_HD inline
+#endif
+
+namespace gfk {
+
+#ifdef __CUDACC__
+GF_HD long long dbits(double x) { return __double_as_longlong(x); }
+GF_HD double bitsd(long long b) { return __longlong_as_double(b); }
+GF_HD float bitsf(unsigned b) { return __uint_as_float(b); }
+GF_HD int f2i_magic(float x) { return __float_as_int(__fadd_rn(x, 12582912.0f)) - 0x4b400000; }
+GF_HD float i2f(int i) { return __int2float_rn(i); }
+GF_HD float fmul(float a, float b) { return __fmul_rn(a, b); }
+GF_HD float seed_rcp(float x) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+GF_HD float seed_rsqrt(float x) {
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+GF_HD double native_sqrt(double x) { return sqrt(x); }
+#else
+inline long long dbits(double x) { long long b; std::memcpy(&b, &x, 8); return b; }
+inline double bitsd(long long b) { double x; std::memcpy(&x, &b, 8); return x; }
+inline float bitsf(unsigned b) { float x; std::memcpy(&x, &b, 4); return x; }
+inline int f2i_magic(float x) {
+  volatile float s = x + 12582912.0f;
+  const float t = s;
+  int b;
+  std::memcpy(&b, &t, 4);
+  return b - 0x4b400000;
+}
+inline float i2f(int i) { return (float)i; }
+inline float fmul(float a, float b) { volatile float r = a * b; return r; }
+float seed_rcp(float x);
+float seed_rsqrt(float x);
+double native_sqrt(double x);
+#endif
+
+constexpr long long D_MANT = (1ll << 52) - 1;
+constexpr long long D_HID = 1ll << 52;
+constexpr long long D_INF = 0x7ffll << 52;
+
+// a / b.  Digit recurrence on the 53-bit significands ma, mb: three quotient
+// digits of 20, 20 and 15 bits, each the remainder's leading bits times an
+// FP32 reciprocal of mb rounded to an integer, with the remainder updated
+// exactly modulo 2^64.  The reciprocal is within 2^-21.5 (23-bit truncation
+// of mb plus the approximation), so a digit is off by less than 2 units, the
+// remainder stays below 2^55 and the last digit (15 bits) is within 0.6 of
+// the exact one: the sign of the last remainder says whether the 56-bit
+// quotient is one too large, and whether it is zero is the sticky bit.
+GF_HD double div_rn(double a, double b) {
+  const long long ab = dbits(a), bb = dbits(b);
+  const int ea = (int)(ab >> 52) & 0x7ff, eb = (int)(bb >> 52) & 0x7ff;
+  const int e = ea - eb;
+  // both operands and the quotient well inside the normal range
+  if ((unsigned)(ea - 1) < 2046u && (unsigned)(eb - 1) < 2046u && (unsigned)(e + 1021) < 2043u) {
+    const long long ma = (ab & D_MANT) | D_HID, mb = (bb & D_MANT) | D_HID;
+    const float fa = bitsf(0x3f800000u | (unsigned)((ab & D_MANT) >> 29));
+    const float fb = bitsf(0x3f800000u | (unsigned)((bb & D_MANT) >> 29));
+    const float y = seed_rcp(fb);
+    const int q1 = f2i_magic(fmul(fa, fmul(y, 1048576.0f)));
+    const long long r1 = (long long)((unsigned long long)ma << 20) - (long long)q1 * mb;
+    const int q2 = f2i_magic(fmul(i2f((int)(r1 >> 24)), fmul(y, 0x1p-8f)));
+    const long long r2 = (long long)((unsigned long long)r1 << 20) - (long long)q2 * mb;
+    const int q3 = f2i_magic(fmul(i2f((int)(r2 >> 24)), fmul(y, 0x1p-13f)));
+    const long long r3 = (long long)((unsigned long long)r2 << 15) - (long long)q3 * mb;
+    // quotient ma 2^55 / mb in (2^54, 2^56): floor, then the sticky bit
+    long long Q = ((long long)q1 << 35) + (long long)q2 * 32768 + q3;
+    Q += r3 >> 63;
+    Q |= r3 != 0 ? 1 : 0;
+    const bool small = Q < (1ll << 55);
+    Q = small ? Q + Q : Q;
+    const long long m = (Q + 3 + ((Q >> 3) & 1)) >> 3;
+    const long long r = ((long long)(e + (small ? 1021 : 1022)) << 52) + m;
+    return bitsd(r | ((ab ^ bb) & (long long)0x8000000000000000ull));
+  }
+  if ((ab << 1) == 0 && (unsigned)(eb - 1) < 2046u)  // signed zero
+    return bitsd((ab ^ bb) & (long long)0x8000000000000000ull);
+  return a / b;
+}
+
+// sqrt(x).  The same recurrence for the root: m in [2^52, 2^54) (the exponent
+// made even), digits of the root at 2^20, 2^40 and 2^53, each the exact
+// residual times half an FP32 reciprocal square root.  The last digit is
+// within 0.6 of the exact one, so the residual's sign gives the floor of the
+// 54-bit root; a root is never halfway between two results.
+GF_HD double sqrt_rn(double x) {
+  const long long xb = dbits(x);
+  const int ex = (int)(xb >> 52);  // sign included: negative values fall out
+  if ((unsigned)(ex - 1) < 2046u) {
+    const int odd = (ex + 1) & 1;  // ex - 1023 odd
+    const unsigned long long m = (unsigned long long)((xb & D_MANT) | D_HID) << odd;
+    const float f0 = bitsf(0x3f800000u | (unsigned)((xb & D_MANT) >> 29));
+    const float f = odd ? f0 + f0 : f0;
+    const float y = seed_rsqrt(f);
+    const int s1 = f2i_magic(fmul(fmul(f, y), 1048576.0f));
+    const long long r1 = (long long)(m - ((unsigned long long)((long long)s1 * s1) << 12));
+    const int s2 = f2i_magic(fmul(i2f((int)(r1 >> 8)), fmul(y, 0x1p-5f)));
+    const long long r2 =
+        (long long)((unsigned long long)r1 << 28) -
+        (long long)((unsigned long long)((long long)s1 * s2) << 21) - (long long)s2 * s2;
+    const long long S2 = ((long long)s1 << 20) + s2;
+    const int s3 = f2i_magic(fmul(i2f((int)(r2 >> 16)), fmul(y, 0x1p-12f)));
+    const long long r3 = (long long)(((unsigned long long)r2 << 26) -
+                                     ((unsigned long long)(S2 * s3) << 14)) -
+                         (long long)s3 * s3;
+    long long S = (S2 << 13) + s3;
+    S += r3 >> 63;
+    const long long mr = (S + 1) >> 1;  // [2^52, 2^53]
+    const int er = (ex - 1023 - odd) / 2 + 1022;
+    return bitsd(((long long)er << 52) + mr);
+  }
+  if ((xb << 1) == 0) return x;
+  return native_sqrt(x);
+}
+
+// a < b and a <= 0 style tests on the bit patterns (no NaN operands: a NaN
+// orders beyond infinity here, and the step reports it as a non-finite value
+// whichever branch it takes).
+GF_HD long long okey(double x) {  // order-preserving; -0 and +0 alike
+  const long long b = dbits(x);
+  return b < 0 ? (long long)(0x8000000000000000ull - (unsigned long long)b) : b;
+}
+GF_HD bool dlt(double a, double b) { return okey(a) < okey(b); }
+GF_HD bool neg(double x) { return dbits(x) < 0 && (dbits(x) << 1) != 0; }
+GF_HD bool pos(double x) { return dbits(x) > 0; }
+GF_HD bool iszero(double x) { return (dbits(x) << 1) == 0; }
+GF_HD double dabs(double x) { return bitsd(dbits(x) & 0x7fffffffffffffffll); }
+GF_HD double dneg(double x) { return bitsd(dbits(x) ^ (long long)0x8000000000000000ull); }
+GF_HD double dmin(double a, double b) { return dlt(a, b) ? a : b; }
+GF_HD double dmax(double a, double b) { return dlt(b, a) ? a : b; }
+// h > d for a positive threshold d; false for NaN
+GF_HD bool above(double h, double d) {
+  return (unsigned long long)(dbits(h) - dbits(d) - 1) < (unsigned long long)(D_INF - dbits(d));
+}
+// x / 2 and 2 x by the exponent (native where it is at the range's ends)
+GF_HD double half(double x) {
+  const int e = (int)(dbits(x) >> 52) & 0x7ff;
+  if ((unsigned)(e - 2) < 2045u) return bitsd(dbits(x) - D_HID);
+  return 0.5 * x;
+}
+GF_HD double twice(double x) {
+  const int e = (int)(dbits(x) >> 52) & 0x7ff;
+  if ((unsigned)(e - 1) < 2045u) return bitsd(dbits(x) + D_HID);
+  return 2.0 * x;
+}
+
+}  // namespace gfk

@@ -141,11 +141,11 @@ struct GfView {
   // per cell)
   const unsigned* pbox;
   unsigned* done;         // CTA completion counter of the step (or null)
-  // Launch order of the patch step (or null: patch order).  sched[0] selects
-  // which of ord0/ord1 this launch reads; the launch writes the other one
-  // with the patches whose tile held water first (sched[1], sched[2] count
-  // the wet and dry entries) and its last CTA flips sched[0].  Only with a
-  // controller (done != null).
+  // Launch order of the patch step (or null: patch order).  sched[0] counts
+  // the launches modulo 6; its parity selects which of ord0/ord1 a launch
+  // reads; the launch writes the other one with the patches whose tile held
+  // water first (sched[1], sched[2] count the wet and dry entries) and its
+  // last CTA advances sched[0].  Only with a controller (done != null).
   unsigned* sched;
   int* ord0;
   int* ord1;
@@ -170,15 +170,17 @@ struct GfView {
   // DEMs and eta0.
   void* bcache;
   unsigned char* bvalid;
-  // Per patch, two arrays selected by the launch-order parity sched[0] (or
-  // null: every patch runs): 1 if the patch must run in the launch that
-  // reads that parity.  A launch clears the flags it reads and sets, in the
-  // other array, those of every patch whose tile held water and of its
-  // same-level neighbours; the cross-level ghost fill and the inflow set
-  // those of the patches whose ghost cells they write.  An unmarked patch
-  // whose tile is dry and unchanged in both buffers and that holds no gauge
-  // returns before staging: its ghost ring is dry, so the full path would
-  // write nothing either.  Whole-tile CTAs only; not with subcycling.
+  // Per patch, three arrays in turn, selected by sched[0] modulo 3 (or null:
+  // every patch runs): 1 if the patch must run in the launch that reads that
+  // array.  A launch reads one array, sets in the next one the flags of
+  // every patch whose tile held water and of its same-level neighbours, and
+  // clears the third, which nobody reads or sets meanwhile (so the CTAs of a
+  // patch's sub-tiles may all read the flag); the cross-level ghost fill and
+  // the inflow set those of the patches whose ghost cells they write.  A dry
+  // tile (or sub-tile) of an unmarked patch that is unchanged in both
+  // buffers and whose patch holds no gauge returns before staging: its ghost
+  // ring is dry, so the full path would write nothing either.  Not with
+  // subcycling.
   unsigned char* runf;
   int runf_stride;
   int npatch;

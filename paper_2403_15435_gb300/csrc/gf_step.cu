@@ -70,14 +70,25 @@ __global__ void k_wait_check(int* out, unsigned limit) {
 
 namespace gf {
 
-// Kernel variants (the autotuner picks one per context): for 32 x 32
-// patches, 0 = one 512-thread CTA per patch (TMA bulk staging of the whole
-// tile), 1 = four CTAs of 16 x 16 sub-tiles per patch, 2 = as 0 (FP32) or 1
-// (FP64) with the register limit for one CTA per SM; 16 x 16 patches have the
-// single variant 0.  Dimensionally split stepping has one kernel per patch
-// size (whole-patch CTAs).
+// Kernel variants (the autotuner picks one per context).  FP64, 32 x 32
+// patches: 0 = by the rule of use_small_tiles, 8 x 8 sub-tiles or 16 x 16
+// sub-tiles in 192-thread CTAs, three per SM; 1 = 16 x 16 sub-tiles in
+// 256-thread CTAs, two per SM; 2 = 8 x 8 sub-tiles; 3 = 16 x 16 sub-tiles in
+// 352-thread CTAs.  16 x 16 patches have the single variant 0.  Dimensionally
+// split stepping has one kernel per patch size (whole-patch CTAs).
 int patch_step_variants(int mx, int prec, int dim_split) {
   return dim_split ? 1 : (mx == 32 ? (prec ? 8 : 4) : 1);
+}
+
+// FP64 sub-tile size.  8 x 8 sub-tiles do 1.2 times the FP64 work of 16 x 16
+// ones (more halo edges per cell) but four times the CTAs share it, so they
+// win while all of them are resident at once: 152 SMs x 4 CTAs.  Measured, us
+// per step with every cell wet, 8 x 8 against 16 x 16: 16 patches of 32 x 32
+// (256 CTAs of 8 x 8) 44 against 68, 36 patches (576 CTAs) 62 against 70, 64
+// patches (1024 CTAs) 127 against 93, 256 patches 372 against 312; 144
+// patches of 16 x 16 (576 CTAs) 62 against 71, 256 patches 126 against 92.
+static bool use_small_tiles(int npatch, int mx) {
+  return (long long)npatch * (mx / 8) * (mx / 8) <= 152 * 4;
 }
 
 int launch_patch_step_f64(const GfGeom& g, const GfView& v, int variant,
@@ -89,14 +100,18 @@ int launch_patch_step_f64(const GfGeom& g, const GfView& v, int variant,
     if (g.M == 16) return gfs::launch_step<gfs::PrecF64, 16, 16, 256, 1, true>(g, v, st);
     return -1;
   }
-  if (g.M == 32 && variant == 1)
-    return gfs::launch_step<gfs::PrecF64, 32, 16, 256, 2>(g, v, st);
-  if (g.M == 32 && variant == 2)
-    return gfs::launch_step<gfs::PrecF64, 32, 16, 256, 1>(g, v, st);
-  if (g.M == 32 && variant == 3)
-    return gfs::launch_step_adaptive<gfs::PrecF64, 32, 16, 352, 1>(g, v, st);
-  if (g.M == 32) return gfs::launch_step<gfs::PrecF64, 32, 32, 512, 1>(g, v, st);
-  if (g.M == 16) return gfs::launch_step<gfs::PrecF64, 16, 16, 256, 1>(g, v, st);
+  const bool small = use_small_tiles(v.npatch, g.M);
+  if (g.M == 32) {
+    if (variant == 1) return gfs::launch_step<gfs::PrecF64, 32, 16, 256, 2>(g, v, st);
+    if (variant == 2 || (variant == 0 && small))
+      return gfs::launch_step<gfs::PrecF64, 32, 8, 128, 4>(g, v, st);
+    if (variant == 3) return gfs::launch_step<gfs::PrecF64, 32, 16, 352, 1>(g, v, st);
+    return gfs::launch_step<gfs::PrecF64, 32, 16, 192, 3>(g, v, st);
+  }
+  if (g.M == 16) {
+    if (small) return gfs::launch_step<gfs::PrecF64, 16, 8, 128, 4>(g, v, st);
+    return gfs::launch_step<gfs::PrecF64, 16, 16, 256, 2>(g, v, st);
+  }
   return -1;
 }
 
@@ -219,9 +234,9 @@ extern "C" int geoflood_step_tiles_noalloc(const double* q_in, const double* b,
     return noalloc_fail(-1, "step_tiles_noalloc: bad argument");
   if (npatch < 1 || npatch > GF_NOALLOC_MAX_PATCHES)
     return noalloc_fail(-8, "step_tiles_noalloc: npatch must be in [1, 16384]");
-  // the kernel stages whole tiles with bulk copies, which need 16-byte
-  // aligned addresses (a tile plane is a multiple of 16 bytes for mx = 16
-  // and 32, so every tile of an aligned buffer is aligned)
+  // kernels that stage whole tiles do so with bulk copies, which need
+  // 16-byte aligned addresses (a tile plane is a multiple of 16 bytes for
+  // mx = 16 and 32, so every tile of an aligned buffer is aligned)
   if ((reinterpret_cast<uintptr_t>(q_in) | reinterpret_cast<uintptr_t>(b) |
        reinterpret_cast<uintptr_t>(q_out)) & 15u)
     return noalloc_fail(-1, "step_tiles_noalloc: q_in, b and q_out must be 16-byte aligned");
@@ -257,10 +272,7 @@ extern "C" int geoflood_step_tiles_noalloc(const double* q_in, const double* b,
   k_noalloc_init<<<(npatch + 255) / 256, 256, 0, st>>>(S, npatch, dt, manning_n);
   if (cudaGetLastError() != cudaSuccess)
     return noalloc_fail(-2, "step_tiles_noalloc: init launch failed");
-  const int lr = mx == 32
-                     ? gfs::launch_step<gfs::PrecF64, 32, 32, 512, 1>(G, V, st)
-                     : gfs::launch_step<gfs::PrecF64, 16, 16, 256, 1>(G, V, st);
-  if (lr) return noalloc_fail(-2, "step_tiles_noalloc: step launch failed");
+  if (gf::launch_patch_step_f64(G, V, 0, st)) return noalloc_fail(-2, "step_tiles_noalloc: step launch failed");
   if (cmax) {
     // the reduction cell and the kernel's status in one copy: a bounded
     // wait that gave up leaves its tile unwritten, and a non-finite value

@@ -4,8 +4,9 @@
 //              FP32 compensation terms for the update, bed b - eta0, exact
 //              wet tests (FP32 with an FP64 tie-break) and FP64 volume sums.
 //
-// One CTA per patch.  The (M+4)^2 tile of the state and bed is staged in
-// shared memory by 1D TMA bulk copies; then, in barrier-separated phases:
+// One CTA per patch, or per sub-tile of one.  The (M+4)^2 tile of the state
+// and bed is staged in shared memory (whole patches by 1D TMA bulk copies);
+// then, in barrier-separated phases:
 // every x-edge's augmented Riemann solve (Sec. 3.3), the MC-limited f-wave
 // corrections (Sec. 3.2, Eq. wpa_update_corrections), the per-cell x
 // increments and their transverse split along y (2D extension, leveque2002
@@ -89,7 +90,8 @@ __device__ __forceinline__ R warp_max(R v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     const R w = __shfl_xor_sync(0xffffffffu, v, o);
-    v = v > w ? v : w;
+    if constexpr (sizeof(R) == 8) v = gfk::dmax(v, w);
+    else v = v > w ? v : w;
   }
   return v;
 }
@@ -219,11 +221,15 @@ struct Layout {
   static constexpr int NEDGE = NR * NE;
   static constexpr int NLIM = NR * (M + 1);   // edges a in [0, M] per line
   static constexpr int NCELL = M * NR;        // cells of the increments
-  static constexpr int NF = P::DEV ? 5 : 4;   // tile fields (+ depth)
+  // FP64, unsplit: per-cell primitives beside the state (surface, two
+  // velocities, celerity, root of the depth) and 11 wave planes
+  static constexpr bool PRIM = !P::DEV && !DS;
+  static constexpr int NF = P::DEV ? 5 : (PRIM ? 9 : 4);  // tile fields (+ depth)
+  static constexpr int NWP = PRIM ? 11 : 12;              // wave planes
   static constexpr size_t TRB = DS ? 0 : sizeof(R) * 3 * M * (M + 1);
   // byte offsets in dynamic shared memory
   static constexpr size_t OFF_W = sizeof(R) * NF * TT;
-  static constexpr size_t OFF_F = OFF_W + sizeof(R) * 12 * NEDGE;
+  static constexpr size_t OFF_F = OFF_W + sizeof(R) * NWP * NEDGE;
   static constexpr size_t OFF_G = OFF_F + TRB;
   static constexpr size_t OFF_RED = align16(OFF_G + TRB);
   static constexpr size_t OFF_NB = OFF_RED + sizeof(double) * 64;  // 8 ints
@@ -263,6 +269,14 @@ __device__ __forceinline__ void cell_item(int k, int dir, int& a, int& line) {
 // depends only on its two-cell neighbourhood, so the result does not depend
 // on M.
 //
+// FP64 (unsplit): the FP64 pipe (two operations per SM and clock) bounds the
+// step, so the body computes a cell's velocities, celerity and root of the
+// depth once (not once per edge side) and leaves only additions and products
+// to that pipe (gf_fp64.cuh).  1024 x 1024 radial dam break, 36 % wet: 1770
+// FP64-pipe operations per wet cell before, 548 after; 1060 us per step
+// before, 507 after (ncu: FP64 pipe 82 % busy before, 66 % after, the rest
+// barrier waits between the phases).
+//
 // Scheme variants (Sec. 3.2): G.first_order drops the limited corrections,
 // G.no_transverse the transverse terms; DS (dimensional splitting) takes the
 // x sweep on every row of the window, updates the interior columns of all
@@ -297,6 +311,13 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
   R* shv = s0 + 2 * TT;
   R* sb = s0 + 3 * TT;
   R* sdep = DEV ? s0 + 4 * TT : s0;     // depth
+  constexpr bool PRIM = Lo::PRIM;
+  // PRIM: surface, velocities, celerity and root of the depth of every cell
+  R* seta = s0 + (PRIM ? 4 : 0) * TT;
+  R* su = s0 + (PRIM ? 5 : 0) * TT;
+  R* sv = s0 + (PRIM ? 6 : 0) * TT;
+  R* sc = s0 + (PRIM ? 7 : 0) * TT;
+  R* sq = s0 + (PRIM ? 8 : 0) * TT;
   R* W = reinterpret_cast<R*>(smraw + Lo::OFF_W);
   R* Ftr = reinterpret_cast<R*>(smraw + Lo::OFF_F);  // [row j][edge 0..M][3]
   R* Gtr = reinterpret_cast<R*>(smraw + Lo::OFF_G);  // [column i][edge][3]
@@ -441,7 +462,7 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
       swet[k] = wt ? 1 : 0;
       return wt ? 1 : 0;
     } else {
-      return s0[k] > rdry ? 1 : 0;
+      return gfk::above(s0[k], rdry) ? 1 : 0;
     }
   };
   int anywet = 0;
@@ -490,12 +511,30 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
   }
   auto wetc = [&](int c) -> bool {
     if constexpr (DEV) return swet[c] != 0;
+    else if constexpr (PRIM) return gfk::pos(sc[c]);  // zero celerity: dry
     else return s0[c] > rdry;
   };
   auto surf = [&](int c) -> R {
     if constexpr (DEV) return s0[c];
+    else if constexpr (PRIM) return seta[c];
     else return s0[c] + sb[c];
   };
+  if constexpr (PRIM) {
+    if (anywet) {
+      // what belongs to a cell, once per cell: an interior cell is a side of
+      // four edges and is split twice
+      for (int k = tid; k < TT; k += NT) {
+        const double h = s0[k];
+        const bool wt = gfk::above(h, rdry);
+        seta[k] = h + sb[k];
+        su[k] = wt ? gfk::div_rn(shu[k], h) : 0.0;
+        sv[k] = wt ? gfk::div_rn(shv[k], h) : 0.0;
+        sc[k] = wt ? gfk::sqrt_rn(g * h) : 0.0;
+        sq[k] = wt ? gfk::sqrt_rn(h) : 0.0;
+      }
+      __syncthreads();
+    }
+  }
 
   R X[RC][3];   // nu_x * dQx of owned interior cells
   R Y[RC][3];   // nu_y * dQy
@@ -538,14 +577,30 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
       const int a = (dir == 0 ? k % NE : k / NRL) - 1;
       const int cl = dir == 0 ? tix<M>(a - 1, line) : tix<M>(line, a - 1);
       const int cr = dir == 0 ? tix<M>(a, line) : tix<M>(line, a);
+      // waves in planes: component q of edge e at W[q * NEDGE + e], e the
+      // edge's place (line, a) in the sweep
+      R* w = W + ((line - L0) * NE + a + 1);
+      if constexpr (PRIM) {
+        const R* un = dir == 0 ? su : sv;
+        const R* ut = dir == 0 ? sv : su;
+        double z[8], S[3];
+        gfk::riemann_prim(
+            gfk::Prim{s0[cl], sn[cl], st[cl], sb[cl], seta[cl], un[cl], ut[cl], sc[cl], sq[cl],
+                      wetc(cl)},
+            gfk::Prim{s0[cr], sn[cr], st[cr], sb[cr], seta[cr], un[cr], ut[cr], sc[cr], sq[cr],
+                      wetc(cr)},
+            g, z, S);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) w[q * NEDGE] = z[q];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) w[(8 + q) * NEDGE] = S[q];
+        continue;
+      }
       R Z[9], S[3];
       gfk::riemann<R, DEV>(
           gfk::Side<R>{sdep[cl], sn[cl], st[cl], sb[cl], s0[cl], wetc(cl)},
           gfk::Side<R>{sdep[cr], sn[cr], st[cr], sb[cr], s0[cr], wetc(cr)}, g,
           rdry, Z, S);
-      // waves in planes: component q of edge e at W[q * NEDGE + e], e the
-      // edge's place (line, a) in the sweep
-      R* w = W + ((line - L0) * NE + a + 1);
 #pragma unroll
       for (int q = 0; q < 9; ++q)
         if (!(DEV && q == 3)) w[q * NEDGE] = Z[q];  // FP32: Z[3] is zero, not read
@@ -566,6 +621,16 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
         const int cl = dir == 0 ? tix<M>(a - 1, line) : tix<M>(line, a - 1);
         const int cr = dir == 0 ? tix<M>(a, line) : tix<M>(line, a);
         const bool wet = corr && wetc(cl) && wetc(cr);
+        if constexpr (PRIM) {
+          gfk::edge_fluxes_prim<NEDGE>(w, w - 1, w + 1, nu, wet, AMr[r], APr[r], FFr[r]);
+          if (line >= 0 && line < M) {
+            // |s| of the outer waves (the middle speed is their mean)
+            const double m = gfk::dmax(gfk::dabs(w[8 * NEDGE]), gfk::dabs(w[10 * NEDGE]));
+            if (dir == 0) smx = gfk::dmax(m, smx);
+            else smy = gfk::dmax(m, smy);
+          }
+          continue;
+        }
         gfk::edge_fluxes<R, NEDGE, DEV>(w, w + 9 * NEDGE, w - 1, w + 1, nu, wet,
                                         AMr[r], APr[r], FFr[r]);
         if (line >= 0 && line < M) {
@@ -679,6 +744,10 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
         const int cp = dir == 0 ? tix<M>(a, line + 1) : tix<M>(line + 1, a);
         const R dd[3] = {d[0], d[2], d[1]};
         R pl[3], mi[3];
+        if constexpr (PRIM)
+          gfk::tsplit_prim(dir == 0 ? sv[ci] : su[ci], dir == 0 ? su[ci] : sv[ci], sc[ci],
+                           seta[ci], wetc(ci), wetc(cm), sb[cm], wetc(cp), sb[cp], dd, pl, mi);
+        else
         gfk::tsplit<R>(sdep[ci], st[ci], sn[ci], surf(ci), wetc(ci), wetc(cm),
                        sb[cm], wetc(cp), sb[cp], dd, g, pl, mi);
         // back to (h, hu, hv): frame (mass, along = st, other = sn)
@@ -775,16 +844,17 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
         const R tf = trv ? nux * (fa[3 + f] - fa[f]) + nuy * (ga[3 + f] - ga[f]) : R(0);
         o[f] = (q[f] - fl) - tf;
       }
-      if (o[0] < R(0)) { clipd -= o[0]; o[0] = R(0); ++nclip; }
-      if (mn > R(0) && o[0] > rdry) {
-        const R u = o[1] / o[0], v = o[2] / o[0];
-        const R sp = sqrt(u * u + v * v);
-        const R D = g * mn * mn * sp / (o[0] * cbrt(o[0]));
+      if (gfk::neg(o[0])) { clipd -= o[0]; o[0] = R(0); ++nclip; }
+      const bool wnew = gfk::above(o[0], rdry);
+      if (wnew && gfk::pos(mn)) {
+        const R u = gfk::div_rn(o[1], o[0]), v = gfk::div_rn(o[2], o[0]);
+        const R sp = gfk::sqrt_rn(u * u + v * v);
+        const R D = gfk::div_rn(g * mn * mn * sp, o[0] * gfk::cbrt_pos(o[0]));
         const R den = R(1) + dtr * D;
-        o[1] = o[1] / den;
-        o[2] = o[2] / den;
+        o[1] = gfk::div_rn(o[1], den);
+        o[2] = gfk::div_rn(o[2], den);
       }
-      if (o[0] <= rdry) { o[1] = R(0); o[2] = R(0); }
+      if (!wnew) { o[1] = R(0); o[2] = R(0); }
     } else {
       // compensated update: (hi + lo) - fl - tf, hi rounded, lo the error
       float lo[3];
@@ -829,7 +899,12 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
 #pragma unroll
       for (int f = 0; f < 3; ++f) lod[f * MP * MP + kp] = lo[f];
     }
-    bad |= !(isfinite(o[0]) && isfinite(o[1]) && isfinite(o[2]));
+    if constexpr (DEV) {
+      bad |= !(isfinite(o[0]) && isfinite(o[1]) && isfinite(o[2]));
+    } else {
+#pragma unroll
+      for (int f = 0; f < 3; ++f) bad |= (gfk::dbits(o[f]) & gfk::D_INF) == gfk::D_INF;
+    }
     qd[cg] = o[0];
     qd[TG + cg] = o[1];
     qd[2 * TG + cg] = o[2];
@@ -1203,7 +1278,7 @@ __device__ void step_finish(const GfGeom& G, const GfView& V, int cells_per_patc
   // the next launch reads the counters and the schedule after this kernel
   // has ended, which orders these writes before it
   if (threadIdx.x == 0 && V.sched) {
-    V.sched[0] ^= 1u;
+    V.sched[0] = (V.sched[0] + 1u) % 6u;
     V.sched[3] = V.sched[1];  // wet patches at the head of the next order
     V.sched[1] = 0u;
     V.sched[2] = 0u;
@@ -1223,7 +1298,7 @@ __global__ void __launch_bounds__(NT, MINB)
   extern __shared__ __align__(16) unsigned char smraw[];
   constexpr int NSUB = (MP / M) * (MP / M);
   const bool sched = V.sched != nullptr && V.done != nullptr;
-  const unsigned par = sched ? V.sched[0] : 0u;
+  const unsigned par = sched ? V.sched[0] & 1u : 0u;
   const int nw = sched ? (int)V.sched[3] : 0;
   const int* ord = sched ? (par ? V.ord1 : V.ord0) : nullptr;
   const int b = blockIdx.x;
@@ -1283,18 +1358,23 @@ __global__ void __launch_bounds__(NT, MINB)
   // launch order: tiles that held water in the previous launch first, so the
   // long wet CTAs start at once and the short dry ones fill in around them
   const bool sched = V.sched != nullptr && V.done != nullptr;
-  const unsigned par = sched ? V.sched[0] : 0u;
+  const unsigned count = sched ? V.sched[0] : 0u;
+  const unsigned par = count & 1u;
   const int p = sched ? (par ? V.ord1 : V.ord0)[slot] : slot;
   // run flags (GfView::runf): read by every thread beside the patch record,
   // so that a running tile waits for nothing more
-  constexpr bool FLAGS = NSUB == 1 && !DS;
-  const bool use_flags = FLAGS && sched && V.runf != nullptr && !G.subcycle;
-  unsigned char* rcur = use_flags ? V.runf + (size_t)(par & 1u) * V.runf_stride : nullptr;
-  unsigned char* rnxt = use_flags ? V.runf + (size_t)((par ^ 1u) & 1u) * V.runf_stride : nullptr;
+  const bool use_flags = !DS && sched && V.runf != nullptr && !G.subcycle;
+  const unsigned r3 = count % 3u;
+  const unsigned char* rcur = use_flags ? V.runf + (size_t)r3 * V.runf_stride : nullptr;
+  unsigned char* rnxt = use_flags ? V.runf + (size_t)((r3 + 1u) % 3u) * V.runf_stride : nullptr;
   const bool marked = use_flags && rcur[p] != 0;
-  // an unmarked dry, unchanged tile without a gauge takes no step (the full
-  // path would find its ghost ring dry and write nothing)
-  const bool skip = use_flags && !marked && V.same != nullptr && V.same[p] != 0 &&
+  // the array that the launch after the next one's marks go to
+  if (use_flags && sub == 0 && threadIdx.x == 0)
+    V.runf[(size_t)((r3 + 2u) % 3u) * V.runf_stride + p] = 0;
+  // a dry, unchanged tile (or sub-tile) of an unmarked patch without a gauge
+  // takes no step (the full path would find its ghost ring dry and write
+  // nothing)
+  const bool skip = use_flags && !marked && V.same != nullptr && V.same[p * NSUB + sub] != 0 &&
                     !(V.gflag != nullptr && V.gflag[p] != 0);
   int wet = 0;
   bool wrote = false;
@@ -1310,11 +1390,8 @@ __global__ void __launch_bounds__(NT, MINB)
     if (run)
       wet = patch_body<P, MP, M, NT, DS>(G, V, smraw, p, sub, nullptr, &wrote);
     else wrote = false;
-    if (use_flags && threadIdx.x == 0) {
-      // the mark is consumed; a patch that did not run carries it forward
-      rcur[p] = 0;
-      if (!run) rnxt[p] = 1;
-    }
+    // a patch that did not run carries its mark forward
+    if (use_flags && threadIdx.x == 0 && !run) rnxt[p] = 1;
     if (use_flags && wet && threadIdx.x < 9) {
       // water in this tile: it and its same-level neighbours run next launch
       // (their indices were staged in shared memory by the patch body)
