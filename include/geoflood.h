@@ -352,14 +352,13 @@ int geoflood_counters(geoflood_ctx* ctx, int scenario, long long* cell_updates,
  * NULL).  Variants of 32 x 32 patches, FP64 (CTAs of sub-tiles with their
  * two-cell halo): 0 = 8 x 8 or, from 39 patches on, 16 x 16 sub-tiles (192
  * threads), 1 = 16 x 16 (256 threads), 2 = 8 x 8 (128 threads), 3 = 16 x 16
- * (352 threads).  FP32: 0 = one 512-thread CTA per patch staging the whole
- * tile by TMA bulk copies, 1 = four CTAs per patch, each staging a 16 x 16
- * sub-tile with its two-cell halo, 2 = the shape of 0 with the register
- * budget of one CTA per SM, 3 = one 1024-thread CTA per patch, 4 = the
- * sub-tiles of 1 with three 352-thread CTAs per SM, 5 = with four 320-thread
- * CTAs per SM, 6 = adaptive (four sub-tile CTAs for each patch that held
- * water in the previous step, one CTA that checks the whole tile for every
- * other patch), 7 = one 608-thread CTA per patch, two per SM.  Results do not depend on
+ * (352 threads).  FP32: 0 = by the forest's size 8 x 8 (up to 38 patches) or
+ * 16 x 16 (up to 152) sub-tiles or whole tiles staged by TMA bulk copies (320
+ * threads, two CTAs per SM), 1 = 16 x 16 sub-tiles (192 threads, four CTAs per
+ * SM), 2 = whole tiles (640 threads), 3 = whole tiles (320 threads, one CTA
+ * per SM), 4 = 16 x 16 sub-tiles (192 threads, three per SM), 5 = 8 x 8
+ * sub-tiles (96 threads), 6 = 16 x 16 sub-tiles (96 threads), 7 = whole tiles
+ * (384 threads, two per SM).  Results do not depend on
  * the variant. */
 int geoflood_autotune(geoflood_ctx* ctx, int reps, int* variant,
                       double* ms_per_variant);

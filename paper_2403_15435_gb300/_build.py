@@ -23,7 +23,8 @@ SOURCES = [
     # FP32 kernels: approximate single-precision division and square root
     # (a few ulp; the FP32 path is held to absolute tolerances, and a lake at
     # rest still gives exactly zero waves), denormals flushed to zero
-    ("gf_step32.cu", ["-prec-div=false", "-prec-sqrt=false", "-ftz=true"]),
+    ("gf_step32.cu", ["-fmad=false", "-prec-div=false", "-prec-sqrt=false", "-ftz=true"]),
+    ("gf_step32s.cu", ["-prec-div=false", "-prec-sqrt=false", "-ftz=true"]),
     ("gf_amr.cu", ["-fmad=false"]),
     ("gf_cnn.cu", []),
     ("gf_forest.cpp", []),

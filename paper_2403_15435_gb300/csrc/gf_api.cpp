@@ -89,10 +89,8 @@ struct geoflood_ctx {
   unsigned* d_sched = nullptr;        // launch-order parity and counters
   int* d_ord[2] = {nullptr, nullptr}; // launch orders of the patch step
   unsigned char* d_same = nullptr;    // per work unit: buffers agree
-  unsigned char* d_runf = nullptr;    // [3][cap] run flags (see GfView::runf)
+  unsigned char* d_runf = nullptr;    // [3][cap] run flags, then GfView::inactive
   unsigned char* d_gflag = nullptr;   // per patch: holds a gauge
-  unsigned* d_pwet = nullptr;         // adaptive variant: per-patch flags
-  unsigned* d_pcnt = nullptr;
   int* d_rlist = nullptr;   // regrid: new slots to compute
   int* d_rpairs = nullptr;  // regrid: (new, old) slots to copy
   int* d_glist[2] = {nullptr, nullptr};  // ghost regions next to a level change
@@ -188,6 +186,12 @@ int fail(geoflood_ctx* c, int code, const std::string& msg) {
     }                                                                     \
   } while (0)
 
+// Run flags of the patch step: three arrays, then the word GfView::inactive,
+// which one fill with ones ("every patch runs") sets above any patch count.
+size_t runf_bytes(const geoflood_ctx* c) {
+  return (((size_t)c->cap * 3 + 15) & ~size_t(15)) + 16;
+}
+
 GfView view(geoflood_ctx* c, int t, int bb) {
   GfView v{};
   v.patch = c->d_patch[t];
@@ -206,13 +210,12 @@ GfView view(geoflood_ctx* c, int t, int bb) {
   v.pbox = c->d_pbox[t];
   v.done = c->d_done;
   v.sched = c->d_sched;
+  v.inactive = reinterpret_cast<unsigned*>(c->d_runf + runf_bytes(c) - 16);
   v.ord0 = c->d_ord[0];
   v.ord1 = c->d_ord[1];
   v.same = c->d_same;
   v.push = 1;
-  v.pwet = c->d_pwet;
   v.gflag = c->d_gflag;
-  v.pcnt = c->d_pcnt;
   v.bcache = c->d_bcache;
   v.bvalid = c->d_bvalid;
   v.runf = c->d_runf;
@@ -463,10 +466,8 @@ int upload_tables(geoflood_ctx* ctx, int t,
                      cudaMemcpyDeviceToDevice, ctx->st));
   CK(cudaMemsetAsync(ctx->d_sched, 0, 8 * sizeof(unsigned), ctx->st));
   CK(cudaMemsetAsync(ctx->d_same, 0, (size_t)ctx->cap * kUnits, ctx->st));
-  CK(cudaMemsetAsync(ctx->d_runf, 1, (size_t)ctx->cap * 3, ctx->st));
-  CK(cudaMemsetAsync(ctx->d_pwet, 0, (size_t)ctx->cap * sizeof(unsigned), ctx->st));
+  CK(cudaMemsetAsync(ctx->d_runf, 1, runf_bytes(ctx), ctx->st));
   CK(cudaMemsetAsync(ctx->d_gflag, 0, (size_t)ctx->cap, ctx->st));
-  CK(cudaMemsetAsync(ctx->d_pcnt, 0, (size_t)ctx->cap * sizeof(unsigned), ctx->st));
   rc |= upload_put(ctx, ctx->d_patch[t], hp.data(), sizeof(GfPatch) * total);
   rc |= upload_put(ctx, ctx->d_lut[t], lut.data(), sizeof(int) * lut.size());
   rc |= upload_put(ctx, ctx->d_scen, ctx->h_scen.data(), sizeof(GfScenario) * ctx->nscen);
@@ -498,7 +499,7 @@ int check_errflag(geoflood_ctx* ctx) {
 int ghost_fill_all(geoflood_ctx* ctx) {
   gf::set_errflag(ctx->d_err);
   // ghost cells rewritten from scratch: every patch runs next
-  CK(cudaMemsetAsync(ctx->d_runf, 1, (size_t)ctx->cap * 3, ctx->st));
+  CK(cudaMemsetAsync(ctx->d_runf, 1, runf_bytes(ctx), ctx->st));
   ProfRec r;
   prof_begin(ctx, "ghost_fill", &r);
   CKL(gf::launch_ghost_fill(ctx->G, view(ctx), 0, ctx->st), "ghost_fill");
@@ -518,7 +519,7 @@ int ghost_fill_all(geoflood_ctx* ctx) {
 int forget_same(geoflood_ctx* ctx) {
   CK(cudaMemsetAsync(ctx->d_same, 0, (size_t)ctx->cap * kUnits, ctx->st));
   // every patch runs until the marks of two launches have built up again
-  CK(cudaMemsetAsync(ctx->d_runf, 1, (size_t)ctx->cap * 3, ctx->st));
+  CK(cudaMemsetAsync(ctx->d_runf, 1, runf_bytes(ctx), ctx->st));
   return 0;
 }
 
@@ -732,6 +733,7 @@ int geoflood_init_forest(const geoflood_config* cfg, void* stream,
   G.gf = (float)c.g;
   G.drytolf = (float)c.drytol;
   G.marginf = (float)(c.drytol * 0x1p-20);
+  G.negzero = -0.0f;
   G.tag_depthf = (float)c.tag_depth;
   G.tag_speedf = (float)c.tag_speed;
   G.tag_detaf = (float)c.tag_deta;
@@ -822,10 +824,8 @@ int geoflood_init_forest(const geoflood_config* cfg, void* stream,
   okk &= alloc((void**)&ctx->d_ord[0], cap * sizeof(int));
   okk &= alloc((void**)&ctx->d_ord[1], cap * sizeof(int));
   okk &= alloc((void**)&ctx->d_same, cap * kUnits);
-  okk &= alloc((void**)&ctx->d_runf, cap * 3);
-  okk &= alloc((void**)&ctx->d_pwet, cap * sizeof(unsigned));
+  okk &= alloc((void**)&ctx->d_runf, runf_bytes(ctx));
   okk &= alloc((void**)&ctx->d_gflag, cap);
-  okk &= alloc((void**)&ctx->d_pcnt, cap * sizeof(unsigned));
   okk &= alloc((void**)&ctx->d_rlist, cap * sizeof(int));
   okk &= alloc((void**)&ctx->d_rpairs, cap * 2 * sizeof(int));
   okk &= alloc((void**)&ctx->d_glist[0], cap * 8 * sizeof(int));
@@ -931,9 +931,7 @@ void geoflood_destroy(geoflood_ctx* ctx) {
   cudaFree(ctx->d_ord[1]);
   cudaFree(ctx->d_same);
   cudaFree(ctx->d_runf);
-  cudaFree(ctx->d_pwet);
   cudaFree(ctx->d_gflag);
-  cudaFree(ctx->d_pcnt);
   cudaFree(ctx->d_rlist);
   cudaFree(ctx->d_rpairs);
   cudaFree(ctx->d_glist[0]);

@@ -11,7 +11,7 @@
 #define GF_SPIN_LIMIT (1u << 22)  // bounded waits on TMA mbarriers
 
 // One patch: level, position on that level's patch grid, scenario.
-struct GfPatch {
+struct alignas(16) GfPatch {
   int level, px, py, scen;
 };
 
@@ -92,6 +92,7 @@ struct GfGeom {
   double dxl[GF_MAXLEV + 1], dyl[GF_MAXLEV + 1], areal[GF_MAXLEV + 1];
   float inv_dxf[GF_MAXLEV + 1], inv_dyf[GF_MAXLEV + 1];
   float gf, drytolf, marginf;
+  float negzero;  // -0.0f, unknown to the compiler (see mulr2)
   float tag_depthf, tag_speedf, tag_detaf;
   // criterion 2 (|hu| > tag_flux) and criterion 5 (flow grades)
   double tag_flux;
@@ -143,10 +144,14 @@ struct GfView {
   unsigned* done;         // CTA completion counter of the step (or null)
   // Launch order of the patch step (or null: patch order).  sched[0] counts
   // the launches modulo 6; its parity selects which of ord0/ord1 a launch
-  // reads; the launch writes the other one with the patches whose tile held
-  // water first (sched[1], sched[2] count the wet and dry entries) and its
-  // last CTA advances sched[0].  Only with a controller (done != null).
+  // reads; the launch writes the other one with the patches that took the
+  // step first (sched[1], sched[2] count those and the others), and its last
+  // CTA advances sched[0] and stores the number of the others in *inactive.
+  // (Without run flags: the patches whose tile held water first.)  A value
+  // of *inactive above npatch means that nothing is known yet: every patch
+  // then gets its own CTAs.  Only with a controller (done != null).
   unsigned* sched;
+  unsigned* inactive;
   int* ord0;
   int* ord1;
   // Per CTA work unit (patch * sub-tiles + sub-tile): 1 when both state
@@ -157,10 +162,6 @@ struct GfView {
   // interior into the ghost cells of its same-level neighbours in the next
   // buffer (so the separate ghost fill skips those regions); needs nbr.
   int push;
-  // adaptive variant: per patch, whether a sub-tile held water and how many
-  // of its CTAs have finished (both back to 0 after the patch is reported)
-  unsigned* pwet;
-  unsigned* pcnt;
   // per patch: 1 if a gauge samples in it (or null)
   unsigned char* gflag;
   // Bed tiles by position (or null): slot = the lookup-table index of
@@ -221,6 +222,7 @@ namespace gf {
 int patch_step_variants(int mx, int prec, int dim_split);
 int launch_patch_step_f64(const GfGeom& g, const GfView& v, int variant, void* stream);
 int launch_patch_step_f32(const GfGeom& g, const GfView& v, int variant, void* stream);
+int launch_patch_step_f32_split(const GfGeom& g, const GfView& v, void* stream);
 int launch_ctl_begin(GfCtl* ctl, int nscen, double t_target,
                      long long max_steps, const int* scen_mask, void* stream);
 int launch_ghost_fill(const GfGeom& g, const GfView& v, int only_active,

@@ -598,4 +598,384 @@ __device__ __forceinline__ bool wet_dev(float w, float b, double drytol,
   return wet_dev_tie(w, b, drytol);
 }
 
+// ------------------------------------------------------------------------
+// The FP32 step's own forms.  That kernel is bound by issue slots, so the
+// per-cell quantities come from shared memory (see the FP64 forms).  The unit
+// is compiled without contraction and every fused operation is written out,
+// so all kernel shapes round alike; the operations and the places where they
+// fuse are those the compiler chose for riemann / edge_fluxes / tsplit.
+
+__device__ __forceinline__ float rcpf(float x) { return seed_rcp(x); }
+
+// One side of an edge in the deviation form: stored surface and bed (minus
+// eta0), normal momentum, velocities and the root of the depth (u, v and q
+// are zero in a dry cell).
+struct Prim32 {
+  float w, b, n, u, v, q;
+};
+
+// Waves z[8] as in riemann_prim and the outer speeds s1, s3 (the middle one
+// is their mean): the general case.
+__device__ __forceinline__ void riemann32(Prim32 l, Prim32 r, float g, float (&z)[8],
+                                              float& s1, float& s3) {
+#pragma unroll
+  for (int k = 0; k < 8; ++k) z[k] = 0.0f;
+  s1 = s3 = 0.0f;
+  const bool wl = l.q > 0.0f, wr = r.q > 0.0f;
+  if (!wl && !wr) return;
+  float hl = l.w - l.b, hr = r.w - r.b;
+  int wall = 0;
+  if (wl != wr) {
+    const float el = hl, er = hr;
+    if (!wl) { hl = 0.0f; l.n = 0.0f; }
+    if (!wr) { hr = 0.0f; r.n = 0.0f; }
+    if (wl && r.b > l.w) {
+      const float c = sqrtf(g * hl), sw = fmaxf(c - l.u, c);
+      const float hm = hl + l.n * rcpf(sw);
+      if (r.b >= l.b + hm) {  // a wall: the mirrored state
+        wall = 1;
+        r = l;
+        r.n = -l.n;
+        r.u = -l.u;
+        hr = hl;
+      } else {  // overtopped: the step lowered to the surface
+        r.w = l.w + er;
+        r.b = l.w;
+      }
+    } else if (wr && l.b > r.w) {
+      const float c = sqrtf(g * hr), sw = fmaxf(r.u + c, c);
+      const float hm = hr - r.n * rcpf(sw);
+      if (l.b >= r.b + hm) {
+        wall = -1;
+        l = r;
+        l.n = -r.n;
+        l.u = -r.u;
+        hl = hr;
+      } else {
+        l.w = r.w + el;
+        l.b = r.w;
+      }
+    }
+  }
+  const float sg = sqrtf(g);
+  const float cl = sg * l.q, cr = sg * r.q;
+  const float ghb = g * (0.5f * (hl + hr));
+  if (l.q > 0.0f && r.q > 0.0f) {
+    const float uhat = fmaf(l.q, l.u, r.q * r.u) * rcpf(l.q + r.q);
+    const float chat = sqrtf(ghb);
+    s1 = fminf(l.u - cl, uhat - chat);
+    s3 = fmaxf(r.u + cr, uhat + chat);
+  } else if (l.q > 0.0f) {
+    s1 = l.u - cl;
+    s3 = l.u + 2.0f * cl;
+  } else {
+    s1 = r.u - 2.0f * cr;
+    s3 = r.u + cr;
+  }
+  const float dn = r.n - l.n;
+  const float deta = r.w - l.w;
+  const float den = s3 - s1, rden = rcpf(den);
+  const float hhll = (fmaf(s3, hr, -(s1 * hl)) - dn) * rden;
+  const float x = hhll * den;
+  float dhs = l.b - r.b;
+  bool clamped = false;
+  if (s1 < 0.0f && s3 > 0.0f) {
+    const float lo = x * rcpf(s1), hi = x * rcpf(s3);
+    if (dhs < lo) { dhs = lo; clamped = true; }
+    if (dhs > hi) { dhs = hi; clamped = true; }
+  } else if (s1 >= 0.0f) {
+    const float hi = s1 > 0.0f ? x * rcpf(s1) : dhs;
+    if (dhs > hi) { dhs = hi; clamped = true; }
+    if (dhs < -hl) { dhs = -hl; clamped = true; }
+  } else {
+    const float lo = s3 < 0.0f ? x * rcpf(s3) : dhs;
+    if (dhs < lo) { dhs = lo; clamped = true; }
+    if (dhs > hr) { dhs = hr; clamped = true; }
+  }
+  const float d1 = clamped ? (hr - hl) - dhs : deta;
+  const float d3 = fmaf(ghb, deta, fmaf(r.n, r.u, -(l.n * l.u)));
+  const float b1 = fmaf(s3, d1, -dn) * rden;
+  const float b3 = fmaf(-s1, d1, dn) * rden;
+  const float q1 = s1 * s1, q3 = s3 * s3;
+  z[0] = s1 * b1;
+  z[1] = q1 * b1;
+  z[2] = l.v * z[0];
+  z[5] = s3 * b3;
+  z[6] = q3 * b3;
+  z[7] = r.v * z[5];
+  z[3] = d3 - (z[1] + z[6]);
+  z[4] = fmaf(r.n, r.v, -(l.n * l.v)) - (z[2] + z[7]);
+  if (wall == 1) z[3] = z[4] = z[5] = z[6] = z[7] = 0.0f;
+  else if (wall == -1) z[0] = z[1] = z[2] = z[3] = z[4] = 0.0f;
+}
+
+// ---------------------------------------------------------------- pairs
+//
+// Two neighbouring edges (or cells) per thread: the additions, products and
+// fused products of both in one packed instruction (f32x2), which halves the
+// issue slots of the arithmetic, the index work and the shared-memory
+// instructions.  Each half rounds as the scalar instruction does.
+
+typedef unsigned long long f2;
+__device__ __forceinline__ f2 pk(float a, float b) {
+  f2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void upk(f2 v, float& a, float& b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ f2 pk1(float a) { return pk(a, a); }
+__device__ __forceinline__ f2 add2(f2 a, f2 b) {
+  f2 r;
+  asm("add.rn.ftz.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f2 mul2(f2 a, f2 b) {
+  f2 r;
+  asm("mul.rn.ftz.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
+  f2 r;
+  asm("fma.rn.ftz.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+// A product that is rounded on its own although it feeds an addition: the
+// assembler fuses mul2 and add2 (whatever their rounding modifiers), so it is
+// written as a fused product with an addend nz of negative zero that the
+// compiler does not know (GfGeom::negzero).
+__device__ __forceinline__ f2 mulr2(f2 a, f2 b, f2 nz) { return fma2(a, b, nz); }
+__device__ __forceinline__ f2 neg2(f2 a) { return a ^ 0x8000000080000000ull; }
+__device__ __forceinline__ f2 sub2(f2 a, f2 b) { return add2(a, neg2(b)); }
+__device__ __forceinline__ f2 rcp2(f2 a) {
+  float x, y;
+  upk(a, x, y);
+  return pk(seed_rcp(x), seed_rcp(y));
+}
+__device__ __forceinline__ f2 sqrt2(f2 a) {
+  float x, y;
+  upk(a, x, y);
+  return pk(sqrtf(x), sqrtf(y));
+}
+__device__ __forceinline__ f2 min2(f2 a, f2 b) {
+  float x, y, u, v;
+  upk(a, x, y);
+  upk(b, u, v);
+  return pk(fminf(x, u), fminf(y, v));
+}
+__device__ __forceinline__ f2 max2(f2 a, f2 b) {
+  float x, y, u, v;
+  upk(a, x, y);
+  upk(b, u, v);
+  return pk(fmaxf(x, u), fmaxf(y, v));
+}
+// per half: c ? a : b
+__device__ __forceinline__ f2 sel2(bool c0, bool c1, f2 a, f2 b) {
+  float x, y, u, v;
+  upk(a, x, y);
+  upk(b, u, v);
+  return pk(c0 ? x : u, c1 ? y : v);
+}
+__device__ __forceinline__ f2 ld2(const float* p) { return *reinterpret_cast<const f2*>(p); }
+__device__ __forceinline__ void st2(float* p, f2 v) { *reinterpret_cast<f2*>(p) = v; }
+
+struct Prim32x2 {
+  f2 w, b, n, u, v, q;
+};
+
+// The general solver for one half, outputs through a pointer (rare: an edge
+// touching a dry cell, or one whose stationary wave may be clamped).
+static __device__ __noinline__ void riemann32_one(Prim32 l, Prim32 r, float g, float* out) {
+  float z[8], s1, s3;
+  riemann32(l, r, g, z, s1, s3);
+#pragma unroll
+  for (int k = 0; k < 8; ++k) out[k] = z[k];
+  out[8] = s1;
+  out[9] = s3;
+}
+
+// Two edges between wet cells whose stationary waves are inside their bounds
+// (tested with a margin far above the rounding of the exact bounds); a half
+// that is not goes through riemann32.  sg = sqrt(g).
+__device__ __forceinline__ void riemann32x2(const Prim32x2& l, const Prim32x2& r, float g,
+                                            float sg, f2 nz, f2 (&z)[8], f2& s1, f2& s3) {
+  const f2 hl = sub2(l.w, l.b), hr = sub2(r.w, r.b);
+  const f2 cl = mulr2(pk1(sg), l.q, nz), cr = mulr2(pk1(sg), r.q, nz);
+  const f2 ghb = mul2(pk1(g), mul2(pk1(0.5f), add2(hl, hr)));
+  const f2 uhat = mulr2(fma2(l.q, l.u, mul2(r.q, r.u)), rcp2(add2(l.q, r.q)), nz);
+  const f2 chat = sqrt2(ghb);
+  s1 = min2(sub2(l.u, cl), sub2(uhat, chat));
+  s3 = max2(add2(r.u, cr), add2(uhat, chat));
+  const f2 dn = sub2(r.n, l.n), deta = sub2(r.w, l.w);
+  const f2 rden = rcp2(sub2(s3, s1));
+  const f2 ns1 = neg2(s1);
+  const f2 x = sub2(fma2(s3, hr, mul2(ns1, hl)), dn);
+  const f2 dhs = sub2(l.b, r.b), xm = mul2(pk1(0.9999f), x);
+  const f2 ok = min2(min2(min2(sub2(xm, mul2(dhs, s1)), sub2(xm, mul2(dhs, s3))), x),
+                     min2(min2(add2(dhs, hl), sub2(hr, dhs)), min2(l.q, r.q)));
+  const f2 d3 = fma2(ghb, deta, fma2(r.n, r.u, neg2(mul2(l.n, l.u))));
+  const f2 b1 = mul2(fma2(s3, deta, neg2(dn)), rden);
+  const f2 b3 = mul2(fma2(ns1, deta, dn), rden);
+  z[0] = mul2(s1, b1);
+  z[1] = mulr2(mul2(s1, s1), b1, nz);
+  z[2] = mulr2(l.v, z[0], nz);
+  z[5] = mul2(s3, b3);
+  z[6] = mulr2(mul2(s3, s3), b3, nz);
+  z[7] = mulr2(r.v, z[5], nz);
+  z[3] = sub2(d3, add2(z[1], z[6]));
+  z[4] = sub2(fma2(r.n, r.v, neg2(mul2(l.n, l.v))), add2(z[2], z[7]));
+  float ok0, ok1;
+  upk(ok, ok0, ok1);
+  if (!(ok0 > 0.0f && ok1 > 0.0f)) {
+#pragma unroll 1
+    for (int h = 0; h < 2; ++h) {
+      if ((h ? ok1 : ok0) > 0.0f) continue;
+      auto half = [&](f2 v) { return __uint_as_float((unsigned)(h ? v >> 32 : v)); };
+      float o[10];
+      riemann32_one(
+          Prim32{half(l.w), half(l.b), half(l.n), half(l.u), half(l.v), half(l.q)},
+          Prim32{half(r.w), half(r.b), half(r.n), half(r.u), half(r.v), half(r.q)}, g, o);
+      auto put = [&](f2& v, float a) {
+        const f2 b = __float_as_uint(a);
+        v = h ? ((v & 0xffffffffull) | (b << 32)) : ((v & ~0xffffffffull) | b);
+      };
+#pragma unroll
+      for (int k = 0; k < 8; ++k) put(z[k], o[k]);
+      put(s1, o[8]);
+      put(s3, o[9]);
+    }
+  }
+}
+
+// Limiter coefficients of one wave of two edges: hs = half the sign of the
+// speed (zero at zero speed), m = 1 - nu |s|.  The smallest normal number
+// keeps a vanishing wave's ratio finite.
+__device__ __forceinline__ f2 limit32x2(f2 num, f2 zz, f2 hs, f2 m, f2 nz) {
+  const f2 th = mulr2(num, rcp2(add2(zz, pk1(1.17549435e-38f))), nz);
+  const f2 a = mul2(pk1(0.5f), add2(pk1(1.0f), th));
+  const f2 phi = max2(min2(min2(a, pk1(2.0f)), add2(th, th)), pk1(0.0f));
+  return mul2(mul2(hs, m), phi);
+}
+
+// edge_fluxes for the edges at w and w + 1 (planes of pitch ST, SE the place
+// of the next edge of a line); wet0, wet1: both cells of the edge are wet.
+template <int ST, int SE>
+__device__ __forceinline__ void edge32x2(const float* w, float nu, bool wet0, bool wet1, f2 nz,
+                                         f2 (&am)[3], f2 (&ap)[3], f2 (&ff)[3]) {
+  f2 z[8];
+#pragma unroll
+  for (int c = 0; c < 8; ++c) z[c] = ld2(w + c * ST);
+  const f2 s1 = ld2(w + 8 * ST), s3 = ld2(w + 9 * ST);
+  const f2 s2 = mul2(pk1(0.5f), add2(s1, s3));
+  float a1, b1, a2, b2, a3, b3;
+  upk(s1, a1, b1);
+  upk(s2, a2, b2);
+  upk(s3, a3, b3);
+  f2 u[8];       // the upwind edges' waves
+  f2 h1, h2, h3;  // half the signs
+  if (fmaxf(a1, b1) < 0.0f && fminf(a3, b3) > 0.0f && a2 != 0.0f && b2 != 0.0f) {
+    // first wave leftwards, third rightwards, the middle one to one side
+    const bool n0 = a2 < 0.0f, n1 = b2 < 0.0f;
+    am[0] = z[0];
+    ap[0] = z[5];
+#pragma unroll
+    for (int k = 1; k < 3; ++k) {
+      const f2 x = add2(sel2(n0, n1, z[k], z[5 + k]), z[2 + k]);
+      am[k] = sel2(n0, n1, x, z[k]);
+      ap[k] = sel2(n0, n1, z[5 + k], x);
+    }
+    if constexpr (SE % 2 == 0) {
+#pragma unroll
+      for (int c = 0; c < 3; ++c) u[c] = ld2(w + c * ST + SE);
+#pragma unroll
+      for (int c = 5; c < 8; ++c) u[c] = ld2(w + c * ST - SE);
+    } else {
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        float lo, hi;
+        upk(z[c], lo, hi);
+        u[c] = pk(hi, w[c * ST + 2]);
+      }
+#pragma unroll
+      for (int c = 5; c < 8; ++c) {
+        float lo, hi;
+        upk(z[c], lo, hi);
+        u[c] = pk(w[c * ST - 1], lo);
+      }
+    }
+    h1 = pk1(-0.5f);
+    h3 = pk1(0.5f);
+    h2 = pk(n0 ? -0.5f : 0.5f, n1 ? -0.5f : 0.5f);
+  } else {
+    auto side = [](float s) { return s < 0.0f ? 1.0f : (s == 0.0f ? 0.5f : 0.0f); };
+    const f2 m1 = pk(side(a1), side(b1)), m2 = pk(side(a2), side(b2)), m3 = pk(side(a3), side(b3));
+    const f2 one = pk1(1.0f);
+    const f2 p1 = sub2(one, m1), p2 = sub2(one, m2), p3 = sub2(one, m3);
+    am[0] = add2(mul2(m1, z[0]), mul2(m3, z[5]));
+    ap[0] = add2(mul2(p1, z[0]), mul2(p3, z[5]));
+#pragma unroll
+    for (int k = 1; k < 3; ++k) {
+      am[k] = add2(add2(mul2(m1, z[k]), mul2(m3, z[5 + k])), mul2(m2, z[2 + k]));
+      ap[k] = add2(add2(mul2(p1, z[k]), mul2(p3, z[5 + k])), mul2(p2, z[2 + k]));
+    }
+    const int o10 = a1 > 0.0f ? -SE : SE, o11 = (b1 > 0.0f ? -SE : SE) + 1;
+    const int o30 = a3 > 0.0f ? -SE : SE, o31 = (b3 > 0.0f ? -SE : SE) + 1;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) u[c] = pk(w[c * ST + o10], w[c * ST + o11]);
+#pragma unroll
+    for (int c = 5; c < 8; ++c) u[c] = pk(w[c * ST + o30], w[c * ST + o31]);
+    auto hsign = [](float s) { return s > 0.0f ? 0.5f : (s < 0.0f ? -0.5f : 0.0f); };
+    h1 = pk(hsign(a1), hsign(b1));
+    h2 = pk(hsign(a2), hsign(b2));
+    h3 = pk(hsign(a3), hsign(b3));
+  }
+  const int o20 = a2 > 0.0f ? -SE : SE, o21 = (b2 > 0.0f ? -SE : SE) + 1;
+#pragma unroll
+  for (int c = 3; c < 5; ++c) u[c] = pk(w[c * ST + o20], w[c * ST + o21]);
+  const f2 one = pk1(1.0f), nn = pk1(-nu);
+  auto abs2 = [](f2 v) { return v & 0x7fffffff7fffffffull; };
+  f2 k1 = limit32x2(fma2(u[2], z[2], fma2(u[0], z[0], mul2(u[1], z[1]))),
+                    fma2(z[2], z[2], fma2(z[0], z[0], mul2(z[1], z[1]))), h1,
+                    fma2(nn, abs2(s1), one), nz);
+  f2 k2 = limit32x2(fma2(u[3], z[3], mul2(u[4], z[4])), fma2(z[3], z[3], mul2(z[4], z[4])), h2,
+                    fma2(nn, abs2(s2), one), nz);
+  f2 k3 = limit32x2(fma2(u[7], z[7], fma2(u[5], z[5], mul2(u[6], z[6]))),
+                    fma2(z[7], z[7], fma2(z[5], z[5], mul2(z[6], z[6]))), h3,
+                    fma2(nn, abs2(s3), one), nz);
+  if (!(wet0 && wet1)) {
+    k1 = sel2(wet0, wet1, k1, 0ull);
+    k2 = sel2(wet0, wet1, k2, 0ull);
+    k3 = sel2(wet0, wet1, k3, 0ull);
+  }
+  ff[0] = add2(mulr2(k1, z[0], nz), mulr2(k3, z[5], nz));
+  ff[1] = add2(add2(mulr2(k1, z[1], nz), mulr2(k3, z[6], nz)), mulr2(k2, z[3], nz));
+  ff[2] = add2(add2(mulr2(k1, z[2], nz), mulr2(k3, z[7], nz)), mulr2(k2, z[4], nz));
+}
+
+// tsplit of two cells' increments d = (mass, along, other); w, z: velocities
+// along the split direction and across it, h: depths.  A dry half's result
+// is not used.
+__device__ __forceinline__ void tsplit32x2(f2 w, f2 z, f2 h, float g, f2 nz, const f2 (&d)[3],
+                                           f2 (&plus)[3], f2 (&minus)[3]) {
+  const f2 c = sqrt2(mul2(pk1(g), h));
+  const f2 l1 = sub2(w, c), l3 = add2(w, c), r2c = rcp2(add2(c, c));
+  const f2 c1 = mul2(l1, mul2(fma2(l3, d[0], neg2(d[1])), r2c));
+  const f2 c3 = mul2(l3, mul2(fma2(neg2(l1), d[0], d[1]), r2c));
+  const f2 c2 = mul2(w, fma2(neg2(z), d[0], d[2]));
+  float l1a, l1b, l3a, l3b, wa, wb;
+  upk(l1, l1a, l1b);
+  upk(l3, l3a, l3b);
+  upk(w, wa, wb);
+  const f2 p1 = sel2(l1a > 0.0f, l1b > 0.0f, c1, 0ull), q1 = sel2(l1a < 0.0f, l1b < 0.0f, c1, 0ull);
+  const f2 p3 = sel2(l3a > 0.0f, l3b > 0.0f, c3, 0ull), q3 = sel2(l3a < 0.0f, l3b < 0.0f, c3, 0ull);
+  const f2 p2 = sel2(wa > 0.0f, wb > 0.0f, c2, 0ull), q2 = sel2(wa < 0.0f, wb < 0.0f, c2, 0ull);
+  plus[0] = add2(p1, p3);
+  plus[1] = add2(mulr2(p1, l1, nz), mulr2(p3, l3, nz));
+  plus[2] = add2(add2(mulr2(p1, z, nz), mulr2(p3, z, nz)), p2);
+  minus[0] = add2(q1, q3);
+  minus[1] = add2(mulr2(q1, l1, nz), mulr2(q3, l3, nz));
+  minus[2] = add2(add2(mulr2(q1, z, nz), mulr2(q3, z, nz)), q2);
+}
+
 }  // namespace gfk

@@ -1,6 +1,7 @@
-// FP32 surface-deviation patch step (instantiation of gf_step_kernel.cuh).
-// Compiled with fused multiply-add allowed: this path is checked against the
-// FP64 oracle with absolute depth and momentum tolerances, not bit for bit.
+// FP32 surface-deviation patch step, unsplit (instantiation of
+// gf_step_kernel.cuh).  Compiled without contraction: the fused operations of
+// this path are written out, so that every kernel shape rounds alike.  It is
+// checked against the FP64 oracle with absolute depth and momentum tolerances.
 #include <cuda_runtime.h>
 
 #include "gf_internal.h"
@@ -8,37 +9,41 @@
 
 namespace gf {
 
+// Shapes (variants of 32 x 32 patches): 0 = by the rule below; whole tiles
+// with 3 = 320 threads, one CTA per SM, 7 = 384 threads, two, 2 = 640
+// threads, one; 16 x 16 sub-tiles with 1 = 192 threads, four CTAs per SM, 4 =
+// three, 6 = 96 threads, six; 5 = 8 x 8 sub-tiles with 96 threads.
+//
+// The rule for variant 0: whole tiles with 320 threads, two CTAs per SM (115
+// KB of shared memory each), except where the sub-tiles of all patches are
+// resident at once (152 SMs x 4 CTAs): a tile's chain of barriers, not the
+// arithmetic, is then the launch's time, and smaller tiles have shorter ones.
+// Measured, us per step of a third-wet grid, whole / 16 x 16 / 8 x 8: 16
+// patches 23.8 / 17.7 / 16.4, 36 patches 25.1 / 17.8 / 17.0, 64 patches 23.9 /
+// 17.9 / 17.7, 144 patches 24.8 / 20.8 / 23.8, 256 patches 26.0 / 25.0 / 34.0
+// (every cell wet: 24.7 / 31.7 / 48.5), 1024 patches 45.9 / 54.6 / 87.2.
 int launch_patch_step_f32(const GfGeom& g, const GfView& v, int variant,
                           void* stream) {
   if (v.npatch <= 0) return 0;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  if (g.dim_split) {
-    if (g.M == 32) return gfs::launch_step<gfs::PrecF32, 32, 32, 512, 2, true>(g, v, st);
-    if (g.M == 16) return gfs::launch_step<gfs::PrecF32, 16, 16, 352, 2, true>(g, v, st);
-    return -1;
+  if (g.dim_split) return launch_patch_step_f32_split(g, v, stream);
+  if (g.M == 32) {
+    // sub-tiles for small forests: see the rule above
+    const int shape = variant != 0 ? variant
+                      : v.npatch * 16 <= 152 * 4 ? 5
+                      : v.npatch * 4 <= 152 * 4 ? 1 : 0;
+    switch (shape) {
+      case 1: return gfs::launch_step<gfs::PrecF32, 32, 16, 192, 4>(g, v, st);
+      case 2: return gfs::launch_step<gfs::PrecF32, 32, 32, 640, 1>(g, v, st);
+      case 3: return gfs::launch_step<gfs::PrecF32, 32, 32, 320, 1>(g, v, st);
+      case 4: return gfs::launch_step<gfs::PrecF32, 32, 16, 192, 3>(g, v, st);
+      case 5: return gfs::launch_step<gfs::PrecF32, 32, 8, 96, 8>(g, v, st);
+      case 6: return gfs::launch_step<gfs::PrecF32, 32, 16, 96, 6>(g, v, st);
+      case 7: return gfs::launch_step<gfs::PrecF32, 32, 32, 384, 2>(g, v, st);
+      default: return gfs::launch_step<gfs::PrecF32, 32, 32, 320, 2>(g, v, st);
+    }
   }
-  if (g.M == 32 && variant == 1)
-    return gfs::launch_step<gfs::PrecF32, 32, 16, 352, 2>(g, v, st);
-  if (g.M == 32 && variant == 2)
-    return gfs::launch_step<gfs::PrecF32, 32, 32, 512, 1>(g, v, st);
-  if (g.M == 32 && variant == 3)
-    return gfs::launch_step<gfs::PrecF32, 32, 32, 1024, 1>(g, v, st);
-  // 16 x 16 sub-tiles with more CTAs per SM: 352 threads, three CTAs (one
-  // round per sweep phase, 56 registers); 320 threads, four CTAs
-  if (g.M == 32 && variant == 4)
-    return gfs::launch_step<gfs::PrecF32, 32, 16, 352, 3>(g, v, st);
-  if (g.M == 32 && variant == 5)
-    return gfs::launch_step<gfs::PrecF32, 32, 16, 320, 4>(g, v, st);
-  // adaptive: four 16 x 16 sub-tile CTAs for each patch wet in the previous
-  // launch, one whole-tile check (and dry update) for every other patch
-  if (g.M == 32 && variant == 6)
-    return gfs::launch_step_adaptive<gfs::PrecF32, 32, 16, 352, 1>(g, v, st);
-  // 608 threads, two CTAs per SM: every sweep phase in two rounds instead of
-  // three (48 registers, a few bytes spilled)
-  if (g.M == 32 && variant == 7)
-    return gfs::launch_step<gfs::PrecF32, 32, 32, 608, 2>(g, v, st);
-  if (g.M == 32) return gfs::launch_step<gfs::PrecF32, 32, 32, 512, 2>(g, v, st);
-  if (g.M == 16) return gfs::launch_step<gfs::PrecF32, 16, 16, 352, 2>(g, v, st);
+  if (g.M == 16) return gfs::launch_step<gfs::PrecF32, 16, 16, 192, 4>(g, v, st);
   return -1;
 }
 

@@ -61,6 +61,11 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src,
       : "memory");
 }
 
+// Ask for `bytes` (a multiple of 16) at a 16-byte aligned address in L2.
+__device__ __forceinline__ void bulk_prefetch(const void* src, unsigned bytes) {
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
+}
+
 // Bounded wait for the completion of the barrier's phase with the given
 // parity; returns false on timeout.
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, unsigned limit,
@@ -79,10 +84,20 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, unsigned limit,
 }
 
 // Phases of the two staging barriers of a CTA that stages one tile after
-// another (persistent variant): the parity each barrier completes next.
+// another: the parity each barrier completes next.
 struct TmaPhase {
   unsigned b0, b1;
   bool init;
+};
+
+// What a tile's chain of loads starts from, read by the kernel in as few
+// round trips as possible.
+struct TileHdr {
+  GfPatch Pt;
+  int cur, accepted;
+  double dt;      // dt_use
+  bool same_in;   // both buffers hold the same dry interior
+  bool has_gauge;
 };
 
 template <typename R>
@@ -101,6 +116,11 @@ __device__ __forceinline__ double warp_sum_tree(double v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
   return v;
 }
+
+// Patches that took no step in the previous launch share a CTA in groups of
+// this many.  Valley of 10496 patches, 5480 of them dry: their CTAs, two to an
+// SM because of the wet tiles' shared memory, were 43 of a launch's 358 us.
+#define GF_STEP_GROUP 16
 
 constexpr size_t align16(size_t x) { return (x + 15) & ~size_t(15); }
 
@@ -218,15 +238,21 @@ struct Layout {
   // most lines in one sweep: one ghost line each side (unsplit) or two
   static constexpr int NR = DS ? M + 4 : M + 2;
   static constexpr int NE = M + 3;  // edges per line, a in [-1, M+1]
-  static constexpr int NEDGE = NR * NE;
+  // places of a wave plane.  FP32, unsplit: rows of pitch M + 4, so that
+  // pairs of edges are 8-byte aligned
+  static constexpr bool FAST = P::DEV && !DS;
+  static constexpr int NEDGE = FAST ? (M + 3) * (M + 4) : NR * NE;
   static constexpr int NLIM = NR * (M + 1);   // edges a in [0, M] per line
   static constexpr int NCELL = M * NR;        // cells of the increments
   // FP64, unsplit: per-cell primitives beside the state (surface, two
   // velocities, celerity, root of the depth) and 11 wave planes
   static constexpr bool PRIM = !P::DEV && !DS;
-  static constexpr int NF = P::DEV ? 5 : (PRIM ? 9 : 4);  // tile fields (+ depth)
-  static constexpr int NWP = PRIM ? 11 : 12;              // wave planes
-  static constexpr size_t TRB = DS ? 0 : sizeof(R) * 3 * M * (M + 1);
+  // FP32, unsplit: velocities and root of the depth beside the state, 10
+  // wave planes, 6 planes of transverse parts
+  static constexpr int NF = FAST ? 7 : (P::DEV ? 5 : (PRIM ? 9 : 4));  // tile fields
+  static constexpr int NWP = FAST ? 10 : (PRIM ? 11 : 12);             // wave planes
+  static constexpr size_t TRB =
+      DS ? 0 : (FAST ? sizeof(R) * 3 * M * (M + 4) : sizeof(R) * 3 * M * (M + 1));
   // byte offsets in dynamic shared memory
   static constexpr size_t OFF_W = sizeof(R) * NF * TT;
   static constexpr size_t OFF_F = OFF_W + sizeof(R) * NWP * NEDGE;
@@ -234,7 +260,7 @@ struct Layout {
   static constexpr size_t OFF_RED = align16(OFF_G + TRB);
   static constexpr size_t OFF_NB = OFF_RED + sizeof(double) * 64;  // 8 ints
   static constexpr size_t OFF_WET = OFF_NB + 32;
-  static constexpr size_t OFF_BAR = align16(OFF_WET + (P::DEV ? TT : 0));
+  static constexpr size_t OFF_BAR = align16(OFF_WET + (P::DEV && DS ? TT : 16));
   static constexpr size_t BYTES = OFF_BAR + 16;
 };
 
@@ -277,6 +303,17 @@ __device__ __forceinline__ void cell_item(int k, int dir, int& a, int& line) {
 // before, 507 after (ncu: FP64 pipe 82 % busy before, 66 % after, the rest
 // barrier waits between the phases).
 //
+// FP32 (unsplit): bound by issue slots and by the tile's chain of barriers
+// (115 KB of shared memory allow two whole tiles per SM).  A thread takes two
+// neighbouring edges or cells: packed instructions for their arithmetic, one
+// index and one 8-byte shared-memory access for both; the cell's velocities
+// and root of the depth are computed once per cell while its state is looked
+// at; the six transverse parts of a cell are written once and read by its
+// neighbours; the copies of the edge cells follow the update side by side.
+// 4 km x 2 km valley, 10496 patches, 5012 of them with water: 269 M -> 191 M
+// warp instructions, 393 -> 312 us per launch; 17 km x 9 km canyon of 19350 16
+// x 16 patches, 1837 with water: 182 -> 75 us.  Results keep every bit.
+//
 // Scheme variants (Sec. 3.2): G.first_order drops the limited corrections,
 // G.no_transverse the transverse terms; DS (dimensional splitting) takes the
 // x sweep on every row of the window, updates the interior columns of all
@@ -285,8 +322,8 @@ __device__ __forceinline__ void cell_item(int k, int dir, int& a, int& line) {
 template <class P, int MP, int M, int NT, bool DS = false>
 __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
                                           unsigned char* smraw, const int p,
-                                          const int sub, TmaPhase* tp = nullptr,
-                                          bool* wrote = nullptr) {
+                                          const int sub, const TileHdr& H, TmaPhase* tp,
+                                          bool* wrote) {
   using R = typename P::R;
   constexpr bool DEV = P::DEV;
   using Lo = Layout<P, M, DS>;
@@ -294,13 +331,20 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
   constexpr int TGW = MP + 2 * GF_NG, TG = TGW * TGW;  // patch tile
   constexpr int NS1 = MP / M, NSUB = NS1 * NS1;
   constexpr int RL = (Lo::NLIM + NT - 1) / NT;    // limiter items per thread
-  constexpr int RC = (M * M + NT - 1) / NT;       // interior cells per thread
+  // FAST: a thread's cells are pairs: columns 2 (tid % (M / 2)) and the next
+  // of rows tid / (M / 2), + TLC, ..., in both sweeps and the update; rows M
+  // and M + 1 stand for the ghost rows -1 and M, so that their pairs fill
+  // warps of their own
+  constexpr bool FAST = Lo::FAST;
+  constexpr int M2 = M / 2, TLC = NT / M2;
+  static_assert(!FAST || NT % M2 == 0, "whole rows of pairs per round");
+  constexpr int RC = FAST ? (M + 2 + TLC - 1) / TLC : (M * M + NT - 1) / NT;  // cells per thread
   constexpr int RX = (Lo::NCELL + NT - 1) / NT;   // increment cells per thread
 
   const int unit = p * NSUB + sub;  // CTA work unit: volume slot, same[] flag
-  const bool has_gauge = V.gflag != nullptr && V.gflag[p] != 0;
+  const bool has_gauge = H.has_gauge;
   const int ox = (sub % NS1) * M, oy = (sub / NS1) * M;
-  const GfPatch Pt = V.patch[p];
+  const GfPatch Pt = H.Pt;
   GfCtl* C = V.ctl + Pt.scen;
   // global tile index of local cell (i, j), and interior index in the patch
   auto gix = [&](int i, int j) { return (ox + i + GF_NG) + (oy + j + GF_NG) * TGW; };
@@ -310,14 +354,14 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
   R* shu = s0 + TT;
   R* shv = s0 + 2 * TT;
   R* sb = s0 + 3 * TT;
-  R* sdep = DEV ? s0 + 4 * TT : s0;     // depth
+  R* sdep = DEV && DS ? s0 + 4 * TT : s0;  // depth
   constexpr bool PRIM = Lo::PRIM;
   // PRIM: surface, velocities, celerity and root of the depth of every cell
   R* seta = s0 + (PRIM ? 4 : 0) * TT;
-  R* su = s0 + (PRIM ? 5 : 0) * TT;
-  R* sv = s0 + (PRIM ? 6 : 0) * TT;
+  R* su = s0 + (PRIM ? 5 : (FAST ? 4 : 0)) * TT;
+  R* sv = s0 + (PRIM ? 6 : (FAST ? 5 : 0)) * TT;
   R* sc = s0 + (PRIM ? 7 : 0) * TT;
-  R* sq = s0 + (PRIM ? 8 : 0) * TT;
+  R* sq = s0 + (PRIM ? 8 : (FAST ? 6 : 0)) * TT;
   R* W = reinterpret_cast<R*>(smraw + Lo::OFF_W);
   R* Ftr = reinterpret_cast<R*>(smraw + Lo::OFF_F);  // [row j][edge 0..M][3]
   R* Gtr = reinterpret_cast<R*>(smraw + Lo::OFF_G);  // [column i][edge][3]
@@ -325,6 +369,8 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
   unsigned char* swet = smraw + Lo::OFF_WET;
   int* snb = reinterpret_cast<int*>(smraw + Lo::OFF_NB);  // same-level neighbours
   uint64_t* bar = reinterpret_cast<uint64_t*>(smraw + Lo::OFF_BAR);
+  // FAST: set by a thread whose bounded wait gave up
+  volatile int* sflag = reinterpret_cast<volatile int*>(smraw + Lo::OFF_WET);
 
   const int tid = threadIdx.x;
   // level subcycling: this level's period in fine substeps, its buffer
@@ -332,8 +378,8 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
   // step (the macro step's share for the level)
   const bool subc = G.subcycle != 0;
   const int per = subc ? 1 << (G.maxlevel - Pt.level) : 1;
-  const int cur = subc ? C->cur ^ ((C->sub_k / per) & 1) : C->cur;
-  const double dtp = subc ? (C->dt_use / (double)G.sub_K) * (double)per : C->dt_use;
+  const int cur = subc ? H.cur ^ ((C->sub_k / per) & 1) : H.cur;
+  const double dtp = subc ? (H.dt / (double)G.sub_K) * (double)per : H.dt;
   const R* qs;
   R* qd;
   const R* bs;
@@ -350,7 +396,7 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
   // A tile whose interior is the same in both buffers (it was dry and copied)
   // needs only its surface and bed to find out whether it is still dry; its
   // momenta are fetched only if water has arrived.
-  const bool same_in = V.same != nullptr && V.same[unit] != 0;
+  const bool same_in = H.same_in;
   bool mom_issued = false;
   // staging barrier phases (a CTA that stages several tiles keeps them in tp)
   const bool fresh = tp == nullptr || !tp->init;
@@ -363,6 +409,7 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
         mbar_init(bar, 1);
         mbar_init(bar + 1, 1);
       }
+      if constexpr (FAST) *sflag = 0;
       mbar_expect_tx(bar, 2u * TT * sizeof(R));
       bulk_g2s(s0, qs, TT * sizeof(R), bar);
       bulk_g2s(sb, bs, TT * sizeof(R), bar);
@@ -370,23 +417,45 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
         mbar_expect_tx(bar + 1, 2u * TT * sizeof(R));
         bulk_g2s(shu, qs + TT, TT * sizeof(R), bar + 1);
         bulk_g2s(shv, qs + 2 * TT, TT * sizeof(R), bar + 1);
+        if constexpr (FAST)  // the update's compensation terms, towards L2
+          bulk_prefetch(V.lof[cur] + (size_t)p * 3 * MP * MP, 3u * MP * MP * sizeof(float));
       }
     }
     mom_issued = !same_in;
     if (tp) tp->init = true;
-    __syncthreads();
     // every wait is bounded; the decision to give up is taken by the whole CTA
-    if (!__syncthreads_and(mbar_wait(bar, GF_SPIN_LIMIT, ph0) ? 1 : 0)) {
-      if (tid == 0) C->status = -7;  // GEOFLOOD_ERR_TIMEOUT
-      mbar_wait(bar, GF_SPIN_LIMIT, ph0);
-      if (mom_issued) mbar_wait(bar + 1, GF_SPIN_LIMIT, ph1);
+    // (FAST: the first wait comes after the scalars below)
+    if constexpr (!FAST) {
       __syncthreads();
-      return -1;
+      if (!__syncthreads_and(mbar_wait(bar, GF_SPIN_LIMIT, ph0) ? 1 : 0)) {
+        if (tid == 0) C->status = -7;  // GEOFLOOD_ERR_TIMEOUT
+        mbar_wait(bar, GF_SPIN_LIMIT, ph0);
+        if (mom_issued) mbar_wait(bar + 1, GF_SPIN_LIMIT, ph1);
+        __syncthreads();
+        return -1;
+      }
+      if (tp) tp->b0 ^= 1u;
     }
-    if (tp) tp->b0 ^= 1u;
   } else {
     // sub-tile: the (M+4)^2 window of each field, row segments read with
     // consecutive threads on consecutive addresses
+    if constexpr (FAST) {
+      // 16-byte pieces (tile rows and sub-tile origins are multiples of 16 B)
+      constexpr int Q = Lo::T / 4;
+      for (int k = tid; k < Q * Lo::T; k += NT) {
+        const int li = 4 * (k % Q), lj = k / Q;
+        const int g = (ox + li) + (oy + lj) * TGW, c = li + lj * Lo::T;
+        const float4 a0 = *reinterpret_cast<const float4*>(qs + g);
+        const float4 a1 = *reinterpret_cast<const float4*>(qs + TG + g);
+        const float4 a2 = *reinterpret_cast<const float4*>(qs + 2 * TG + g);
+        const float4 a3 = *reinterpret_cast<const float4*>(bs + g);
+        *reinterpret_cast<float4*>(s0 + c) = a0;
+        *reinterpret_cast<float4*>(shu + c) = a1;
+        *reinterpret_cast<float4*>(shv + c) = a2;
+        *reinterpret_cast<float4*>(sb + c) = a3;
+      }
+      if (tid == 0) *sflag = 0;
+    } else
     for (int k = tid; k < TT; k += NT) {
       const int li = k % Lo::T, lj = k / Lo::T;
       const int g = (ox + li) + (oy + lj) * TGW;
@@ -457,15 +526,81 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
   auto examine = [&](int k) -> int {
     if constexpr (DEV) {
       const float w = s0[k], b = sb[k];
-      sdep[k] = w - b;
       const bool wt = gfk::wet_dev(w, b, drytol, dtf, margin);
-      swet[k] = wt ? 1 : 0;
+      if constexpr (FAST) {
+        sq[k] = wt ? sqrtf(w - b) : 0.0f;  // zero: dry
+      } else {
+        sdep[k] = w - b;
+        swet[k] = wt ? 1 : 0;
+      }
       return wt ? 1 : 0;
     } else {
       return gfk::above(s0[k], rdry) ? 1 : 0;
     }
   };
   int anywet = 0;
+  // FAST: a quad of cells: wet tests, roots of the depths and velocities
+  [[maybe_unused]] auto cells4 = [&](int k, bool velocities) {
+    if constexpr (FAST) {
+      const float4 w = *reinterpret_cast<const float4*>(s0 + k);
+      const float4 b = *reinterpret_cast<const float4*>(sb + k);
+      float4 q;
+      auto one = [&](float wk, float bk) {
+        const bool wt = gfk::wet_dev(wk, bk, drytol, dtf, margin);
+        anywet |= wt ? 1 : 0;
+        return wt ? sqrtf(wk - bk) : 0.0f;  // zero: dry
+      };
+      q.x = one(w.x, b.x);
+      q.y = one(w.y, b.y);
+      q.z = one(w.z, b.z);
+      q.w = one(w.w, b.w);
+      *reinterpret_cast<float4*>(sq + k) = q;
+      if (!velocities) return;
+      const float4 hu = *reinterpret_cast<const float4*>(shu + k);
+      const float4 hv = *reinterpret_cast<const float4*>(shv + k);
+      float4 u, v;
+      auto vel = [](float qk, float h, float a, float c, float& x, float& y) {
+        const float rh = gfk::rcpf(h);
+        x = qk > 0.0f ? __fmul_rn(a, rh) : 0.0f;
+        y = qk > 0.0f ? __fmul_rn(c, rh) : 0.0f;
+      };
+      vel(q.x, w.x - b.x, hu.x, hv.x, u.x, v.x);
+      vel(q.y, w.y - b.y, hu.y, hv.y, u.y, v.y);
+      vel(q.z, w.z - b.z, hu.z, hv.z, u.z, v.z);
+      vel(q.w, w.w - b.w, hu.w, hv.w, u.w, v.w);
+      *reinterpret_cast<float4*>(su + k) = u;
+      *reinterpret_cast<float4*>(sv + k) = v;
+    }
+  };
+  if constexpr (FAST) {
+    if constexpr (M == MP) {
+      bool ok = mbar_wait(bar, GF_SPIN_LIMIT, ph0);
+      if (mom_issued) ok = mbar_wait(bar + 1, GF_SPIN_LIMIT, ph1) && ok;
+      if (!ok) *sflag = 1;
+      if (tp) {
+        tp->b0 ^= 1u;
+        if (mom_issued) tp->b1 ^= 1u;
+      }
+    }
+    if (M == MP && same_in) {
+      // an unchanged dry interior: only the ghost cells can have taken water
+      for (int k = tid; k < NRING; k += NT) anywet |= examine(ring_cell(k));
+    } else {
+      for (int k = 4 * tid; k < TT; k += 4 * NT) cells4(k, true);
+    }
+    anywet = __syncthreads_or(anywet);
+    if (*sflag) {
+      // some wait gave up: wait (again with a limit) for the copies in
+      // flight, then give the tile up
+      if (tid == 0) C->status = -7;  // GEOFLOOD_ERR_TIMEOUT
+      if constexpr (M == MP) {
+        mbar_wait(bar, GF_SPIN_LIMIT, ph0);
+        if (mom_issued) mbar_wait(bar + 1, GF_SPIN_LIMIT, ph1);
+      }
+      __syncthreads();
+      return -1;
+    }
+  } else {
   if (same_in) {
     for (int k = tid; k < NRING; k += NT) anywet |= examine(ring_cell(k));
     anywet = __syncthreads_or(anywet);
@@ -478,10 +613,12 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
     for (int k = tid; k < TT; k += NT) anywet |= examine(k);
     anywet = __syncthreads_or(anywet);
   }
+  }
   if constexpr (M == MP) {
     // the momenta: requested now if water arrived at a copied dry tile, and
     // waited for whenever they were requested
-    if (anywet && !mom_issued) {
+    const bool late = anywet && !mom_issued;
+    if (late) {
       if (tid == 0) {
         mbar_expect_tx(bar + 1, 2u * TT * sizeof(R));
         bulk_g2s(shu, qs + TT, TT * sizeof(R), bar + 1);
@@ -489,19 +626,26 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
       }
       mom_issued = true;
     }
-    if (mom_issued && !__syncthreads_and(mbar_wait(bar + 1, GF_SPIN_LIMIT, ph1) ? 1 : 0)) {
+    if ((FAST ? late : mom_issued) &&
+        !__syncthreads_and(mbar_wait(bar + 1, GF_SPIN_LIMIT, ph1) ? 1 : 0)) {
       if (tid == 0) C->status = -7;  // GEOFLOOD_ERR_TIMEOUT
       mbar_wait(bar + 1, GF_SPIN_LIMIT, ph1);
       __syncthreads();
       return -1;
     }
-    if (mom_issued && tp) tp->b1 ^= 1u;
+    if ((FAST ? late : mom_issued) && tp) tp->b1 ^= 1u;
+    if constexpr (FAST) {
+      if (late) {
+        for (int k = 4 * tid; k < TT; k += 4 * NT) cells4(k, true);
+        __syncthreads();
+      }
+    }
   }
   // a dry tile whose interior is already the same in both buffers writes
   // nothing (its update is the identity on the surface, zero momenta)
   const bool skip_writes = same_in && !anywet;
   if (V.same != nullptr && tid == 0) V.same[unit] = anywet ? 0 : 1;
-  if (has_gauge && C->accepted && (!subc || C->sub_k == 0))
+  if (has_gauge && H.accepted && (!subc || C->sub_k == 0))
     sample_gauges<R, DEV, MP, M>(V, Pt.scen, C, p, ox, oy, s0, shu, shv, sb,
                                  M != MP || mom_issued);
   if (skip_writes) {
@@ -510,7 +654,8 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
     return 0;
   }
   auto wetc = [&](int c) -> bool {
-    if constexpr (DEV) return swet[c] != 0;
+    if constexpr (FAST) return sq[c] > R(0);
+    else if constexpr (DEV) return swet[c] != 0;
     else if constexpr (PRIM) return gfk::pos(sc[c]);  // zero celerity: dry
     else return s0[c] > rdry;
   };
@@ -536,8 +681,8 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
     }
   }
 
-  R X[RC][3];   // nu_x * dQx of owned interior cells
-  R Y[RC][3];   // nu_y * dQy
+  R X[FAST ? 1 : RC][3];   // nu_x * dQx of owned interior cells
+  R Y[FAST ? 1 : RC][3];   // nu_y * dQy
   // dimensional splitting, deviation form: compensation terms of the
   // intermediate state of owned interior cells
   float LO1[DS && DEV ? RC : 1][3];
@@ -559,7 +704,267 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
   // without the sweeps; the results are identical.
   // one sweep; the direction is a compile-time constant so that the index
   // arithmetic of the two sweeps is resolved statically
-  auto sweep = [&](auto dirc) {
+  using gfk::f2;
+  // FAST: of the pairs of owned cells, nu dQ summed over the sweeps and the
+  // transverse fluxes' change
+  [[maybe_unused]] f2 XP[FAST ? RC : 1][3], TP[FAST ? RC : 1][3];
+  [[maybe_unused]] auto sweep32 = [&](auto dirc) {
+    constexpr int dir = decltype(dirc)::value;
+    if constexpr (FAST) {
+    // Edge a in [-1, M + 1] of line l in [-1, M].  In both sweeps threads take
+    // pairs of neighbours along a tile row: two edges of a row in the x
+    // sweep, the edges of two columns (from column -2 on) in the y sweep.
+    // Place of an edge in a wave plane: tile-like rows of pitch PW.
+    constexpr int PW = M + 4;
+    constexpr int SE = dir == 0 ? 1 : PW;        // place of the next edge of a line
+    constexpr int CS = dir == 0 ? 1 : Lo::T;     // tile step along the sweep
+    constexpr int CL = dir == 0 ? Lo::T : 1;     // and across it
+    const R* sn = dir == 0 ? shu : shv;
+    const R* un = dir == 0 ? su : sv;
+    const R* ut = dir == 0 ? sv : su;
+    const float nu = dir == 0 ? nux : nuy;
+    const float sg = sqrtf(g);
+    const f2 nz = gfk::pk1(G.negzero);
+    float smax = dir == 0 ? smx : smy;
+    // phase 1: Riemann solves.  x: row l, edges a = -1 + 2 m and the next;
+    // y: edge row a, columns -2 + 2 m and the next
+    constexpr int N1 = dir == 0 ? (M + 2) * PW / 2 : (M + 3) * PW / 2;
+#pragma unroll 1
+    for (int k = tid; k < N1; k += NT) {
+      const int m = k % (PW / 2), row = k / (PW / 2);  // row: l + 1, or a + 1
+      const int e = row * PW + 2 * m;
+      // tile cell left of (below) the first edge
+      const int c = dir == 0 ? (row + 1) * Lo::T + 2 * m : row * Lo::T + 2 * m;
+      auto pair_l = [&](const R* p) { return gfk::ld2(p + c); };
+      auto pair_r = [&](const R* p, f2 l) {
+        if constexpr (dir == 0) {
+          float x, y;
+          gfk::upk(l, x, y);
+          return gfk::pk(y, p[c + 2]);
+        } else {
+          (void)l;
+          return gfk::ld2(p + c + CS);
+        }
+      };
+      gfk::Prim32x2 L{pair_l(s0), pair_l(sb), pair_l(sn), pair_l(un), pair_l(ut), pair_l(sq)};
+      gfk::Prim32x2 Rt{pair_r(s0, L.w), pair_r(sb, L.b), pair_r(sn, L.n),
+                       pair_r(un, L.u), pair_r(ut, L.v), pair_r(sq, L.q)};
+      f2 z[8], s1, s3;
+      gfk::riemann32x2(L, Rt, g, sg, nz, z, s1, s3);
+      R* w = W + e;
+#pragma unroll
+      for (int q = 0; q < 8; ++q) gfk::st2(w + q * NEDGE, z[q]);
+      gfk::st2(w + 8 * NEDGE, s1);
+      gfk::st2(w + 9 * NEDGE, s3);
+      // CFL rate: edges of interior lines that bound interior cells
+      float s1a, s1b, s3a, s3b;
+      gfk::upk(s1, s1a, s1b);
+      gfk::upk(s3, s3a, s3b);
+      const float ma = fmaxf(fabsf(s1a), fabsf(s3a)), mb = fmaxf(fabsf(s1b), fabsf(s3b));
+      if constexpr (dir == 0) {
+        if ((unsigned)(row - 1) < (unsigned)M) {  // a = 2 m - 1, 2 m
+          if (m > 0 && m <= M2) smax = fmaxf(smax, ma);
+          if (m <= M2) smax = fmaxf(smax, mb);
+        }
+      } else {
+        if ((unsigned)(row - 1) <= (unsigned)M && m > 0 && m <= M2)
+          smax = fmaxf(smax, fmaxf(ma, mb));
+      }
+    }
+    if (dir == 0) smx = smax;
+    else smy = smax;
+    __syncthreads();
+    // phase 2: limited fluxes of edges 0..M, kept until every wave was read.
+    // x: pairs from a = -1 on; y: rows a = 0..M
+    constexpr int N2 = dir == 0 ? (M + 2) * (M2 + 1) : (M + 1) * PW / 2;
+    constexpr int RE = (N2 + NT - 1) / NT;
+    f2 am[RE][3], ap[RE][3], ff[RE][3];
+#pragma unroll
+    for (int r = 0; r < RE; ++r) {
+      const int k = tid + r * NT;
+      if (k < N2) {
+        const int m = dir == 0 ? k % (M2 + 1) : k % (PW / 2);
+        const int row = dir == 0 ? k / (M2 + 1) : k / (PW / 2) + 1;  // l + 1, or a + 1
+        const int e = row * PW + 2 * m;
+        const int c = dir == 0 ? (row + 1) * Lo::T + 2 * m : row * Lo::T + 2 * m;
+        float q0, q1, q2, q3;
+        gfk::upk(gfk::ld2(sq + c), q0, q1);
+        if constexpr (dir == 0) {
+          q3 = sq[c + 2];
+          q2 = q1;
+        } else {
+          gfk::upk(gfk::ld2(sq + c + CS), q2, q3);
+        }
+        gfk::edge32x2<NEDGE, SE>(W + e, nu, corr && fminf(q0, q2) > 0.0f,
+                                 corr && fminf(q1, q3) > 0.0f, nz, am[r], ap[r], ff[r]);
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < RE; ++r) {
+      const int k = tid + r * NT;
+      if (k < N2) {
+        const int m = dir == 0 ? k % (M2 + 1) : k % (PW / 2);
+        const int row = dir == 0 ? k / (M2 + 1) : k / (PW / 2) + 1;
+        R* w = W + row * PW + 2 * m;
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+          gfk::st2(w + q * NEDGE, am[r][q]);
+          gfk::st2(w + (3 + q) * NEDGE, ap[r][q]);
+          gfk::st2(w + (6 + q) * NEDGE, ff[r][q]);
+        }
+      }
+    }
+    __syncthreads();
+    // phase 3: increments and their transverse split.  The x sweep covers
+    // rows -1..M of the thread's columns; in the y sweep the threads of the
+    // two ghost rows take the two ghost columns instead (two rows each).
+    // Transverse parts (plus, minus; mass, hu, hv) in planes of pitch PT.
+    constexpr int PTP = M * (M + 4);          // one plane
+    constexpr int PT = dir == 0 ? M : M + 4;  // its rows
+    R* Tr = Ftr;
+    auto tplace = [&](int i, int j) { return dir == 0 ? (j + 1) * M + i : j * PT + i + 2; };
+    f2 opl[RC][3], omi[RC][3];
+#pragma unroll
+    for (int r = 0; r < RC; ++r) {
+      const int lane = tid % M2, Lx = tid / M2 + r * TLC;
+      const bool inner = Lx < M;
+      const int Lr = inner ? Lx : (Lx == M ? -1 : M);
+      if (!(Lx <= M + 1 && (inner || trv))) continue;
+      const bool col = dir == 1 && !inner;  // a pair down a ghost column
+      const int i = col ? Lr : 2 * lane, j = col ? 2 * lane : Lr;
+      f2 d[3];  // mass, normal (sweep) momentum, transverse
+      if constexpr (dir == 0) {
+        const R* w = W + (j + 1) * PW + i + 1;  // edge a = i (odd place)
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+          const f2 apl = gfk::pk(w[(3 + q) * NEDGE], w[(3 + q) * NEDGE + 1]);
+          const f2 fr = gfk::ld2(w + (6 + q) * NEDGE + 1);
+          float f1, f2v;
+          gfk::upk(fr, f1, f2v);
+          const f2 fl = gfk::pk(w[(6 + q) * NEDGE], f1);
+          d[q] = gfk::add2(gfk::add2(apl, gfk::ld2(w + q * NEDGE + 1)), gfk::sub2(fr, fl));
+        }
+      } else {
+        const R* w = W + (j + 1) * PW + i + 2;  // edge a = j of column i
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+          const R *wa = w + q * NEDGE + PW, *wp = w + (3 + q) * NEDGE, *wf = w + (6 + q) * NEDGE;
+          f2 amr, apl, fl, fr;
+          if (col) {
+            amr = gfk::pk(wa[0], wa[PW]);
+            apl = gfk::pk(wp[0], wp[PW]);
+            fl = gfk::pk(wf[0], wf[PW]);
+            fr = gfk::pk(wf[PW], wf[2 * PW]);
+          } else {
+            amr = gfk::ld2(wa);
+            apl = gfk::ld2(wp);
+            fl = gfk::ld2(wf);
+            fr = gfk::ld2(wf + PW);
+          }
+          d[q] = gfk::add2(gfk::add2(apl, amr), gfk::sub2(fr, fl));
+        }
+      }
+      if (inner) {
+        // (mass, hu, hv)
+        const f2 n2 = gfk::pk1(nu);
+        if constexpr (dir == 0) {
+          XP[r][0] = gfk::mulr2(n2, d[0], nz);
+          XP[r][1] = gfk::mulr2(n2, d[1], nz);
+          XP[r][2] = gfk::mulr2(n2, d[2], nz);
+        } else {
+          XP[r][0] = gfk::add2(XP[r][0], gfk::mulr2(n2, d[0], nz));
+          XP[r][1] = gfk::add2(XP[r][1], gfk::mulr2(n2, d[2], nz));
+          XP[r][2] = gfk::add2(XP[r][2], gfk::mulr2(n2, d[1], nz));
+        }
+      }
+      if (!trv) continue;
+      const int c = tix<M>(i, j);
+      const int c1 = col ? c + Lo::T : c + 1;  // the pair's second cell
+      auto cells = [&](const R* p) {
+        return col ? gfk::pk(p[c], p[c1]) : gfk::ld2(p + c);
+      };
+      const f2 w2 = cells(s0);
+      float q0, q1;
+      gfk::upk(cells(sq), q0, q1);
+      f2 pl[3], mi[3];
+      const f2 dd[3] = {d[0], d[2], d[1]};
+      gfk::tsplit32x2(cells(ut), cells(un), gfk::sub2(w2, cells(sb)), g, nz, dd, pl, mi);
+      // nothing from a dry cell, nor into a dry neighbour across the sweep
+      // whose bed is above the cell's surface
+      const float qp0 = sq[c + CL], qm0 = sq[c - CL], qp1 = sq[c1 + CL], qm1 = sq[c1 - CL];
+      if (!(fminf(fminf(fminf(qp0, qm0), fminf(qp1, qm1)), fminf(q0, q1)) > 0.0f)) {
+        float w0, w1;
+        gfk::upk(w2, w0, w1);
+        const bool p0 = q0 > 0.0f && (qp0 > 0.0f || !(sb[c + CL] > w0));
+        const bool p1 = q1 > 0.0f && (qp1 > 0.0f || !(sb[c1 + CL] > w1));
+        const bool m0 = q0 > 0.0f && (qm0 > 0.0f || !(sb[c - CL] > w0));
+        const bool m1 = q1 > 0.0f && (qm1 > 0.0f || !(sb[c1 - CL] > w1));
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+          pl[q] = gfk::sel2(p0, p1, pl[q], 0ull);
+          mi[q] = gfk::sel2(m0, m1, mi[q], 0ull);
+        }
+      }
+      // (mass, hu, hv): "along" is the transverse momentum
+      const int hu = dir == 0 ? 2 : 1, hv = dir == 0 ? 1 : 2;
+      const f2 po[3] = {pl[0], pl[hu], pl[hv]}, mo[3] = {mi[0], mi[hu], mi[hv]};
+      R* o = Tr + tplace(i, j);
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        if (col) {
+          float x, y;
+          gfk::upk(po[q], x, y);
+          o[q * PTP] = x;
+          o[q * PTP + PT] = y;
+          gfk::upk(mo[q], x, y);
+          o[(3 + q) * PTP] = x;
+          o[(3 + q) * PTP + PT] = y;
+        } else {
+          gfk::st2(o + q * PTP, po[q]);
+          gfk::st2(o + (3 + q) * PTP, mo[q]);
+        }
+        opl[r][q] = po[q];
+        omi[r][q] = mo[q];
+      }
+    }
+    __syncthreads();
+    // transverse fluxes through the cell's two edges across the sweep:
+    // -nu/2 of what enters each from both sides; their difference
+    if (trv) {
+      const f2 kt = gfk::pk1(-0.5f * nu), nx2 = gfk::pk1(nux);
+#pragma unroll
+      for (int r = 0; r < RC; ++r) {
+        const int i = 2 * (tid % M2), j = tid / M2 + r * TLC;
+        if ((unsigned)j >= (unsigned)M) continue;
+        const R* o = Tr + tplace(i, j);
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+          f2 mn, pp;  // minus of the next line's cells, plus of the previous
+          if constexpr (dir == 0) {
+            mn = gfk::ld2(o + (3 + q) * PTP + PT);
+            pp = gfk::ld2(o + q * PTP - PT);
+          } else {
+            float x, y;
+            gfk::upk(omi[r][q], x, y);
+            mn = gfk::pk(y, o[(3 + q) * PTP + 2]);
+            gfk::upk(opl[r][q], x, y);
+            pp = gfk::pk(o[q * PTP - 1], x);
+          }
+          const f2 hi = gfk::mulr2(kt, gfk::add2(opl[r][q], mn), nz);
+          const f2 lo = gfk::mulr2(kt, gfk::add2(pp, omi[r][q]), nz);
+          const f2 df = gfk::sub2(hi, lo);
+          if constexpr (dir == 0) TP[r][q] = gfk::mul2(gfk::pk1(nuy), df);
+          else TP[r][q] = gfk::fma2(nx2, df, TP[r][q]);
+        }
+      }
+    } else {
+#pragma unroll
+      for (int r = 0; r < RC; ++r) TP[r][0] = TP[r][1] = TP[r][2] = 0ull;
+    }
+    }
+  };
+  [[maybe_unused]] auto sweep = [&](auto dirc) {
     constexpr int dir = decltype(dirc)::value;
     // lines swept: -1..M (unsplit), -2..M+1 (split, x), 0..M-1 (split, y)
     constexpr int NRL = DS ? (dir == 0 ? M + 4 : M) : M + 2;
@@ -781,9 +1186,19 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
     __syncthreads();
   };
   if (anywet) {
-    sweep(std::integral_constant<int, 0>{});
-    sweep(std::integral_constant<int, 1>{});
+    if constexpr (FAST) {
+      sweep32(std::integral_constant<int, 0>{});
+      sweep32(std::integral_constant<int, 1>{});
+    } else {
+      sweep(std::integral_constant<int, 0>{});
+      sweep(std::integral_constant<int, 1>{});
+    }
   }
+  // interior cell of round r (or -1): its index in the M x M tile
+  auto owned = [&](int r) -> int {
+    const int k = tid + r * NT;
+    return k < M * M ? k : -1;
+  };
 
   // New values of a cell near the patch edge also go to the ghost cells that
   // copy or mirror it (same-level neighbours, physical boundaries).
@@ -800,21 +1215,146 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
   bool bad = false;
   // the compensation terms of every owned cell requested at once, so that
   // their global loads overlap instead of one wait per cell
-  float lpre[DEV && !DS ? RC : 1][3];
-  if constexpr (DEV && !DS) {
+  if constexpr (FAST) {
+    if (anywet) {
+      f2 lpre[RC][3];
 #pragma unroll
-    for (int r = 0; r < RC; ++r) {
-      const int k = tid + r * NT;
-      const int kp = k < M * M ? pix(k % M, k / M) : 0;
+      for (int r = 0; r < RC; ++r) {
+        const int i = 2 * (tid % M2), j = tid / M2 + r * TLC;
+        if ((unsigned)j >= (unsigned)M) continue;
 #pragma unroll
-      for (int f = 0; f < 3; ++f)
-        lpre[r][f] = (anywet && k < M * M) ? los[f * MP * MP + kp] : 0.0f;
+        for (int f = 0; f < 3; ++f) lpre[r][f] = gfk::ld2(los + f * MP * MP + pix(i, j));
+      }
+      // new values of the tile for the edge cells' copies below; the wave
+      // planes are free since the last barrier
+      R* nv = W;
+#pragma unroll
+      for (int r = 0; r < RC; ++r) {
+        const int i = 2 * (tid % M2), j = tid / M2 + r * TLC;
+        if ((unsigned)j >= (unsigned)M) continue;
+        const int c = tix<M>(i, j), cg = gix(i, j), kp = pix(i, j);
+        // compensated update: (hi + lo) - change, hi rounded, lo the error
+        f2 o2[3], l2[3];
+#pragma unroll
+        for (int f = 0; f < 3; ++f) {
+          const f2 q = gfk::ld2((f == 0 ? s0 : (f == 1 ? shu : shv)) + c);
+          const f2 x = gfk::sub2(gfk::sub2(lpre[r][f], XP[r][f]), TP[r][f]);
+          const f2 sum = gfk::add2(q, x), bb = gfk::sub2(sum, q);
+          l2[f] = gfk::add2(gfk::sub2(q, gfk::sub2(sum, bb)), gfk::sub2(x, bb));
+          o2[f] = sum;
+        }
+        float o[2][3], lo[2][3], bc[2], qc[2];
+#pragma unroll
+        for (int f = 0; f < 3; ++f) {
+          gfk::upk(o2[f], o[0][f], o[1][f]);
+          gfk::upk(l2[f], lo[0][f], lo[1][f]);
+        }
+        gfk::upk(gfk::ld2(sb + c), bc[0], bc[1]);
+        gfk::upk(gfk::ld2(sq + c), qc[0], qc[1]);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          nwet += qc[h] > 0.0f ? 1u : 0u;
+          if (o[h][0] < bc[h]) {  // negative depth: reset to a dry bed
+            clipf += bc[h] - o[h][0];
+            o[h][0] = bc[h];
+            lo[h][0] = 0.0f;
+            ++nclip;
+          }
+          const bool wnew = gfk::wet_dev(o[h][0], bc[h], drytol, dtf, margin);
+          if (mn > 0.0f && wnew) {
+            // approximate reciprocals and h^(-4/3) by the fast power
+            // (relative error about 1e-6, far inside this path's tolerance)
+            const float d = o[h][0] - bc[h];
+            const float rh = gfk::rcpf(d);
+            const float u = __fmul_rn(o[h][1], rh), v = __fmul_rn(o[h][2], rh);
+            const float sp = sqrtf(fmaf(u, u, __fmul_rn(v, v)));
+            const float D = g * mn * mn * sp * __powf(d, -4.0f / 3.0f);
+            const float rden = gfk::rcpf(fmaf(dtr, D, 1.0f));
+            o[h][1] = __fmul_rn(o[h][1], rden);
+            o[h][2] = __fmul_rn(o[h][2], rden);
+            lo[h][1] = __fmul_rn(lo[h][1], rden);
+            lo[h][2] = __fmul_rn(lo[h][2], rden);
+          }
+          if (!wnew) { o[h][1] = 0.0f; o[h][2] = 0.0f; lo[h][1] = 0.0f; lo[h][2] = 0.0f; }
+          bad |= !(isfinite(o[h][0]) && isfinite(o[h][1]) && isfinite(o[h][2]));
+        }
+#pragma unroll
+        for (int f = 0; f < 3; ++f) {
+          const f2 v = gfk::pk(o[0][f], o[1][f]);
+          gfk::st2(lod + f * MP * MP + kp, gfk::pk(lo[0][f], lo[1][f]));
+          gfk::st2(qd + f * TG + cg, v);
+          gfk::st2(nv + f * M * M + j * M + i, v);
+        }
+      }
+      __syncthreads();
+      // Copies of the cells within two of the tile's edge.  Away from the
+      // domain's boundary every copy goes to one same-level neighbour: the
+      // ghost cells of the bottom and top neighbours (2 M each, along x), the
+      // left and right ones, then the corners.
+      if (M == MP && Pt.px > 0 && Pt.px < nxp - 1 && Pt.py > 0 && Pt.py < nyp - 1) {
+        for (int k = push ? tid : 8 * M + 16; k < 8 * M + 16; k += NT) {
+          int r, i, j;
+          if (k < 4 * M) {
+            r = 2 + k / (2 * M);
+            i = k % M;
+            j = k / M + (r == 3 ? M - 4 : 0);
+          } else if (k < 8 * M) {
+            const int x = k - 4 * M;
+            r = x / (2 * M);
+            i = x % 2 + (r ? M - 2 : 0);
+            j = x / 2 % M;
+          } else {
+            const int x = k - 8 * M;
+            r = 4 + x / 4;
+            i = x % 2 + (r & 1 ? M - 2 : 0);
+            j = x / 2 % 2 + (r & 2 ? M - 2 : 0);
+          }
+          const int pn = snb[r];
+          if (pn < 0) continue;
+          const R* v = nv + j * M + i;
+          // towards the neighbour: its cell beyond its own opposite edge
+          const int di = r == 0 || r == 4 || r == 6 ? M : (r == 1 || r == 5 || r == 7 ? -M : 0);
+          const int dj = r == 2 || r == 4 || r == 5 ? M : (r == 3 || r == 6 || r == 7 ? -M : 0);
+          R* d = qnext + (size_t)pn * 3 * TG + tix<M>(i + di, j + dj);
+          d[0] = v[0];
+          d[TG] = v[M * M];
+          d[2 * TG] = v[2 * M * M];
+        }
+      } else
+      // otherwise cell by cell, side by side, so that a warp takes cells of
+      // the same kind (updating and copying in one loop sent every warp
+      // through the copies for its two outer columns)
+      for (int k = tid; k < 8 * M - 16; k += NT) {
+        int i, j;
+        if (k < 4 * M) {
+          i = k % M;
+          j = k < 2 * M ? k / M : M - 4 + k / M;
+        } else {
+          const int r = k - 4 * M, x = r / (M - 4);
+          j = 2 + r % (M - 4);
+          i = x < 2 ? x : M - 4 + x;
+        }
+        const R* v = nv + j * M + i;
+        push_edge(ox + i, oy + j, v[0], v[M * M], v[2 * M * M]);
+      }
+    } else if (!skip_writes) {
+      for (int k = tid; k < M * M; k += NT) {
+        const int i = k % M, j = k / M, cg = gix(i, j), kp = pix(i, j);
+        const float w = s0[tix<M>(i, j)];
+        qd[cg] = w;
+        qd[TG + cg] = 0.0f;
+        qd[2 * TG + cg] = 0.0f;
+        push_edge(ox + i, oy + j, w, 0.0f, 0.0f);
+        lod[kp] = los[kp];
+        lod[MP * MP + kp] = 0.0f;
+        lod[2 * MP * MP + kp] = 0.0f;
+      }
     }
   }
 #pragma unroll
-  for (int r = 0; r < RC; ++r) {
-    const int k = tid + r * NT;
-    if (k >= M * M) continue;
+  for (int r = 0; r < (FAST ? 0 : RC); ++r) {
+    const int k = owned(r);
+    if (k < 0) continue;
     const int i = k % M, j = k / M;
     const int c = tix<M>(i, j);
     const int cg = gix(i, j), kp = pix(i, j);
@@ -860,13 +1400,7 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
       float lo[3];
 #pragma unroll
       for (int f = 0; f < 3; ++f) {
-        const float fl = DS ? Y[r][f] : X[r][f] + Y[r][f];
-        const float* fa = Ftr + 3 * (j * (M + 1) + i);
-        const float* ga = Gtr + 3 * (i * (M + 1) + j);
-        const float tf =
-            trv ? nux * (fa[3 + f] - fa[f]) + nuy * (ga[3 + f] - ga[f]) : 0.0f;
-        const float lin = DS ? LO1[DS && DEV ? r : 0][f] : lpre[DS ? 0 : r][f];
-        const float x = (lin - fl) - tf;
+        const float x = LO1[DS && DEV ? r : 0][f] - Y[DS ? r : 0][f];
         const float s = q[f] + x;
         const float bb = s - q[f];
         lo[f] = (q[f] - (s - bb)) + (x - bb);
@@ -887,9 +1421,9 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
         const float h = o[0] - bc;
         const float rh = __fdividef(1.0f, h);
         const float u = __fmul_rn(o[1], rh), v = __fmul_rn(o[2], rh);
-        const float sp = sqrtf(u * u + v * v);
+        const float sp = sqrtf(fmaf(u, u, __fmul_rn(v, v)));
         const float D = g * mn * mn * sp * __powf(h, -4.0f / 3.0f);
-        const float rden = __fdividef(1.0f, 1.0f + dtr * D);
+        const float rden = __fdividef(1.0f, fmaf(dtr, D, 1.0f));
         o[1] = __fmul_rn(o[1], rden);
         o[2] = __fmul_rn(o[2], rden);
         lo[1] = __fmul_rn(lo[1], rden);
@@ -977,100 +1511,6 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
   }
   if (bad) C->nonfinite = 1;
   return anywet;
-}
-
-// Whole-patch pass of the adaptive variant for a patch expected to be dry:
-// one CTA stages the surface and bed of the MP x MP tile (two TMA bulk
-// copies), decides whether any cell of the tile holds water and, if none
-// does, applies the dry update (copy the surface, zero the momenta) to the
-// whole patch.  Returns 1 if the tile held water (the caller then runs the
-// M x M sub-tiles one after the other; the result does not depend on the
-// split).
-template <class P, int MP, int M, int NT>
-__device__ __forceinline__ int whole_tile(const GfGeom& G, const GfView& V,
-                                          unsigned char* smraw, const int p) {
-  using R = typename P::R;
-  constexpr bool DEV = P::DEV;
-  using Lo = Layout<P, M>;
-  constexpr int TGW = MP + 2 * GF_NG, TG = TGW * TGW;
-  constexpr int NS1 = MP / M, NSUB = NS1 * NS1;
-  static_assert(2 * TG * sizeof(R) <= Lo::OFF_RED, "tile staging fits the sub-tile layout");
-  const int tid = threadIdx.x;
-  const GfPatch Pt = V.patch[p];
-  GfCtl* C = V.ctl + Pt.scen;
-  const int cur = C->cur;
-  R* s0 = reinterpret_cast<R*>(smraw);
-  R* sb = s0 + TG;
-  int* snb = reinterpret_cast<int*>(smraw + Lo::OFF_NB);
-  uint64_t* bar = reinterpret_cast<uint64_t*>(smraw + Lo::OFF_BAR);
-  const R* qs;
-  R* qd;
-  R* qnext;
-  const R* bs;
-  if constexpr (DEV) {
-    qs = V.qf[cur] + (size_t)p * 3 * TG;
-    qnext = V.qf[cur ^ 1];
-    bs = V.bf + (size_t)p * TG;
-  } else {
-    qs = V.q[cur] + (size_t)p * 3 * TG;
-    qnext = V.q[cur ^ 1];
-    bs = V.b + (size_t)p * TG;
-  }
-  qd = qnext + (size_t)p * 3 * TG;
-  bool same_in = V.same != nullptr;
-  if (same_in)
-    for (int u = 0; u < NSUB; ++u) same_in = same_in && V.same[p * NSUB + u] != 0;
-  const bool push = V.push != 0 && V.nbr != nullptr;
-  if (tid == 0) {
-    mbar_init(bar, 1);
-    mbar_expect_tx(bar, 2u * TG * sizeof(R));
-    bulk_g2s(s0, qs, TG * sizeof(R), bar);
-    bulk_g2s(sb, bs, TG * sizeof(R), bar);
-  }
-  if (push && tid < 8) snb[tid] = V.nbr[(size_t)p * 8 + tid];
-  __syncthreads();
-  if (!__syncthreads_and(mbar_wait(bar, GF_SPIN_LIMIT) ? 1 : 0)) {
-    if (tid == 0) C->status = -7;  // GEOFLOOD_ERR_TIMEOUT
-    mbar_wait(bar, GF_SPIN_LIMIT);
-    __syncthreads();
-    return 0;
-  }
-  const double drytol = G.drytol;
-  int anywet = 0;
-  for (int k = tid; k < TG; k += NT) {
-    if constexpr (DEV) anywet |= gfk::wet_dev(s0[k], sb[k], drytol, G.drytolf, G.marginf) ? 1 : 0;
-    else anywet |= s0[k] > drytol ? 1 : 0;
-  }
-  anywet = __syncthreads_or(anywet);
-  if (anywet) return 1;  // the caller runs the sub-tiles
-  if (V.gflag != nullptr && V.gflag[p] != 0 && C->accepted)
-    sample_gauges<R, DEV, MP, MP>(V, Pt.scen, C, p, 0, 0, s0, s0, s0, sb, false);
-  // dry update of the whole patch (skipped when both buffers already agree)
-  const float* los = nullptr;
-  float* lod = nullptr;
-  if constexpr (DEV) {
-    los = V.lof[cur] + (size_t)p * 3 * MP * MP;
-    lod = V.lof[cur ^ 1] + (size_t)p * 3 * MP * MP;
-  }
-  if (!same_in) {
-    for (int k = tid; k < MP * MP; k += NT) {
-      const int i = k % MP, j = k / MP;
-      const int c = (i + GF_NG) + (j + GF_NG) * TGW;
-      const R w = s0[c];
-      qd[c] = w;
-      qd[TG + c] = R(0);
-      qd[2 * TG + c] = R(0);
-      if constexpr (DEV) {
-        lod[k] = los[k];
-        lod[MP * MP + k] = 0.0f;
-        lod[2 * MP * MP + k] = 0.0f;
-      }
-      emit_edge<R, MP>(qnext, p, Pt.px, Pt.py, G.mi << Pt.level, G.mj << Pt.level, snb, G.bc,
-                       push, i, j, w, R(0), R(0));
-    }
-  }
-  if (tid < NSUB && V.same != nullptr) V.same[p * NSUB + tid] = 1;
-  return 0;
 }
 
 // Controller of a subcycled macro step (one thread of the last CTA of each
@@ -1245,13 +1685,13 @@ static __device__ void ctl_finish(const GfGeom& G, GfCtl* Cp, unsigned long long
   }
 }
 
-// End of a step: the last CTA to finish applies the CFL rule to every active
+// End of a step: the last of the nctas working CTAs to finish applies the CFL rule to every active
 // scenario, one thread per scenario (the scenarios' rules are independent).
 // The volume of the state is not part of the step; geoflood_mass computes it
 // on demand.
 template <int NT>
-__device__ void step_finish(const GfGeom& G, const GfView& V, int cells_per_patch,
-                            bool wrote = true) {
+__device__ void step_finish(const GfGeom& G, const GfView& V, int cells_per_patch, bool wrote,
+                            unsigned nctas) {
   __shared__ int last;
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -1259,7 +1699,7 @@ __device__ void step_finish(const GfGeom& G, const GfView& V, int cells_per_patc
     // before it counts itself done; one that did not needs no fence
     if (wrote) __threadfence();
     const unsigned t = atomicAdd(V.done, 1u);
-    last = t == gridDim.x - 1;
+    last = t == nctas - 1u;
   }
   __syncthreads();
   if (!last) return;
@@ -1279,73 +1719,23 @@ __device__ void step_finish(const GfGeom& G, const GfView& V, int cells_per_patc
   // has ended, which orders these writes before it
   if (threadIdx.x == 0 && V.sched) {
     V.sched[0] = (V.sched[0] + 1u) % 6u;
-    V.sched[3] = V.sched[1];  // wet patches at the head of the next order
+    // patches that took no step, at the tail of the next order
+    if (V.inactive) *V.inactive = V.sched[2];
     V.sched[1] = 0u;
     V.sched[2] = 0u;
   }
   if (threadIdx.x == 0) *V.done = 0u;
 }
 
-// Adaptive variant: the previous launch's wet patches (the head of its
-// launch order, sched[3] of them) get NSUB CTAs each, one per M x M
-// sub-tile; every other patch gets one CTA that checks the whole tile and
-// takes the dry update, or the sub-tiles in turn if water has arrived.  The
-// grid has NSUB CTAs per patch; those beyond the work exit at once.
-template <class P, int MP, int M, int NT, int MINB>
-__global__ void __launch_bounds__(NT, MINB)
-    k_patch_step_adaptive(const __grid_constant__ GfGeom G,
-                          const __grid_constant__ GfView V) {
+// patch_body out of line, for the rare tiles that a CTA takes one after the
+// other: inlined into a loop, everything that does not depend on the tile
+// would be kept in registers across the tiles and spilled (1.6 KB a thread).
+template <class P, int MP, int M, int NT, bool DS>
+__device__ __noinline__ int patch_body_call(const GfGeom& G, const GfView& V, const int p,
+                                            const int sub, const TileHdr& H, TmaPhase* tp,
+                                            bool* wrote) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  constexpr int NSUB = (MP / M) * (MP / M);
-  const bool sched = V.sched != nullptr && V.done != nullptr;
-  const unsigned par = sched ? V.sched[0] & 1u : 0u;
-  const int nw = sched ? (int)V.sched[3] : 0;
-  const int* ord = sched ? (par ? V.ord1 : V.ord0) : nullptr;
-  const int b = blockIdx.x;
-  int p = -1, wet = 0;
-  int s_lo = 0, s_hi = 0;  // sub-tiles this CTA computes
-  bool whole = false, active = false;
-  if (b < nw * NSUB) {
-    p = ord[b / NSUB];
-    s_lo = b % NSUB;
-    s_hi = s_lo + 1;
-  } else if (b < nw * NSUB + (V.npatch - nw)) {
-    p = sched ? ord[nw + (b - nw * NSUB)] : b;
-    whole = true;
-  }
-  if (p >= 0) active = V.ctl[V.patch[p].scen].active != 0;
-  if (whole && active && whole_tile<P, MP, M, NT>(G, V, smraw, p)) {
-    wet = 1;
-    s_lo = 0;
-    s_hi = NSUB;
-  }
-  if (!active) s_hi = s_lo;
-  // one call site of the sub-tile body
-  for (int sub = s_lo; sub < s_hi; ++sub) {
-    wet |= patch_body<P, MP, M, NT>(G, V, smraw, p, sub);
-    __syncthreads();
-  }
-  bool report = whole && threadIdx.x == 0;
-  if (!whole && p >= 0 && threadIdx.x == 0) {
-    // the last of the patch's CTAs reports whether any sub-tile held water
-    if (wet) V.pwet[p] = 1u;
-    __threadfence();
-    const unsigned c = atomicAdd(V.pcnt + p, 1u);
-    if (c == NSUB - 1) {
-      __threadfence();
-      wet = *(volatile unsigned*)(V.pwet + p) != 0u;
-      V.pwet[p] = 0u;
-      V.pcnt[p] = 0u;
-      report = true;
-    }
-  }
-  if (sched && report) {
-    int* nxt = par ? V.ord0 : V.ord1;
-    if (wet) nxt[atomicAdd(V.sched + 1, 1u)] = p;
-    else nxt[V.npatch - 1 - (int)atomicAdd(V.sched + 2, 1u)] = p;
-  }
-  if (V.done)
-    step_finish<NT>(G, V, MP * MP);
+  return patch_body<P, MP, M, NT, DS>(G, V, smraw, p, sub, H, tp, wrote);
 }
 
 template <class P, int MP, int M, int NT, int MINB, bool DS = false>
@@ -1353,61 +1743,152 @@ __global__ void __launch_bounds__(NT, MINB)
     k_patch_step(const __grid_constant__ GfGeom G,
                  const __grid_constant__ GfView V) {
   extern __shared__ __align__(16) unsigned char smraw[];
+  using Lo = Layout<P, M, DS>;
   constexpr int NSUB = (MP / M) * (MP / M);
+  // (the FP64 tiles' own time hides their dry neighbours' CTAs)
+  constexpr bool GROUPS = Lo::FAST;
+  constexpr int GRP = GF_STEP_GROUP;
   const int slot = blockIdx.x / NSUB, sub = blockIdx.x % NSUB;
-  // launch order: tiles that held water in the previous launch first, so the
-  // long wet CTAs start at once and the short dry ones fill in around them
+  // The launch order (see GfView::sched): first the patches that took the
+  // step in the previous launch, one CTA each (or one per sub-tile), then
+  // those that did not, GRP to a CTA, which usually finds that none of them
+  // has to; the CTAs beyond return.  Among the first, short dry tiles stay
+  // between the wet ones: with the wet ones strictly ahead the CTAs of an SM
+  // run through their phases side by side and wait for the same unit
+  // (1024 x 1024 grid: 47.6 us a step against 42.7, FP64 568 against 525).  A CTA is a chain of dependent loads, so
+  // what the later ones need is read together: the counter, both orders'
+  // entries and, when there is one scenario, its controller.
   const bool sched = V.sched != nullptr && V.done != nullptr;
-  const unsigned count = sched ? V.sched[0] : 0u;
-  const unsigned par = count & 1u;
-  const int p = sched ? (par ? V.ord1 : V.ord0)[slot] : slot;
-  // run flags (GfView::runf): read by every thread beside the patch record,
-  // so that a running tile waits for nothing more
   const bool use_flags = !DS && sched && V.runf != nullptr && !G.subcycle;
-  const unsigned r3 = count % 3u;
-  const unsigned char* rcur = use_flags ? V.runf + (size_t)r3 * V.runf_stride : nullptr;
-  unsigned char* rnxt = use_flags ? V.runf + (size_t)((r3 + 1u) % 3u) * V.runf_stride : nullptr;
-  const bool marked = use_flags && rcur[p] != 0;
-  // the array that the launch after the next one's marks go to
-  if (use_flags && sub == 0 && threadIdx.x == 0)
-    V.runf[(size_t)((r3 + 2u) % 3u) * V.runf_stride + p] = 0;
-  // a dry, unchanged tile (or sub-tile) of an unmarked patch without a gauge
-  // takes no step (the full path would find its ghost ring dry and write
-  // nothing)
-  const bool skip = use_flags && !marked && V.same != nullptr && V.same[p * NSUB + sub] != 0 &&
-                    !(V.gflag != nullptr && V.gflag[p] != 0);
-  int wet = 0;
+  const bool one = G.nscen == 1;
+  unsigned count = 0u;
+  int inactive = 0, e0 = slot, e1 = slot;
+  if (sched) {
+    count = V.sched[0];
+    e0 = V.ord0[slot];
+    e1 = V.ord1[slot];
+    if (GROUPS && use_flags) inactive = (int)*V.inactive;
+  }
+  if (inactive > V.npatch) inactive = 0;  // unknown: every patch by itself
+  const int nact = V.npatch - inactive;
+  const unsigned working =
+      GROUPS ? (unsigned)(nact + (inactive + GRP - 1) / GRP) * NSUB : gridDim.x;
+  if (GROUPS && blockIdx.x >= working) return;
+  int act = 0, cur = 0, acc = 0;
+  double dt = 0.0;
+  if (one) {
+    const GfCtl& C = V.ctl[0];
+    act = C.active;
+    cur = C.cur;
+    acc = C.accepted;
+    dt = C.dt_use;
+  }
+  const unsigned par = count & 1u, r3 = count % 3u;
+  const int* ord = par ? V.ord1 : V.ord0;
+  // run flags (GfView::runf): this launch's, the next one's, and the array
+  // that is cleared for the one after
+  auto flags = [&](unsigned k) { return V.runf + (size_t)((r3 + k) % 3u) * V.runf_stride; };
+  int first = slot, n = 1;
+  const bool group = GROUPS && slot >= nact;
+  if (group) {
+    first = nact + (slot - nact) * GRP;
+    n = V.npatch - first < GRP ? V.npatch - first : GRP;
+  }
+  // lane l of every warp looks at patch l of the CTA: its run flag and
+  // whether it may stand still (a dry, unchanged tile or sub-tile of an
+  // unmarked patch without a gauge: the full path would find its ghost ring
+  // dry and write nothing)
+  const int lane = threadIdx.x & 31;
+  int pl = -1;
+  int4 rec = make_int4(0, 0, 0, 0);  // its patch record
+  bool marked = false, same = false, gauge = false, skip = false;
+  if (lane < n) {
+    pl = group ? ord[first + lane] : (par ? e1 : e0);
+    marked = use_flags && flags(0u)[pl] != 0;
+    same = V.same != nullptr && V.same[pl * NSUB + sub] != 0;
+    gauge = V.gflag != nullptr && V.gflag[pl] != 0;
+    rec = *reinterpret_cast<const int4*>(V.patch + pl);
+    skip = use_flags && !marked && same && !gauge;
+    if (use_flags && sub == 0 && threadIdx.x < 32) {
+      flags(2u)[pl] = 0;
+      if (skip) {
+        int* nxt = par ? V.ord0 : V.ord1;
+        nxt[V.npatch - 1 - (int)atomicAdd(V.sched + 2, 1u)] = pl;
+      }
+    }
+  }
+  unsigned todo = __ballot_sync(0xffffffffu, lane < n && !skip);
   bool wrote = false;
-  if (!skip) {
-    const GfPatch Pt = V.patch[p];
-    bool run = V.ctl[Pt.scen].active != 0;
+  // patch of lane l; body runs its tile
+  auto take = [&](int l, auto body) -> int {
+    const int p = __shfl_sync(0xffffffffu, pl, l);
+    TileHdr H;
+    H.Pt = GfPatch{__shfl_sync(0xffffffffu, rec.x, l), __shfl_sync(0xffffffffu, rec.y, l),
+                   __shfl_sync(0xffffffffu, rec.z, l), __shfl_sync(0xffffffffu, rec.w, l)};
+    H.same_in = __shfl_sync(0xffffffffu, same ? 1 : 0, l) != 0;
+    H.has_gauge = __shfl_sync(0xffffffffu, gauge ? 1 : 0, l) != 0;
+    if (!one) {
+      const GfCtl& C = V.ctl[H.Pt.scen];
+      act = C.active;
+      cur = C.cur;
+      acc = C.accepted;
+      dt = C.dt_use;
+    }
+    H.cur = cur;
+    H.accepted = acc;
+    H.dt = dt;
+    bool run = act != 0;
     if (run && G.subcycle) {
       // level subcycling: only the levels due at this substep step
-      const GfCtl& C = V.ctl[Pt.scen];
-      run = !C.sub_rej && C.sub_k % (1 << (G.maxlevel - Pt.level)) == 0;
+      const GfCtl& C = V.ctl[H.Pt.scen];
+      run = !C.sub_rej && C.sub_k % (1 << (G.maxlevel - H.Pt.level)) == 0;
     }
-    wrote = true;
-    if (run)
-      wet = patch_body<P, MP, M, NT, DS>(G, V, smraw, p, sub, nullptr, &wrote);
-    else wrote = false;
-    // a patch that did not run carries its mark forward
-    if (use_flags && threadIdx.x == 0 && !run) rnxt[p] = 1;
-    if (use_flags && wet && threadIdx.x < 9) {
-      // water in this tile: it and its same-level neighbours run next launch
-      // (their indices were staged in shared memory by the patch body)
-      using Lo = Layout<P, M, DS>;
-      const int* snb = reinterpret_cast<const int*>(smraw + Lo::OFF_NB);
-      const int q = threadIdx.x == 8 ? p : snb[threadIdx.x];
-      if (q >= 0) rnxt[q] = 1;
+    int wet = 0;
+    if (run) {
+      bool w = true;
+      wet = body(p, H, &w);
+      wrote |= w;
+    }
+    if (use_flags) {
+      // a patch that did not run carries its mark forward
+      if (threadIdx.x == 0 && !run) flags(1u)[p] = 1;
+      if (wet && threadIdx.x < 9) {
+        // water in this tile: it and its same-level neighbours run next
+        // launch (their indices were staged in shared memory by patch_body)
+        const int* snb = reinterpret_cast<const int*>(smraw + Lo::OFF_NB);
+        const int q = threadIdx.x == 8 ? p : snb[threadIdx.x];
+        if (q >= 0) flags(1u)[q] = 1;
+      }
+    }
+    if (sched && sub == 0 && threadIdx.x == 0) {
+      int* nxt = par ? V.ord0 : V.ord1;
+      if (use_flags || wet) nxt[atomicAdd(V.sched + 1, 1u)] = p;
+      else nxt[V.npatch - 1 - (int)atomicAdd(V.sched + 2, 1u)] = p;
+    }
+    return wet;
+  };
+  if (!group) {
+    if (todo)
+      take(0, [&](int p, const TileHdr& H, bool* w) {
+        return patch_body<P, MP, M, NT, DS>(G, V, smraw, p, sub, H, nullptr, w);
+      });
+  }
+  if constexpr (GROUPS) {
+  if (group && todo) {
+    TmaPhase tp{0u, 0u, false};
+    while (todo) {
+      const int wet = take(__ffs(todo) - 1, [&](int p, const TileHdr& H, bool* w) {
+        return patch_body_call<P, MP, M, NT, DS>(G, V, p, sub, H, &tp, w);
+      });
+      todo = wet < 0 ? 0u : todo & (todo - 1u);  // a wait gave up: the launch has failed
+      // shared memory is reused, first by the next tile's bulk copies
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      __syncthreads();
     }
   }
-  if (sched && sub == 0 && threadIdx.x == 0) {
-    int* nxt = par ? V.ord0 : V.ord1;
-    if (wet) nxt[atomicAdd(V.sched + 1, 1u)] = p;
-    else nxt[V.npatch - 1 - (int)atomicAdd(V.sched + 2, 1u)] = p;
   }
   if (V.done)
-    step_finish<NT>(G, V, MP * MP, wrote);
+    step_finish<NT>(G, V, MP * MP, wrote, working);
 }
 
 // Launch the patch step on every patch: MP x MP patches, M x M sub-tiles
@@ -1425,24 +1906,6 @@ int launch_step(const GfGeom& g, const GfView& v, cudaStream_t st) {
   }
   constexpr int NSUB = (MP / M) * (MP / M);
   k_patch_step<P, MP, M, NT, MINB, DS><<<v.npatch * NSUB, NT, bytes, st>>>(g, v);
-  return cudaGetLastError() == cudaSuccess ? 0 : -2;
-}
-
-// Launch the adaptive variant (NSUB CTAs per patch, see
-// k_patch_step_adaptive).
-template <class P, int MP, int M, int NT, int MINB>
-int launch_step_adaptive(const GfGeom& g, const GfView& v, cudaStream_t st) {
-  constexpr size_t bytes = Layout<P, M>::BYTES;
-  static bool attr = false;
-  if (!attr) {
-    if (cudaFuncSetAttribute(k_patch_step_adaptive<P, MP, M, NT, MINB>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)bytes) != cudaSuccess)
-      return -2;
-    attr = true;
-  }
-  constexpr int NSUB = (MP / M) * (MP / M);
-  k_patch_step_adaptive<P, MP, M, NT, MINB><<<v.npatch * NSUB, NT, bytes, st>>>(g, v);
   return cudaGetLastError() == cudaSuccess ? 0 : -2;
 }
 
