@@ -1101,7 +1101,7 @@ __global__ void __launch_bounds__(256, 1) k_ghost_other(const __grid_constant__ 
 // Bilinear interpolant of DEM k at (x, y), constant beyond its edges.
 __device__ double dem_eval(const GfScenario& S, int k, double x, double y) {
   const int nx = S.dnx[k], ny = S.dny[k];
-  double fx = (x - S.dx0[k]) / S.ddx[k], fy = (y - S.dy0[k]) / S.ddy[k];
+  double fx = gfk::div_rn(x - S.dx0[k], S.ddx[k]), fy = gfk::div_rn(y - S.dy0[k], S.ddy[k]);
   if (fx < 0.0) fx = 0.0;
   if (fx > (double)(nx - 1)) fx = (double)(nx - 1);
   if (fy < 0.0) fy = 0.0;
@@ -1143,7 +1143,7 @@ __device__ double next_break(const GfScenario& S, bool xaxis, double v, double b
     const double o = xaxis ? S.dx0[k] : S.dy0[k];
     const double d = xaxis ? S.ddx[k] : S.ddy[k];
     const int n = xaxis ? S.dnx[k] : S.dny[k];
-    double f = floor((v - o) / d) + 1.0;
+    double f = floor(gfk::div_rn(v - o, d)) + 1.0;
     if (f < 0.0) f = 0.0;
     if (f > (double)n) f = (double)n;
     int i = (int)f;
@@ -1157,6 +1157,7 @@ __device__ double next_break(const GfScenario& S, bool xaxis, double v, double b
   return best;
 }
 
+// (Quotients in the integer pipe: the FP64 pipe bounds this kernel.)
 // Exact average over [xa,xb]x[ya,yb] of the composite interpolant: the node
 // lines of all DEMs cut the cell into pieces on which it is bilinear; each
 // piece contributes its area times its midpoint value.  Rows of pieces in
@@ -1177,11 +1178,16 @@ __device__ double dem_average(const GfScenario& S, double xa, double xb,
     }
     y0 = y1;
   }
-  return sum / ((xb - xa) * (yb - ya));
+  return gfk::div_rn(sum, (xb - xa) * (yb - ya));
 }
 
+// One CTA per patch.  448 threads (three rounds of the 1296 cells of a 32 x 32
+// patch's tile, one of a 16 x 16 patch's 400) instead of 128: a forest of
+// some hundred patches gives an SM one CTA, whose warps are all that hides
+// the FP64 latency.  116 patches on an 8 m DEM: 253 -> 164 us, 1856: 1150 ->
+// 717 us.
 template <typename T>
-__global__ void k_topo(const __grid_constant__ GfGeom G, const __grid_constant__ GfView V, int first,
+__global__ void __launch_bounds__(448) k_topo(const __grid_constant__ GfGeom G, const __grid_constant__ GfView V, int first,
                        const int* list) {
   const int p = list ? list[blockIdx.x] : first + blockIdx.x;
   const GfPatch P = V.patch[p];
@@ -1199,7 +1205,7 @@ __global__ void k_topo(const __grid_constant__ GfGeom G, const __grid_constant__
     return;
   }
   const long long NX = e.nx(P.level), NY = e.ny(P.level);
-  const double dx = e.dx(P.level), dy = e.dy(P.level);
+  const double dx = G.dxl[P.level], dy = G.dyl[P.level];
   for (int k = threadIdx.x; k < TT; k += blockDim.x) {
     const int i = k % T_ - GF_NG, j = k / T_ - GF_NG;
     const long long I = (long long)P.px * M + i, J = (long long)P.py * M + j;
@@ -1643,7 +1649,9 @@ __global__ void k_gauges(const __grid_constant__ GfGeom G, const __grid_constant
   const GfCtl* C = V.ctl + s;
   if (only_accepted && !C->accepted) return;
   Geo<T> e(G, V);
-  const GfGaugeRef r = gauge_locate(e, G, V, S, g);
+  // the stencil as k_gauge_refs left it for this forest (locating the gauge
+  // again, level by level in FP64, took 8 of this kernel's 12.5 us)
+  const GfGaugeRef r = S.gref[g];
   double* o = S.gout + 5 * g;
   o[0] = C->t;
   if (r.p < 0) { o[1] = o[2] = o[3] = o[4] = 0.0; return; }
@@ -2148,8 +2156,8 @@ int launch_topo(const GfGeom& g, const GfView& v, int first, int count,
                 void* stream, const int* list) {
   if (count <= 0) return 0;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  if (v.prec) k_topo<float><<<count, 128, 0, st>>>(g, v, first, list);
-  else k_topo<double><<<count, 128, 0, st>>>(g, v, first, list);
+  if (v.prec) k_topo<float><<<count, 448, 0, st>>>(g, v, first, list);
+  else k_topo<double><<<count, 448, 0, st>>>(g, v, first, list);
   return ok();
 }
 
