@@ -1488,7 +1488,11 @@ int regrid_impl(geoflood_ctx* ctx, int* misses) {
     changed[s] = same ? 0 : 1;
   };
   const auto t_host = std::chrono::steady_clock::now();
-  const int nthreads = std::min(ctx->nscen, std::max(1, std::min(16, (int)std::thread::hardware_concurrency())));
+  // one thread per 4000 leaves: starting a thread takes longer than the trees
+  // of a thousand (16 scenarios of 116-128 leaves: 0.85 ms on 16 threads, 0.08
+  // ms on one)
+  const int nthreads = std::min({ctx->nscen, 1 + ctx->npatch / 4000,
+                                 std::max(1, std::min(16, (int)std::thread::hardware_concurrency()))});
   if (nthreads <= 1) {
     for (int s = 0; s < ctx->nscen; ++s) regrid_one(s);
   } else {
@@ -1605,35 +1609,46 @@ int geoflood_mass(geoflood_ctx* ctx, int s, double* mass) {
   return 0;
 }
 
-int geoflood_set_gauges(geoflood_ctx* ctx, int s, const double* xy, int n) {
-  if (!valid_scen(ctx, s) || n < 0 || n > ctx->cfg.max_gauges || (n > 0 && !xy))
-    return fail(ctx, GEOFLOOD_ERR_ARG, "set_gauges: bad argument");
-  cudaFree(ctx->d_gxy[s]);
-  cudaFree(ctx->d_gout[s]);
-  cudaFree(ctx->d_garr[s]);
-  cudaFree(ctx->d_gref[s]);
-  ctx->d_gxy[s] = ctx->d_gout[s] = ctx->d_garr[s] = nullptr;
-  ctx->d_gref[s] = nullptr;
-  const int m = n > 0 ? n : 1;
-  CK(cudaMalloc(&ctx->d_gxy[s], 2 * m * sizeof(double)));
-  CK(cudaMalloc(&ctx->d_gout[s], 5 * m * sizeof(double)));
-  CK(cudaMalloc(&ctx->d_garr[s], m * sizeof(double)));
-  CK(cudaMalloc(&ctx->d_gref[s], m * sizeof(GfGaugeRef)));
-  if (n > 0)
-    CK(cudaMemcpyAsync(ctx->d_gxy[s], xy, 2 * n * sizeof(double), cudaMemcpyHostToDevice, ctx->st));
-  CK(cudaMemsetAsync(ctx->d_gout[s], 0, 5 * m * sizeof(double), ctx->st));
-  std::vector<double> neg(m, -1.0);
-  CK(cudaMemcpyAsync(ctx->d_garr[s], neg.data(), m * sizeof(double), cudaMemcpyHostToDevice, ctx->st));
+// Buffers for n gauges of scenario s (kept where their number is the same)
+// and its record; the caller uploads the record.
+static int gauge_buffers(geoflood_ctx* ctx, int s, int n) {
   GfScenario& S = ctx->h_scen[s];
+  const int m = n > 0 ? n : 1;
+  if (!ctx->d_gref[s] || S.ngauge != n) {
+    cudaFree(ctx->d_gxy[s]);
+    cudaFree(ctx->d_gout[s]);
+    cudaFree(ctx->d_garr[s]);
+    cudaFree(ctx->d_gref[s]);
+    ctx->d_gxy[s] = ctx->d_gout[s] = ctx->d_garr[s] = nullptr;
+    ctx->d_gref[s] = nullptr;
+    S.ngauge = 0;
+    CK(cudaMalloc(&ctx->d_gxy[s], 2 * m * sizeof(double)));
+    CK(cudaMalloc(&ctx->d_gout[s], 5 * m * sizeof(double)));
+    CK(cudaMalloc(&ctx->d_garr[s], m * sizeof(double)));
+    CK(cudaMalloc(&ctx->d_gref[s], m * sizeof(GfGaugeRef)));
+  }
   S.ngauge = n;
   S.gxy = ctx->d_gxy[s];
   S.gout = ctx->d_gout[s];
   S.garr = ctx->d_garr[s];
   S.gref = ctx->d_gref[s];
-  int rc = upload_scen(ctx);
-  if (rc) return rc;
   ctx->max_gauges_used = 0;
   for (auto& sc : ctx->h_scen) ctx->max_gauges_used = std::max(ctx->max_gauges_used, sc.ngauge);
+  return 0;
+}
+
+int geoflood_set_gauges(geoflood_ctx* ctx, int s, const double* xy, int n) {
+  if (!valid_scen(ctx, s) || n < 0 || n > ctx->cfg.max_gauges || (n > 0 && !xy))
+    return fail(ctx, GEOFLOOD_ERR_ARG, "set_gauges: bad argument");
+  int rc = gauge_buffers(ctx, s, n);
+  if (rc) return rc;
+  const int m = n > 0 ? n : 1;
+  if (n > 0)
+    CK(cudaMemcpyAsync(ctx->d_gxy[s], xy, 2 * n * sizeof(double), cudaMemcpyHostToDevice, ctx->st));
+  CK(cudaMemsetAsync(ctx->d_gout[s], 0, 5 * m * sizeof(double), ctx->st));
+  std::vector<double> neg(m, -1.0);
+  CK(cudaMemcpyAsync(ctx->d_garr[s], neg.data(), m * sizeof(double), cudaMemcpyHostToDevice, ctx->st));
+  if ((rc = upload_scen(ctx))) return rc;
   CK(cudaMemsetAsync(ctx->d_gflag, 0, (size_t)ctx->cap, ctx->st));
   CKL(gf::launch_gauge_refs(ctx->G, view(ctx), ctx->max_gauges_used, ctx->st), "gauge_refs");
   CKL(gf::launch_gauges(ctx->G, view(ctx), 0, ctx->max_gauges_used, ctx->st), "gauges");
@@ -2152,6 +2167,13 @@ struct Reader {
     at += k;
   }
   template <typename T> T val() { T v{}; get(&v, sizeof(T)); return v; }
+  // k bytes in place (any alignment), or null at the end of the record
+  const unsigned char* skip(size_t k) {
+    if (!ok || k > n - at) { ok = false; return nullptr; }
+    const unsigned char* q = p + at;
+    at += k;
+    return q;
+  }
 };
 
 const char kMagic[4] = {'G', 'F', 'C', 'K'};
@@ -2253,14 +2275,15 @@ int geoflood_load(geoflood_ctx* ctx, const void* buf, size_t size) {
   const size_t esz = ctx->prec ? sizeof(float) : sizeof(double);
   struct Scen {
     double manning, eta0;
-    std::vector<std::vector<double>> z;
+    // the large arrays stay in the caller's buffer and are copied from there
+    std::vector<const unsigned char*> z;
     std::vector<int> nx, ny;
     std::vector<double> x0, y0, dx, dy;
     std::vector<gf::Leaf> leaves;
     GfCtl ctl{};
     int ngauge = 0;
     std::vector<double> gxy, gout, garr;
-    std::vector<unsigned char> q, lo;
+    const unsigned char *q = nullptr, *lo = nullptr;
   };
   std::vector<Scen> sc(ctx->nscen);
   size_t total = 0;
@@ -2277,8 +2300,7 @@ int geoflood_load(geoflood_ctx* ctx, const void* buf, size_t size) {
       if (!r.ok || x.nx.back() < 2 || x.ny.back() < 2 ||
           (size_t)x.nx.back() * x.ny.back() * 8 > size)
         return fail(ctx, GEOFLOOD_ERR_ARG, "load: corrupt DEM");
-      x.z.emplace_back((size_t)x.nx.back() * x.ny.back());
-      r.get(x.z.back().data(), x.z.back().size() * 8);
+      x.z.push_back(r.skip((size_t)x.nx.back() * x.ny.back() * 8));
     }
     const int nl = r.val<int>();
     if (!r.ok || nl < 1 || nl > ctx->cap) return fail(ctx, GEOFLOOD_ERR_ARG, "load: corrupt leaf list");
@@ -2302,12 +2324,8 @@ int geoflood_load(geoflood_ctx* ctx, const void* buf, size_t size) {
     r.get(x.gxy.data(), x.gxy.size() * 8);
     r.get(x.gout.data(), x.gout.size() * 8);
     r.get(x.garr.data(), x.garr.size() * 8);
-    x.q.resize((size_t)nl * 3 * TT * esz);
-    r.get(x.q.data(), x.q.size());
-    if (ctx->prec) {
-      x.lo.resize((size_t)nl * 3 * MM * sizeof(float));
-      r.get(x.lo.data(), x.lo.size());
-    }
+    x.q = r.skip((size_t)nl * 3 * TT * esz);
+    if (ctx->prec) x.lo = r.skip((size_t)nl * 3 * MM * sizeof(float));
     total += (size_t)nl;
   }
   const int nprm = gf::cnn_nparam();
@@ -2344,16 +2362,27 @@ int geoflood_load(geoflood_ctx* ctx, const void* buf, size_t size) {
   ctx->generation++;
   // DEMs (stored in priority order already) and beds
   for (int s = 0; s < ctx->nscen; ++s) {
-    for (auto p : ctx->d_dem[s]) cudaFree(p);
-    ctx->d_dem[s].clear();
     GfScenario& S = ctx->h_scen[s];
+    // the device copies of DEMs of the same sizes are overwritten in place
+    bool fits = ctx->d_dem[s].size() == sc[s].z.size() && S.ndem == (int)sc[s].z.size();
+    for (size_t k = 0; fits && k < sc[s].z.size(); ++k)
+      fits = S.dem[k] == ctx->d_dem[s][k] && S.dnx[k] == sc[s].nx[k] && S.dny[k] == sc[s].ny[k];
+    if (!fits) {
+      for (auto p : ctx->d_dem[s]) cudaFree(p);
+      ctx->d_dem[s].clear();
+    }
     S.ndem = 0;
     for (size_t k = 0; k < sc[s].z.size(); ++k) {
+      const size_t bytes = (size_t)sc[s].nx[k] * sc[s].ny[k] * 8;
       double* d = nullptr;
-      if (cudaMalloc(&d, sc[s].z[k].size() * 8) != cudaSuccess)
-        return fail(ctx, GEOFLOOD_ERR_OOM, "load: DEM allocation");
-      ctx->d_dem[s].push_back(d);
-      CK(cudaMemcpyAsync(d, sc[s].z[k].data(), sc[s].z[k].size() * 8, cudaMemcpyHostToDevice, ctx->st));
+      if (fits) {
+        d = ctx->d_dem[s][k];
+      } else {
+        if (cudaMalloc(&d, bytes) != cudaSuccess)
+          return fail(ctx, GEOFLOOD_ERR_OOM, "load: DEM allocation");
+        ctx->d_dem[s].push_back(d);
+      }
+      CK(cudaMemcpyAsync(d, sc[s].z[k], bytes, cudaMemcpyHostToDevice, ctx->st));
       S.dem[k] = d;
       S.dnx[k] = sc[s].nx[k]; S.dny[k] = sc[s].ny[k];
       S.dx0[k] = sc[s].x0[k]; S.dy0[k] = sc[s].y0[k];
@@ -2371,9 +2400,10 @@ int geoflood_load(geoflood_ctx* ctx, const void* buf, size_t size) {
     const GfScenario& S = ctx->h_scen[s];
     const size_t off = (size_t)S.poff;
     void* q = ctx->prec ? (void*)(ctx->qf[0] + off * 3 * TT) : (void*)(ctx->q[0] + off * 3 * TT);
-    CK(cudaMemcpyAsync(q, sc[s].q.data(), sc[s].q.size(), cudaMemcpyHostToDevice, ctx->st));
+    const size_t nl = sc[s].leaves.size();
+    CK(cudaMemcpyAsync(q, sc[s].q, nl * 3 * TT * esz, cudaMemcpyHostToDevice, ctx->st));
     if (ctx->prec)
-      CK(cudaMemcpyAsync(ctx->lof[0] + off * 3 * MM, sc[s].lo.data(), sc[s].lo.size(),
+      CK(cudaMemcpyAsync(ctx->lof[0] + off * 3 * MM, sc[s].lo, nl * 3 * MM * sizeof(float),
                          cudaMemcpyHostToDevice, ctx->st));
     GfCtl& C = ctx->h_ctl[s];
     const GfCtl& X = sc[s].ctl;
@@ -2384,14 +2414,24 @@ int geoflood_load(geoflood_ctx* ctx, const void* buf, size_t size) {
     C.sub_k = 0; C.sub_rej = 0; C.rmax_bits = 0ull;
   }
   if ((rc = sync_ctl_up(ctx))) return rc;
+  // the gauges of every scenario, their stencils located once for all
+  for (int s = 0; s < ctx->nscen; ++s)
+    if ((rc = gauge_buffers(ctx, s, sc[s].ngauge))) return rc;
+  if ((rc = upload_scen(ctx))) return rc;
   for (int s = 0; s < ctx->nscen; ++s) {
-    if ((rc = geoflood_set_gauges(ctx, s, sc[s].gxy.data(), sc[s].ngauge))) return rc;
     if (sc[s].ngauge > 0) {
+      CK(cudaMemcpyAsync(ctx->d_gxy[s], sc[s].gxy.data(), sc[s].gxy.size() * 8,
+                         cudaMemcpyHostToDevice, ctx->st));
       CK(cudaMemcpyAsync(ctx->d_gout[s], sc[s].gout.data(), sc[s].gout.size() * 8,
                          cudaMemcpyHostToDevice, ctx->st));
       CK(cudaMemcpyAsync(ctx->d_garr[s], sc[s].garr.data(), sc[s].garr.size() * 8,
                          cudaMemcpyHostToDevice, ctx->st));
     }
+  }
+  CK(cudaMemsetAsync(ctx->d_gflag, 0, (size_t)ctx->cap, ctx->st));
+  if (ctx->max_gauges_used > 0) {
+    CKL(gf::launch_gauge_refs(ctx->G, view(ctx), ctx->max_gauges_used, ctx->st), "gauge_refs");
+    ctx->launches++;
   }
   // the network
   if (has_net) {
