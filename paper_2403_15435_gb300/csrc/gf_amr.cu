@@ -237,14 +237,14 @@ __device__ void interp_children(const Geo<T>& e, int s, int L, long long ic, lon
       for (int dj = 0; dj < 3; ++dj)
         for (int di = 0; di < 3; ++di)
           if (in[dj][di]) {
-            const double u = nb[dj][di][k + 1] / nb[dj][di][0];
+            const double u = gfk::div_rn(nb[dj][di][k + 1], nb[dj][di][0]);
             lo = fmin(lo, u);
             hi = fmax(hi, u);
           }
       for (int b = 0; b < 2; ++b)
         for (int a = 0; a < 2; ++a)
           if (d[b][a] > drytol) {
-            const double u = m[b][a][k] / d[b][a];
+            const double u = gfk::div_rn(m[b][a][k], d[b][a]);
             if (u < lo || u > hi) split[k] = true;
           }
     }
@@ -255,7 +255,7 @@ __device__ void interp_children(const Geo<T>& e, int s, int L, long long ic, lon
       out[b0][a0][0] = hf;
       for (int k = 0; k < 2; ++k)
         out[b0][a0][k + 1] = !split[k] ? m[b0][a0][k]
-                                       : (S > 0.0 ? (4.0 * qc[k + 1]) * (hf / S) : 0.0);
+                                       : (S > 0.0 ? (4.0 * qc[k + 1]) * gfk::div_rn(hf, S) : 0.0);
       if (hf <= drytol) {
         out[b0][a0][1] = 0.0;
         out[b0][a0][2] = 0.0;
@@ -838,36 +838,56 @@ __device__ __forceinline__ bool wet_f32(const GfGeom& G, float w, float b) {
 }
 
 // interp_children in FP32: out[b][a] = (w, hu, hv) of child (2 ic + a,
-// 2 jc + b) of level L, whose bed is bs[b][a].
+// 2 jc + b) of level L, whose bed is bs[b][a].  own >= 0: the children are
+// ghost cells of patch own (level L), child (0, 0) at its local cell (li, lj);
+// the neighbours that lie in that patch are the means of its own cells, found
+// without lookups (three of the nine along a side).
 __device__ void interp_children_f32(const Geo<float>& e, int s, int cur, int L, long long ic,
                                     long long jc, const float (&bs)[2][2],
-                                    float (&out)[2][2][3], int* err) {
+                                    float (&out)[2][2][3], int* err, int own = -1, int li = 0,
+                                    int lj = 0) {
   const GfGeom& G = e.G;
   const long long NXc = e.nx(L - 1), NYc = e.ny(L - 1);
   float nb[3][3][4];
   bool in[3][3], wt[3][3];
-  // the neighbourhood in three straight-line passes, so that the loads of
-  // the nine cells overlap: the leaves of level L - 1 holding them, the
-  // values of those found, then the others (surf_near_f32's rarer cases)
+  // the neighbourhood in straight-line passes, so that the loads of the nine
+  // cells overlap: the cells of the own patch, the leaves of level L - 1
+  // holding the others, the values of those found, then the rest
+  // (surf_near_f32)
   int pl[3][3];
+  constexpr int OWN = -2;
 #pragma unroll
   for (int dj = 0; dj < 3; ++dj)
 #pragma unroll
     for (int di = 0; di < 3; ++di) {
       const long long x = ic + di - 1, y = jc + dj - 1;
       in[dj][di] = x >= 0 && y >= 0 && x < NXc && y < NYc;
-      pl[dj][di] = in[dj][di] ? e.leaf(s, L - 1, x, y) : -1;
+      const bool mine = own >= 0 && (unsigned)(li + 2 * (di - 1)) < (unsigned)G.M &&
+                        (unsigned)(lj + 2 * (dj - 1)) < (unsigned)G.M;
+      pl[dj][di] = mine ? OWN : (in[dj][di] ? e.leaf(s, L - 1, x, y) : -1);
     }
 #pragma unroll
   for (int dj = 0; dj < 3; ++dj)
 #pragma unroll
     for (int di = 0; di < 3; ++di)
-      if (pl[dj][di] >= 0) load_surf(e, pl[dj][di], cur, e.local(ic + di - 1, jc + dj - 1), nb[dj][di]);
+      if (pl[dj][di] == OWN) {
+        // patch origins are even: the four cells are two 8-byte pairs
+        const int c = e.tix(li + 2 * (di - 1), lj + 2 * (dj - 1)), TT = G.T * G.T;
+        const float* q = e.V.qf[cur] + (size_t)own * 3 * TT + c;
+        const float* bo = e.V.bf + (size_t)own * TT + c;
+#pragma unroll
+        for (int f = 0; f < 4; ++f) {
+          const float* v = f < 3 ? q + f * TT : bo;
+          const float2 a = *reinterpret_cast<const float2*>(v);
+          const float2 b = *reinterpret_cast<const float2*>(v + G.T);
+          nb[dj][di][f] = 0.25f * ((a.x + a.y) + (b.x + b.y));
+        }
+      } else if (pl[dj][di] >= 0) load_surf(e, pl[dj][di], cur, e.local(ic + di - 1, jc + dj - 1), nb[dj][di]);
 #pragma unroll
   for (int dj = 0; dj < 3; ++dj)
 #pragma unroll
     for (int di = 0; di < 3; ++di) {
-      if (in[dj][di] && pl[dj][di] < 0)
+      if (in[dj][di] && pl[dj][di] == -1)
         surf_near_f32(e, s, cur, L - 1, ic + di - 1, jc + dj - 1, nb[dj][di], err);
       wt[dj][di] = in[dj][di] && wet_f32(G, nb[dj][di][0], nb[dj][di][3]);
     }
@@ -995,6 +1015,59 @@ __device__ void fill_cell_f32(const Geo<float>& e, int s, int cur, int L, long l
   }
 }
 
+// (w, hu, hv) of a cell (the mean of four finer cells on leaves of level
+// L + 1, or else whatever fill_cell_f32 finds): fill_cell_f32's usual case
+// for a region next to finer leaves, its general form out of line.
+struct Cell3 {
+  float v[3];
+  int err;
+};
+__device__ __noinline__ Cell3 fill_cell_call(const GfGeom* G, const GfView* V, int s, int cur,
+                                             int L, long long I, long long J, float b00,
+                                             float b01, float b10, float b11) {
+  const Geo<float> e(*G, *V);
+  const float bs[2][2] = {{b00, b01}, {b10, b11}};
+  Cell3 r{};
+  fill_cell_f32(e, s, cur, L, I, J, bs, r.v, &r.err);
+  return r;
+}
+__device__ __forceinline__ void fill_finer_f32(const Geo<float>& e, int s, int cur, int L,
+                                               long long I, long long J,
+                                               const float (&bs)[2][2], float (&out)[3],
+                                               int* err) {
+  int pc[4];
+#pragma unroll
+  for (int ch = 0; ch < 4; ++ch) pc[ch] = e.leaf(s, L + 1, 2 * I + (ch & 1), 2 * J + (ch >> 1));
+  // a leaf of level L + 1 covers the cell or none does
+  if (min(min(pc[0], pc[1]), min(pc[2], pc[3])) < 0) {
+    const Cell3 r = fill_cell_call(&e.G, &e.V, s, cur, L, I, J, bs[0][0], bs[0][1], bs[1][0],
+                                   bs[1][1]);
+#pragma unroll
+    for (int f = 0; f < 3; ++f) out[f] = r.v[f];
+    if (r.err) *err = 1;
+    return;
+  }
+  const float bt = bs[J & 1][I & 1];
+  float v[4][4];
+#pragma unroll
+  for (int ch = 0; ch < 4; ++ch)
+    load_surf(e, pc[ch], cur, e.local(2 * I + (ch & 1), 2 * J + (ch >> 1)), v[ch]);
+  bool all = true;
+#pragma unroll
+  for (int ch = 0; ch < 4; ++ch) all = all && wet_f32(e.G, v[ch][0], v[ch][3]);
+#pragma unroll
+  for (int f = 1; f < 3; ++f) out[f] = 0.25f * ((v[0][f] + v[1][f]) + (v[2][f] + v[3][f]));
+  if (all) {
+    const float w = 0.25f * ((v[0][0] + v[1][0]) + (v[2][0] + v[3][0]));
+    out[0] = w > bt ? w : bt;
+  } else {
+    float h[4];
+#pragma unroll
+    for (int ch = 0; ch < 4; ++ch) h[ch] = v[ch][0] - v[ch][3];
+    out[0] = 0.25f * ((h[0] + h[1]) + (h[2] + h[3])) + bt;
+  }
+}
+
 // Store (w, hu, hv) into ghost cell (i, j) of patch P's tile q (bed bt),
 // then mark and mirror as store_ghost does.
 __device__ void store_ghost_f32(const Geo<float>& e, const GfView& V, float* q,
@@ -1007,6 +1080,11 @@ __device__ void store_ghost_f32(const Geo<float>& e, const GfView& V, float* q,
   mark_and_mirror(e, V, q, P, p, i, j, out[0] > bt);
 }
 
+// Threads per CTA of the level-change ghosts: a warp's path is long (some
+// thousand instructions, few of them shared between warps that wait for the
+// same fetch), so few warps to an SM.
+#define GF_GHOST_NT 64
+
 // Ghost cells of regions without a same-level neighbour, after each step.
 // regs[0, nquad) are regions next to a coarser leaf: one thread per 2 x 2
 // block of ghost cells (the children of one coarser cell, interpolated
@@ -1016,21 +1094,23 @@ __device__ void store_ghost_f32(const Geo<float>& e, const GfView& V, float* q,
 // 1 right, 2 bottom, 3 top (2 x M cells each), 4-7 the corners (2 x 2).
 // F32: the FP32 operators above (FP32 forests without subcycling).
 template <typename T, bool F32>
-__global__ void __launch_bounds__(256, 1) k_ghost_other(const __grid_constant__ GfGeom G, const __grid_constant__ GfView V,
+__global__ void __launch_bounds__(GF_GHOST_NT, 1) k_ghost_other(const __grid_constant__ GfGeom G, const __grid_constant__ GfView V,
                               const int* regs, int nquad, int nreg, int* errflag) {
-  const int M = G.M;
-  const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const long long nq_items = (long long)nquad * (M / 2);
+  // M is 16 or 32: the item's region and place by shifts (64-bit divisions
+  // are some 70 instructions each, of a path whose length is its time)
+  const int M = G.M, sh = M == 32 ? 4 : 3;
+  const unsigned idx = blockIdx.x * blockDim.x + threadIdx.x;
+  const unsigned nq_items = (unsigned)nquad << sh;
   const bool quad = idx < nq_items;
   int code, k;
   if (quad) {
-    code = regs[idx / (M / 2)];
-    k = (int)(idx % (M / 2));
+    code = regs[idx >> sh];
+    k = (int)(idx & ((1u << sh) - 1u));
   } else {
-    const long long r2 = idx - nq_items;
-    if (r2 >= (long long)(nreg - nquad) * 2 * M) return;
-    code = regs[nquad + r2 / (2 * M)];
-    k = (int)(r2 % (2 * M));
+    const unsigned r2 = idx - nq_items;
+    if (r2 >= (unsigned)(nreg - nquad) << (sh + 2)) return;
+    code = regs[nquad + (r2 >> (sh + 2))];
+    k = (int)(r2 & ((4u << sh) - 1u));
   }
   const int p = code >> 3, r = code & 7;
   int i, j;
@@ -1072,7 +1152,7 @@ __global__ void __launch_bounds__(256, 1) k_ghost_other(const __grid_constant__ 
     int err = 0;
     if (quad) {
       float out4[2][2][3];
-      interp_children_f32(e, P.scen, cur, P.level, I >> 1, J >> 1, bs, out4, &err);
+      interp_children_f32(e, P.scen, cur, P.level, I >> 1, J >> 1, bs, out4, &err, p, i, j);
       if (err && errflag) *errflag = 1;
       for (int b = 0; b < 2; ++b)
         for (int a = 0; a < 2; ++a)
@@ -1080,7 +1160,7 @@ __global__ void __launch_bounds__(256, 1) k_ghost_other(const __grid_constant__ 
       return;
     }
     float out[3];
-    fill_cell_f32(e, P.scen, cur, P.level, I, J, bs, out, &err);
+    fill_finer_f32(e, P.scen, cur, P.level, I, J, bs, out, &err);
     if (err && errflag) *errflag = 1;
     store_ghost_f32(e, V, q, P, p, i, j, out, bs[j & 1][i & 1]);
     return;
@@ -2131,12 +2211,12 @@ int launch_ghost_rest(const GfGeom& g, const GfView& v, const int* regs, int nqu
   if (nreg <= 0) return 0;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const long long total = (long long)nquad * (g.M / 2) + (long long)(nreg - nquad) * 2 * g.M;
-  const int blocks = (int)((total + 255) / 256);
+  const int blocks = (int)((total + GF_GHOST_NT - 1) / GF_GHOST_NT);
   if (v.prec && !g.subcycle)
-    k_ghost_other<float, true><<<blocks, 256, 0, st>>>(g, v, regs, nquad, nreg, g_errflag);
+    k_ghost_other<float, true><<<blocks, GF_GHOST_NT, 0, st>>>(g, v, regs, nquad, nreg, g_errflag);
   else if (v.prec)
-    k_ghost_other<float, false><<<blocks, 256, 0, st>>>(g, v, regs, nquad, nreg, g_errflag);
-  else k_ghost_other<double, false><<<blocks, 256, 0, st>>>(g, v, regs, nquad, nreg, g_errflag);
+    k_ghost_other<float, false><<<blocks, GF_GHOST_NT, 0, st>>>(g, v, regs, nquad, nreg, g_errflag);
+  else k_ghost_other<double, false><<<blocks, GF_GHOST_NT, 0, st>>>(g, v, regs, nquad, nreg, g_errflag);
   return ok();
 }
 
