@@ -160,16 +160,27 @@ GF_HD double dmax(double a, double b) { return dlt(b, a) ? a : b; }
 GF_HD bool above(double h, double d) {
   return (unsigned long long)(dbits(h) - dbits(d) - 1) < (unsigned long long)(D_INF - dbits(d));
 }
-// x / 2 and 2 x by the exponent (native where it is at the range's ends)
+// x / 2 and 2 x by the exponent, at the ends of the range too (a product
+// there, however rare, would take a slot of the FP64 pipe each time: the
+// compiler predicates it)
 GF_HD double half(double x) {
-  const int e = (int)(dbits(x) >> 52) & 0x7ff;
-  if ((unsigned)(e - 2) < 2045u) return bitsd(dbits(x) - D_HID);
-  return 0.5 * x;
+  const long long b = dbits(x), m = b & 0x7fffffffffffffffll;
+  // below twice the smallest normal number: the significand halved, to even
+  const long long lo = (m >> 1) + ((m & 3) == 3 ? 1 : 0);
+  const long long hi = m >= D_INF ? m : m - D_HID;
+  return bitsd((m < 2 * D_HID ? lo : hi) | (b & (long long)0x8000000000000000ull));
 }
 GF_HD double twice(double x) {
-  const int e = (int)(dbits(x) >> 52) & 0x7ff;
-  if ((unsigned)(e - 1) < 2045u) return bitsd(dbits(x) + D_HID);
-  return 2.0 * x;
+  const long long b = dbits(x), m = b & 0x7fffffffffffffffll;
+  const long long hi = m >= D_INF - D_HID ? (m > D_INF ? m : D_INF) : m + D_HID;
+  return bitsd((m < D_HID ? 2 * m : hi) | (b & (long long)0x8000000000000000ull));
+}
+// Marks a rare branch: keeps the compiler from executing its FP64 operations
+// under a predicate (each would take its slot of the FP64 pipe all the same).
+GF_HD void rare() {
+#ifdef __CUDACC__
+  asm volatile("");
+#endif
 }
 
 }  // namespace gfk

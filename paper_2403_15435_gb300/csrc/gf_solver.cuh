@@ -382,9 +382,11 @@ __device__ __forceinline__ void riemann_prim(Prim l, Prim r, double g, double (&
     s1 = dmin(l.u - l.c, uhat - chat);
     s3 = dmax(r.u + r.c, uhat + chat);
   } else if (pl) {
+    rare();
     s1 = l.u - l.c;
     s3 = l.u + twice(l.c);
   } else {
+    rare();
     s1 = r.u - twice(r.c);
     s3 = r.u + r.c;
   }
@@ -405,6 +407,7 @@ __device__ __forceinline__ void riemann_prim(Prim l, Prim r, double g, double (&
     const bool inside = xf > 1e-25f && df * trunc_f32(s1) < 0.9999f * xf &&
                         df * trunc_f32(s3) < 0.9999f * xf;
     if (!inside) {
+      rare();
       const double lo = div_rn(x, s1), hi = div_rn(x, s3);
       if (dlt(dhs, lo)) { dhs = lo; clamped = true; }
       if (dlt(hi, dhs)) { dhs = hi; clamped = true; }
@@ -419,7 +422,10 @@ __device__ __forceinline__ void riemann_prim(Prim l, Prim r, double g, double (&
     if (dlt(r.h, dhs)) { dhs = r.h; clamped = true; }
   }
   double d1 = deta;
-  if (clamped) d1 = (r.h - l.h) - dhs;
+  if (clamped) {
+    rare();
+    d1 = (r.h - l.h) - dhs;
+  }
   const double d3 = (r.n * r.u - l.n * l.u) + ghb * deta;
   const double b1 = div_rn(s3 * d1 - dn, den);
   const double b3 = div_rn(dn - s1 * d1, den);
@@ -476,6 +482,7 @@ __device__ __forceinline__ void edge_fluxes_prim(const double* Z, const double* 
     ap[1] = n2 ? z[6] : x1;
     ap[2] = n2 ? z[7] : x2;
   } else {
+    rare();
     const double wm[3] = {neg(s[0]) ? 1.0 : (iszero(s[0]) ? 0.5 : 0.0),
                           n2 ? 1.0 : (iszero(s[1]) ? 0.5 : 0.0),
                           neg(s[2]) ? 1.0 : (iszero(s[2]) ? 0.5 : 0.0)};
@@ -543,6 +550,7 @@ __device__ __forceinline__ void tsplit_prim(double w, double z, double c, double
     p[0] = W3[0]; p[1] = W3[1]; p[2] = pos(w) ? x : W3[2];
     q[0] = W1[0]; q[1] = W1[1]; q[2] = neg(w) ? x : W1[2];
   } else {
+    rare();
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
       p[k] = (pos(l1) ? W1[k] : 0.0) + (pos(l3) ? W3[k] : 0.0);

@@ -257,6 +257,8 @@ extern "C" int geoflood_step_tiles_noalloc(const double* q_in, const double* b,
   G.mi = 1; G.mj = 1; G.M = mx; G.T = mx + 2 * GF_NG;
   G.xlower = 0.0; G.xupper = dx * mx;
   G.ylower = 0.0; G.yupper = dy * mx;
+  G.dxl[0] = G.xupper / mx;
+  G.dyl[0] = G.yupper / mx;
   G.g = g; G.drytol = drytol;
   G.cfl_desired = 0.9; G.cfl_max = 1.0; G.dt_max = 1e300;
   G.nscen = 1;

@@ -379,7 +379,7 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
   const bool subc = G.subcycle != 0;
   const int per = subc ? 1 << (G.maxlevel - Pt.level) : 1;
   const int cur = subc ? H.cur ^ ((C->sub_k / per) & 1) : H.cur;
-  const double dtp = subc ? (H.dt / (double)G.sub_K) * (double)per : H.dt;
+  const double dtp = subc ? (gfk::div_rn(H.dt, (double)G.sub_K)) * (double)per : H.dt;
   const R* qs;
   R* qd;
   const R* bs;
@@ -485,14 +485,11 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
       fscal[0] = G.drytolf;
       fscal[1] = G.marginf;
     } else {
-      const long long NXL = (long long)G.mi * MP << Pt.level;
-      const long long NYL = (long long)G.mj * MP << Pt.level;
-      const double dx0 = (G.xupper - G.xlower) / (double)NXL;
-      const double dy0 = (G.yupper - G.ylower) / (double)NYL;
+      const double dx0 = G.dxl[Pt.level], dy0 = G.dyl[Pt.level];
       scal[0] = dx0;
       scal[1] = dy0;
-      scal[2] = dtp / dx0;
-      scal[3] = dtp / dy0;
+      scal[2] = gfk::div_rn(dtp, dx0);
+      scal[3] = gfk::div_rn(dtp, dy0);
       rscal[0] = (R)G.g;
       rscal[1] = (R)G.drytol;
       rscal[2] = (R)scal[2];
@@ -1384,7 +1381,7 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
         const R tf = trv ? nux * (fa[3 + f] - fa[f]) + nuy * (ga[3 + f] - ga[f]) : R(0);
         o[f] = (q[f] - fl) - tf;
       }
-      if (gfk::neg(o[0])) { clipd -= o[0]; o[0] = R(0); ++nclip; }
+      if (gfk::neg(o[0])) { gfk::rare(); clipd -= o[0]; o[0] = R(0); ++nclip; }
       const bool wnew = gfk::above(o[0], rdry);
       if (wnew && gfk::pos(mn)) {
         const R u = gfk::div_rn(o[1], o[0]), v = gfk::div_rn(o[2], o[0]);
@@ -1494,13 +1491,12 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
       double mx = 0.0, my = 0.0;
       unsigned nw = 0u;
       for (int w = 0; w < NW; ++w) {
-        mx = red[w] > mx ? red[w] : mx;
-        my = red[NW + w] > my ? red[NW + w] : my;
+        mx = gfk::dmax(red[w], mx);
+        my = gfk::dmax(red[NW + w], my);
         nw += redu[w];
       }
-      const double cx = mx / dx, cy = my / dy;
-      double cm = cx > cy ? cx : cy;
-      if (subc) cm = cm * (double)per / (double)G.sub_K;  // cmax / n_L
+      double cm = gfk::dmax(gfk::div_rn(mx, dx), gfk::div_rn(my, dy));
+      if (subc) cm = gfk::div_rn(cm * (double)per, (double)G.sub_K);  // cmax / n_L
       atomicMax(&C->cmax_bits, (unsigned long long)__double_as_longlong(cm));
       if (nw) atomicAdd(&C->wet_updates, (unsigned long long)nw);
     }
@@ -1552,7 +1548,7 @@ static __device__ void subcycle_finish(const GfGeom& G, const GfView& V, GfCtl* 
   if (sub_rej) {
     Cp->accepted = 0;
   } else if (k == 0 && DT * rate > G.cfl_max) {
-    dtn = G.cfl_desired / rate;
+    dtn = gfk::div_rn(G.cfl_desired, rate);
     Cp->dt_next = dtn;
     Cp->rejects = rejects + 1;
     Cp->accepted = 0;
@@ -1591,7 +1587,7 @@ static __device__ void subcycle_finish(const GfGeom& G, const GfView& V, GfCtl* 
       const double r = __longlong_as_double((long long)rb);
       rb = 0ull;
       if (r > 0.0) {
-        const double dn = G.cfl_desired / r;
+        const double dn = gfk::div_rn(G.cfl_desired, r);
         dtn = dn < G.dt_max ? dn : G.dt_max;
         Cp->dt_next = dtn;
       }
@@ -1645,7 +1641,7 @@ static __device__ void ctl_finish(const GfGeom& G, GfCtl* Cp, unsigned long long
   double tn = t, dtn = dt_next0;
   long long tk = taken;
   if (dt * cmax > G.cfl_max) {
-    dtn = G.cfl_desired / cmax;
+    dtn = gfk::div_rn(G.cfl_desired, cmax);
     Cp->dt_next = dtn;
     Cp->rejects = rejects + 1;
     Cp->accepted = 0;
@@ -1671,7 +1667,7 @@ static __device__ void ctl_finish(const GfGeom& G, GfCtl* Cp, unsigned long long
     Cp->step_clipvol = 0.0;
     Cp->accepted = 1;
     if (cmax > 0.0) {
-      const double dn = G.cfl_desired / cmax;
+      const double dn = gfk::div_rn(G.cfl_desired, cmax);
       dtn = dn < G.dt_max ? dn : G.dt_max;
       Cp->dt_next = dtn;
     }
