@@ -350,9 +350,10 @@ int geoflood_counters(geoflood_ctx* ctx, int scenario, long long* cell_updates,
  * ms_per_variant (one entry per variant, at most 16: eight for 32 x 32
  * patches in FP32, four in FP64, one for 16 x 16; either pointer may be
  * NULL).  Variants of 32 x 32 patches, FP64 (CTAs of sub-tiles with their
- * two-cell halo): 0 = 8 x 8 or, from 39 patches on, 16 x 16 sub-tiles (192
- * threads), 1 = 16 x 16 (256 threads), 2 = 8 x 8 (128 threads), 3 = 16 x 16
- * (352 threads).  FP32: 0 = by the forest's size 8 x 8 (up to 38 patches) or
+ * two-cell halo): 0 = by the forest's size 8 x 8 (256
+ * threads, up to 38 patches) or 16 x 16 sub-tiles (256 threads up to 152
+ * patches, 192 beyond), 1 = 16 x 16 (256 threads), 2 = 8 x 8 (256 threads), 3 =
+ * 16 x 16 (352 threads).  FP32: 0 = by the forest's size 8 x 8 (up to 38 patches) or
  * 16 x 16 (up to 152) sub-tiles or whole tiles staged by TMA bulk copies (320
  * threads, two CTAs per SM), 1 = 16 x 16 sub-tiles (192 threads, four CTAs per
  * SM), 2 = whole tiles (640 threads), 3 = whole tiles (320 threads, one CTA

@@ -21,8 +21,12 @@
 
 #ifdef __CUDACC__
 #define GF_HD __device__ __forceinline__
+// out of line: a quotient or root is some sixty instructions, and the FP64
+// kernels hold dozens of them
+#define GF_HD_CALL static __device__ __noinline__
 #else
 #define GF_HD inline
+#define GF_HD_CALL inline
 #endif
 
 namespace gfk {
@@ -75,7 +79,7 @@ constexpr long long D_INF = 0x7ffll << 52;
 // remainder stays below 2^55 and the last digit (15 bits) is within 0.6 of
 // the exact one: the sign of the last remainder says whether the 56-bit
 // quotient is one too large, and whether it is zero is the sticky bit.
-GF_HD double div_rn(double a, double b) {
+GF_HD_CALL double div_rn(double a, double b) {
   const long long ab = dbits(a), bb = dbits(b);
   const int ea = (int)(ab >> 52) & 0x7ff, eb = (int)(bb >> 52) & 0x7ff;
   const int e = ea - eb;
@@ -111,7 +115,7 @@ GF_HD double div_rn(double a, double b) {
 // residual times half an FP32 reciprocal square root.  The last digit is
 // within 0.6 of the exact one, so the residual's sign gives the floor of the
 // 54-bit root; a root is never halfway between two results.
-GF_HD double sqrt_rn(double x) {
+GF_HD_CALL double sqrt_rn(double x) {
   const long long xb = dbits(x);
   const int ex = (int)(xb >> 52);  // sign included: negative values fall out
   if ((unsigned)(ex - 1) < 2046u) {

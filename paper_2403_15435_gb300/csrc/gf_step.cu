@@ -71,8 +71,8 @@ __global__ void k_wait_check(int* out, unsigned limit) {
 namespace gf {
 
 // Kernel variants (the autotuner picks one per context).  FP64, 32 x 32
-// patches: 0 = by the rule of use_small_tiles, 8 x 8 sub-tiles or 16 x 16
-// sub-tiles in 192-thread CTAs, three per SM; 1 = 16 x 16 sub-tiles in
+// patches: 0 = by the forest's size, 8 x 8 sub-tiles (use_small_tiles) or 16 x
+// 16 sub-tiles in 256-thread CTAs, two per SM, or in 192-thread CTAs, three; 1 = 16 x 16 sub-tiles in
 // 256-thread CTAs, two per SM; 2 = 8 x 8 sub-tiles; 3 = 16 x 16 sub-tiles in
 // 352-thread CTAs.  16 x 16 patches have the single variant 0.  Dimensionally
 // split stepping has one kernel per patch size (whole-patch CTAs).
@@ -81,12 +81,13 @@ int patch_step_variants(int mx, int prec, int dim_split) {
 }
 
 // FP64 sub-tile size.  8 x 8 sub-tiles do 1.2 times the FP64 work of 16 x 16
-// ones (more halo edges per cell) but four times the CTAs share it, so they
-// win while all of them are resident at once: 152 SMs x 4 CTAs.  Measured, us
-// per step with every cell wet, 8 x 8 against 16 x 16: 16 patches of 32 x 32
-// (256 CTAs of 8 x 8) 44 against 68, 36 patches (576 CTAs) 62 against 70, 64
-// patches (1024 CTAs) 127 against 93, 256 patches 372 against 312; 144
-// patches of 16 x 16 (576 CTAs) 62 against 71, 256 patches 126 against 92.
+// ones (more halo edges per cell) but four times the CTAs share it, and their
+// two sweeps run side by side, so they win while all of them are resident at
+// once: 152 SMs x 4 CTAs.  Measured, us per step with every cell wet, 8 x 8
+// against 16 x 16: 4 patches of 32 x 32 (64 CTAs of 8 x 8) 28 against 68, 16
+// patches 37 against 68, 36 patches (576 CTAs) 67 against 67 (a third wet 42
+// against 72), 64 patches (1024 CTAs) 120 against 92, 256 patches 399 against
+// 298; 64 patches of 16 x 16 36 against 71, 144 patches (576 CTAs) 66 against 71.
 static bool use_small_tiles(int npatch, int mx) {
   return (long long)npatch * (mx / 8) * (mx / 8) <= 152 * 4;
 }
@@ -102,14 +103,19 @@ int launch_patch_step_f64(const GfGeom& g, const GfView& v, int variant,
   }
   const bool small = use_small_tiles(v.npatch, g.M);
   if (g.M == 32) {
-    if (variant == 1) return gfs::launch_step<gfs::PrecF64, 32, 16, 256, 2>(g, v, st);
+    // 16 x 16 sub-tiles of up to 152 patches fit two to an SM in two rounds
+    // with 256 threads; three 192-thread CTAs per SM are ahead on larger
+    // forests (121 patches 170 against 199 us a step, 1024 patches 1064
+    // against 988)
+    if (variant == 1 || (variant == 0 && !small && v.npatch * 4 <= 152 * 4))
+      return gfs::launch_step<gfs::PrecF64, 32, 16, 256, 2>(g, v, st);
     if (variant == 2 || (variant == 0 && small))
-      return gfs::launch_step<gfs::PrecF64, 32, 8, 128, 4>(g, v, st);
+      return gfs::launch_step<gfs::PrecF64, 32, 8, 256, 2>(g, v, st);
     if (variant == 3) return gfs::launch_step<gfs::PrecF64, 32, 16, 352, 1>(g, v, st);
     return gfs::launch_step<gfs::PrecF64, 32, 16, 192, 3>(g, v, st);
   }
   if (g.M == 16) {
-    if (small) return gfs::launch_step<gfs::PrecF64, 16, 8, 128, 4>(g, v, st);
+    if (small) return gfs::launch_step<gfs::PrecF64, 16, 8, 256, 2>(g, v, st);
     return gfs::launch_step<gfs::PrecF64, 16, 16, 256, 2>(g, v, st);
   }
   return -1;

@@ -255,7 +255,10 @@ struct Layout {
       DS ? 0 : (FAST ? sizeof(R) * 3 * M * (M + 4) : sizeof(R) * 3 * M * (M + 1));
   // byte offsets in dynamic shared memory
   static constexpr size_t OFF_W = sizeof(R) * NF * TT;
-  static constexpr size_t OFF_F = OFF_W + sizeof(R) * NWP * NEDGE;
+  // FP64 8 x 8 sub-tiles: half the threads take the x sweep while the others
+  // take the y sweep, each half with wave planes of its own
+  static constexpr bool BOTH = PRIM && M == 8;
+  static constexpr size_t OFF_F = OFF_W + sizeof(R) * NWP * NEDGE * (BOTH ? 2 : 1);
   static constexpr size_t OFF_G = OFF_F + TRB;
   static constexpr size_t OFF_RED = align16(OFF_G + TRB);
   static constexpr size_t OFF_NB = OFF_RED + sizeof(double) * 64;  // 8 ints
@@ -298,10 +301,12 @@ __device__ __forceinline__ void cell_item(int k, int dir, int& a, int& line) {
 // FP64 (unsplit): the FP64 pipe (two operations per SM and clock) bounds the
 // step, so the body computes a cell's velocities, celerity and root of the
 // depth once (not once per edge side) and leaves only additions and products
-// to that pipe (gf_fp64.cuh).  1024 x 1024 radial dam break, 36 % wet: 1770
-// FP64-pipe operations per wet cell before, 548 after; 1060 us per step
-// before, 507 after (ncu: FP64 pipe 82 % busy before, 66 % after, the rest
-// barrier waits between the phases).
+// to that pipe (gf_fp64.cuh).  Both sweeps share one copy of the code and the
+// quotients and roots are calls, since instruction fetch shows too; 8 x 8
+// sub-tiles take both sweeps at once.  1024 x 1024 radial dam break, 36 % wet:
+// 1770 -> 520 FP64-pipe operations per wet cell, 1060 -> 470 us per step (ncu:
+// FP64 pipe 82 % busy before, 65 % after, the rest barrier waits between the
+// phases); a 64 x 64 basin 270 -> 30 us per step.
 //
 // FP32 (unsplit): bound by issue slots and by the tile's chain of barriers
 // (115 KB of shared memory allow two whole tiles per SM).  A thread takes two
@@ -679,7 +684,7 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
   }
 
   R X[FAST ? 1 : RC][3];   // nu_x * dQx of owned interior cells
-  R Y[FAST ? 1 : RC][3];   // nu_y * dQy
+  R Y[FAST || PRIM ? 1 : RC][3];   // nu_y * dQy (PRIM: added to X)
   // dimensional splitting, deviation form: compensation terms of the
   // intermediate state of owned interior cells
   float LO1[DS && DEV ? RC : 1][3];
@@ -961,6 +966,164 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
     }
     }
   };
+  // PRIM: one sweep, the direction a run-time value so that both sweeps share
+  // one copy of the code (this kernel's instruction fetch shows in its time).
+  // ht: the thread's number among the HN that take this sweep; Wd: their
+  // wave planes.  Every thread of the CTA passes the same barriers.
+  constexpr bool BOTH = Lo::BOTH;
+  constexpr int HN = BOTH ? NT / 2 : NT;
+  [[maybe_unused]] auto sweep64 = [&](const int dir, const int ht, R* const Wd) {
+    if constexpr (PRIM) {
+    constexpr int NRL = M + 2;
+    constexpr int RL6 = (NRL * (M + 1) + HN - 1) / HN;
+    constexpr int RX6 = (M * NRL + HN - 1) / HN;
+    const bool xs = dir == 0;
+    const int CS = xs ? 1 : Lo::T, CL = xs ? Lo::T : 1;  // tile steps along, across
+    const R* sn = xs ? shu : shv;  // normal momentum
+    const R* st = xs ? shv : shu;  // transverse momentum
+    const R* un = xs ? su : sv;
+    const R* ut = xs ? sv : su;
+    const R nu = xs ? nux : nuy;
+    // tile cell (position a along the sweep, line across it)
+    auto at = [&](int a, int line) { return tix<M>(0, 0) + a * CS + line * CL; };
+    // phase 1: Riemann solves on the lines -1..M, edges -1..M+1
+    for (int k = ht; k < NRL * NE; k += HN) {
+      const int line = (xs ? k / NE : k % NRL) - 1;
+      const int a = (xs ? k % NE : k / NRL) - 1;
+      const int cr = at(a, line), cl = cr - CS;
+      R* w = Wd + ((line + 1) * NE + a + 1);
+      double z[8], S[3];
+      gfk::riemann_prim(gfk::Prim{s0[cl], sn[cl], st[cl], sb[cl], seta[cl], un[cl], ut[cl],
+                                  sc[cl], sq[cl], wetc(cl)},
+                        gfk::Prim{s0[cr], sn[cr], st[cr], sb[cr], seta[cr], un[cr], ut[cr],
+                                  sc[cr], sq[cr], wetc(cr)},
+                        g, z, S);
+#pragma unroll
+      for (int q = 0; q < 8; ++q) w[q * NEDGE] = z[q];
+#pragma unroll
+      for (int q = 0; q < 3; ++q) w[(8 + q) * NEDGE] = S[q];
+    }
+    __syncthreads();
+    // phase 2: fluctuations and limited corrections on edges 0..M
+    R AMr[RL6][3], APr[RL6][3], FFr[RL6][3];
+    R smax = R(0);
+#pragma unroll
+    for (int r = 0; r < RL6; ++r) {
+      const int k = ht + r * HN;
+      if (k < NRL * (M + 1)) {
+        const int line = k / (M + 1) - 1, a = k % (M + 1);
+        const R* w = Wd + ((line + 1) * NE + a + 1);
+        const int cr = at(a, line);
+        const bool wet = corr && wetc(cr - CS) && wetc(cr);
+        gfk::edge_fluxes_prim<NEDGE>(w, w - 1, w + 1, nu, wet, AMr[r], APr[r], FFr[r]);
+        // |s| of the outer waves (the middle speed is their mean)
+        if (line >= 0 && line < M)
+          smax = gfk::dmax(smax, gfk::dmax(gfk::dabs(w[8 * NEDGE]), gfk::dabs(w[10 * NEDGE])));
+      }
+    }
+    if (xs) smx = gfk::dmax(smx, smax);
+    else smy = gfk::dmax(smy, smax);
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < RL6; ++r) {
+      const int k = ht + r * HN;
+      if (k < NRL * (M + 1)) {
+        R* w = Wd + ((k / (M + 1)) * NE + k % (M + 1) + 1);
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+          w[q * NEDGE] = AMr[r][q];
+          w[(3 + q) * NEDGE] = APr[r][q];
+          w[(6 + q) * NEDGE] = FFr[r][q];
+        }
+      }
+    }
+    __syncthreads();
+    // phase 3: per-cell increments and their transverse split
+    R* Tr = xs ? Gtr : Ftr;
+    R MIr[RX6][3];
+    R Yb[BOTH ? RC : 1][3];
+#pragma unroll
+    for (int r = 0; r < RX6; ++r) {
+      const int k = ht + r * HN;
+      if (k < M * NRL) {
+        // interior cells in the fixed order of the update, then ghost lines
+        const int kk = k - M * M, i = k % M, j = k / M;
+        const int line = k < M * M ? (xs ? j : i) : (kk < M ? -1 : M);
+        const int a = k < M * M ? (xs ? i : j) : kk % M;
+        const R* wl = Wd + ((line + 1) * NE + a + 1);  // edge a
+        const R* wr = wl + 1;                           // edge a+1
+        R d[3];  // frame: mass, normal (sweep) momentum, transverse
+#pragma unroll
+        for (int q = 0; q < 3; ++q)
+          d[q] = (wl[(3 + q) * NEDGE] + wr[q * NEDGE]) +
+                 (wr[(6 + q) * NEDGE] - wl[(6 + q) * NEDGE]);
+        if (r < RC && k < M * M) {
+          // nu * dQ in (h, hu, hv) order
+          const R v1 = nu * d[1], v2 = nu * d[2];
+          const R v[3] = {nu * d[0], xs ? v1 : v2, xs ? v2 : v1};
+#pragma unroll
+          for (int q = 0; q < 3; ++q) {
+            if constexpr (BOTH) {
+              if (xs) X[r][q] = v[q];
+              else Yb[r][q] = v[q];
+            } else {
+              X[r][q] = xs ? v[q] : X[r][q] + v[q];
+            }
+          }
+        }
+        if (trv) {
+          const int ci = at(a, line), cm = ci - CL, cp = ci + CL;
+          const R dd[3] = {d[0], d[2], d[1]};
+          R pl[3], mi[3];
+          gfk::tsplit_prim(ut[ci], un[ci], sc[ci], seta[ci], wetc(ci), wetc(cm), sb[cm], wetc(cp),
+                           sb[cp], dd, pl, mi);
+          // back to (h, hu, hv): "along" is the sweep's transverse momentum
+          MIr[r][0] = mi[0];
+          MIr[r][1] = xs ? mi[2] : mi[1];
+          MIr[r][2] = xs ? mi[1] : mi[2];
+          if (line + 1 <= M) {
+            R* o = Tr + 3 * (a * (M + 1) + line + 1);
+            o[0] = pl[0];
+            o[1] = xs ? pl[2] : pl[1];
+            o[2] = xs ? pl[1] : pl[2];
+          }
+        }
+      }
+    }
+    __syncthreads();
+    if (trv) {
+      const R kt = R(-0.5) * nu;
+#pragma unroll
+      for (int r = 0; r < RX6; ++r) {
+        const int k = ht + r * HN;
+        if (k < M * NRL) {
+          const int kk = k - M * M, i = k % M, j = k / M;
+          const int line = k < M * M ? (xs ? j : i) : (kk < M ? -1 : M);
+          const int a = k < M * M ? (xs ? i : j) : kk % M;
+          if (line >= 0) {
+            R* o = Tr + 3 * (a * (M + 1) + line);
+#pragma unroll
+            for (int q = 0; q < 3; ++q) o[q] = kt * (o[q] + MIr[r][q]);
+          }
+        }
+      }
+    }
+    if constexpr (BOTH) {
+      // the y half's increments, for the threads that own the cells
+      if (!xs) {
+#pragma unroll
+        for (int r = 0; r < RC; ++r) {
+          const int k = ht + r * HN;
+          if (k < M * M) {
+#pragma unroll
+            for (int q = 0; q < 3; ++q) Wd[q * NEDGE + k] = Yb[r][q];
+          }
+        }
+      }
+    }
+    __syncthreads();
+    }
+  };
   [[maybe_unused]] auto sweep = [&](auto dirc) {
     constexpr int dir = decltype(dirc)::value;
     // lines swept: -1..M (unsplit), -2..M+1 (split, x), 0..M-1 (split, y)
@@ -982,22 +1145,6 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
       // waves in planes: component q of edge e at W[q * NEDGE + e], e the
       // edge's place (line, a) in the sweep
       R* w = W + ((line - L0) * NE + a + 1);
-      if constexpr (PRIM) {
-        const R* un = dir == 0 ? su : sv;
-        const R* ut = dir == 0 ? sv : su;
-        double z[8], S[3];
-        gfk::riemann_prim(
-            gfk::Prim{s0[cl], sn[cl], st[cl], sb[cl], seta[cl], un[cl], ut[cl], sc[cl], sq[cl],
-                      wetc(cl)},
-            gfk::Prim{s0[cr], sn[cr], st[cr], sb[cr], seta[cr], un[cr], ut[cr], sc[cr], sq[cr],
-                      wetc(cr)},
-            g, z, S);
-#pragma unroll
-        for (int q = 0; q < 8; ++q) w[q * NEDGE] = z[q];
-#pragma unroll
-        for (int q = 0; q < 3; ++q) w[(8 + q) * NEDGE] = S[q];
-        continue;
-      }
       R Z[9], S[3];
       gfk::riemann<R, DEV>(
           gfk::Side<R>{sdep[cl], sn[cl], st[cl], sb[cl], s0[cl], wetc(cl)},
@@ -1023,16 +1170,6 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
         const int cl = dir == 0 ? tix<M>(a - 1, line) : tix<M>(line, a - 1);
         const int cr = dir == 0 ? tix<M>(a, line) : tix<M>(line, a);
         const bool wet = corr && wetc(cl) && wetc(cr);
-        if constexpr (PRIM) {
-          gfk::edge_fluxes_prim<NEDGE>(w, w - 1, w + 1, nu, wet, AMr[r], APr[r], FFr[r]);
-          if (line >= 0 && line < M) {
-            // |s| of the outer waves (the middle speed is their mean)
-            const double m = gfk::dmax(gfk::dabs(w[8 * NEDGE]), gfk::dabs(w[10 * NEDGE]));
-            if (dir == 0) smx = gfk::dmax(m, smx);
-            else smy = gfk::dmax(m, smy);
-          }
-          continue;
-        }
         gfk::edge_fluxes<R, NEDGE, DEV>(w, w + 9 * NEDGE, w - 1, w + 1, nu, wet,
                                         AMr[r], APr[r], FFr[r]);
         if (line >= 0 && line < M) {
@@ -1146,10 +1283,6 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
         const int cp = dir == 0 ? tix<M>(a, line + 1) : tix<M>(line + 1, a);
         const R dd[3] = {d[0], d[2], d[1]};
         R pl[3], mi[3];
-        if constexpr (PRIM)
-          gfk::tsplit_prim(dir == 0 ? sv[ci] : su[ci], dir == 0 ? su[ci] : sv[ci], sc[ci],
-                           seta[ci], wetc(ci), wetc(cm), sb[cm], wetc(cp), sb[cp], dd, pl, mi);
-        else
         gfk::tsplit<R>(sdep[ci], st[ci], sn[ci], surf(ci), wetc(ci), wetc(cm),
                        sb[cm], wetc(cp), sb[cp], dd, g, pl, mi);
         // back to (h, hu, hv): frame (mass, along = st, other = sn)
@@ -1186,6 +1319,12 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
     if constexpr (FAST) {
       sweep32(std::integral_constant<int, 0>{});
       sweep32(std::integral_constant<int, 1>{});
+    } else if constexpr (BOTH) {
+      const int half = tid / HN;
+      sweep64(half, tid % HN, W + half * Lo::NWP * NEDGE);
+    } else if constexpr (PRIM) {
+#pragma unroll 1
+      for (int dir = 0; dir < 2; ++dir) sweep64(dir, tid, W);
     } else {
       sweep(std::integral_constant<int, 0>{});
       sweep(std::integral_constant<int, 1>{});
@@ -1375,7 +1514,9 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
     if constexpr (!DEV) {
 #pragma unroll
       for (int f = 0; f < 3; ++f) {
-        const R fl = DS ? Y[r][f] : X[r][f] + Y[r][f];
+        R fl;
+        if constexpr (BOTH) fl = X[r][f] + W[(Lo::NWP + f) * NEDGE + k];
+        else fl = DS ? Y[DS ? r : 0][f] : X[r][f];
         const R* fa = Ftr + 3 * (j * (M + 1) + i);
         const R* ga = Gtr + 3 * (i * (M + 1) + j);
         const R tf = trv ? nux * (fa[3 + f] - fa[f]) + nuy * (ga[3 + f] - ga[f]) : R(0);
