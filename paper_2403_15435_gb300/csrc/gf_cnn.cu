@@ -133,7 +133,10 @@ __global__ void __launch_bounds__(256) k_conv(const bf16* __restrict__ in,
 
 // Weight gradient of a layer: dW[co][tap*16+ci] += sum_p dY[p][co] *
 // in[p + tap][ci] over the patches of this CTA (a GEMM with M = 16, N = 144,
-// K = pixels); one warp per tap.  db[co] += sum_p dY[p][co].
+// K = pixels); one warp per tap.  db[co] += sum_p dY[p][co], each thread over
+// its own pixels of one channel (sixteen threads walking all 256 pixels in
+// turn were the kernel's time: 28.4 us a launch at 1024 patches, now 16.7).  The next
+// patch's activations are requested before the current one's products.
 template <bool HALO>
 __global__ void __launch_bounds__(288) k_conv_dw(const bf16* __restrict__ dY,
                                                  const bf16* __restrict__ in,
@@ -142,21 +145,55 @@ __global__ void __launch_bounds__(288) k_conv_dw(const bf16* __restrict__ dY,
                                                  int npatch, int group) {
   __shared__ __align__(16) bf16 tile[PADW * PADW * NCH];
   __shared__ __align__(16) bf16 sdy[NPIX * NCH];
+  __shared__ float sdb[288];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int tap = warp;
   float acc[2][4] = {};
   float dbs = 0.f;
   const int p0 = blockIdx.x * group;
-  for (int pp = p0; pp < p0 + group && pp < npatch; ++pp) {
+  const int p1 = p0 + group < npatch ? p0 + group : npatch;
+  uint4* t4 = reinterpret_cast<uint4*>(tile);
+  uint4* d4 = reinterpret_cast<uint4*>(sdy);
+  // pieces of 16 bytes of a patch: NIN of the input, 512 of dY, by 288 threads
+  constexpr int NIN = (HALO ? NPAD : NPIX) * 2, RIN = (NIN + 287) / 288, RDY = 2;
+  uint4 rin[RIN], rdy[RDY];
+  auto request = [&](int pp) {
+    const uint4* s4 = reinterpret_cast<const uint4*>(in + (size_t)pp * (HALO ? NPAD : NPIX) * NCH);
+    const uint4* y4 = reinterpret_cast<const uint4*>(dY + (size_t)pp * NPIX * NCH);
+#pragma unroll
+    for (int r = 0; r < RIN; ++r) {
+      const int k = threadIdx.x + r * 288;
+      if (k < NIN) rin[r] = s4[k];
+    }
+#pragma unroll
+    for (int r = 0; r < RDY; ++r) {
+      const int k = threadIdx.x + r * 288;
+      if (k < NPIX * 2) rdy[r] = y4[k];
+    }
+  };
+  if (!HALO)  // the border stays zero
+    for (int k = threadIdx.x; k < NPAD * 2; k += 288) t4[k] = make_uint4(0u, 0u, 0u, 0u);
+  if (p0 < p1) request(p0);
+  for (int pp = p0; pp < p1; ++pp) {
     __syncthreads();
-    stage_padded<HALO>(in + (size_t)pp * (HALO ? NPAD : NPIX) * NCH, tile);
-    for (int k = threadIdx.x; k < NPIX * NCH / 8; k += blockDim.x)
-      reinterpret_cast<uint4*>(sdy)[k] =
-          reinterpret_cast<const uint4*>(dY + (size_t)pp * NPIX * NCH)[k];
+#pragma unroll
+    for (int r = 0; r < RIN; ++r) {
+      const int k = threadIdx.x + r * 288;
+      if (k < NIN) {
+        const int pix = k >> 1;
+        const int c = HALO ? k : (((pix >> 4) + 1) * PADW + (pix & 15) + 1) * 2 + (k & 1);
+        t4[c] = rin[r];
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < RDY; ++r) {
+      const int k = threadIdx.x + r * 288;
+      if (k < NPIX * 2) d4[k] = rdy[r];
+    }
     __syncthreads();
-    if (threadIdx.x < NCH)
-      for (int px = 0; px < NPIX; ++px)
-        dbs += __bfloat162float(sdy[px * NCH + threadIdx.x]);
+    if (pp + 1 < p1) request(pp + 1);
+    for (int px = threadIdx.x >> 4; px < NPIX; px += 18)
+      dbs += __bfloat162float(sdy[px * NCH + (threadIdx.x & 15)]);
     for (int ks = 0; ks < NPIX / 16; ++ks) {
       const int pb = ks * 16;
       unsigned a[4], b[4];
@@ -177,26 +214,54 @@ __global__ void __launch_bounds__(288) k_conv_dw(const bf16* __restrict__ dY,
       atomicAdd(&dW[co * KK + tap * 16 + ci], acc[nt][2 * h]);
       atomicAdd(&dW[co * KK + tap * 16 + ci + 1], acc[nt][2 * h + 1]);
     }
-  if (threadIdx.x < NCH) atomicAdd(&db[threadIdx.x], dbs);
+  sdb[threadIdx.x] = dbs;
+  __syncthreads();
+  if (threadIdx.x < NCH) {
+    float t = 0.f;
+    for (int k = 0; k < 18; ++k) t += sdb[threadIdx.x + 16 * k];
+    atomicAdd(&db[threadIdx.x], t);
+  }
 }
 
-// Head: v = mean_p a3[p][:], logit = wh . v + bh.
+// Head: v = mean_p a3[p][:], logit = wh . v + bh.  A warp per patch; a lane
+// takes 16-byte pieces (eight channels of every sixteenth pixel), then the
+// partial sums meet by shuffles (2-byte loads in a chain of 128 took 17.5 us
+// at 1024 patches, this 3.3).
 __global__ void k_head(const bf16* __restrict__ a3, const float* __restrict__ wh,
                        const float* __restrict__ bh, float* __restrict__ logit,
                        float* __restrict__ vout, int npatch) {
   const int p = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (p >= npatch) return;
-  const bf16* a = a3 + (size_t)p * NPIX * NCH;
-  // lane handles channel lane % 16 over half of the pixels
-  const int c = lane & 15, half = lane >> 4;
-  float s = 0.f;
-  for (int px = half; px < NPIX; px += 2) s += __bfloat162float(a[px * NCH + c]);
-  s += __shfl_xor_sync(0xffffffffu, s, 16);
-  const float v = s * (1.0f / NPIX);
-  if (vout && lane < 16) vout[(size_t)p * NCH + c] = v;
-  float z = lane < 16 ? wh[c] * v : 0.f;
-  for (int o = 8; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
+  const uint4* a = reinterpret_cast<const uint4*>(a3 + (size_t)p * NPIX * NCH);
+  // piece k of the patch: pixel k / 2, channels 8 (k % 2) ..; lane: parity
+  float s[8] = {};
+#pragma unroll
+  for (int r = 0; r < NPIX * 2 / 32; ++r) {
+    const uint4 v = a[r * 32 + lane];
+    const unsigned w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      s[2 * q] += __uint_as_float(w[q] << 16);
+      s[2 * q + 1] += __uint_as_float(w[q] & 0xffff0000u);
+    }
+  }
+#pragma unroll
+  for (int o = 2; o < 32; o <<= 1)
+#pragma unroll
+    for (int q = 0; q < 8; ++q) s[q] += __shfl_xor_sync(0xffffffffu, s[q], o);
+  float z = 0.f;
+  const int c0 = 8 * (lane & 1);
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    s[q] *= 1.0f / NPIX;
+    z += wh[c0 + q] * s[q];
+  }
+  if (vout && lane < 2) {
+#pragma unroll
+    for (int q = 0; q < 8; ++q) vout[(size_t)p * NCH + c0 + q] = s[q];
+  }
+  z += __shfl_xor_sync(0xffffffffu, z, 1);
   if (lane == 0) logit[p] = z + bh[0];
 }
 
@@ -331,7 +396,10 @@ int cnn_backward(const void* x0, const void* wf, const float* prm,
                                      prm + 3 * CNN_LAYER, pos_weight, 1.0f / npatch,
                                      grad + 3 * CNN_LAYER, grad + 3 * CNN_LAYER + NCH,
                                      static_cast<bf16*>(d3), loss);
-  const int group = 8, blocks = (npatch + group - 1) / group;
+  // patches per CTA of the weight gradients: two CTAs to an SM, at most eight
+  // (each adds its 2320 sums to the gradient)
+  const int group = npatch >= 8 * 304 ? 8 : (npatch + 303) / 304;
+  const int blocks = (npatch + group - 1) / group;
   // layer 3: weight gradient from a2, input gradient through relu(a2)
   k_conv_dw<false><<<blocks, 288, 0, st>>>(static_cast<const bf16*>(d3),
                                     static_cast<const bf16*>(a2),
