@@ -81,13 +81,13 @@ FP64_LANES_PER_SM = 2  # measured: DFMA throughput 1.20 TFLOP/s on 152 SMs
 N_SM = 152
 # DRAM bytes (read + write) of one patch-step launch, from the ncu captures
 # summarised in profiles/ (cold caches); None when the kernel has changed
-# since.  Valley: the launch at t = 30 s (6827 patches) of the 608-thread
-# variant that the autotuner picks there, 341 667 840 B over 6 990 848
-# cells, scaled to the cells of an average timed launch.  Uniform workload:
-# launch 151 (t = 29.5 s), 4 629 504 B.
-TRAFFIC_PER_LAUNCH_FP32 = 4629504
+# since (the uniform workloads).  Valley: the launch at t = 30 s (6815
+# patches) of variant 0, which the autotuner picks there, 82 736 640 B read
+# and 31 502 336 B written over 6 978 560 cells, scaled to the cells of an
+# average timed launch.
+TRAFFIC_PER_LAUNCH_FP32 = None
 TRAFFIC_PER_LAUNCH_FP64 = None
-TRAFFIC_PER_CELL_VALLEY_FP32 = 341667840 / 6990848
+TRAFFIC_PER_CELL_VALLEY_FP32 = (82736640 + 31502336) / 6978560
 
 
 def parse():
