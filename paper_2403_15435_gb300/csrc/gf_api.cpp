@@ -40,8 +40,6 @@ struct CnnState {
   float scale[4] = {10.f, 10.f, 10.f, 10.f};
   // inference over the current patches (sized to the patch capacity)
   void* x = nullptr;
-  void* a[3] = {nullptr, nullptr, nullptr};
-  float* pool = nullptr;
   float* logit = nullptr;
   // pending samples: features at a snapshot, labels OR'ed over checks
   void* px = nullptr;
@@ -56,9 +54,6 @@ struct CnnState {
   void* xb = nullptr;
   float* yb = nullptr;
   int* idx = nullptr;
-  void* ta[3] = {nullptr, nullptr, nullptr};
-  void* td[3] = {nullptr, nullptr, nullptr};
-  float* tv = nullptr;
   float* tlogit = nullptr;
   float* loss = nullptr;
   int bcap = 0, idx_cap = 0;
@@ -554,7 +549,6 @@ int cnn_alloc(geoflood_ctx* ctx, void** p, size_t bytes) {
 }
 
 const size_t CNN_X_BYTES = (size_t)gf::CNN_IN_PIX * gf::CNN_CH * 2;
-const size_t CNN_A_BYTES = (size_t)gf::CNN_PIX * gf::CNN_CH * 2;
 
 int cnn_params_alloc(geoflood_ctx* ctx) {
   CnnState& n = ctx->cnn;
@@ -575,8 +569,6 @@ int cnn_infer_alloc(geoflood_ctx* ctx) {
   const size_t cap = (size_t)ctx->cap;
   int rc = 0;
   rc |= cnn_alloc(ctx, &n.x, cap * CNN_X_BYTES);
-  for (int l = 0; l < 3; ++l) rc |= cnn_alloc(ctx, &n.a[l], cap * CNN_A_BYTES);
-  rc |= cnn_alloc(ctx, (void**)&n.pool, cap * 16 * 4);
   rc |= cnn_alloc(ctx, (void**)&n.logit, cap * 4);
   return rc ? GEOFLOOD_ERR_OOM : 0;
 }
@@ -584,20 +576,13 @@ int cnn_infer_alloc(geoflood_ctx* ctx) {
 int cnn_batch_alloc(geoflood_ctx* ctx, int b) {
   CnnState& n = ctx->cnn;
   if (b <= n.bcap) return 0;
-  for (void* p : {n.xb, (void*)n.yb, n.ta[0], n.ta[1], n.ta[2], n.td[0], n.td[1], n.td[2],
-                  (void*)n.tv, (void*)n.tlogit})
+  for (void* p : {n.xb, (void*)n.yb, (void*)n.tlogit})
     cudaFree(p);
-  n.xb = nullptr; n.yb = nullptr; n.tv = nullptr; n.tlogit = nullptr;
-  for (int l = 0; l < 3; ++l) n.ta[l] = n.td[l] = nullptr;
+  n.xb = nullptr; n.yb = nullptr; n.tlogit = nullptr;
   n.bcap = 0;
   int rc = 0;
   rc |= cnn_alloc(ctx, &n.xb, (size_t)b * CNN_X_BYTES);
   rc |= cnn_alloc(ctx, (void**)&n.yb, (size_t)b * 4);
-  for (int l = 0; l < 3; ++l) {
-    rc |= cnn_alloc(ctx, &n.ta[l], (size_t)b * CNN_A_BYTES);
-    rc |= cnn_alloc(ctx, &n.td[l], (size_t)b * CNN_A_BYTES);
-  }
-  rc |= cnn_alloc(ctx, (void**)&n.tv, (size_t)b * 16 * 4);
   rc |= cnn_alloc(ctx, (void**)&n.tlogit, (size_t)b * 4);
   if (rc) return GEOFLOOD_ERR_OOM;
   n.bcap = b;
@@ -611,10 +596,8 @@ int cnn_infer(geoflood_ctx* ctx, int first, int count) {
   if (rc) return rc;
   CKL(gf::launch_cnn_features(ctx->G, view(ctx), first, count, n.scale, n.x, ctx->st),
       "cnn_features");
-  CKL(gf::cnn_forward(n.x, n.wb, n.prm, n.a[0], n.a[1], n.a[2], n.pool, n.logit, count,
-                      ctx->st),
-      "cnn_forward");
-  ctx->launches += 5;
+  CKL(gf::cnn_forward(n.x, n.wb, n.prm, n.logit, count, ctx->st), "cnn_forward");
+  ctx->launches += 2;
   return 0;
 }
 
@@ -963,9 +946,8 @@ void geoflood_destroy(geoflood_ctx* ctx) {
   for (auto e : ctx->pool) cudaEventDestroy(e);
   CnnState& n = ctx->cnn;
   for (void* p : {(void*)n.prm, n.wb, n.wf, (void*)n.grad, (void*)n.am, (void*)n.av, n.x,
-                  n.a[0], n.a[1], n.a[2], (void*)n.pool, (void*)n.logit, n.px, (void*)n.py,
-                  n.dx, (void*)n.dy, n.xb, (void*)n.yb, (void*)n.idx, n.ta[0], n.ta[1],
-                  n.ta[2], n.td[0], n.td[1], n.td[2], (void*)n.tv, (void*)n.tlogit,
+                  (void*)n.logit, n.px, (void*)n.py,
+                  n.dx, (void*)n.dy, n.xb, (void*)n.yb, (void*)n.idx, (void*)n.tlogit,
                   (void*)n.loss, (void*)n.misses})
     cudaFree(p);
   delete ctx;
@@ -1869,12 +1851,10 @@ int geoflood_cnn_grad(geoflood_ctx* ctx, const uint16_t* x, const float* label, 
   CK(cudaMemcpyAsync(c.yb, label, (size_t)n * 4, cudaMemcpyHostToDevice, ctx->st));
   CK(cudaMemsetAsync(c.grad, 0, (size_t)np * 4, ctx->st));
   CK(cudaMemsetAsync(c.loss, 0, 4, ctx->st));
-  CKL(gf::cnn_forward(c.xb, c.wb, c.prm, c.ta[0], c.ta[1], c.ta[2], c.tv, c.tlogit, n, ctx->st),
-      "cnn_forward");
-  CKL(gf::cnn_backward(c.xb, c.wf, c.prm, c.ta[0], c.ta[1], c.ta[2], c.tv, c.tlogit, c.yb,
-                       pos_weight, c.grad, c.loss, c.td[0], c.td[1], c.td[2], n, ctx->st),
-      "cnn_backward");
-  ctx->launches += 11;
+  CKL(gf::cnn_grad(c.xb, nullptr, c.wb, c.wf, c.prm, c.yb, pos_weight, c.tlogit, c.grad, c.loss,
+                   n, ctx->st),
+      "cnn_grad");
+  ctx->launches++;
   if (logit) CK(cudaMemcpyAsync(logit, c.tlogit, (size_t)n * 4, cudaMemcpyDeviceToHost, ctx->st));
   if (grad) CK(cudaMemcpyAsync(grad, c.grad, (size_t)np * 4, cudaMemcpyDeviceToHost, ctx->st));
   if (loss) CK(cudaMemcpyAsync(loss, c.loss, 4, cudaMemcpyDeviceToHost, ctx->st));
@@ -2004,19 +1984,13 @@ int geoflood_cnn_train(geoflood_ctx* ctx, int epochs, int batch, float lr, float
     }
     CK(cudaMemcpyAsync(c.idx, perm.data(), (size_t)N * 4, cudaMemcpyHostToDevice, ctx->st));
     for (int b = 0; b < nb; ++b) {
-      CKL(gf::cnn_gather(c.dx, c.dy, c.idx + (size_t)b * batch, batch, c.xb, c.yb, ctx->st),
-          "cnn_gather");
       CK(cudaMemsetAsync(c.grad, 0, (size_t)np * 4, ctx->st));
-      CKL(gf::cnn_forward(c.xb, c.wb, c.prm, c.ta[0], c.ta[1], c.ta[2], c.tv, c.tlogit, batch,
-                          ctx->st),
-          "cnn_forward");
-      CKL(gf::cnn_backward(c.xb, c.wf, c.prm, c.ta[0], c.ta[1], c.ta[2], c.tv, c.tlogit, c.yb,
-                           pos_weight, c.grad, c.loss + e, c.td[0], c.td[1], c.td[2], batch,
-                           ctx->st),
-          "cnn_backward");
+      CKL(gf::cnn_grad(c.dx, c.idx + (size_t)b * batch, c.wb, c.wf, c.prm, c.dy, pos_weight,
+                       c.tlogit, c.grad, c.loss + e, batch, ctx->st),
+          "cnn_grad");
       CKL(gf::cnn_adam(c.prm, c.grad, c.am, c.av, lr, ++c.adam_t, ctx->st), "cnn_adam");
       CKL(gf::cnn_cast(c.prm, c.wb, c.wf, ctx->st), "cnn_cast");
-      ctx->launches += 14;
+      ctx->launches += 3;
     }
     // the host vector is rewritten next epoch: wait for its copy
     CK(cudaStreamSynchronize(ctx->st));

@@ -7,8 +7,8 @@
 // a_1 = relu(conv3x3_valid(x0; W_1) + b_1) on the 16 x 16 pixels, a_l =
 // relu(conv3x3(a_{l-1}; W_l) + b_l) with zero padding for l = 2, 3, 16
 // channels each; v = mean over pixels of a_3; logit = wh . v + bh.
-// Layouts: activations [patch][256][16] BF16 (pixel-major, pixel = y*16 +
-// x); conv weights [16 co][144 k] with k = tap*16 + ci and tap = (dy+1)*3 +
+// Layouts: features [patch][324][16] BF16 (pixel-major, pixel = y*18 + x);
+// conv weights [16 co][144 k] with k = tap*16 + ci and tap = (dy+1)*3 +
 // (dx+1).  Every conv is an implicit GEMM with M = 256 pixels, N = 16,
 // K = 144; the weight gradient is a GEMM with M = 16, N = 144 and K =
 // pixels x patches.
@@ -49,252 +49,279 @@ __device__ __forceinline__ void mma16816(float (&d)[4], const unsigned (&a)[4],
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-// Stage one patch's activations into an 18 x 18 x 16 tile: the input grid
-// itself when it carries its ring (HALO), else 16 x 16 with a zero border.
-template <bool HALO>
-__device__ void stage_padded(const bf16* __restrict__ src, bf16* tile) {
-  uint4* t4 = reinterpret_cast<uint4*>(tile);  // 2 x uint4 per pixel
-  const uint4* s4 = reinterpret_cast<const uint4*>(src);
-  if (HALO) {
-    for (int k = threadIdx.x; k < PADW * PADW * 2; k += blockDim.x) t4[k] = s4[k];
-    return;
-  }
-  const uint4 z = make_uint4(0u, 0u, 0u, 0u);
-  for (int k = threadIdx.x; k < PADW * PADW * 2; k += blockDim.x) t4[k] = z;
-  __syncthreads();
-  for (int k = threadIdx.x; k < NPIX * 2; k += blockDim.x) {
-    const int pix = k >> 1, half = k & 1;
-    const int y = pix >> 4, x = pix & 15;
-    t4[((y + 1) * PADW + (x + 1)) * 2 + half] = s4[k];
-  }
+// A patch's activations in shared memory: 18 x 18 pixels of 16 channels, two
+// 16-byte pieces a pixel.  The pieces of a pixel change places with bit 2 of
+// the pixel's index, so that the eight rows of an ldmatrix (eight pixels in a
+// row, one piece each) fall into eight different bank groups.
+constexpr int TILE = NPAD * 2;  // 16-byte pieces
+constexpr int WROW = KK + 8;    // weight row in shared memory (conflict-free)
+
+__device__ __forceinline__ int piece(int pix, int half) {
+  return pix * 2 + (half ^ ((pix >> 2) & 1));
 }
 
-__device__ __forceinline__ const bf16* tap_row(const bf16* tile, int pix,
-                                               int tap) {
-  const int y = pix >> 4, x = pix & 15;
-  const int dy = tap / 3 - 1, dx = tap % 3 - 1;
-  return tile + ((y + dy + 1) * PADW + (x + dx + 1)) * NCH;
+// Pixel (y, x) of the 16 x 16 in the padded tile, moved by (dy, dx).
+__device__ __forceinline__ int padded(int y, int x, int dy = 0, int dx = 0) {
+  return (y + dy + 1) * PADW + x + dx + 1;
 }
 
-// Convolution layer (also the input-gradient pass with flipped weights):
-// out[p][co] = sum_{tap,ci} W[co][tap*16+ci] * in[p + tap][ci] (+ bias),
-// then relu, or multiplied by (mask > 0).  One CTA (8 warps) per patch.
-template <bool BIAS, bool RELU, bool MASK, bool HALO>
-__global__ void __launch_bounds__(256) k_conv(const bf16* __restrict__ in,
-                                              const bf16* __restrict__ W,
-                                              const float* __restrict__ bias,
-                                              const bf16* __restrict__ mask,
-                                              bf16* __restrict__ out) {
-  __shared__ __align__(16) bf16 tile[PADW * PADW * NCH];
-  __shared__ __align__(16) bf16 sw[NCH * KK];
-  const int p = blockIdx.x;
-  stage_padded<HALO>(in + (size_t)p * (HALO ? NPAD : NPIX) * NCH, tile);
-  for (int k = threadIdx.x; k < NCH * KK / 8; k += blockDim.x)
-    reinterpret_cast<uint4*>(sw)[k] = reinterpret_cast<const uint4*>(W)[k];
-  __syncthreads();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+// 3 x 3 convolution of a tile by warps 0..7, 32 pixels each (M = 256, N = 16,
+// K = 144); done(pixel, channel pair's half, word, value, value) gets every
+// output.
+template <typename F>
+__device__ __forceinline__ void conv(const uint4* in, const bf16* w, int warp, int lane, F done) {
   float acc[2][2][4] = {};
+  const bf16* wl = w + ((lane & 7) + 8 * (lane >> 4)) * WROW + 8 * ((lane >> 3) & 1);
+  const int x = (lane & 7) + 8 * ((lane >> 3) & 1);
+#pragma unroll 3
   for (int tap = 0; tap < 9; ++tap) {
     unsigned b[4];
-    ldsm_x4(b, sw + ((lane & 7) + 8 * (lane >> 4)) * KK + tap * 16 +
-                   8 * ((lane >> 3) & 1));
+    ldsm_x4(b, wl + tap * 16);
 #pragma unroll
     for (int mt = 0; mt < 2; ++mt) {
-      const int pix = warp * 32 + mt * 16 + (lane & 7) + 8 * ((lane >> 3) & 1);
       unsigned a[4];
-      ldsm_x4(a, tap_row(tile, pix, tap) + 8 * (lane >> 4));
+      ldsm_x4(a, in + piece(padded(warp * 2 + mt, x, tap / 3 - 1, tap % 3 - 1), lane >> 4));
       mma16816(acc[mt][0], a, b[0], b[1]);
       mma16816(acc[mt][1], a, b[2], b[3]);
     }
   }
-  bf16* o = out + (size_t)p * NPIX * NCH;
-  const bf16* mk = MASK ? mask + (size_t)p * NPIX * NCH : nullptr;
 #pragma unroll
   for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
-    for (int nt = 0; nt < 2; ++nt)
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int pix = warp * 32 + mt * 16 + (lane >> 2) + 8 * h;
-        const int co = nt * 8 + (lane & 3) * 2;
-        float v0 = acc[mt][nt][2 * h], v1 = acc[mt][nt][2 * h + 1];
-        if (BIAS) { v0 += bias[co]; v1 += bias[co + 1]; }
-        if (RELU) { v0 = fmaxf(v0, 0.f); v1 = fmaxf(v1, 0.f); }
-        if (MASK) {
-          if (!(__bfloat162float(mk[pix * NCH + co]) > 0.f)) v0 = 0.f;
-          if (!(__bfloat162float(mk[pix * NCH + co + 1]) > 0.f)) v1 = 0.f;
-        }
-        __nv_bfloat162 r;
-        r.x = __float2bfloat16_rn(v0);
-        r.y = __float2bfloat16_rn(v1);
-        *reinterpret_cast<__nv_bfloat162*>(o + pix * NCH + co) = r;
-      }
-}
-
-// Weight gradient of a layer: dW[co][tap*16+ci] += sum_p dY[p][co] *
-// in[p + tap][ci] over the patches of this CTA (a GEMM with M = 16, N = 144,
-// K = pixels); one warp per tap.  db[co] += sum_p dY[p][co], each thread over
-// its own pixels of one channel (sixteen threads walking all 256 pixels in
-// turn were the kernel's time: 28.4 us a launch at 1024 patches, now 16.7).  The next
-// patch's activations are requested before the current one's products.
-template <bool HALO>
-__global__ void __launch_bounds__(288) k_conv_dw(const bf16* __restrict__ dY,
-                                                 const bf16* __restrict__ in,
-                                                 float* __restrict__ dW,
-                                                 float* __restrict__ db,
-                                                 int npatch, int group) {
-  __shared__ __align__(16) bf16 tile[PADW * PADW * NCH];
-  __shared__ __align__(16) bf16 sdy[NPIX * NCH];
-  __shared__ float sdb[288];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int tap = warp;
-  float acc[2][4] = {};
-  float dbs = 0.f;
-  const int p0 = blockIdx.x * group;
-  const int p1 = p0 + group < npatch ? p0 + group : npatch;
-  uint4* t4 = reinterpret_cast<uint4*>(tile);
-  uint4* d4 = reinterpret_cast<uint4*>(sdy);
-  // pieces of 16 bytes of a patch: NIN of the input, 512 of dY, by 288 threads
-  constexpr int NIN = (HALO ? NPAD : NPIX) * 2, RIN = (NIN + 287) / 288, RDY = 2;
-  uint4 rin[RIN], rdy[RDY];
-  auto request = [&](int pp) {
-    const uint4* s4 = reinterpret_cast<const uint4*>(in + (size_t)pp * (HALO ? NPAD : NPIX) * NCH);
-    const uint4* y4 = reinterpret_cast<const uint4*>(dY + (size_t)pp * NPIX * NCH);
-#pragma unroll
-    for (int r = 0; r < RIN; ++r) {
-      const int k = threadIdx.x + r * 288;
-      if (k < NIN) rin[r] = s4[k];
-    }
-#pragma unroll
-    for (int r = 0; r < RDY; ++r) {
-      const int k = threadIdx.x + r * 288;
-      if (k < NPIX * 2) rdy[r] = y4[k];
-    }
-  };
-  if (!HALO)  // the border stays zero
-    for (int k = threadIdx.x; k < NPAD * 2; k += 288) t4[k] = make_uint4(0u, 0u, 0u, 0u);
-  if (p0 < p1) request(p0);
-  for (int pp = p0; pp < p1; ++pp) {
-    __syncthreads();
-#pragma unroll
-    for (int r = 0; r < RIN; ++r) {
-      const int k = threadIdx.x + r * 288;
-      if (k < NIN) {
-        const int pix = k >> 1;
-        const int c = HALO ? k : (((pix >> 4) + 1) * PADW + (pix & 15) + 1) * 2 + (k & 1);
-        t4[c] = rin[r];
-      }
-    }
-#pragma unroll
-    for (int r = 0; r < RDY; ++r) {
-      const int k = threadIdx.x + r * 288;
-      if (k < NPIX * 2) d4[k] = rdy[r];
-    }
-    __syncthreads();
-    if (pp + 1 < p1) request(pp + 1);
-    for (int px = threadIdx.x >> 4; px < NPIX; px += 18)
-      dbs += __bfloat162float(sdy[px * NCH + (threadIdx.x & 15)]);
-    for (int ks = 0; ks < NPIX / 16; ++ks) {
-      const int pb = ks * 16;
-      unsigned a[4], b[4];
-      ldsm_x4_t(a, sdy + (pb + (lane & 7) + 8 * (lane >> 4)) * NCH +
-                       8 * ((lane >> 3) & 1));
-      ldsm_x4_t(b, tap_row(tile, pb + (lane & 7) + 8 * ((lane >> 3) & 1), tap) +
-                       8 * (lane >> 4));
-      mma16816(acc[0], a, b[0], b[1]);
-      mma16816(acc[1], a, b[2], b[3]);
-    }
-  }
-#pragma unroll
-  for (int nt = 0; nt < 2; ++nt)
-#pragma unroll
     for (int h = 0; h < 2; ++h) {
-      const int co = (lane >> 2) + 8 * h;
-      const int ci = nt * 8 + (lane & 3) * 2;
-      atomicAdd(&dW[co * KK + tap * 16 + ci], acc[nt][2 * h]);
-      atomicAdd(&dW[co * KK + tap * 16 + ci + 1], acc[nt][2 * h + 1]);
+      const int pix = padded(warp * 2 + mt, (lane >> 2) + 8 * h);
+#pragma unroll
+      for (int nt = 0; nt < 2; ++nt)
+        done(piece(pix, nt) * 4 + (lane & 3), nt * 8 + (lane & 3) * 2, acc[mt][nt][2 * h],
+             acc[mt][nt][2 * h + 1]);
     }
-  sdb[threadIdx.x] = dbs;
-  __syncthreads();
-  if (threadIdx.x < NCH) {
-    float t = 0.f;
-    for (int k = 0; k < 18; ++k) t += sdb[threadIdx.x + 16 * k];
-    atomicAdd(&db[threadIdx.x], t);
+}
+
+__device__ __forceinline__ __nv_bfloat162 pair_bf16(float a, float b) {
+  __nv_bfloat162 r;
+  r.x = __float2bfloat16_rn(a);
+  r.y = __float2bfloat16_rn(b);
+  return r;
+}
+
+// One patch's part of a weight gradient, dW[co][tap*16+ci] += sum_p dY[p][co]
+// in[p + tap][ci] (M = 16, N = 144, K = 256), one warp per tap, and of the
+// bias gradient, each thread over its own pixels of two channels.
+__device__ __forceinline__ void conv_dw(const uint4* dy, const uint4* in, int tap, int lane,
+                                        float (&acc)[2][4], float2& db) {
+  const int xa = (lane & 7) + 8 * (lane >> 4), xb = (lane & 7) + 8 * ((lane >> 3) & 1);
+  const int ty = tap / 3 - 1, tx = tap % 3 - 1;
+#pragma unroll 2
+  for (int y = 0; y < 16; ++y) {
+    unsigned a[4], b[4];
+    ldsm_x4_t(a, dy + piece(padded(y, xa), (lane >> 3) & 1));
+    ldsm_x4_t(b, in + piece(padded(y, xb, ty, tx), lane >> 4));
+    mma16816(acc[0], a, b[0], b[1]);
+    mma16816(acc[1], a, b[2], b[3]);
+  }
+  const unsigned* w = reinterpret_cast<const unsigned*>(dy);
+  for (int px = threadIdx.x >> 3; px < NPIX; px += 36) {
+    const unsigned v =
+        w[piece(padded(px >> 4, px & 15), (threadIdx.x >> 2) & 1) * 4 + (threadIdx.x & 3)];
+    db.x += __uint_as_float(v << 16);
+    db.y += __uint_as_float(v & 0xffff0000u);
   }
 }
 
-// Head: v = mean_p a3[p][:], logit = wh . v + bh.  A warp per patch; a lane
-// takes 16-byte pieces (eight channels of every sixteenth pixel), then the
-// partial sums meet by shuffles (2-byte loads in a chain of 128 took 17.5 us
-// at 1024 patches, this 3.3).
-__global__ void k_head(const bf16* __restrict__ a3, const float* __restrict__ wh,
-                       const float* __restrict__ bh, float* __restrict__ logit,
-                       float* __restrict__ vout, int npatch) {
-  const int p = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (p >= npatch) return;
-  const uint4* a = reinterpret_cast<const uint4*>(a3 + (size_t)p * NPIX * NCH);
-  // piece k of the patch: pixel k / 2, channels 8 (k % 2) ..; lane: parity
-  float s[8] = {};
-#pragma unroll
-  for (int r = 0; r < NPIX * 2 / 32; ++r) {
-    const uint4 v = a[r * 32 + lane];
-    const unsigned w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      s[2 * q] += __uint_as_float(w[q] << 16);
-      s[2 * q + 1] += __uint_as_float(w[q] & 0xffff0000u);
-    }
-  }
-#pragma unroll
-  for (int o = 2; o < 32; o <<= 1)
-#pragma unroll
-    for (int q = 0; q < 8; ++q) s[q] += __shfl_xor_sync(0xffffffffu, s[q], o);
-  float z = 0.f;
-  const int c0 = 8 * (lane & 1);
-#pragma unroll
-  for (int q = 0; q < 8; ++q) {
-    s[q] *= 1.0f / NPIX;
-    z += wh[c0 + q] * s[q];
-  }
-  if (vout && lane < 2) {
-#pragma unroll
-    for (int q = 0; q < 8; ++q) vout[(size_t)p * NCH + c0 + q] = s[q];
-  }
-  z += __shfl_xor_sync(0xffffffffu, z, 1);
-  if (lane == 0) logit[p] = z + bh[0];
-}
-
-// Head backward for binary cross-entropy on the logits: dlogit =
+// The network on whole patches: every layer of a patch in one CTA, the
+// activations in shared memory, the weights staged once per CTA, the patches
+// p, p + gridDim.x, ... one after another.  GRAD adds the backward pass of
+// the weighted cross-entropy: weight gradients stay in registers over the
+// CTA's patches and are added to grad once at its end.  What bounds it is a
+// patch's chain of eight phases between barriers, so as many CTAs share an SM
+// as shared memory allows (72 KB: three; forward alone 46 KB: four).
+// 1024 samples' loss and gradient on the device: nine launches with the
+// activations written and read between them about 120 us, this one 51; the
+// whole call 268 -> 175 us.
+//
+// Head: v = mean_p a3[p][:], logit = wh . v + bh.  Backward: dlogit =
 // w_y (sigmoid(z) - y) / n; dwh += dlogit v; dbh += dlogit;
-// dA3[p][c] = dlogit wh[c] / 256 where a3 > 0 (relu), else 0.
-__global__ void k_head_bwd(const float* __restrict__ logit,
-                           const float* __restrict__ label,
-                           const float* __restrict__ v,
-                           const bf16* __restrict__ a3,
-                           const float* __restrict__ wh, float pos_weight,
-                           float inv_n, float* __restrict__ dwh,
-                           float* __restrict__ dbh, bf16* __restrict__ dY3,
-                           float* __restrict__ loss) {
-  const int p = blockIdx.x;
-  const float z = logit[p], y = label[p];
-  const float sg = 1.f / (1.f + expf(-z));
-  const float w = y > 0.5f ? pos_weight : 1.f;
-  const float dz = w * (sg - y) * inv_n;
-  if (threadIdx.x < NCH) atomicAdd(&dwh[threadIdx.x], dz * v[(size_t)p * NCH + threadIdx.x]);
-  if (threadIdx.x == 0) {
-    atomicAdd(dbh, dz);
-    // softplus form of the cross-entropy
-    const float l = fmaxf(z, 0.f) - z * y + log1pf(expf(-fabsf(z)));
-    atomicAdd(loss, w * l * inv_n);
+// da3[p][c] = dlogit wh[c] / 256; each d through its layer's relu.
+template <bool GRAD>
+struct Net {
+  static constexpr int NT = GRAD ? 288 : 256;  // a warp per tap | 32 pixels per warp
+  static constexpr int NTILE = GRAD ? 5 : 3;
+  static constexpr int NW = GRAD ? 5 : 3;
+  static constexpr int PER_SM = GRAD ? 3 : 4;
+  static constexpr size_t smem() { return (size_t)NTILE * TILE * 16 + (size_t)NW * NCH * WROW * 2; }
+};
+
+template <bool GRAD>
+__global__ void __launch_bounds__(Net<GRAD>::NT, Net<GRAD>::PER_SM)
+    k_net(const bf16* __restrict__ x0, const int* __restrict__ idx, const bf16* __restrict__ wb,
+          const bf16* __restrict__ wf, const float* __restrict__ prm,
+          const float* __restrict__ label, float pos_weight, float inv_n,
+          float* __restrict__ logit, float* __restrict__ grad, float* __restrict__ loss,
+          int npatch) {
+  constexpr int NT = Net<GRAD>::NT, LAYER = NCH * KK + NCH;
+  extern __shared__ __align__(16) uint4 smem[];
+  __shared__ float sprm[3 * NCH + NCH + 1];  // biases, head weights, head bias
+  __shared__ float shead[NCH + 2];           // sums of dwh, dbh, loss
+  __shared__ float sdz;
+  uint4* X = smem;
+  uint4* A1 = X + TILE;
+  uint4* A2 = A1 + TILE;
+  uint4* A3 = GRAD ? A2 + TILE : A1;      // then d3, then d1
+  uint4* D2 = A2 + 2 * TILE;              // GRAD only
+  bf16* w = reinterpret_cast<bf16*>(smem + Net<GRAD>::NTILE * TILE);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+
+  for (int k = threadIdx.x; k < (Net<GRAD>::NTILE - 1) * TILE; k += NT)
+    A1[k] = make_uint4(0u, 0u, 0u, 0u);  // the borders stay zero
+  constexpr int ROWP = KK / 8;  // 16-byte pieces of a weight row
+  for (int k = threadIdx.x; k < Net<GRAD>::NW * NCH * ROWP; k += NT) {
+    const int row = k / ROWP, c = k % ROWP;
+    // the flipped weights of layers 2 and 3 after the three layers'
+    const bf16* src = row < 3 * NCH ? wb + row * KK : wf + (row - 2 * NCH) * KK;
+    *reinterpret_cast<uint4*>(w + row * WROW + c * 8) = reinterpret_cast<const uint4*>(src)[c];
   }
-  const bf16* a = a3 + (size_t)p * NPIX * NCH;
-  bf16* d = dY3 + (size_t)p * NPIX * NCH;
-  for (int k = threadIdx.x; k < NPIX * NCH; k += blockDim.x) {
-    const int c = k & 15;
-    const float g = __bfloat162float(a[k]) > 0.f ? dz * wh[c] * (1.0f / NPIX) : 0.f;
-    d[k] = __float2bfloat16_rn(g);
+  for (int k = threadIdx.x; k < 3 * NCH + NCH + 1; k += NT)
+    sprm[k] = k < 3 * NCH ? prm[(k >> 4) * LAYER + NCH * KK + (k & 15)]
+                          : prm[3 * LAYER + k - 3 * NCH];
+  if (GRAD && threadIdx.x < NCH + 2) shead[threadIdx.x] = 0.f;
+  float dw[3][2][4] = {};
+  float2 db[3] = {};
+
+  for (int p = blockIdx.x; p < npatch; p += gridDim.x) {
+    const int src = idx ? idx[p] : p;
+    const uint4* s4 = reinterpret_cast<const uint4*>(x0 + (size_t)src * NPAD * NCH);
+    if (p != (int)blockIdx.x) __syncthreads();  // the last patch's tiles are done with
+    for (int k = threadIdx.x; k < TILE; k += NT) X[piece(k >> 1, k & 1)] = s4[k];
+    __syncthreads();
+    auto layer = [&](const uint4* in, uint4* out, int l) {
+      unsigned* o = reinterpret_cast<unsigned*>(out);
+      if (warp < 8)
+        conv(in, w + l * NCH * WROW, warp, lane, [&](int at, int co, float v0, float v1) {
+          const float* b = sprm + l * NCH + co;
+          *reinterpret_cast<__nv_bfloat162*>(o + at) =
+              pair_bf16(fmaxf(v0 + b[0], 0.f), fmaxf(v1 + b[1], 0.f));
+        });
+      __syncthreads();
+    };
+    layer(X, A1, 0);
+    layer(A1, A2, 1);
+    layer(A2, A3, 2);
+    if (warp == 0) {
+      // a lane takes the same eight channels of every sixteenth pixel
+      float s[8] = {};
+      const int half = lane & 1;
+#pragma unroll 4
+      for (int r = 0; r < 16; ++r) {
+        const uint4 v = A3[piece(padded(r, lane >> 1), half)];
+        const unsigned q4[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          s[2 * q] += __uint_as_float(q4[q] << 16);
+          s[2 * q + 1] += __uint_as_float(q4[q] & 0xffff0000u);
+        }
+      }
+#pragma unroll
+      for (int o = 2; o < 32; o <<= 1)
+#pragma unroll
+        for (int q = 0; q < 8; ++q) s[q] += __shfl_xor_sync(0xffffffffu, s[q], o);
+      const float* wh = sprm + 3 * NCH + 8 * half;
+      float z = 0.f;
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        s[q] *= 1.0f / NPIX;
+        z += wh[q] * s[q];
+      }
+      z += __shfl_xor_sync(0xffffffffu, z, 1);
+      z += sprm[4 * NCH];
+      if (lane == 0) logit[p] = z;
+      if (GRAD && lane < 2) {
+        const float y = label[src];
+        const float sg = 1.f / (1.f + expf(-z));
+        const float wy = y > 0.5f ? pos_weight : 1.f;
+        const float dz = wy * (sg - y) * inv_n;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) shead[8 * half + q] += dz * s[q];
+        if (lane == 0) {
+          sdz = dz;
+          shead[NCH] += dz;
+          // softplus form of the cross-entropy
+          const float l = fmaxf(z, 0.f) - z * y + log1pf(expf(-fabsf(z)));
+          shead[NCH + 1] += wy * l * inv_n;
+        }
+      }
+    }
+    if constexpr (GRAD) {
+      __syncthreads();
+      {  // d3 in place of a3
+        const float dz = sdz;
+        const float* wh = sprm + 3 * NCH + 8 * (threadIdx.x & 1);
+        __nv_bfloat162 g[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          g[q] = pair_bf16(dz * wh[2 * q] * (1.0f / NPIX), dz * wh[2 * q + 1] * (1.0f / NPIX));
+        for (int k = threadIdx.x; k < NPIX * 2; k += NT) {
+          uint4* c = A3 + piece(padded(k >> 5, (k >> 1) & 15), k & 1);
+          uint4 v = *c;
+          unsigned* q4 = &v.x;
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const unsigned gq = *reinterpret_cast<const unsigned*>(&g[q]);
+            const unsigned lo = __uint_as_float(q4[q] << 16) > 0.f ? gq & 0xffffu : 0u;
+            const unsigned hi = __uint_as_float(q4[q] & 0xffff0000u) > 0.f ? gq & 0xffff0000u : 0u;
+            q4[q] = lo | hi;
+          }
+          *c = v;
+        }
+      }
+      __syncthreads();
+      // weight gradient of a layer, and the gradient of its input through the
+      // relu that made it (act), which both only read d
+      auto back = [&](const uint4* d, const uint4* act, uint4* out, int l) {
+        conv_dw(d, act, warp, lane, dw[l], db[l]);
+        if (warp < 8) {
+          const unsigned* m = reinterpret_cast<const unsigned*>(act);
+          unsigned* o = reinterpret_cast<unsigned*>(out);
+          conv(d, w + (2 + l) * NCH * WROW, warp, lane, [&](int at, int, float v0, float v1) {
+            const unsigned a = m[at];
+            if (!(__uint_as_float(a << 16) > 0.f)) v0 = 0.f;
+            if (!(__uint_as_float(a & 0xffff0000u) > 0.f)) v1 = 0.f;
+            *reinterpret_cast<__nv_bfloat162*>(o + at) = pair_bf16(v0, v1);
+          });
+        }
+        __syncthreads();
+      };
+      back(A3, A2, D2, 2);
+      back(D2, A1, A3, 1);
+      conv_dw(A3, X, warp, lane, dw[0], db[0]);
+    }
   }
+  if constexpr (GRAD) {
+    // the CTA's sums to the gradient: channel pairs are neighbours in dW
+#pragma unroll
+    for (int l = 0; l < 3; ++l)
+#pragma unroll
+      for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int co = (lane >> 2) + 8 * h, ci = nt * 8 + (lane & 3) * 2;
+          atomicAdd(reinterpret_cast<float2*>(grad + l * LAYER + co * KK + warp * 16 + ci),
+                    make_float2(dw[l][nt][2 * h], dw[l][nt][2 * h + 1]));
+        }
+    __syncthreads();
+    float2* sdb = reinterpret_cast<float2*>(X);  // [3][36 pixels][8 channel pairs]
+#pragma unroll
+    for (int l = 0; l < 3; ++l) sdb[l * 288 + threadIdx.x] = db[l];
+    __syncthreads();
+    if (threadIdx.x < 3 * NCH) {
+      const int l = threadIdx.x >> 4, c = threadIdx.x & 15;
+      const float* f = reinterpret_cast<const float*>(sdb + l * 288) + c;
+      float t = 0.f;
+      for (int k = 0; k < 36; ++k) t += f[k * 16];
+      atomicAdd(&grad[l * LAYER + NCH * KK + c], t);
+    } else if (threadIdx.x >= 64 && threadIdx.x < 64 + NCH + 2) {
+      const int k = threadIdx.x - 64;
+      atomicAdd(k <= NCH ? &grad[3 * LAYER + k] : loss, shead[k]);
+    }  }
 }
 
 // Adam on the FP32 master parameters, then the BF16 copies of the conv
@@ -332,16 +359,20 @@ __global__ void k_to_bf16(const float* __restrict__ x, bf16* __restrict__ y,
   if (k < n) y[k] = __float2bfloat16_rn(x[k]);
 }
 
-// Minibatch gather: xb[k] = x[idx[k]] (one CTA per sample), yb[k] = y[idx[k]].
-__global__ void k_gather(const bf16* __restrict__ x, const float* __restrict__ y,
-                         const int* __restrict__ idx, bf16* __restrict__ xb,
-                         float* __restrict__ yb) {
-  const int k = blockIdx.x;
-  const int src = idx[k];
-  const uint4* s4 = reinterpret_cast<const uint4*>(x + (size_t)src * NPAD * NCH);
-  uint4* d4 = reinterpret_cast<uint4*>(xb + (size_t)k * NPAD * NCH);
-  for (int t = threadIdx.x; t < NPAD * 2; t += blockDim.x) d4[t] = s4[t];
-  if (threadIdx.x == 0) yb[k] = y[src];
+template <bool GRAD>
+int launch_net(const void* x0, const int* idx, const void* wb, const void* wf, const float* prm,
+               const float* label, float pos_weight, float* logit, float* grad, float* loss,
+               int npatch, cudaStream_t st) {
+  constexpr size_t bytes = Net<GRAD>::smem();
+  if (cudaFuncSetAttribute(k_net<GRAD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)bytes) != cudaSuccess)
+    return -2;
+  const int fit = 152 * Net<GRAD>::PER_SM;
+  k_net<GRAD><<<npatch < fit ? npatch : fit, Net<GRAD>::NT, bytes, st>>>(
+      static_cast<const bf16*>(x0), idx, static_cast<const bf16*>(wb),
+      static_cast<const bf16*>(wf), prm, label, pos_weight, 1.0f / npatch, logit, grad, loss,
+      npatch);
+  return cudaGetLastError() == cudaSuccess ? 0 : -2;
 }
 
 inline int ok() { return cudaGetLastError() == cudaSuccess ? 0 : -2; }
@@ -357,70 +388,23 @@ constexpr int CNN_NPARAM = 3 * CNN_LAYER + NCH + 1;
 
 int cnn_nparam() { return CNN_NPARAM; }
 
-// Forward pass of npatch feature tiles x0 (BF16) with the BF16 weights wb:
-// fills a1, a2, a3, the pooled features v and the logits.
-int cnn_forward(const void* x0, const void* wb, const float* prm, void* a1,
-                void* a2, void* a3, float* v, float* logit, int npatch,
+// Logits of npatch feature tiles x0 (BF16) with the BF16 weights wb.
+int cnn_forward(const void* x0, const void* wb, const float* prm, float* logit, int npatch,
                 void* stream) {
   if (npatch <= 0) return 0;
-  cudaStream_t st = static_cast<cudaStream_t>(stream);
-  const bf16* W = static_cast<const bf16*>(wb);
-  k_conv<true, true, false, true><<<npatch, 256, 0, st>>>(
-      static_cast<const bf16*>(x0), W, prm + NCH * KK, nullptr, static_cast<bf16*>(a1));
-  k_conv<true, true, false, false><<<npatch, 256, 0, st>>>(
-      static_cast<const bf16*>(a1), W + NCH * KK, prm + CNN_LAYER + NCH * KK, nullptr,
-      static_cast<bf16*>(a2));
-  k_conv<true, true, false, false><<<npatch, 256, 0, st>>>(
-      static_cast<const bf16*>(a2), W + 2 * NCH * KK, prm + 2 * CNN_LAYER + NCH * KK,
-      nullptr, static_cast<bf16*>(a3));
-  k_head<<<(npatch + 7) / 8, 256, 0, st>>>(static_cast<const bf16*>(a3),
-                                            prm + 3 * CNN_LAYER,
-                                            prm + 3 * CNN_LAYER + NCH, logit, v,
-                                            npatch);
-  return ok();
+  return launch_net<false>(x0, nullptr, wb, nullptr, prm, nullptr, 1.f, logit, nullptr, nullptr,
+                           npatch, static_cast<cudaStream_t>(stream));
 }
 
-// Backward pass after cnn_forward: accumulates the gradient of the mean
-// weighted cross-entropy into grad (FP32, same layout as the parameters)
-// and the loss into *loss.  d1, d2, d3 are BF16 scratch of the activations'
-// shape.
-int cnn_backward(const void* x0, const void* wf, const float* prm,
-                 const void* a1, const void* a2, const void* a3, const float* v,
-                 const float* logit, const float* label, float pos_weight,
-                 float* grad, float* loss, void* d1, void* d2, void* d3,
-                 int npatch, void* stream) {
+// Forward and backward pass: logits, the gradient of the mean weighted
+// cross-entropy added to grad (FP32, same layout as the parameters) and the
+// loss to *loss.  Sample p is row idx[p] of x0 and label (idx null: row p).
+int cnn_grad(const void* x0, const int* idx, const void* wb, const void* wf, const float* prm,
+             const float* label, float pos_weight, float* logit, float* grad, float* loss,
+             int npatch, void* stream) {
   if (npatch <= 0) return 0;
-  cudaStream_t st = static_cast<cudaStream_t>(stream);
-  const bf16* Wf = static_cast<const bf16*>(wf);
-  k_head_bwd<<<npatch, 256, 0, st>>>(logit, label, v, static_cast<const bf16*>(a3),
-                                     prm + 3 * CNN_LAYER, pos_weight, 1.0f / npatch,
-                                     grad + 3 * CNN_LAYER, grad + 3 * CNN_LAYER + NCH,
-                                     static_cast<bf16*>(d3), loss);
-  // patches per CTA of the weight gradients: two CTAs to an SM, at most eight
-  // (each adds its 2320 sums to the gradient)
-  const int group = npatch >= 8 * 304 ? 8 : (npatch + 303) / 304;
-  const int blocks = (npatch + group - 1) / group;
-  // layer 3: weight gradient from a2, input gradient through relu(a2)
-  k_conv_dw<false><<<blocks, 288, 0, st>>>(static_cast<const bf16*>(d3),
-                                    static_cast<const bf16*>(a2),
-                                    grad + 2 * CNN_LAYER, grad + 2 * CNN_LAYER + NCH * KK,
-                                    npatch, group);
-  k_conv<false, false, true, false><<<npatch, 256, 0, st>>>(
-      static_cast<const bf16*>(d3), Wf + 2 * NCH * KK, nullptr,
-      static_cast<const bf16*>(a2), static_cast<bf16*>(d2));
-  // layer 2
-  k_conv_dw<false><<<blocks, 288, 0, st>>>(static_cast<const bf16*>(d2),
-                                    static_cast<const bf16*>(a1),
-                                    grad + CNN_LAYER, grad + CNN_LAYER + NCH * KK,
-                                    npatch, group);
-  k_conv<false, false, true, false><<<npatch, 256, 0, st>>>(
-      static_cast<const bf16*>(d2), Wf + NCH * KK, nullptr,
-      static_cast<const bf16*>(a1), static_cast<bf16*>(d1));
-  // layer 1: weight gradient from the input features
-  k_conv_dw<true><<<blocks, 288, 0, st>>>(static_cast<const bf16*>(d1),
-                                    static_cast<const bf16*>(x0), grad,
-                                    grad + NCH * KK, npatch, group);
-  return ok();
+  return launch_net<true>(x0, idx, wb, wf, prm, label, pos_weight, logit, grad, loss, npatch,
+                          static_cast<cudaStream_t>(stream));
 }
 
 int cnn_adam(float* prm, const float* grad, float* m, float* v, float lr,
@@ -438,14 +422,6 @@ int cnn_cast(const float* prm, void* wb, void* wf, void* stream) {
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   k_cast_weights<<<dim3((NCH * KK + 255) / 256, 3), 256, 0, st>>>(
       prm, CNN_LAYER, static_cast<bf16*>(wb), static_cast<bf16*>(wf));
-  return ok();
-}
-
-int cnn_gather(const void* x, const float* y, const int* idx, int n, void* xb,
-               float* yb, void* stream) {
-  if (n <= 0) return 0;
-  k_gather<<<n, 256, 0, static_cast<cudaStream_t>(stream)>>>(
-      static_cast<const bf16*>(x), y, idx, static_cast<bf16*>(xb), yb);
   return ok();
 }
 

@@ -278,21 +278,15 @@ int launch_cnn_features(const GfGeom& g, const GfView& v, int first, int count,
                         const float* scale, void* out, void* stream);
 // learned refinement predictor (gf_cnn.cu)
 int cnn_nparam();
-int cnn_forward(const void* x0, const void* wb, const float* prm, void* a1,
-                void* a2, void* a3, float* v, float* logit, int npatch,
+int cnn_forward(const void* x0, const void* wb, const float* prm, float* logit, int npatch,
                 void* stream);
-int cnn_backward(const void* x0, const void* wf, const float* prm,
-                 const void* a1, const void* a2, const void* a3, const float* v,
-                 const float* logit, const float* label, float pos_weight,
-                 float* grad, float* loss, void* d1, void* d2, void* d3,
-                 int npatch, void* stream);
+int cnn_grad(const void* x0, const int* idx, const void* wb, const void* wf, const float* prm,
+             const float* label, float pos_weight, float* logit, float* grad, float* loss,
+             int npatch, void* stream);
 int cnn_adam(float* prm, const float* grad, float* m, float* v, float lr,
              int t, void* stream);
 int cnn_cast(const float* prm, void* wb, void* wf, void* stream);
 int cnn_to_bf16(const float* x, void* y, size_t n, void* stream);
-int cnn_gather(const void* x, const float* y, const int* idx, int n, void* xb,
-               float* yb, void* stream);
 constexpr int CNN_IN_PIX = 324;  // 18 x 18 input pixels per patch
-constexpr int CNN_PIX = 256;     // 16 x 16 activation pixels per patch
 constexpr int CNN_CH = 16;
 }  // namespace gf
