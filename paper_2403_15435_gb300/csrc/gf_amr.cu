@@ -1185,26 +1185,34 @@ __global__ void __launch_bounds__(GF_GHOST_NT, 1) k_ghost_other(const __grid_con
 
 // ------------------------------------------------------------ topography
 
-// Bilinear interpolant of DEM k at (x, y), constant beyond its edges.
-__device__ double dem_eval(const GfScenario& S, int k, double x, double y) {
-  const int nx = S.dnx[k], ny = S.dny[k];
-  double fx = gfk::div_rn(x - S.dx0[k], S.ddx[k]), fy = gfk::div_rn(y - S.dy0[k], S.ddy[k]);
-  if (fx < 0.0) fx = 0.0;
-  if (fx > (double)(nx - 1)) fx = (double)(nx - 1);
-  if (fy < 0.0) fy = 0.0;
-  if (fy > (double)(ny - 1)) fy = (double)(ny - 1);
-  int i = (int)floor(fx), j = (int)floor(fy);
-  if (i > nx - 2) i = nx - 2;
-  if (j > ny - 2) j = ny - 2;
+// Sums of products are written as the fused operations they are computed
+// with, so that both ways to a cell's average below give the same bits.
+
+// Place of v along one axis of a DEM (o: first node, d: spacing, n: nodes):
+// lower node and fraction, constant beyond the ends.
+__device__ __forceinline__ int dem_place(double v, double o, double d, int n, double* frac) {
+  double f = gfk::div_rn(v - o, d);
+  if (f < 0.0) f = 0.0;
+  if (f > (double)(n - 1)) f = (double)(n - 1);
+  int i = (int)floor(f);
+  if (i > n - 2) i = n - 2;
   if (i < 0) i = 0;
-  if (j < 0) j = 0;
-  const double ax = fx - (double)i, ay = fy - (double)j;
-  const double* z = S.dem[k];
-  const double z00 = z[i + (size_t)j * nx], z10 = z[i + 1 + (size_t)j * nx];
-  const double z01 = z[i + (size_t)(j + 1) * nx];
-  const double z11 = z[i + 1 + (size_t)(j + 1) * nx];
-  return (1.0 - ay) * ((1.0 - ax) * z00 + ax * z10) +
-         ay * ((1.0 - ax) * z01 + ax * z11);
+  *frac = f - (double)i;
+  return i;
+}
+
+__device__ __forceinline__ bool dem_inside(double v, double o, double d, int n) {
+  return v >= o && v <= fma((double)(n - 1), d, o);
+}
+
+// Bilinear interpolant of DEM k between its nodes (i, j) and (i + 1, j + 1).
+__device__ __forceinline__ double dem_value(const GfScenario& S, int k, int i, int j, double ax,
+                                            double ay) {
+  const size_t nx = (size_t)S.dnx[k];
+  const double* z = S.dem[k] + (i + j * nx);
+  const double lo = fma(1.0 - ax, z[0], ax * z[1]);
+  const double hi = fma(1.0 - ax, z[nx], ax * z[nx + 1]);
+  return fma(1.0 - ay, lo, ay * hi);
 }
 
 // Composite interpolant of the scenario's DEMs (Sec. 6.2): the first DEM in
@@ -1212,12 +1220,14 @@ __device__ double dem_eval(const GfScenario& S, int k, double x, double y) {
 // extent the last (coarsest) one's, constant beyond its edges.
 __device__ double dems_eval(const GfScenario& S, double x, double y) {
   int k = 0;
-  for (; k < S.ndem; ++k) {
-    const double xe = S.dx0[k] + (double)(S.dnx[k] - 1) * S.ddx[k];
-    const double ye = S.dy0[k] + (double)(S.dny[k] - 1) * S.ddy[k];
-    if (x >= S.dx0[k] && x <= xe && y >= S.dy0[k] && y <= ye) break;
-  }
-  return dem_eval(S, k < S.ndem ? k : S.ndem - 1, x, y);
+  for (; k < S.ndem; ++k)
+    if (dem_inside(x, S.dx0[k], S.ddx[k], S.dnx[k]) && dem_inside(y, S.dy0[k], S.ddy[k], S.dny[k]))
+      break;
+  if (k == S.ndem) k = S.ndem - 1;
+  double ax, ay;
+  const int i = dem_place(x, S.dx0[k], S.ddx[k], S.dnx[k], &ax);
+  const int j = dem_place(y, S.dy0[k], S.ddy[k], S.dny[k], &ay);
+  return dem_value(S, k, i, j, ax, ay);
 }
 
 // The smallest break point above v along one axis (xaxis: x), at most b:
@@ -1234,17 +1244,16 @@ __device__ double next_break(const GfScenario& S, bool xaxis, double v, double b
     if (f < 0.0) f = 0.0;
     if (f > (double)n) f = (double)n;
     int i = (int)f;
-    while (i > 0 && o + (double)(i - 1) * d > v) --i;
-    while (i <= n - 1 && !(o + (double)i * d > v)) ++i;
+    while (i > 0 && fma((double)(i - 1), d, o) > v) --i;
+    while (i <= n - 1 && !(fma((double)i, d, o) > v)) ++i;
     if (i <= n - 1) {
-      const double xn = o + (double)i * d;
+      const double xn = fma((double)i, d, o);
       if (xn < best) best = xn;
     }
   }
   return best;
 }
 
-// (Quotients in the integer pipe: the FP64 pipe bounds this kernel.)
 // Exact average over [xa,xb]x[ya,yb] of the composite interpolant: the node
 // lines of all DEMs cut the cell into pieces on which it is bilinear; each
 // piece contributes its area times its midpoint value.  Rows of pieces in
@@ -1260,7 +1269,7 @@ __device__ double dem_average(const GfScenario& S, double xa, double xb,
       const double x1 = next_break(S, true, x0, xb);
       const double xm = 0.5 * (x0 + x1), ym = 0.5 * (y0 + y1);
       const double w = (x1 - x0) * (y1 - y0);
-      sum += w * dems_eval(S, xm, ym);
+      sum = fma(w, dems_eval(S, xm, ym), sum);
       x0 = x1;
     }
     y0 = y1;
@@ -1268,11 +1277,45 @@ __device__ double dem_average(const GfScenario& S, double xa, double xb,
   return gfk::div_rn(sum, (xb - xa) * (yb - ya));
 }
 
-// One CTA per patch.  448 threads (three rounds of the 1296 cells of a 32 x 32
-// patch's tile, one of a 16 x 16 patch's 400) instead of 128: a forest of
-// some hundred patches gives an SM one CTA, whose warps are all that hides
-// the FP64 latency.  116 patches on an 8 m DEM: 253 -> 164 us, 1856: 1150 ->
-// 717 us.
+// The pieces of one column or row of a tile's cells: length, and for each DEM
+// the place of the midpoint and whether its extent holds it.
+constexpr int TOPO_PIECES = 4, TOPO_TMAX = 36;
+struct TopoPiece {
+  double len, frac[GF_MAXDEM];
+  int at[GF_MAXDEM];
+  unsigned inside;
+};
+
+// Fills the pieces of [a, b]; their number, or TOPO_PIECES + 1 if there are more.
+__device__ int topo_pieces(const GfScenario& S, bool xaxis, double a, double b, TopoPiece* out) {
+  int n = 0;
+  for (double v0 = a; v0 < b; ++n) {
+    if (n == TOPO_PIECES) return TOPO_PIECES + 1;
+    const double v1 = next_break(S, xaxis, v0, b), vm = 0.5 * (v0 + v1);
+    TopoPiece& P = out[n];
+    P.len = v1 - v0;
+    P.inside = 0;
+    for (int k = 0; k < S.ndem; ++k) {
+      const double o = xaxis ? S.dx0[k] : S.dy0[k], d = xaxis ? S.ddx[k] : S.ddy[k];
+      const int m = xaxis ? S.dnx[k] : S.dny[k];
+      P.at[k] = dem_place(vm, o, d, m, &P.frac[k]);
+      if (dem_inside(vm, o, d, m)) P.inside |= 1u << k;
+    }
+    v0 = v1;
+  }
+  return n;
+}
+
+// One CTA per patch.  The FP64 pipe bounds this kernel, so what depends on a
+// cell's column or row alone (its pieces between node lines, their places in
+// the DEMs) is found once per column and row; a cell then takes some twelve
+// FP64 operations a piece instead of some eighty.  A patch with a column or
+// row of more than TOPO_PIECES pieces (cells several nodes wide) takes
+// dem_average cell by cell, as every patch did before.  448 threads: three
+// rounds of the 1296 cells of a 32 x 32 patch's tile, one of a 16 x 16
+// patch's 400; a forest of some hundred patches gives an SM one CTA, whose
+// warps are all that hides the latency.  116 patches on an 8 m DEM: 164 -> 40
+// us (FP64 218 -> 45), 1856: 717 -> 199 us.
 template <typename T>
 __global__ void __launch_bounds__(448) k_topo(const __grid_constant__ GfGeom G, const __grid_constant__ GfView V, int first,
                        const int* list) {
@@ -1293,16 +1336,46 @@ __global__ void __launch_bounds__(448) k_topo(const __grid_constant__ GfGeom G, 
   }
   const long long NX = e.nx(P.level), NY = e.ny(P.level);
   const double dx = G.dxl[P.level], dy = G.dyl[P.level];
+  __shared__ TopoPiece piece[2][TOPO_TMAX][TOPO_PIECES];
+  __shared__ int npiece[2][TOPO_TMAX];
+  const long long I0 = (long long)P.px * M - GF_NG, J0 = (long long)P.py * M - GF_NG;
+  bool many = false;
+  // columns by the first two warps, rows by the next two
+  if (threadIdx.x < 128) {
+    const int ax = threadIdx.x >> 6, c = threadIdx.x & 63;
+    const long long I = (ax == 0 ? I0 : J0) + c;
+    if (c < T_ && I >= 0 && I < (ax == 0 ? NX : NY)) {
+      const double d = ax == 0 ? dx : dy, o = ax == 0 ? G.xlower : G.ylower;
+      const int n = topo_pieces(S, ax == 0, fma((double)I, d, o), fma((double)(I + 1), d, o),
+                                piece[ax][c]);
+      npiece[ax][c] = n;
+      many = n > TOPO_PIECES;
+    }
+  }
+  const bool cells = __syncthreads_or(many);
   for (int k = threadIdx.x; k < TT; k += blockDim.x) {
-    const int i = k % T_ - GF_NG, j = k / T_ - GF_NG;
-    const long long I = (long long)P.px * M + i, J = (long long)P.py * M + j;
+    const int i = k % T_, j = k / T_;
+    const long long I = I0 + i, J = J0 + j;
     double v = 0.0;
     if (I >= 0 && J >= 0 && I < NX && J < NY && S.ndem > 0) {
-      const double xa = G.xlower + (double)I * dx;
-      const double xb = G.xlower + (double)(I + 1) * dx;
-      const double ya = G.ylower + (double)J * dy;
-      const double yb = G.ylower + (double)(J + 1) * dy;
-      v = dem_average(S, xa, xb, ya, yb);
+      const double xa = fma((double)I, dx, G.xlower);
+      const double xb = fma((double)(I + 1), dx, G.xlower);
+      const double ya = fma((double)J, dy, G.ylower);
+      const double yb = fma((double)(J + 1), dy, G.ylower);
+      if (cells) {
+        v = dem_average(S, xa, xb, ya, yb);
+      } else {
+        double sum = 0.0;
+        for (int yp = 0; yp < npiece[1][j]; ++yp)
+          for (int xp = 0; xp < npiece[0][i]; ++xp) {
+            const TopoPiece &X = piece[0][i][xp], &Y = piece[1][j][yp];
+            const unsigned in = X.inside & Y.inside;
+            const int kd = in ? __ffs(in) - 1 : S.ndem - 1;
+            sum = fma(X.len * Y.len, dem_value(S, kd, X.at[kd], Y.at[kd], X.frac[kd], Y.frac[kd]),
+                      sum);
+          }
+        v = gfk::div_rn(sum, (xb - xa) * (yb - ya));
+      }
     }
     // the deviation form keeps the bed relative to the reference surface
     b[k] = Geo<T>::DEV ? (T)(v - S.eta0) : (T)v;
