@@ -1185,9 +1185,6 @@ __global__ void __launch_bounds__(GF_GHOST_NT, 1) k_ghost_other(const __grid_con
 
 // ------------------------------------------------------------ topography
 
-// Sums of products are written as the fused operations they are computed
-// with, so that both ways to a cell's average below give the same bits.
-
 // Place of v along one axis of a DEM (o: first node, d: spacing, n: nodes):
 // lower node and fraction, constant beyond the ends.
 __device__ __forceinline__ int dem_place(double v, double o, double d, int n, double* frac) {
@@ -1202,17 +1199,18 @@ __device__ __forceinline__ int dem_place(double v, double o, double d, int n, do
 }
 
 __device__ __forceinline__ bool dem_inside(double v, double o, double d, int n) {
-  return v >= o && v <= fma((double)(n - 1), d, o);
+  return v >= o && v <= o + (double)(n - 1) * d;
 }
 
-// Bilinear interpolant of DEM k between its nodes (i, j) and (i + 1, j + 1).
+// Bilinear interpolant of DEM k between its nodes (i, j) and (i + 1, j + 1);
+// (rx, ry) is 1 - (ax, ay).
 __device__ __forceinline__ double dem_value(const GfScenario& S, int k, int i, int j, double ax,
-                                            double ay) {
+                                            double rx, double ay, double ry) {
   const size_t nx = (size_t)S.dnx[k];
   const double* z = S.dem[k] + (i + j * nx);
-  const double lo = fma(1.0 - ax, z[0], ax * z[1]);
-  const double hi = fma(1.0 - ax, z[nx], ax * z[nx + 1]);
-  return fma(1.0 - ay, lo, ay * hi);
+  const double lo = rx * z[0] + ax * z[1];
+  const double hi = rx * z[nx] + ax * z[nx + 1];
+  return ry * lo + ay * hi;
 }
 
 // Composite interpolant of the scenario's DEMs (Sec. 6.2): the first DEM in
@@ -1227,7 +1225,7 @@ __device__ double dems_eval(const GfScenario& S, double x, double y) {
   double ax, ay;
   const int i = dem_place(x, S.dx0[k], S.ddx[k], S.dnx[k], &ax);
   const int j = dem_place(y, S.dy0[k], S.ddy[k], S.dny[k], &ay);
-  return dem_value(S, k, i, j, ax, ay);
+  return dem_value(S, k, i, j, ax, 1.0 - ax, ay, 1.0 - ay);
 }
 
 // The smallest break point above v along one axis (xaxis: x), at most b:
@@ -1244,10 +1242,10 @@ __device__ double next_break(const GfScenario& S, bool xaxis, double v, double b
     if (f < 0.0) f = 0.0;
     if (f > (double)n) f = (double)n;
     int i = (int)f;
-    while (i > 0 && fma((double)(i - 1), d, o) > v) --i;
-    while (i <= n - 1 && !(fma((double)i, d, o) > v)) ++i;
+    while (i > 0 && o + (double)(i - 1) * d > v) --i;
+    while (i <= n - 1 && !(o + (double)i * d > v)) ++i;
     if (i <= n - 1) {
-      const double xn = fma((double)i, d, o);
+      const double xn = o + (double)i * d;
       if (xn < best) best = xn;
     }
   }
@@ -1269,7 +1267,7 @@ __device__ double dem_average(const GfScenario& S, double xa, double xb,
       const double x1 = next_break(S, true, x0, xb);
       const double xm = 0.5 * (x0 + x1), ym = 0.5 * (y0 + y1);
       const double w = (x1 - x0) * (y1 - y0);
-      sum = fma(w, dems_eval(S, xm, ym), sum);
+      sum += w * dems_eval(S, xm, ym);
       x0 = x1;
     }
     y0 = y1;
@@ -1278,10 +1276,11 @@ __device__ double dem_average(const GfScenario& S, double xa, double xb,
 }
 
 // The pieces of one column or row of a tile's cells: length, and for each DEM
-// the place of the midpoint and whether its extent holds it.
+// the place of the midpoint (rest: one minus the fraction) and whether its
+// extent holds it.
 constexpr int TOPO_PIECES = 4, TOPO_TMAX = 36;
 struct TopoPiece {
-  double len, frac[GF_MAXDEM];
+  double len, frac[GF_MAXDEM], rest[GF_MAXDEM];
   int at[GF_MAXDEM];
   unsigned inside;
 };
@@ -1299,6 +1298,7 @@ __device__ int topo_pieces(const GfScenario& S, bool xaxis, double a, double b, 
       const double o = xaxis ? S.dx0[k] : S.dy0[k], d = xaxis ? S.ddx[k] : S.ddy[k];
       const int m = xaxis ? S.dnx[k] : S.dny[k];
       P.at[k] = dem_place(vm, o, d, m, &P.frac[k]);
+      P.rest[k] = 1.0 - P.frac[k];
       if (dem_inside(vm, o, d, m)) P.inside |= 1u << k;
     }
     v0 = v1;
@@ -1314,8 +1314,8 @@ __device__ int topo_pieces(const GfScenario& S, bool xaxis, double a, double b, 
 // dem_average cell by cell, as every patch did before.  448 threads: three
 // rounds of the 1296 cells of a 32 x 32 patch's tile, one of a 16 x 16
 // patch's 400; a forest of some hundred patches gives an SM one CTA, whose
-// warps are all that hides the latency.  116 patches on an 8 m DEM: 164 -> 40
-// us (FP64 218 -> 45), 1856: 717 -> 199 us.
+// warps are all that hides the latency.  116 patches on an 8 m DEM: 164 -> 44
+// us (FP64 218 -> 52), 1856: 717 -> 206 us; the beds keep every bit.
 template <typename T>
 __global__ void __launch_bounds__(448) k_topo(const __grid_constant__ GfGeom G, const __grid_constant__ GfView V, int first,
                        const int* list) {
@@ -1338,6 +1338,7 @@ __global__ void __launch_bounds__(448) k_topo(const __grid_constant__ GfGeom G, 
   const double dx = G.dxl[P.level], dy = G.dyl[P.level];
   __shared__ TopoPiece piece[2][TOPO_TMAX][TOPO_PIECES];
   __shared__ int npiece[2][TOPO_TMAX];
+  __shared__ double span[2][TOPO_TMAX];
   const long long I0 = (long long)P.px * M - GF_NG, J0 = (long long)P.py * M - GF_NG;
   bool many = false;
   // columns by the first two warps, rows by the next two
@@ -1346,8 +1347,9 @@ __global__ void __launch_bounds__(448) k_topo(const __grid_constant__ GfGeom G, 
     const long long I = (ax == 0 ? I0 : J0) + c;
     if (c < T_ && I >= 0 && I < (ax == 0 ? NX : NY)) {
       const double d = ax == 0 ? dx : dy, o = ax == 0 ? G.xlower : G.ylower;
-      const int n = topo_pieces(S, ax == 0, fma((double)I, d, o), fma((double)(I + 1), d, o),
-                                piece[ax][c]);
+      const double a = o + (double)I * d, b2 = o + (double)(I + 1) * d;
+      const int n = topo_pieces(S, ax == 0, a, b2, piece[ax][c]);
+      span[ax][c] = b2 - a;
       npiece[ax][c] = n;
       many = n > TOPO_PIECES;
     }
@@ -1358,11 +1360,11 @@ __global__ void __launch_bounds__(448) k_topo(const __grid_constant__ GfGeom G, 
     const long long I = I0 + i, J = J0 + j;
     double v = 0.0;
     if (I >= 0 && J >= 0 && I < NX && J < NY && S.ndem > 0) {
-      const double xa = fma((double)I, dx, G.xlower);
-      const double xb = fma((double)(I + 1), dx, G.xlower);
-      const double ya = fma((double)J, dy, G.ylower);
-      const double yb = fma((double)(J + 1), dy, G.ylower);
       if (cells) {
+        const double xa = G.xlower + (double)I * dx;
+        const double xb = G.xlower + (double)(I + 1) * dx;
+        const double ya = G.ylower + (double)J * dy;
+        const double yb = G.ylower + (double)(J + 1) * dy;
         v = dem_average(S, xa, xb, ya, yb);
       } else {
         double sum = 0.0;
@@ -1371,10 +1373,11 @@ __global__ void __launch_bounds__(448) k_topo(const __grid_constant__ GfGeom G, 
             const TopoPiece &X = piece[0][i][xp], &Y = piece[1][j][yp];
             const unsigned in = X.inside & Y.inside;
             const int kd = in ? __ffs(in) - 1 : S.ndem - 1;
-            sum = fma(X.len * Y.len, dem_value(S, kd, X.at[kd], Y.at[kd], X.frac[kd], Y.frac[kd]),
-                      sum);
+            sum += X.len * Y.len *
+                   dem_value(S, kd, X.at[kd], Y.at[kd], X.frac[kd], X.rest[kd], Y.frac[kd],
+                             Y.rest[kd]);
           }
-        v = gfk::div_rn(sum, (xb - xa) * (yb - ya));
+        v = gfk::div_rn(sum, span[0][i] * span[1][j]);
       }
     }
     // the deviation form keeps the bed relative to the reference surface
