@@ -153,9 +153,9 @@ struct geoflood_ctx {
 
 namespace {
 
-// Device memory the bed cache may take (all scenarios, all levels).
 // work units (sub-tile CTAs) a patch can have: 8 x 8 sub-tiles of 32 x 32
 constexpr size_t kUnits = 16;
+// Device memory the bed cache may take (all scenarios, all levels).
 constexpr size_t kBedCacheBudget = size_t(16) << 30;
 
 int fail(geoflood_ctx* c, int code, const std::string& msg) {
@@ -2271,8 +2271,9 @@ int geoflood_load(geoflood_ctx* ctx, const void* buf, size_t size) {
       x.nx.push_back(r.val<int>()); x.ny.push_back(r.val<int>());
       x.x0.push_back(r.val<double>()); x.y0.push_back(r.val<double>());
       x.dx.push_back(r.val<double>()); x.dy.push_back(r.val<double>());
+      // (the product of the two counts cannot wrap, eight times it can)
       if (!r.ok || x.nx.back() < 2 || x.ny.back() < 2 ||
-          (size_t)x.nx.back() * x.ny.back() * 8 > size)
+          (size_t)x.nx.back() * x.ny.back() > size / 8)
         return fail(ctx, GEOFLOOD_ERR_ARG, "load: corrupt DEM");
       x.z.push_back(r.skip((size_t)x.nx.back() * x.ny.back() * 8));
     }
@@ -2352,8 +2353,10 @@ int geoflood_load(geoflood_ctx* ctx, const void* buf, size_t size) {
       if (fits) {
         d = ctx->d_dem[s][k];
       } else {
-        if (cudaMalloc(&d, bytes) != cudaSuccess)
+        if (cudaMalloc(&d, bytes) != cudaSuccess) {
+          cudaStreamSynchronize(ctx->st);  // copies out of the caller's buffer
           return fail(ctx, GEOFLOOD_ERR_OOM, "load: DEM allocation");
+        }
         ctx->d_dem[s].push_back(d);
       }
       CK(cudaMemcpyAsync(d, sc[s].z[k], bytes, cudaMemcpyHostToDevice, ctx->st));

@@ -134,7 +134,7 @@ __device__ __forceinline__ void conv_dw(const uint4* dy, const uint4* in, int ta
 // the weighted cross-entropy: weight gradients stay in registers over the
 // CTA's patches and are added to grad once at its end.  What bounds it is a
 // patch's chain of eight phases between barriers, so as many CTAs share an SM
-// as shared memory allows (72 KB: three; forward alone 46 KB: four).
+// as shared memory and registers allow (74 KB: three; forward alone 45 KB: four).
 // 1024 samples' loss and gradient on the device: nine launches with the
 // activations written and read between them about 120 us, this one 51; the
 // whole call 268 -> 175 us.
@@ -321,7 +321,8 @@ __global__ void __launch_bounds__(Net<GRAD>::NT, Net<GRAD>::PER_SM)
     } else if (threadIdx.x >= 64 && threadIdx.x < 64 + NCH + 2) {
       const int k = threadIdx.x - 64;
       atomicAdd(k <= NCH ? &grad[3 * LAYER + k] : loss, shead[k]);
-    }  }
+    }
+  }
 }
 
 // Adam on the FP32 master parameters, then the BF16 copies of the conv

@@ -261,8 +261,9 @@ class Forest:
     def load(self, data):
         """Resume from a checkpoint of save() (same configuration)."""
         # bytes are read in place; other buffers are copied into some
-        buf = C.c_char_p(data if isinstance(data, bytes) else bytes(data))
-        self._check(lib().geoflood_load(self._h, C.cast(buf, C.c_void_p), memoryview(data).nbytes))
+        buf = (C.c_char_p(data) if isinstance(data, bytes)
+               else (C.c_ubyte * len(data)).from_buffer_copy(data))
+        self._check(lib().geoflood_load(self._h, C.cast(buf, C.c_void_p), len(data)))
 
     def set_topo(self, dem, s=0):
         """One DEM, or a list of up to 4 overlapping DEMs (Sec. 6.2)."""
