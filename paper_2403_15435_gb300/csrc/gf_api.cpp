@@ -181,8 +181,9 @@ int fail(geoflood_ctx* c, int code, const std::string& msg) {
     }                                                                     \
   } while (0)
 
-// Run flags of the patch step: three arrays, then the word GfView::inactive,
-// which one fill with ones ("every patch runs") sets above any patch count.
+// Run flags of the patch step: three arrays, then the two words of
+// GfView::inactive, which one fill with ones ("every patch runs") sets above
+// any patch count.
 size_t runf_bytes(const geoflood_ctx* c) {
   return (((size_t)c->cap * 3 + 15) & ~size_t(15)) + 16;
 }
@@ -1202,12 +1203,12 @@ int geoflood_get_time(geoflood_ctx* ctx, int s, double* t, double* dt_next,
 static int step_core(geoflood_ctx* ctx, double t_target, int max_steps, double* t_out,
                      int* steps_out, int* misses) {
   if (!ctx || max_steps < 0) return fail(ctx, GEOFLOOD_ERR_ARG, "step: bad argument");
+  GfView v = view(ctx);
   CKL(gf::launch_ctl_begin(ctx->d_ctl, ctx->nscen, t_target, max_steps,
-                           nullptr, ctx->st),
+                           nullptr, v.inactive, ctx->st),
       "ctl_begin");
   ctx->launches++;
   gf::set_errflag(ctx->d_err);
-  const GfView v = view(ctx);
   // The steps run in chunks of K captured as one CUDA graph (patch step with
   // the fused CFL controller, ghost fill, gauges); the device controller
   // deactivates a scenario when it reaches t_target or max_steps accepted
@@ -1253,6 +1254,8 @@ static int step_core(geoflood_ctx* ctx, double t_target, int max_steps, double* 
           rg.b = pool_event(ctx);
           cudaEventRecordWithFlags(r.a, ctx->st, cudaEventRecordExternal);
         }
+        // the last launch writes inactive[1]
+        v.parity = (unsigned)(K * ctx->G.sub_K - 1 - (it * ctx->G.sub_K + sub)) & 1u;
         lrc |= ctx->prec ? gf::launch_patch_step_f32(ctx->G, v, ctx->variant, ctx->st)
                          : gf::launch_patch_step_f64(ctx->G, v, ctx->variant, ctx->st);
         if (sample) {

@@ -146,12 +146,21 @@ struct GfView {
   // the launches modulo 6; its parity selects which of ord0/ord1 a launch
   // reads; the launch writes the other one with the patches that took the
   // step first (sched[1], sched[2] count those and the others), and its last
-  // CTA advances sched[0] and stores the number of the others in *inactive.
-  // (Without run flags: the patches whose tile held water first.)  A value
-  // of *inactive above npatch means that nothing is known yet: every patch
-  // then gets its own CTAs.  Only with a controller (done != null).
+  // CTA advances sched[0] and stores the number of the others in
+  // inactive[parity ^ 1].  (Without run flags: the patches whose tile held
+  // water first.)  Only with a controller (done != null).
+  //
+  // A launch reads inactive[parity]; the host alternates parity from launch
+  // to launch, so that no launch writes the word it reads: every CTA of it,
+  // however late it starts, counts the same working CTAs.  The value decides
+  // only how the order is shared out, never which patches run: above npatch
+  // (nothing known yet) every patch gets its own CTAs, and an older launch's
+  // number is right too.  A chunk's last launch writes inactive[1], which the
+  // next chunk reads first if its launches are even in number; otherwise it
+  // reads inactive[0], where ctl_begin has put the same.
   unsigned* sched;
   unsigned* inactive;
+  unsigned parity;
   int* ord0;
   int* ord1;
   // Per CTA work unit (patch * sub-tiles + sub-tile): 1 when both state
@@ -224,7 +233,8 @@ int launch_patch_step_f64(const GfGeom& g, const GfView& v, int variant, void* s
 int launch_patch_step_f32(const GfGeom& g, const GfView& v, int variant, void* stream);
 int launch_patch_step_f32_split(const GfGeom& g, const GfView& v, void* stream);
 int launch_ctl_begin(GfCtl* ctl, int nscen, double t_target,
-                     long long max_steps, const int* scen_mask, void* stream);
+                     long long max_steps, const int* scen_mask, unsigned* inactive,
+                     void* stream);
 int launch_ghost_fill(const GfGeom& g, const GfView& v, int only_active,
                       void* stream);
 // Ghost cells in regions without a same-level neighbour (which the patch

@@ -15,8 +15,9 @@
 namespace {
 
 __global__ void k_ctl_begin(GfCtl* ctl, int nscen, double t_target,
-                            long long max_steps, const int* mask) {
+                            long long max_steps, const int* mask, unsigned* inactive) {
   const int s = blockIdx.x * blockDim.x + threadIdx.x;
+  if (s == 0) inactive[0] = inactive[1];
   if (s >= nscen) return;
   GfCtl* C = ctl + s;
   C->t_target = t_target;
@@ -122,10 +123,11 @@ int launch_patch_step_f64(const GfGeom& g, const GfView& v, int variant,
 }
 
 int launch_ctl_begin(GfCtl* ctl, int nscen, double t_target,
-                     long long max_steps, const int* mask, void* stream) {
+                     long long max_steps, const int* mask, unsigned* inactive,
+                     void* stream) {
   k_ctl_begin<<<(nscen + 127) / 128, 128, 0,
                 static_cast<cudaStream_t>(stream)>>>(ctl, nscen, t_target,
-                                                      max_steps, mask);
+                                                      max_steps, mask, inactive);
   return cudaGetLastError() == cudaSuccess ? 0 : -2;
 }
 

@@ -1857,7 +1857,9 @@ __device__ void step_finish(const GfGeom& G, const GfView& V, int cells_per_patc
   if (threadIdx.x == 0 && V.sched) {
     V.sched[0] = (V.sched[0] + 1u) % 6u;
     // patches that took no step, at the tail of the next order
-    if (V.inactive) *V.inactive = V.sched[2];
+    // (in the word this launch does not read: CTAs beyond the working ones
+    // may start after this and must still find themselves beyond)
+    if (V.inactive) V.inactive[V.parity ^ 1u] = V.sched[2];
     V.sched[1] = 0u;
     V.sched[2] = 0u;
   }
@@ -1904,7 +1906,7 @@ __global__ void __launch_bounds__(NT, MINB)
     count = V.sched[0];
     e0 = V.ord0[slot];
     e1 = V.ord1[slot];
-    if (GROUPS && use_flags) inactive = (int)*V.inactive;
+    if (GROUPS && use_flags) inactive = (int)V.inactive[V.parity];
   }
   if (inactive > V.npatch) inactive = 0;  // unknown: every patch by itself
   const int nact = V.npatch - inactive;
