@@ -67,6 +67,10 @@ float seed_rsqrt(float x);
 double native_sqrt(double x);
 #endif
 
+// Remainders below are exact modulo 2^64 although the products they come from
+// are longer: formed unsigned, read signed.
+typedef unsigned long long u64;
+
 constexpr long long D_MANT = (1ll << 52) - 1;
 constexpr long long D_HID = 1ll << 52;
 constexpr long long D_INF = 0x7ffll << 52;
@@ -85,18 +89,18 @@ GF_HD_CALL double div_rn(double a, double b) {
   const int e = ea - eb;
   // both operands and the quotient well inside the normal range
   if ((unsigned)(ea - 1) < 2046u && (unsigned)(eb - 1) < 2046u && (unsigned)(e + 1021) < 2043u) {
-    const long long ma = (ab & D_MANT) | D_HID, mb = (bb & D_MANT) | D_HID;
+    const u64 ma = (u64)((ab & D_MANT) | D_HID), mb = (u64)((bb & D_MANT) | D_HID);
     const float fa = bitsf(0x3f800000u | (unsigned)((ab & D_MANT) >> 29));
     const float fb = bitsf(0x3f800000u | (unsigned)((bb & D_MANT) >> 29));
     const float y = seed_rcp(fb);
     const int q1 = f2i_magic(fmul(fa, fmul(y, 1048576.0f)));
-    const long long r1 = (long long)((unsigned long long)ma << 20) - (long long)q1 * mb;
+    const long long r1 = (long long)((ma << 20) - (u64)(long long)q1 * mb);
     const int q2 = f2i_magic(fmul(i2f((int)(r1 >> 24)), fmul(y, 0x1p-8f)));
-    const long long r2 = (long long)((unsigned long long)r1 << 20) - (long long)q2 * mb;
+    const long long r2 = (long long)(((u64)r1 << 20) - (u64)(long long)q2 * mb);
     const int q3 = f2i_magic(fmul(i2f((int)(r2 >> 24)), fmul(y, 0x1p-13f)));
-    const long long r3 = (long long)((unsigned long long)r2 << 15) - (long long)q3 * mb;
+    const long long r3 = (long long)(((u64)r2 << 15) - (u64)(long long)q3 * mb);
     // quotient ma 2^55 / mb in (2^54, 2^56): floor, then the sticky bit
-    long long Q = ((long long)q1 << 35) + (long long)q2 * 32768 + q3;
+    long long Q = (long long)((u64)q1 << 35) + (long long)q2 * 32768 + q3;
     Q += r3 >> 63;
     Q |= r3 != 0 ? 1 : 0;
     const bool small = Q < (1ll << 55);
@@ -105,7 +109,7 @@ GF_HD_CALL double div_rn(double a, double b) {
     const long long r = ((long long)(e + (small ? 1021 : 1022)) << 52) + m;
     return bitsd(r | ((ab ^ bb) & (long long)0x8000000000000000ull));
   }
-  if ((ab << 1) == 0 && (unsigned)(eb - 1) < 2046u)  // signed zero
+  if ((u64)ab << 1 == 0 && (unsigned)(eb - 1) < 2046u)  // signed zero
     return bitsd((ab ^ bb) & (long long)0x8000000000000000ull);
   return a / b;
 }
@@ -120,28 +124,26 @@ GF_HD_CALL double sqrt_rn(double x) {
   const int ex = (int)(xb >> 52);  // sign included: negative values fall out
   if ((unsigned)(ex - 1) < 2046u) {
     const int odd = (ex + 1) & 1;  // ex - 1023 odd
-    const unsigned long long m = (unsigned long long)((xb & D_MANT) | D_HID) << odd;
+    const u64 m = (u64)((xb & D_MANT) | D_HID) << odd;
     const float f0 = bitsf(0x3f800000u | (unsigned)((xb & D_MANT) >> 29));
     const float f = odd ? f0 + f0 : f0;
     const float y = seed_rsqrt(f);
     const int s1 = f2i_magic(fmul(fmul(f, y), 1048576.0f));
-    const long long r1 = (long long)(m - ((unsigned long long)((long long)s1 * s1) << 12));
+    const long long r1 = (long long)(m - ((u64)((long long)s1 * s1) << 12));
     const int s2 = f2i_magic(fmul(i2f((int)(r1 >> 8)), fmul(y, 0x1p-5f)));
-    const long long r2 =
-        (long long)((unsigned long long)r1 << 28) -
-        (long long)((unsigned long long)((long long)s1 * s2) << 21) - (long long)s2 * s2;
+    const long long r2 = (long long)(((u64)r1 << 28) - ((u64)((long long)s1 * s2) << 21) -
+                                     (u64)((long long)s2 * s2));
     const long long S2 = ((long long)s1 << 20) + s2;
     const int s3 = f2i_magic(fmul(i2f((int)(r2 >> 16)), fmul(y, 0x1p-12f)));
-    const long long r3 = (long long)(((unsigned long long)r2 << 26) -
-                                     ((unsigned long long)(S2 * s3) << 14)) -
-                         (long long)s3 * s3;
+    const long long r3 = (long long)(((u64)r2 << 26) - ((u64)(S2 * s3) << 14) -
+                                     (u64)((long long)s3 * s3));
     long long S = (S2 << 13) + s3;
     S += r3 >> 63;
     const long long mr = (S + 1) >> 1;  // [2^52, 2^53]
     const int er = (ex - 1023 - odd) / 2 + 1022;
     return bitsd(((long long)er << 52) + mr);
   }
-  if ((xb << 1) == 0) return x;
+  if ((u64)xb << 1 == 0) return x;
   return native_sqrt(x);
 }
 
@@ -153,16 +155,16 @@ GF_HD long long okey(double x) {  // order-preserving; -0 and +0 alike
   return b < 0 ? (long long)(0x8000000000000000ull - (unsigned long long)b) : b;
 }
 GF_HD bool dlt(double a, double b) { return okey(a) < okey(b); }
-GF_HD bool neg(double x) { return dbits(x) < 0 && (dbits(x) << 1) != 0; }
+GF_HD bool neg(double x) { return dbits(x) < 0 && (u64)dbits(x) << 1 != 0; }
 GF_HD bool pos(double x) { return dbits(x) > 0; }
-GF_HD bool iszero(double x) { return (dbits(x) << 1) == 0; }
+GF_HD bool iszero(double x) { return (u64)dbits(x) << 1 == 0; }
 GF_HD double dabs(double x) { return bitsd(dbits(x) & 0x7fffffffffffffffll); }
 GF_HD double dneg(double x) { return bitsd(dbits(x) ^ (long long)0x8000000000000000ull); }
 GF_HD double dmin(double a, double b) { return dlt(a, b) ? a : b; }
 GF_HD double dmax(double a, double b) { return dlt(b, a) ? a : b; }
 // h > d for a positive threshold d; false for NaN
 GF_HD bool above(double h, double d) {
-  return (unsigned long long)(dbits(h) - dbits(d) - 1) < (unsigned long long)(D_INF - dbits(d));
+  return (u64)dbits(h) - (u64)dbits(d) - 1u < (u64)D_INF - (u64)dbits(d);
 }
 // x / 2 and 2 x by the exponent, at the ends of the range too (a product
 // there, however rare, would take a slot of the FP64 pipe each time: the
