@@ -867,23 +867,28 @@ __device__ __forceinline__ f2 limit32x2(f2 num, f2 zz, f2 hs, f2 m, f2 nz) {
 }
 
 // edge_fluxes for the edges at w and w + 1 (planes of pitch ST, SE the place
-// of the next edge of a line); wet0, wet1: both cells of the edge are wet.
+// of the next edge of a line); wet0, wet1: the edge takes a correction (both
+// its cells are wet).  Where neither does, the limiters are left out.
 template <int ST, int SE>
 __device__ __forceinline__ void edge32x2(const float* w, float nu, bool wet0, bool wet1, f2 nz,
                                          f2 (&am)[3], f2 (&ap)[3], f2 (&ff)[3]) {
+#pragma unroll
+  for (int k = 0; k < 3; ++k) am[k] = ap[k] = ff[k] = 0ull;
+  const f2 s1 = ld2(w + 8 * ST), s3 = ld2(w + 9 * ST);
+  if ((s1 | s3) == 0ull) return;  // between dry cells
   f2 z[8];
 #pragma unroll
   for (int c = 0; c < 8; ++c) z[c] = ld2(w + c * ST);
-  const f2 s1 = ld2(w + 8 * ST), s3 = ld2(w + 9 * ST);
   const f2 s2 = mul2(pk1(0.5f), add2(s1, s3));
   float a1, b1, a2, b2, a3, b3;
   upk(s1, a1, b1);
   upk(s2, a2, b2);
   upk(s3, a3, b3);
-  f2 u[8];       // the upwind edges' waves
-  f2 h1, h2, h3;  // half the signs
-  if (fmaxf(a1, b1) < 0.0f && fminf(a3, b3) > 0.0f && a2 != 0.0f && b2 != 0.0f) {
-    // first wave leftwards, third rightwards, the middle one to one side
+  // first wave leftwards, third rightwards, the middle one to one side; an
+  // edge between dry cells beside such a one has zero waves, which may go with it
+  const bool usual = ((a1 < 0.0f && a3 > 0.0f && a2 != 0.0f) || (a1 == 0.0f && a3 == 0.0f)) &&
+                     ((b1 < 0.0f && b3 > 0.0f && b2 != 0.0f) || (b1 == 0.0f && b3 == 0.0f));
+  if (usual) {
     const bool n0 = a2 < 0.0f, n1 = b2 < 0.0f;
     am[0] = z[0];
     ap[0] = z[5];
@@ -893,6 +898,24 @@ __device__ __forceinline__ void edge32x2(const float* w, float nu, bool wet0, bo
       am[k] = sel2(n0, n1, x, z[k]);
       ap[k] = sel2(n0, n1, z[5 + k], x);
     }
+  } else {
+    auto side = [](float s) { return s < 0.0f ? 1.0f : (s == 0.0f ? 0.5f : 0.0f); };
+    const f2 m1 = pk(side(a1), side(b1)), m2 = pk(side(a2), side(b2)), m3 = pk(side(a3), side(b3));
+    const f2 one = pk1(1.0f);
+    const f2 p1 = sub2(one, m1), p2 = sub2(one, m2), p3 = sub2(one, m3);
+    am[0] = add2(mul2(m1, z[0]), mul2(m3, z[5]));
+    ap[0] = add2(mul2(p1, z[0]), mul2(p3, z[5]));
+#pragma unroll
+    for (int k = 1; k < 3; ++k) {
+      am[k] = add2(add2(mul2(m1, z[k]), mul2(m3, z[5 + k])), mul2(m2, z[2 + k]));
+      ap[k] = add2(add2(mul2(p1, z[k]), mul2(p3, z[5 + k])), mul2(p2, z[2 + k]));
+    }
+  }
+  if (!(wet0 || wet1)) return;
+  f2 u[8];        // the upwind edges' waves
+  f2 h1, h2, h3;  // half the signs
+  if (usual) {
+    const bool n0 = a2 < 0.0f, n1 = b2 < 0.0f;
     if constexpr (SE % 2 == 0) {
 #pragma unroll
       for (int c = 0; c < 3; ++c) u[c] = ld2(w + c * ST + SE);
@@ -916,17 +939,6 @@ __device__ __forceinline__ void edge32x2(const float* w, float nu, bool wet0, bo
     h3 = pk1(0.5f);
     h2 = pk(n0 ? -0.5f : 0.5f, n1 ? -0.5f : 0.5f);
   } else {
-    auto side = [](float s) { return s < 0.0f ? 1.0f : (s == 0.0f ? 0.5f : 0.0f); };
-    const f2 m1 = pk(side(a1), side(b1)), m2 = pk(side(a2), side(b2)), m3 = pk(side(a3), side(b3));
-    const f2 one = pk1(1.0f);
-    const f2 p1 = sub2(one, m1), p2 = sub2(one, m2), p3 = sub2(one, m3);
-    am[0] = add2(mul2(m1, z[0]), mul2(m3, z[5]));
-    ap[0] = add2(mul2(p1, z[0]), mul2(p3, z[5]));
-#pragma unroll
-    for (int k = 1; k < 3; ++k) {
-      am[k] = add2(add2(mul2(m1, z[k]), mul2(m3, z[5 + k])), mul2(m2, z[2 + k]));
-      ap[k] = add2(add2(mul2(p1, z[k]), mul2(p3, z[5 + k])), mul2(p2, z[2 + k]));
-    }
     const int o10 = a1 > 0.0f ? -SE : SE, o11 = (b1 > 0.0f ? -SE : SE) + 1;
     const int o30 = a3 > 0.0f ? -SE : SE, o31 = (b3 > 0.0f ? -SE : SE) + 1;
 #pragma unroll
