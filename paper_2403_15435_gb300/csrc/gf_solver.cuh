@@ -615,108 +615,6 @@ __device__ __forceinline__ bool wet_dev(float w, float b, double drytol,
 
 __device__ __forceinline__ float rcpf(float x) { return seed_rcp(x); }
 
-// One side of an edge in the deviation form: stored surface and bed (minus
-// eta0), normal momentum, velocities and the root of the depth (u, v and q
-// are zero in a dry cell).
-struct Prim32 {
-  float w, b, n, u, v, q;
-};
-
-// Waves z[8] as in riemann_prim and the outer speeds s1, s3 (the middle one
-// is their mean): the general case.
-__device__ __forceinline__ void riemann32(Prim32 l, Prim32 r, float g, float (&z)[8],
-                                              float& s1, float& s3) {
-#pragma unroll
-  for (int k = 0; k < 8; ++k) z[k] = 0.0f;
-  s1 = s3 = 0.0f;
-  const bool wl = l.q > 0.0f, wr = r.q > 0.0f;
-  if (!wl && !wr) return;
-  float hl = l.w - l.b, hr = r.w - r.b;
-  int wall = 0;
-  if (wl != wr) {
-    const float el = hl, er = hr;
-    if (!wl) { hl = 0.0f; l.n = 0.0f; }
-    if (!wr) { hr = 0.0f; r.n = 0.0f; }
-    if (wl && r.b > l.w) {
-      const float c = sqrtf(g * hl), sw = fmaxf(c - l.u, c);
-      const float hm = hl + l.n * rcpf(sw);
-      if (r.b >= l.b + hm) {  // a wall: the mirrored state
-        wall = 1;
-        r = l;
-        r.n = -l.n;
-        r.u = -l.u;
-        hr = hl;
-      } else {  // overtopped: the step lowered to the surface
-        r.w = l.w + er;
-        r.b = l.w;
-      }
-    } else if (wr && l.b > r.w) {
-      const float c = sqrtf(g * hr), sw = fmaxf(r.u + c, c);
-      const float hm = hr - r.n * rcpf(sw);
-      if (l.b >= r.b + hm) {
-        wall = -1;
-        l = r;
-        l.n = -r.n;
-        l.u = -r.u;
-        hl = hr;
-      } else {
-        l.w = r.w + el;
-        l.b = r.w;
-      }
-    }
-  }
-  const float sg = sqrtf(g);
-  const float cl = sg * l.q, cr = sg * r.q;
-  const float ghb = g * (0.5f * (hl + hr));
-  if (l.q > 0.0f && r.q > 0.0f) {
-    const float uhat = fmaf(l.q, l.u, r.q * r.u) * rcpf(l.q + r.q);
-    const float chat = sqrtf(ghb);
-    s1 = fminf(l.u - cl, uhat - chat);
-    s3 = fmaxf(r.u + cr, uhat + chat);
-  } else if (l.q > 0.0f) {
-    s1 = l.u - cl;
-    s3 = l.u + 2.0f * cl;
-  } else {
-    s1 = r.u - 2.0f * cr;
-    s3 = r.u + cr;
-  }
-  const float dn = r.n - l.n;
-  const float deta = r.w - l.w;
-  const float den = s3 - s1, rden = rcpf(den);
-  const float hhll = (fmaf(s3, hr, -(s1 * hl)) - dn) * rden;
-  const float x = hhll * den;
-  float dhs = l.b - r.b;
-  bool clamped = false;
-  if (s1 < 0.0f && s3 > 0.0f) {
-    const float lo = x * rcpf(s1), hi = x * rcpf(s3);
-    if (dhs < lo) { dhs = lo; clamped = true; }
-    if (dhs > hi) { dhs = hi; clamped = true; }
-  } else if (s1 >= 0.0f) {
-    const float hi = s1 > 0.0f ? x * rcpf(s1) : dhs;
-    if (dhs > hi) { dhs = hi; clamped = true; }
-    if (dhs < -hl) { dhs = -hl; clamped = true; }
-  } else {
-    const float lo = s3 < 0.0f ? x * rcpf(s3) : dhs;
-    if (dhs < lo) { dhs = lo; clamped = true; }
-    if (dhs > hr) { dhs = hr; clamped = true; }
-  }
-  const float d1 = clamped ? (hr - hl) - dhs : deta;
-  const float d3 = fmaf(ghb, deta, fmaf(r.n, r.u, -(l.n * l.u)));
-  const float b1 = fmaf(s3, d1, -dn) * rden;
-  const float b3 = fmaf(-s1, d1, dn) * rden;
-  const float q1 = s1 * s1, q3 = s3 * s3;
-  z[0] = s1 * b1;
-  z[1] = q1 * b1;
-  z[2] = l.v * z[0];
-  z[5] = s3 * b3;
-  z[6] = q3 * b3;
-  z[7] = r.v * z[5];
-  z[3] = d3 - (z[1] + z[6]);
-  z[4] = fmaf(r.n, r.v, -(l.n * l.v)) - (z[2] + z[7]);
-  if (wall == 1) z[3] = z[4] = z[5] = z[6] = z[7] = 0.0f;
-  else if (wall == -1) z[0] = z[1] = z[2] = z[3] = z[4] = 0.0f;
-}
-
 // ---------------------------------------------------------------- pairs
 //
 // Two neighbouring edges (or cells) per thread: the additions, products and
@@ -788,43 +686,124 @@ __device__ __forceinline__ f2 sel2(bool c0, bool c1, f2 a, f2 b) {
 __device__ __forceinline__ f2 ld2(const float* p) { return *reinterpret_cast<const f2*>(p); }
 __device__ __forceinline__ void st2(float* p, f2 v) { *reinterpret_cast<f2*>(p) = v; }
 
+// One side of two edges in the deviation form: stored surface and bed (minus
+// eta0), normal momentum, velocities and the root of the depth (u, v and q
+// are zero in a dry cell).
 struct Prim32x2 {
   f2 w, b, n, u, v, q;
 };
 
-// The general solver for one half, outputs through a pointer (rare: an edge
-// touching a dry cell, or one whose stationary wave may be clamped).
-static __device__ __noinline__ void riemann32_one(Prim32 l, Prim32 r, float g, float* out) {
-  float z[8], s1, s3;
-  riemann32(l, r, g, z, s1, s3);
-#pragma unroll
-  for (int k = 0; k < 8; ++k) out[k] = z[k];
-  out[8] = s1;
-  out[9] = s3;
+// The depth jump dh of a stationary wave, bounded for non-negative depths
+// (x1, x3: what the outer waves leave over s1 and s3).
+__device__ __forceinline__ float jump_bound(float dh, float s1, float s3, float x1, float x3,
+                                             float hl, float hr, bool& clamped) {
+  // right-going flow: the upper bound first
+  const bool right = s1 >= 0.0f, sub = s1 < 0.0f && s3 > 0.0f;
+  const float lo = sub ? x1 : (right ? -hl : (s3 < 0.0f ? x3 : dh));
+  const float hi = sub ? x3 : (right ? (s1 > 0.0f ? x1 : dh) : hr);
+  clamped = false;
+  if (right && dh > hi) { dh = hi; clamped = true; }
+  if (dh < lo) { dh = lo; clamped = true; }
+  if (!right && dh > hi) { dh = hi; clamped = true; }
+  return dh;
 }
 
-// Two edges between wet cells whose stationary waves are inside their bounds
-// (tested with a margin far above the rounding of the exact bounds); a half
-// that is not goes through riemann32.  sg = sqrt(g).
-__device__ __forceinline__ void riemann32x2(const Prim32x2& l, const Prim32x2& r, float g,
-                                            float sg, f2 nz, f2 (&z)[8], f2& s1, f2& s3) {
-  const f2 hl = sub2(l.w, l.b), hr = sub2(r.w, r.b);
+// Waves z[8] as in riemann_prim of two edges and their outer speeds s1, s3
+// (the middle one is their mean); sg = sqrt(g).  The straight line is that of
+// edges between wet cells whose stationary waves are inside their bounds
+// (tested with a margin far above the rounding of the exact bounds); a wet/dry
+// edge, and one that may be clamped, adds its blocks on the way, by selections
+// for both halves at once.  (One after the other through a general solver of
+// their own such edges doubled the phase's time in a front's tile: 64 patches
+// of 16 x 16 with a front 16.7 us a step, 15.4 so.)
+// DRY = false: both cells of every edge that counts are wet.
+template <bool DRY>
+__device__ __forceinline__ void riemann32x2(Prim32x2 l, Prim32x2 r, float g, float sg, f2 nz,
+                                            f2 (&z)[8], f2& s1, f2& s3) {
+  f2 hl = sub2(l.w, l.b), hr = sub2(r.w, r.b);
+  float ql0, ql1, qr0, qr1;
+  upk(l.q, ql0, ql1);
+  upk(r.q, qr0, qr1);
+  const bool wl0 = ql0 > 0.0f, wl1 = ql1 > 0.0f, wr0 = qr0 > 0.0f, wr1 = qr1 > 0.0f;
+  const bool dry = DRY && !(wl0 && wl1 && wr0 && wr1);
+  f2 dn = sub2(r.n, l.n), deta = sub2(r.w, l.w), dhs = sub2(l.b, r.b);
+  bool k0 = false, k1 = false;  // per half: a wall
+  if (dry) {
+    // the wet side, its velocity and momentum towards the dry one
+    const f2 h = sel2(wl0, wl1, hl, hr), b = sel2(wl0, wl1, l.b, r.b);
+    const f2 w = sel2(wl0, wl1, l.w, r.w), q = sel2(wl0, wl1, l.q, r.q);
+    const f2 u = sel2(wl0, wl1, l.u, neg2(r.u)), n = sel2(wl0, wl1, l.n, neg2(r.n));
+    const f2 c = sqrt2(mul2(pk1(g), h)), sw = max2(sub2(c, u), c);
+    const f2 top = add2(b, add2(h, mulr2(n, rcp2(sw), nz)));  // its HLL middle surface
+    float bd0, bd1, w0, w1, t0, t1;
+    upk(sel2(wl0, wl1, r.b, l.b), bd0, bd1);
+    upk(w, w0, w1);
+    upk(top, t0, t1);
+    const bool a0 = wl0 != wr0 && bd0 > w0, a1 = wl1 != wr1 && bd1 > w1;  // bed above the water
+    k0 = a0 && bd0 >= t0;
+    k1 = a1 && bd1 >= t1;
+    // overtopped: the dry side's step lowered to the surface
+    const bool o0 = a0 && !k0, o1 = a1 && !k1;
+    const f2 rise = sub2(add2(w, sel2(wl0, wl1, hr, hl)), w), fall = sub2(b, w);
+    deta = sel2(o0, o1, sel2(wl0, wl1, rise, neg2(rise)), deta);
+    dhs = sel2(o0, o1, sel2(wl0, wl1, fall, neg2(fall)), dhs);
+    // a wall: the mirrored state on the dry side (in both halves of the
+    // solution, of which the wet side's waves are kept)
+    deta = sel2(k0, k1, 0ull, deta);
+    dhs = sel2(k0, k1, 0ull, dhs);
+    hl = sel2(k0, k1, h, sel2(wl0, wl1, hl, 0ull));
+    hr = sel2(k0, k1, h, sel2(wr0, wr1, hr, 0ull));
+    l.n = sel2(wl0, wl1, l.n, 0ull);
+    r.n = sel2(wr0, wr1, r.n, 0ull);
+    const f2 nn = neg2(n);
+    dn = sel2(k0, k1, add2(nn, nn), sub2(r.n, l.n));
+    l.u = sel2(k0, k1, u, l.u);
+    r.u = sel2(k0, k1, neg2(u), r.u);
+    l.q = sel2(k0, k1, q, l.q);
+    r.q = sel2(k0, k1, q, r.q);
+  }
   const f2 cl = mulr2(pk1(sg), l.q, nz), cr = mulr2(pk1(sg), r.q, nz);
   const f2 ghb = mul2(pk1(g), mul2(pk1(0.5f), add2(hl, hr)));
   const f2 uhat = mulr2(fma2(l.q, l.u, mul2(r.q, r.u)), rcp2(add2(l.q, r.q)), nz);
   const f2 chat = sqrt2(ghb);
   s1 = min2(sub2(l.u, cl), sub2(uhat, chat));
   s3 = max2(add2(r.u, cr), add2(uhat, chat));
-  const f2 dn = sub2(r.n, l.n), deta = sub2(r.w, l.w);
-  const f2 rden = rcp2(sub2(s3, s1));
+  if (dry) {
+    // one side without water: the other's speed and the front's
+    const bool b0 = (wl0 && wr0) || k0, b1 = (wl1 && wr1) || k1;
+    const f2 u = sel2(wl0, wl1, l.u, r.u), c = sel2(wl0, wl1, cl, cr), c2 = add2(c, c);
+    s1 = sel2(b0, b1, s1, sub2(u, sel2(wl0, wl1, c, c2)));
+    s3 = sel2(b0, b1, s3, add2(u, sel2(wl0, wl1, c2, c)));
+  }
+  const f2 den = sub2(s3, s1), rden = rcp2(den);
   const f2 ns1 = neg2(s1);
   const f2 x = sub2(fma2(s3, hr, mul2(ns1, hl)), dn);
-  const f2 dhs = sub2(l.b, r.b), xm = mul2(pk1(0.9999f), x);
+  const f2 xm = mul2(pk1(0.9999f), x);
   const f2 ok = min2(min2(min2(sub2(xm, mul2(dhs, s1)), sub2(xm, mul2(dhs, s3))), x),
                      min2(min2(add2(dhs, hl), sub2(hr, dhs)), min2(l.q, r.q)));
+  float ok0, ok1;
+  upk(ok, ok0, ok1);
+  f2 d1 = deta;
+  if (!(ok0 > 0.0f && ok1 > 0.0f)) {
+    // the stationary wave's depth jump, bounded for non-negative depths
+    const f2 hh = mulr2(mulr2(x, rden, nz), den, nz);
+    const f2 b1 = mul2(hh, rcp2(s1)), b3 = mul2(hh, rcp2(s3));
+    float p0, p1, q0, q1, x10, x11, x30, x31, l0, l1, r0, r1, d0, e0;
+    upk(s1, p0, p1);
+    upk(s3, q0, q1);
+    upk(b1, x10, x11);
+    upk(b3, x30, x31);
+    upk(hl, l0, l1);
+    upk(hr, r0, r1);
+    upk(dhs, d0, e0);
+    bool c0, c1;
+    const float j0 = jump_bound(d0, p0, q0, x10, x30, l0, r0, c0);
+    const float j1 = jump_bound(e0, p1, q1, x11, x31, l1, r1, c1);
+    d1 = sel2(c0 && !(ok0 > 0.0f), c1 && !(ok1 > 0.0f), sub2(sub2(hr, hl), pk(j0, j1)), deta);
+  }
   const f2 d3 = fma2(ghb, deta, fma2(r.n, r.u, neg2(mul2(l.n, l.u))));
-  const f2 b1 = mul2(fma2(s3, deta, neg2(dn)), rden);
-  const f2 b3 = mul2(fma2(ns1, deta, dn), rden);
+  const f2 b1 = mul2(fma2(s3, d1, neg2(dn)), rden);
+  const f2 b3 = mul2(fma2(ns1, d1, dn), rden);
   z[0] = mul2(s1, b1);
   z[1] = mulr2(mul2(s1, s1), b1, nz);
   z[2] = mulr2(l.v, z[0], nz);
@@ -833,27 +812,60 @@ __device__ __forceinline__ void riemann32x2(const Prim32x2& l, const Prim32x2& r
   z[7] = mulr2(r.v, z[5], nz);
   z[3] = sub2(d3, add2(z[1], z[6]));
   z[4] = sub2(fma2(r.n, r.v, neg2(mul2(l.n, l.v))), add2(z[2], z[7]));
-  float ok0, ok1;
-  upk(ok, ok0, ok1);
-  if (!(ok0 > 0.0f && ok1 > 0.0f)) {
-#pragma unroll 1
-    for (int h = 0; h < 2; ++h) {
-      if ((h ? ok1 : ok0) > 0.0f) continue;
-      auto half = [&](f2 v) { return __uint_as_float((unsigned)(h ? v >> 32 : v)); };
-      float o[10];
-      riemann32_one(
-          Prim32{half(l.w), half(l.b), half(l.n), half(l.u), half(l.v), half(l.q)},
-          Prim32{half(r.w), half(r.b), half(r.n), half(r.u), half(r.v), half(r.q)}, g, o);
-      auto put = [&](f2& v, float a) {
-        const f2 b = __float_as_uint(a);
-        v = h ? ((v & 0xffffffffull) | (b << 32)) : ((v & ~0xffffffffull) | b);
-      };
+  if (dry) {
+    // nothing between two dry cells, nor behind a wall
+    const bool e0 = !wl0 && !wr0, e1 = !wl1 && !wr1;
+    const bool f0 = k0 || e0, f1 = k1 || e1;
 #pragma unroll
-      for (int k = 0; k < 8; ++k) put(z[k], o[k]);
-      put(s1, o[8]);
-      put(s3, o[9]);
-    }
+    for (int k = 0; k < 8; ++k)
+      z[k] = sel2(f0 && (k >= 5 ? !wr0 : k >= 3 || !wl0), f1 && (k >= 5 ? !wr1 : k >= 3 || !wl1),
+                  0ull, z[k]);
+    s1 = sel2(e0, e1, 0ull, s1);
+    s3 = sel2(e0, e1, 0ull, s3);
   }
+}
+
+// riemann32x2 of one edge with a wet and a dry cell (fields w, b, n, u, v, q).
+__device__ __forceinline__ void riemann32_front(const float (&l)[6], const float (&r)[6], float g,
+                                                float sg, float (&z)[8], float& s1, float& s3) {
+  const bool wl = l[5] > 0.0f;
+  const float hl = l[0] - l[1], hr = r[0] - r[1];
+  // the wet side, its velocity and momentum towards the dry one
+  const float h = wl ? hl : hr, b = wl ? l[1] : r[1], w = wl ? l[0] : r[0], q = wl ? l[5] : r[5];
+  const float u = wl ? l[3] : -r[3], n = wl ? l[2] : -r[2], v = wl ? l[4] : r[4];
+  const float bd = wl ? r[1] : l[1], e = wl ? hr : hl;
+  const float c = sqrtf(g * h), sw = fmaxf(c - u, c);
+  const bool above = bd > w, wall = above && bd >= b + (h + n * rcpf(sw)), over = above && !wall;
+  // jumps towards the dry side of the surface and minus the bed
+  const float jw = wall ? 0.0f : (over ? (w + e) - w : (wl ? r[0] - l[0] : l[0] - r[0]));
+  const float jb = wall ? 0.0f : (over ? b - w : b - bd);
+  const float deta = wl ? jw : -jw, dhs = wl ? jb : -jb;
+  const float dn = wall ? -n - n : -n;
+  const float cq = sg * q, c2 = 2.0f * cq, us = wl ? u : -u;
+  const float ghb = g * (0.5f * (wall ? h + h : h));
+  const float uhat = fmaf(q, u, -(q * u)) * rcpf(q + q), chat = sqrtf(ghb);
+  s1 = wall ? fminf(u - cq, uhat - chat) : us - (wl ? cq : c2);
+  s3 = wall ? fmaxf(cq - u, uhat + chat) : us + (wl ? c2 : cq);
+  const float gl = wl || wall ? h : 0.0f, gr = !wl || wall ? h : 0.0f;
+  const float den = s3 - s1, rden = rcpf(den);
+  const float hh = ((fmaf(s3, gr, -(s1 * gl)) - dn) * rden) * den;
+  bool clamped;
+  const float dh = jump_bound(dhs, s1, s3, hh * rcpf(s1), hh * rcpf(s3), gl, gr, clamped);
+  const float d1 = clamped ? (gr - gl) - dh : deta;
+  const float nu = n * u, nv = (wl ? n : -n) * v;  // the wet side's fluxes
+  const float d3 = fmaf(ghb, deta, wl ? -nu : nu);
+  const float b1 = fmaf(s3, d1, -dn) * rden, b3 = fmaf(-s1, d1, dn) * rden;
+  z[0] = s1 * b1;
+  z[1] = (s1 * s1) * b1;
+  z[2] = (wl ? v : 0.0f) * z[0];
+  z[5] = s3 * b3;
+  z[6] = (s3 * s3) * b3;
+  z[7] = (wl ? 0.0f : v) * z[5];
+  z[3] = d3 - (z[1] + z[6]);
+  z[4] = (wl ? -nv : nv) - (z[2] + z[7]);
+#pragma unroll
+  for (int k = 0; k < 8; ++k)
+    if (wall && (k >= 3 || !wl) && (k < 5 || wl)) z[k] = 0.0f;
 }
 
 // Limiter coefficients of one wave of two edges: hs = half the sign of the

@@ -98,6 +98,7 @@ struct TileHdr {
   double dt;      // dt_use
   bool same_in;   // both buffers hold the same dry interior
   bool has_gauge;
+  int* order;     // the next launch order (or null: another CTA enters the patch)
 };
 
 template <typename R>
@@ -263,7 +264,10 @@ struct Layout {
   static constexpr size_t OFF_RED = align16(OFF_G + TRB);
   static constexpr size_t OFF_NB = OFF_RED + sizeof(double) * 64;  // 8 ints
   static constexpr size_t OFF_WET = OFF_NB + 32;
-  static constexpr size_t OFF_BAR = align16(OFF_WET + (P::DEV && DS ? TT : 16));
+  // FAST, whole 32 x 32 tiles: edges set aside: their number, then their places
+  static constexpr int ASIDE = FAST && M == 32 ? 240 : 0;
+  static constexpr size_t OFF_ASIDE = align16(OFF_WET + (P::DEV && DS ? TT : 16));
+  static constexpr size_t OFF_BAR = align16(OFF_ASIDE + (FAST ? 4 + 2 * ASIDE : 0));
   static constexpr size_t BYTES = OFF_BAR + 16;
 };
 
@@ -376,6 +380,8 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
   uint64_t* bar = reinterpret_cast<uint64_t*>(smraw + Lo::OFF_BAR);
   // FAST: set by a thread whose bounded wait gave up
   volatile int* sflag = reinterpret_cast<volatile int*>(smraw + Lo::OFF_WET);
+  unsigned* naside = reinterpret_cast<unsigned*>(smraw + Lo::OFF_ASIDE);
+  unsigned short* aside = reinterpret_cast<unsigned short*>(naside + 1);
 
   const int tid = threadIdx.x;
   // level subcycling: this level's period in fine substeps, its buffer
@@ -414,7 +420,7 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
         mbar_init(bar, 1);
         mbar_init(bar + 1, 1);
       }
-      if constexpr (FAST) *sflag = 0;
+      if constexpr (FAST) *sflag = 0, *naside = 0u;
       mbar_expect_tx(bar, 2u * TT * sizeof(R));
       bulk_g2s(s0, qs, TT * sizeof(R), bar);
       bulk_g2s(sb, bs, TT * sizeof(R), bar);
@@ -459,7 +465,7 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
         *reinterpret_cast<float4*>(shv + c) = a2;
         *reinterpret_cast<float4*>(sb + c) = a3;
       }
-      if (tid == 0) *sflag = 0;
+      if (tid == 0) *sflag = 0, *naside = 0u;
     } else
     for (int k = tid; k < TT; k += NT) {
       const int li = k % Lo::T, lj = k / Lo::T;
@@ -471,13 +477,23 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
     }
   }
 
-  // per-patch scalars: computed once by thread 0 (FP64 divisions are slow
-  // on this part, so no thread repeats them) and broadcast through shared
-  // memory
+  const bool push = V.push != 0 && V.nbr != nullptr;
+  // FAST: what comes from global memory is asked for here and stored behind
+  // the next barrier, which then waits for none of it
+  [[maybe_unused]] int nbr = -1;
+  [[maybe_unused]] float mann = 0.0f;
+  constexpr int SCT = FAST ? 32 : 0;
+  if constexpr (FAST) {
+    if (push && tid < 8) nbr = V.nbr[(size_t)p * 8 + tid];
+    if (tid == SCT) mann = V.scen[Pt.scen].manning_f;
+  }
+  // per-patch scalars: computed once by one thread (FP64 divisions are slow
+  // on this part, so no thread repeats them; FAST: not by the one that asks
+  // for the tile) and broadcast through shared memory
   double* scal = red + 48;  // dx, dy, nux, nuy, then the R-typed copies
   R* rscal = reinterpret_cast<R*>(red + 52);  // g, drytol, nux, nuy, n, dt
   float* fscal = reinterpret_cast<float*>(red + 60);  // drytol, margin
-  if (tid == 0) {
+  if (tid == SCT) {
     if constexpr (DEV) {
       // FP32 from the host's per-level tables: one conversion per patch
       const float dtf32 = (float)dtp;
@@ -485,7 +501,7 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
       rscal[1] = G.drytolf;
       rscal[2] = dtf32 * G.inv_dxf[Pt.level];
       rscal[3] = dtf32 * G.inv_dyf[Pt.level];
-      rscal[4] = V.scen[Pt.scen].manning_f;
+      if constexpr (!FAST) rscal[4] = V.scen[Pt.scen].manning_f;
       rscal[5] = dtf32;
       fscal[0] = G.drytolf;
       fscal[1] = G.marginf;
@@ -503,8 +519,9 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
       rscal[5] = (R)dtp;
     }
   }
-  const bool push = V.push != 0 && V.nbr != nullptr;
-  if (push && tid < 8) snb[tid] = V.nbr[(size_t)p * 8 + tid];
+  if constexpr (!FAST) {
+    if (push && tid < 8) snb[tid] = V.nbr[(size_t)p * 8 + tid];
+  }
   const double drytol = G.drytol;
   R smx = R(0), smy = R(0);
 
@@ -590,6 +607,8 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
     } else {
       for (int k = 4 * tid; k < TT; k += 4 * NT) cells4(k, true);
     }
+    if (push && tid < 8) snb[tid] = nbr;
+    if (tid == SCT) rscal[4] = mann;
     anywet = __syncthreads_or(anywet);
     if (*sflag) {
       // some wait gave up: wait (again with a limit) for the copies in
@@ -731,29 +750,40 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
     // phase 1: Riemann solves.  x: row l, edges a = -1 + 2 m and the next;
     // y: edge row a, columns -2 + 2 m and the next
     constexpr int N1 = dir == 0 ? (M + 2) * PW / 2 : (M + 3) * PW / 2;
-#pragma unroll 1
-    for (int k = tid; k < N1; k += NT) {
+    // of pair k: tile cell left of (below) its first edge, and its cells
+    auto cell_of = [&](int k) {
       const int m = k % (PW / 2), row = k / (PW / 2);  // row: l + 1, or a + 1
-      const int e = row * PW + 2 * m;
-      // tile cell left of (below) the first edge
-      const int c = dir == 0 ? (row + 1) * Lo::T + 2 * m : row * Lo::T + 2 * m;
+      return dir == 0 ? (row + 1) * Lo::T + 2 * m : row * Lo::T + 2 * m;
+    };
+    auto pair_r = [&](const R* p, int c, f2 l) {
+      if constexpr (dir == 0) {
+        float x, y;
+        gfk::upk(l, x, y);
+        return gfk::pk(y, p[c + 2]);
+      } else {
+        (void)l;
+        return gfk::ld2(p + c + CS);
+      }
+    };
+    auto solve = [&](int k, unsigned both, auto dryc) {
+      const int m = k % (PW / 2), row = k / (PW / 2);
+      const int c = cell_of(k);
       auto pair_l = [&](const R* p) { return gfk::ld2(p + c); };
-      auto pair_r = [&](const R* p, f2 l) {
-        if constexpr (dir == 0) {
-          float x, y;
-          gfk::upk(l, x, y);
-          return gfk::pk(y, p[c + 2]);
-        } else {
-          (void)l;
-          return gfk::ld2(p + c + CS);
-        }
-      };
-      gfk::Prim32x2 L{pair_l(s0), pair_l(sb), pair_l(sn), pair_l(un), pair_l(ut), pair_l(sq)};
-      gfk::Prim32x2 Rt{pair_r(s0, L.w), pair_r(sb, L.b), pair_r(sn, L.n),
-                       pair_r(un, L.u), pair_r(ut, L.v), pair_r(sq, L.q)};
+      const gfk::Prim32x2 L{pair_l(s0), pair_l(sb), pair_l(sn),
+                            pair_l(un), pair_l(ut), pair_l(sq)};
+      const gfk::Prim32x2 Rt{pair_r(s0, c, L.w), pair_r(sb, c, L.b), pair_r(sn, c, L.n),
+                             pair_r(un, c, L.u), pair_r(ut, c, L.v), pair_r(sq, c, L.q)};
       f2 z[8], s1, s3;
-      gfk::riemann32x2(L, Rt, g, sg, nz, z, s1, s3);
-      R* w = W + e;
+      constexpr bool DRY = decltype(dryc)::value;
+      gfk::riemann32x2<DRY>(L, Rt, g, sg, nz, z, s1, s3);
+      if (!DRY && both != 3u) {  // nothing (yet) where a cell is dry
+        const bool b0 = both & 1u, b1 = both & 2u;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) z[q] = gfk::sel2(b0, b1, z[q], 0ull);
+        s1 = gfk::sel2(b0, b1, s1, 0ull);
+        s3 = gfk::sel2(b0, b1, s3, 0ull);
+      }
+      R* w = W + row * PW + 2 * m;
 #pragma unroll
       for (int q = 0; q < 8; ++q) gfk::st2(w + q * NEDGE, z[q]);
       gfk::st2(w + 8 * NEDGE, s1);
@@ -771,6 +801,75 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
       } else {
         if ((unsigned)(row - 1) <= (unsigned)M && m > 0 && m <= M2)
           smax = fmaxf(smax, fmaxf(ma, mb));
+      }
+    };
+    // Edges between a wet and a dry cell: the blocks they add to a pair cost a
+    // warp the same for one lane as for all.  With one pair to a thread they
+    // are taken on the way; with several (whole 32 x 32 tiles, where a front
+    // touches nearly every warp in every round) they are set aside and taken
+    // together, one edge to a thread.  256 patches with a front: 22.2 us a
+    // step on the way, 21.5 so.
+    constexpr bool LATER = Lo::ASIDE > 0 && N1 > NT;
+    // the wet sides of pair k: bits 0, 1 left (below), 2, 3 right
+    auto wetness = [&](int k) {
+      const int c = cell_of(k);
+      const f2 ql = gfk::ld2(sq + c), qr = pair_r(sq, c, ql);
+      float a0, a1, b0, b1;
+      gfk::upk(ql, a0, a1);
+      gfk::upk(qr, b0, b1);
+      return (a0 > 0.0f ? 1u : 0u) | (a1 > 0.0f ? 2u : 0u) | (b0 > 0.0f ? 4u : 0u) |
+             (b1 > 0.0f ? 8u : 0u);
+    };
+#pragma unroll 1
+    for (int k = tid; k < N1; k += NT) {
+      const unsigned wn = wetness(k), both = wn & (wn >> 2);
+      if (LATER ? both == 0u : wn == 0u) {
+        R* w = W + (k / (PW / 2)) * PW + 2 * (k % (PW / 2));
+#pragma unroll
+        for (int q = 0; q < 10; ++q) gfk::st2(w + q * NEDGE, 0ull);
+      } else {
+        solve(k, both, std::bool_constant<!LATER>{});
+      }
+      if constexpr (LATER) {
+        const unsigned mixed = (wn ^ (wn >> 2)) & 3u, now = __activemask();
+        if (__any_sync(now, mixed != 0u)) {
+          const unsigned m0 = __ballot_sync(now, mixed & 1u), m1 = __ballot_sync(now, mixed & 2u);
+          const int lane = tid & 31, lead = __ffs(now) - 1;
+          unsigned at = 0u;
+          if (lane == lead) at = atomicAdd(naside, (unsigned)(__popc(m0) + __popc(m1)));
+          at = __shfl_sync(now, at, lead);
+          const unsigned below = (1u << lane) - 1u;
+          const unsigned at0 = at + __popc(m0 & below);
+          const unsigned at1 = at + __popc(m0) + __popc(m1 & below);
+          const int e = (k / (PW / 2)) * PW + 2 * (k % (PW / 2));
+          if ((mixed & 1u) && at0 < (unsigned)Lo::ASIDE) aside[at0] = (unsigned short)e;
+          if ((mixed & 2u) && at1 < (unsigned)Lo::ASIDE) aside[at1] = (unsigned short)(e + 1);
+        }
+      }
+    }
+    if constexpr (LATER) {
+      // the tile's rows are the planes', so the cell left of or below an edge
+      // is at the same place, a row up in the x sweep
+      static_assert(PW == Lo::T, "an edge's place gives its cells");
+      __syncthreads();
+      const unsigned na = *naside;
+      const bool full = na > (unsigned)Lo::ASIDE;  // more than the list holds
+#pragma unroll 1
+      for (int x = tid; x < (full ? 2 * N1 : (int)na); x += NT) {
+        const int e = full ? x : aside[x], c = dir == 0 ? e + Lo::T : e, row = e / PW, at = e % PW;
+        if (full && (sq[c] > 0.0f) == (sq[c + CS] > 0.0f)) continue;
+        const float l[6] = {s0[c], sb[c], sn[c], un[c], ut[c], sq[c]};
+        const float r[6] = {s0[c + CS], sb[c + CS], sn[c + CS], un[c + CS], ut[c + CS], sq[c + CS]};
+        float z[8], s1, s3;
+        gfk::riemann32_front(l, r, g, sg, z, s1, s3);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) W[q * NEDGE + e] = z[q];
+        W[8 * NEDGE + e] = s1;
+        W[9 * NEDGE + e] = s3;
+        const bool counts =
+            dir == 0 ? (unsigned)(row - 1) < (unsigned)M && (unsigned)(at - 1) <= (unsigned)M
+                     : (unsigned)(row - 1) <= (unsigned)M && (unsigned)(at - 2) < (unsigned)M;
+        if (counts) smax = fmaxf(smax, fmaxf(fabsf(s1), fabsf(s3)));
       }
     }
     if (dir == 0) smx = smax;
@@ -802,6 +901,7 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
       }
     }
     __syncthreads();
+    if (LATER && tid == 0) *naside = 0u;
 #pragma unroll
     for (int r = 0; r < RE; ++r) {
       const int k = tid + r * NT;
@@ -822,6 +922,11 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
     // rows -1..M of the thread's columns; in the y sweep the threads of the
     // two ghost rows take the two ghost columns instead (two rows each).
     // Transverse parts (plus, minus; mass, hu, hv) in planes of pitch PT.
+    // The last warp has no rows in the second round: its last thread enters
+    // the patch in the next launch order meanwhile (at the tile's end the
+    // round trip would be waited for)
+    if (dir == 1 && tid == NT - 1 && H.order != nullptr)
+      H.order[atomicAdd(V.sched + 1, 1u)] = p;
     constexpr int PTP = M * (M + 4);          // one plane
     constexpr int PT = dir == 0 ? M : M + 4;  // its rows
     R* Tr = Ftr;
@@ -1423,13 +1528,15 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
         }
       }
       __syncthreads();
-      // Copies of the cells within two of the tile's edge.  Away from the
-      // domain's boundary every copy goes to one same-level neighbour: the
-      // ghost cells of the bottom and top neighbours (2 M each, along x), the
-      // left and right ones, then the corners.
-      if (M == MP && Pt.px > 0 && Pt.px < nxp - 1 && Pt.py > 0 && Pt.py < nyp - 1) {
-        for (int k = push ? tid : 8 * M + 16; k < 8 * M + 16; k += NT) {
-          int r, i, j;
+      // Copies of the cells within two of the tile's edge.
+      if (M == MP) {
+        // Every ghost cell that takes one of this patch's values, region by
+        // region: bottom and top (2 M each, along x), left and right, then the
+        // corners.  In the domain it is a cell of the neighbour there; beyond
+        // its boundary a mirror cell of this patch or, at a corner beyond one
+        // side only, of the neighbour along the other.
+        for (int k = tid; k < 8 * M + 16; k += NT) {
+          int r, i, j;  // region, source cell
           if (k < 4 * M) {
             r = 2 + k / (2 * M);
             i = k % M;
@@ -1445,16 +1552,35 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
             i = x % 2 + (r & 1 ? M - 2 : 0);
             j = x / 2 % 2 + (r & 2 ? M - 2 : 0);
           }
-          const int pn = snb[r];
+          // its direction
+          const int sx = r == 0 || r == 4 || r == 6 ? -1 : (r == 1 || r == 5 || r == 7 ? 1 : 0);
+          const int sy = r == 2 || r == 4 || r == 5 ? -1 : (r == 3 || r == 6 || r == 7 ? 1 : 0);
+          const bool bx = sx != 0 && (unsigned)(Pt.px + sx) >= (unsigned)nxp;
+          const bool by = sy != 0 && (unsigned)(Pt.py + sy) >= (unsigned)nyp;
+          // the patch that holds it
+          const int rr = r < 4 ? r : (bx ? (sy < 0 ? 2 : 3) : (by ? (sx < 0 ? 0 : 1) : r));
+          const bool self = (bx || sx == 0) && (by || sy == 0);
+          const int pn = self ? p : (push ? snb[rr] : -1);
           if (pn < 0) continue;
+          // its cell there: beyond the opposite edge, or the mirror (wall: the
+          // n-th ghost takes the n-th cell, extrapolation: the first)
+          int gi = i - sx * M, gj = j - sy * M;
+          R fx = R(1), fy = R(1);
+          if (bx) {
+            gi = sx < 0 ? -1 - i : 2 * M - 1 - i;
+            if (G.bc[sx < 0 ? 0 : 1] == 0) fx = R(-1);
+            else i = sx < 0 ? 0 : M - 1;
+          }
+          if (by) {
+            gj = sy < 0 ? -1 - j : 2 * M - 1 - j;
+            if (G.bc[sy < 0 ? 2 : 3] == 0) fy = R(-1);
+            else j = sy < 0 ? 0 : M - 1;
+          }
           const R* v = nv + j * M + i;
-          // towards the neighbour: its cell beyond its own opposite edge
-          const int di = r == 0 || r == 4 || r == 6 ? M : (r == 1 || r == 5 || r == 7 ? -M : 0);
-          const int dj = r == 2 || r == 4 || r == 5 ? M : (r == 3 || r == 6 || r == 7 ? -M : 0);
-          R* d = qnext + (size_t)pn * 3 * TG + tix<M>(i + di, j + dj);
+          R* d = qnext + (size_t)pn * 3 * TG + tix<M>(gi, gj);
           d[0] = v[0];
-          d[TG] = v[M * M];
-          d[2 * TG] = v[2 * M * M];
+          d[TG] = fx * v[M * M];
+          d[2 * TG] = fy * v[2 * M * M];
         }
       } else
       // otherwise cell by cell, side by side, so that a warp takes cells of
@@ -1589,8 +1715,14 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
   static_assert(NW <= 32, "one warp reduces the per-warp partials");
   // the partials fit below the broadcast scalars at red + 48
   static_assert(DEV ? 3 * NW <= 96 : 3 * NW <= 48, "reduction area");
-  smx = warp_max(smx);
-  smy = warp_max(smy);
+  // (speeds are not negative: their bits order as they do)
+  if constexpr (DEV) {
+    smx = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(smx)));
+    smy = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(smy)));
+  } else {
+    smx = warp_max(smx);
+    smy = warp_max(smy);
+  }
   nwet = __reduce_add_sync(0xffffffffu, nwet);
   if constexpr (DEV) {
     float* redf = reinterpret_cast<float*>(red);
@@ -1605,8 +1737,8 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
       float mx = lane < NW ? redf[lane] : 0.0f;
       float my = lane < NW ? redf[NW + lane] : 0.0f;
       const unsigned nw = __reduce_add_sync(0xffffffffu, lane < NW ? redu[lane] : 0u);
-      mx = warp_max(mx);
-      my = warp_max(my);
+      mx = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(mx)));
+      my = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(my)));
       if (lane == 0) {
         const float cx = mx * G.inv_dxf[Pt.level], cy = my * G.inv_dyf[Pt.level];
         double cm = (double)(cx > cy ? cx : cy);
@@ -1676,6 +1808,10 @@ static __device__ void subcycle_finish(const GfGeom& G, const GfView& V, GfCtl* 
   const long long max_steps = __ldcg(&Cp->max_steps);
   const int inrow = __ldcg(&Cp->inrow), lastf = __ldcg(&Cp->last);
   const int nonfinite = __ldcg(&Cp->nonfinite);
+  if (!__ldcg(&Cp->active)) {
+    Cp->accepted = 0;
+    return;
+  }
   Cp->cmax_bits = 0ull;
   const bool end = k == K - 1;
   double tn = t, dtn = dt_next0;
@@ -1771,6 +1907,10 @@ static __device__ void ctl_finish(const GfGeom& G, GfCtl* Cp, unsigned long long
   const long long max_steps = __ldcg(&Cp->max_steps);
   const int cur = __ldcg(&Cp->cur), lastf = __ldcg(&Cp->last);
   const int inrow = __ldcg(&Cp->inrow), nonfinite = __ldcg(&Cp->nonfinite);
+  if (!__ldcg(&Cp->active)) {
+    Cp->accepted = 0;
+    return;
+  }
   Cp->cell_updates = cell_updates + cells;
   Cp->cmax_bits = 0ull;
   if (nonfinite) {
@@ -1843,18 +1983,15 @@ __device__ void step_finish(const GfGeom& G, const GfView& V, int cells_per_patc
   __threadfence();
   for (int s = threadIdx.x; s < G.nscen; s += NT) {
     GfCtl* Cp = V.ctl + s;
-    if (!__ldcg(&Cp->active)) {
-      Cp->accepted = 0;
-      continue;
-    }
     if (G.subcycle)
       subcycle_finish(G, V, Cp, s, cells_per_patch);
     else
       ctl_finish(G, Cp, (unsigned long long)V.scen[s].pcount * (unsigned long long)cells_per_patch);
   }
   // the next launch reads the counters and the schedule after this kernel
-  // has ended, which orders these writes before it
-  if (threadIdx.x == 0 && V.sched) {
+  // has ended, which orders these writes before it (a thread without a
+  // scenario, if there is one: its loads go beside the controller's)
+  if (threadIdx.x == NT - 1 && V.sched) {
     V.sched[0] = (V.sched[0] + 1u) % 6u;
     // patches that took no step, at the tail of the next order
     // (in the word this launch does not read: CTAs beyond the working ones
@@ -1982,6 +2119,8 @@ __global__ void __launch_bounds__(NT, MINB)
       const GfCtl& C = V.ctl[H.Pt.scen];
       run = !C.sub_rej && C.sub_k % (1 << (G.maxlevel - H.Pt.level)) == 0;
     }
+    int* nxt = sched && sub == 0 ? (par ? V.ord0 : V.ord1) : nullptr;
+    H.order = nxt;
     int wet = 0;
     if (run) {
       bool w = true;
@@ -1999,8 +2138,7 @@ __global__ void __launch_bounds__(NT, MINB)
         if (q >= 0) flags(1u)[q] = 1;
       }
     }
-    if (sched && sub == 0 && threadIdx.x == 0) {
-      int* nxt = par ? V.ord0 : V.ord1;
+    if (nxt != nullptr && threadIdx.x == 0 && !(Lo::FAST && wet > 0)) {
       if (use_flags || wet) nxt[atomicAdd(V.sched + 1, 1u)] = p;
       else nxt[V.npatch - 1 - (int)atomicAdd(V.sched + 2, 1u)] = p;
     }
