@@ -16,6 +16,7 @@
 // errors the device's approximations may have.
 #pragma once
 
+#include <cmath>
 #include <cstdint>
 #include <cstring>
 
@@ -48,7 +49,11 @@ GF_HD float seed_rsqrt(float x) {
   asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
+GF_HD float seed_cbrt(float x) { return exp2f(log2f(x) * (1.0f / 3.0f)); }
 GF_HD double native_sqrt(double x) { return sqrt(x); }
+GF_HD double native_cbrt(double x) { return cbrt(x); }
+GF_HD double ffma(double a, double b, double c) { return __fma_rn(a, b, c); }
+GF_HD unsigned fbits(float x) { return __float_as_uint(x); }
 #else
 inline long long dbits(double x) { long long b; std::memcpy(&b, &x, 8); return b; }
 inline double bitsd(long long b) { double x; std::memcpy(&x, &b, 8); return x; }
@@ -64,7 +69,11 @@ inline float i2f(int i) { return (float)i; }
 inline float fmul(float a, float b) { volatile float r = a * b; return r; }
 float seed_rcp(float x);
 float seed_rsqrt(float x);
+float seed_cbrt(float x);
 double native_sqrt(double x);
+double native_cbrt(double x);
+inline double ffma(double a, double b, double c) { return std::fma(a, b, c); }
+inline unsigned fbits(float x) { unsigned b; std::memcpy(&b, &x, 4); return b; }
 #endif
 
 // Remainders below are exact modulo 2^64 although the products they come from
@@ -145,6 +154,37 @@ GF_HD_CALL double sqrt_rn(double x) {
   }
   if ((u64)xb << 1 == 0) return x;
   return native_sqrt(x);
+}
+
+// x rounded towards zero to FP32, without the FP64 pipe's conversion: zero
+// below 2^-126, NaN from 2^127 on.
+GF_HD float trunc_f32(double x) {
+  const u64 b = (u64)dbits(x);
+  const int t = (int)((b >> 32) & 0x7fffffffu) - 0x38000000;
+  // the exponent's bias off, the significand's first 23 bits up to its place
+  const float f = bitsf(((unsigned)t << 3 | (unsigned)b >> 29) | ((unsigned)(b >> 32) & 0x80000000u));
+  return t < 0x00100000 ? 0.0f : (t >= 0x0fe00000 ? bitsf(0x7fffffffu) : f);
+}
+
+// Cube root of a positive number, within an ulp: the FP32 estimate (2^-20)
+// corrected by two terms of the binomial series of the exact residual ratio
+// d = x / y^3 - 1, y (1 + d/3 - d^2/9), whose third term is below 2^-59 of y.
+// (At the ends of the range, and for anything else, the native function.)
+GF_HD double cbrt_pos(double x) {
+  const int e = (int)(dbits(x) >> 52);  // biased exponent
+  if ((unsigned)(e - 4) >= 2040u) return native_cbrt(x);
+  const int k = (e - 1023 + 1533) / 3 - 511;          // floor((e - 1023) / 3)
+  const double m = bitsd(dbits(x) - 3 * k * D_HID);   // [1, 8)
+  const unsigned fb = fbits(seed_cbrt(trunc_f32(m)));
+  // the estimate to FP64 by its bits
+  const double y = bitsd(((long long)((fb >> 23) + 896u) << 52) | ((long long)(fb & 0x7fffffu) << 29));
+  const double y2 = y * y;  // exact: 48 bits
+  const double y3 = y2 * y;
+  const double r = ffma(-y2, y, m);
+  const double d = div_rn(r, y3);
+  const double c = d * ffma(d, -1.0 / 9.0, 1.0 / 3.0);
+  const double t = ffma(y, c, y);
+  return bitsd(dbits(t) + k * D_HID);
 }
 
 // a < b and a <= 0 style tests on the bit patterns (no NaN operands: a NaN

@@ -320,15 +320,6 @@ struct Prim {
   bool wet;
 };
 
-// x rounded towards zero to FP32 (0 below its range, NaN above), without the
-// FP64 pipe's conversion
-__device__ __forceinline__ float trunc_f32(double x) {
-  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-  const int t = (int)(hi & 0x7fffffffu) - 0x38000000;
-  const float f = bitsf(__funnelshift_l(lo, (unsigned)t, 3) | (hi & 0x80000000u));
-  return t < 0x00100000 ? 0.0f : (t >= 0x0fe00000 ? __int_as_float(0x7fffffff) : f);
-}
-
 // Waves z[8]: (mass, normal, transverse) of the first and third wave and
 // (normal, transverse) of the middle one, whose mass part is zero:
 // z[0..2], z[3..4], z[5..7]; speeds s[3].
@@ -564,27 +555,6 @@ __device__ __forceinline__ void tsplit_prim(double w, double z, double c, double
     if (openp) plus[k] = p[k];
     if (openm) minus[k] = q[k];
   }
-}
-
-// Cube root of a positive normal number: the FP32 estimate (2^-20) corrected
-// by two terms of the binomial series of the exact residual ratio
-// d = x / y^3 - 1, y (1 + d/3 - d^2/9), whose third term is below 2^-63.
-__device__ __forceinline__ double cbrt_pos(double x) {
-  const int e = (int)(dbits(x) >> 52);  // biased exponent
-  if ((unsigned)(e - 4) >= 2040u) return cbrt(x);
-  const int k = (e - 1023 + 1533) / 3 - 511;             // floor((e - 1023) / 3)
-  const double m = bitsd(dbits(x) - ((long long)(3 * k) << 52));  // [1, 8)
-  const float yf = exp2f(log2f(trunc_f32(m)) * (1.0f / 3.0f));
-  const unsigned fb = __float_as_uint(yf);
-  // yf to FP64 by its bits
-  const double y = bitsd(((long long)((fb >> 23) + 896u) << 52) | ((long long)(fb & 0x7fffffu) << 29));
-  const double y2 = y * y;  // exact: 48 bits
-  const double y3 = y2 * y;
-  const double r = __fma_rn(-y2, y, m);
-  const double d = div_rn(r, y3);
-  const double c = d * __fma_rn(d, -1.0 / 9.0, 1.0 / 3.0);
-  const double t = __fma_rn(y, c, y);
-  return bitsd(dbits(t) + ((long long)k << 52));
 }
 
 // Exact wet test of a stored surface-deviation cell: depth = w - b (both
