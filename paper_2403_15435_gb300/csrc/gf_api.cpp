@@ -56,7 +56,7 @@ struct CnnState {
   int* idx = nullptr;
   float* tlogit = nullptr;
   float* loss = nullptr;
-  int bcap = 0, idx_cap = 0;
+  int bcap = 0, lcap = 0, idx_cap = 0;
   int tagger = GEOFLOOD_TAGGER_PLAIN;
   float logit_thr = 0.f;
   unsigned* misses = nullptr;
@@ -574,17 +574,28 @@ int cnn_infer_alloc(geoflood_ctx* ctx) {
   return rc ? GEOFLOOD_ERR_OOM : 0;
 }
 
+// Logits of a batch of b samples.
+int cnn_logit_alloc(geoflood_ctx* ctx, int b) {
+  CnnState& n = ctx->cnn;
+  if (b <= n.lcap) return 0;
+  cudaFree(n.tlogit);
+  n.tlogit = nullptr;
+  n.lcap = 0;
+  if (cnn_alloc(ctx, (void**)&n.tlogit, (size_t)b * 4)) return GEOFLOOD_ERR_OOM;
+  n.lcap = b;
+  return 0;
+}
+
+// A batch of b samples from the host, and its logits.
 int cnn_batch_alloc(geoflood_ctx* ctx, int b) {
   CnnState& n = ctx->cnn;
-  if (b <= n.bcap) return 0;
-  for (void* p : {n.xb, (void*)n.yb, (void*)n.tlogit})
-    cudaFree(p);
-  n.xb = nullptr; n.yb = nullptr; n.tlogit = nullptr;
+  int rc = cnn_logit_alloc(ctx, b);
+  if (rc || b <= n.bcap) return rc;
+  for (void* p : {n.xb, (void*)n.yb}) cudaFree(p);
+  n.xb = nullptr; n.yb = nullptr;
   n.bcap = 0;
-  int rc = 0;
   rc |= cnn_alloc(ctx, &n.xb, (size_t)b * CNN_X_BYTES);
   rc |= cnn_alloc(ctx, (void**)&n.yb, (size_t)b * 4);
-  rc |= cnn_alloc(ctx, (void**)&n.tlogit, (size_t)b * 4);
   if (rc) return GEOFLOOD_ERR_OOM;
   n.bcap = b;
   return 0;
@@ -1965,7 +1976,7 @@ int geoflood_cnn_train(geoflood_ctx* ctx, int epochs, int batch, float lr, float
   const int N = c.ds_n;
   if (N < 1) return fail(ctx, GEOFLOOD_ERR_STATE, "cnn_train: empty dataset");
   batch = std::min(batch, N);
-  int rc = cnn_batch_alloc(ctx, batch);
+  int rc = cnn_logit_alloc(ctx, batch);
   if (rc) return rc;
   if (N > c.idx_cap) {
     cudaFree(c.idx);

@@ -1,8 +1,9 @@
 // Device-side building blocks of the wave-propagation step: the augmented
 // Riemann solver (Sec. 3.3), the MC limiter (Sec. 3.2) and the transverse
-// eigen-split of the 2D extension (Sec. 3.2, leveque2002).  Templates on the
-// real type; the FP64 translation units are compiled with -fmad=false so
-// that every operation rounds as written.
+// eigen-split of the 2D extension (Sec. 3.2, leveque2002).  First the forms
+// of the dimensionally split step, templates on the real type; then the
+// unsplit step's own, in FP64 and in FP32.  The FP64 translation units are
+// compiled with -fmad=false so that every operation rounds as written.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -264,53 +265,14 @@ __device__ __forceinline__ void edge_fluxes(const R* Z, const R* S,
   }
 }
 
-// Transverse split of an increment d = (mass, momentum along the split
-// direction, other momentum) in a cell with depth h, momenta ma (along) and
-// mo (other): eigenvectors of the split direction's Jacobian with speeds
-// w - c, w, w + c.  plus/minus are returned in the same frame.  A part
-// entering a dry neighbour whose bed is above the cell's surface is dropped;
-// a dry cell splits nothing.  Wet tests and the surface come from the caller:
-// wet, wetm, wetp for the cell and its neighbours at -1 and +1, eta the
-// cell's surface, bm, bp the neighbours' beds (same datum as eta).
-template <typename R>
-__device__ __forceinline__ void tsplit(R h, R ma, R mo, R eta, bool wet,
-                                       bool wetm, R bm, bool wetp, R bp,
-                                       const R (&d)[3], R g, R (&plus)[3],
-                                       R (&minus)[3]) {
-  plus[0] = plus[1] = plus[2] = R(0);
-  minus[0] = minus[1] = minus[2] = R(0);
-  if (!wet) return;
-  const R w = qdiv(ma, h);
-  const R z = qdiv(mo, h);
-  const R c = qsqrt(g * h);
-  const R a1 = qdiv((w + c) * d[0] - d[1], R(2) * c);
-  const R a3 = qdiv(d[1] - (w - c) * d[0], R(2) * c);
-  const R a2 = d[2] - z * d[0];
-  const R l1 = w - c, l2 = w, l3 = w + c;
-  const R c1 = l1 * a1, c3 = l3 * a3, c2 = l2 * a2;
-  const R W1[3] = {c1, c1 * l1, c1 * z};
-  const R W3[3] = {c3, c3 * l3, c3 * z};
-  const R W2[3] = {R(0), R(0), c2};
-  const bool openp = !(!wetp && (bp > eta));
-  const bool openm = !(!wetm && (bm > eta));
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    const R p1 = l1 > R(0) ? W1[k] : R(0), q1 = l1 < R(0) ? W1[k] : R(0);
-    const R p3 = l3 > R(0) ? W3[k] : R(0), q3 = l3 < R(0) ? W3[k] : R(0);
-    const R p2 = l2 > R(0) ? W2[k] : R(0), q2 = l2 < R(0) ? W2[k] : R(0);
-    if (openp) plus[k] = (p1 + p3) + p2;
-    if (openm) minus[k] = (q1 + q3) + q2;
-  }
-}
-
 // ------------------------------------------------------------------------
 // The FP64 step's own forms.  The FP64 pipe bounds that kernel, so whatever
 // belongs to a cell (velocities, celerity, square root of the depth, surface)
 // is computed once per cell instead of once per edge side, and everything but
 // additions and products (comparisons, selections, scalings by two, quotients,
 // roots) runs in the integer and FP32 pipes.  The operations and their order
-// are those of riemann / edge_fluxes / tsplit above, so the values agree bit
-// for bit up to the sign of zeros.
+// are those of riemann / edge_fluxes above, so the values agree bit for bit up
+// to the sign of zeros.
 
 // One side of an edge.  A dry cell has zero u, v, c and q; h, n, t, b and eta
 // are its stored values.
@@ -518,8 +480,14 @@ __device__ __forceinline__ void edge_fluxes_prim(const double* Z, const double* 
   ff[2] = (f1[2] + f3[2]) + f2[2];
 }
 
-// Transverse split of an increment; see tsplit.  w, z: the cell's velocities
-// along the split direction and across it; c: its celerity (zero when dry).
+// Transverse split of an increment d = (mass, momentum along the split
+// direction, other momentum) in a cell with velocities w along the split
+// direction and z across it and celerity c (zero when dry): eigenvectors of
+// the split direction's Jacobian with speeds w - c, w, w + c.  plus/minus are
+// returned in the same frame.  A part entering a dry neighbour whose bed is
+// above the cell's surface is dropped; a dry cell splits nothing.  wet, wetm,
+// wetp: the cell and its neighbours at -1 and +1; eta the cell's surface, bm,
+// bp the neighbours' beds.
 __device__ __forceinline__ void tsplit_prim(double w, double z, double c, double eta, bool wet,
                                             bool wetm, double bm, bool wetp, double bp,
                                             const double (&d)[3], double (&plus)[3],
@@ -581,7 +549,7 @@ __device__ __forceinline__ bool wet_dev(float w, float b, double drytol,
 // per-cell quantities come from shared memory (see the FP64 forms).  The unit
 // is compiled without contraction and every fused operation is written out,
 // so all kernel shapes round alike; the operations and the places where they
-// fuse are those the compiler chose for riemann / edge_fluxes / tsplit.
+// fuse are those the compiler chooses for riemann / edge_fluxes.
 
 __device__ __forceinline__ float rcpf(float x) { return seed_rcp(x); }
 
@@ -955,7 +923,7 @@ __device__ __forceinline__ void edge32x2(const float* w, float nu, bool wet0, bo
   ff[2] = add2(add2(mulr2(k1, z[2], nz), mulr2(k3, z[7], nz)), mulr2(k2, z[4], nz));
 }
 
-// tsplit of two cells' increments d = (mass, along, other); w, z: velocities
+// tsplit_prim of two cells' increments d = (mass, along, other); w, z: velocities
 // along the split direction and across it, h: depths.  A dry half's result
 // is not used.
 __device__ __forceinline__ void tsplit32x2(f2 w, f2 z, f2 h, float g, f2 nz, const f2 (&d)[3],

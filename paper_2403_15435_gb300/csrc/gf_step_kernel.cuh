@@ -276,7 +276,7 @@ __device__ __forceinline__ int tix(int i, int j) {
   return (i + GF_NG) + (j + GF_NG) * (M + 2 * GF_NG);
 }
 
-// Increment cell of item k in a sweep over NRL lines: items below M*M are
+// Increment cell of item k in a split sweep over NRL lines: items below M*M are
 // interior cells in the fixed order (i = k % M, j = k / M) used by the final
 // update, so each thread owns the same cells in both sweeps; then the ghost
 // lines before the interior (from line L0 on) and those after it.  a is the
@@ -702,8 +702,8 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
     }
   }
 
-  R X[FAST ? 1 : RC][3];   // nu_x * dQx of owned interior cells
-  R Y[FAST || PRIM ? 1 : RC][3];   // nu_y * dQy (PRIM: added to X)
+  R X[PRIM ? RC : 1][3];  // PRIM: nu dQ of owned interior cells
+  R Y[DS ? RC : 1][3];    // split: nu_y * dQy
   // dimensional splitting, deviation form: compensation terms of the
   // intermediate state of owned interior cells
   float LO1[DS && DEV ? RC : 1][3];
@@ -1229,11 +1229,11 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
     __syncthreads();
     }
   };
+  // dimensional splitting: one sweep
   [[maybe_unused]] auto sweep = [&](auto dirc) {
     constexpr int dir = decltype(dirc)::value;
-    // lines swept: -1..M (unsplit), -2..M+1 (split, x), 0..M-1 (split, y)
-    constexpr int NRL = DS ? (dir == 0 ? M + 4 : M) : M + 2;
-    constexpr int L0 = DS ? (dir == 0 ? -2 : 0) : -1;
+    // lines swept: -2..M+1 (x), 0..M-1 (y)
+    constexpr int NRL = dir == 0 ? M + 4 : M, L0 = dir == 0 ? -2 : 0;
     const R* sn = dir == 0 ? shu : shv;  // normal momentum
     const R* st = dir == 0 ? shv : shu;  // transverse momentum
     const R nu = dir == 0 ? nux : nuy;
@@ -1306,10 +1306,7 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
       }
     }
     __syncthreads();
-    // phase 3: per-cell increments and their transverse split (unsplit),
-    // or the intermediate state of the x sweep (split)
-    R* Tr = dir == 0 ? Gtr : Ftr;
-    R MIr[RX][3];
+    // phase 3: per-cell increments, and the intermediate state of the x sweep
 #pragma unroll
     for (int r = 0; r < RX; ++r) {
       const int k = tid + r * NT;
@@ -1323,98 +1320,54 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
         for (int q = 0; q < 3; ++q)
           d[q] = (wl[(3 + q) * NEDGE] + wr[q * NEDGE]) +
                  (wr[(6 + q) * NEDGE] - wl[(6 + q) * NEDGE]);
-        if (r < RC && k < M * M) {
-          // store nu * dQ in (h, hu, hv) order
-          if (dir == 0) {
-            X[r][0] = nu * d[0]; X[r][1] = nu * d[1]; X[r][2] = nu * d[2];
-          } else {
-            Y[r][0] = nu * d[0]; Y[r][1] = nu * d[2]; Y[r][2] = nu * d[1];
-          }
+        if (dir == 1 && r < RC) {  // nu * dQ in (h, hu, hv) order
+          Y[r][0] = nu * d[0]; Y[r][1] = nu * d[2]; Y[r][2] = nu * d[1];
         }
-        if constexpr (DS) {
-          if constexpr (dir == 0) {
-            // intermediate state of cell (a, line) in place: every read of
-            // the window in this sweep is behind the barriers above
-            const int c = tix<M>(a, line);
-            const bool inner = k < M * M;
-            const R xs[3] = {nu * d[0], nu * d[1], nu * d[2]};
-            const R q[3] = {s0[c], shu[c], shv[c]};
-            R o[3];
-            if (inner) nwet += wetc(c) ? 1u : 0u;
-            if constexpr (!DEV) {
+        if constexpr (dir == 0) {
+          // intermediate state of cell (a, line) in place: every read of
+          // the window in this sweep is behind the barriers above
+          const int c = tix<M>(a, line);
+          const bool inner = k < M * M;
+          const R xs[3] = {nu * d[0], nu * d[1], nu * d[2]};
+          const R q[3] = {s0[c], shu[c], shv[c]};
+          R o[3];
+          if (inner) nwet += wetc(c) ? 1u : 0u;
+          if constexpr (!DEV) {
 #pragma unroll
-              for (int f = 0; f < 3; ++f) o[f] = q[f] - xs[f];
-              if (o[0] < R(0)) {
-                if (inner) { clipd -= o[0]; ++nclip; }
-                o[0] = R(0);
-              }
-              if (o[0] <= rdry) { o[1] = R(0); o[2] = R(0); }
-            } else {
-              const int kp = pix(a, line);
-              float lo[3];
-#pragma unroll
-              for (int f = 0; f < 3; ++f) {
-                const float x = (inner ? los[f * MP * MP + kp] : 0.0f) - xs[f];
-                const float s = q[f] + x;
-                const float bb = s - q[f];
-                lo[f] = (q[f] - (s - bb)) + (x - bb);
-                o[f] = s;
-              }
-              const float bc = sb[c];
-              if (o[0] < bc) {
-                if (inner) { clipf += bc - o[0]; ++nclip; }
-                o[0] = bc;
-                lo[0] = 0.0f;
-              }
-              const bool wnew = gfk::wet_dev(o[0], bc, drytol, dtf, margin);
-              if (!wnew) { o[1] = 0.0f; o[2] = 0.0f; lo[1] = 0.0f; lo[2] = 0.0f; }
-              sdep[c] = o[0] - bc;
-              swet[c] = wnew ? 1 : 0;
-              if (inner && r < RC) {
-                LO1[r][0] = lo[0]; LO1[r][1] = lo[1]; LO1[r][2] = lo[2];
-              }
+            for (int f = 0; f < 3; ++f) o[f] = q[f] - xs[f];
+            if (o[0] < R(0)) {
+              if (inner) { clipd -= o[0]; ++nclip; }
+              o[0] = R(0);
             }
-            s0[c] = o[0];
-            shu[c] = o[1];
-            shv[c] = o[2];
+            if (o[0] <= rdry) { o[1] = R(0); o[2] = R(0); }
+          } else {
+            const int kp = pix(a, line);
+            float lo[3];
+#pragma unroll
+            for (int f = 0; f < 3; ++f) {
+              const float x = (inner ? los[f * MP * MP + kp] : 0.0f) - xs[f];
+              const float s = q[f] + x;
+              const float bb = s - q[f];
+              lo[f] = (q[f] - (s - bb)) + (x - bb);
+              o[f] = s;
+            }
+            const float bc = sb[c];
+            if (o[0] < bc) {
+              if (inner) { clipf += bc - o[0]; ++nclip; }
+              o[0] = bc;
+              lo[0] = 0.0f;
+            }
+            const bool wnew = gfk::wet_dev(o[0], bc, drytol, dtf, margin);
+            if (!wnew) { o[1] = 0.0f; o[2] = 0.0f; lo[1] = 0.0f; lo[2] = 0.0f; }
+            sdep[c] = o[0] - bc;
+            swet[c] = wnew ? 1 : 0;
+            if (inner && r < RC) {
+              LO1[r][0] = lo[0]; LO1[r][1] = lo[1]; LO1[r][2] = lo[2];
+            }
           }
-          continue;
-        }
-        if (!trv) continue;
-        // split along the other direction: in that frame the "along"
-        // momentum is this sweep's transverse momentum
-        const int ci = dir == 0 ? tix<M>(a, line) : tix<M>(line, a);
-        const int cm = dir == 0 ? tix<M>(a, line - 1) : tix<M>(line - 1, a);
-        const int cp = dir == 0 ? tix<M>(a, line + 1) : tix<M>(line + 1, a);
-        const R dd[3] = {d[0], d[2], d[1]};
-        R pl[3], mi[3];
-        gfk::tsplit<R>(sdep[ci], st[ci], sn[ci], surf(ci), wetc(ci), wetc(cm),
-                       sb[cm], wetc(cp), sb[cp], dd, g, pl, mi);
-        // back to (h, hu, hv): frame (mass, along = st, other = sn)
-        const R plh[3] = {pl[0], dir == 0 ? pl[2] : pl[1],
-                          dir == 0 ? pl[1] : pl[2]};
-        MIr[r][0] = mi[0];
-        MIr[r][1] = dir == 0 ? mi[2] : mi[1];
-        MIr[r][2] = dir == 0 ? mi[1] : mi[2];
-        if (line + 1 <= M) {
-          R* o = Tr + 3 * (a * (M + 1) + line + 1);
-          o[0] = plh[0]; o[1] = plh[1]; o[2] = plh[2];
-        }
-      }
-    }
-    __syncthreads();
-    if (DS || !trv) return;
-    const R nut = dir == 0 ? nux : nuy;
-#pragma unroll
-    for (int r = 0; r < RX; ++r) {
-      const int k = tid + r * NT;
-      if (k < M * NRL) {
-        int a, line;
-        cell_item<M, NRL, L0>(k, dir, a, line);
-        if (line >= 0) {
-          R* o = Tr + 3 * (a * (M + 1) + line);
-#pragma unroll
-          for (int q = 0; q < 3; ++q) o[q] = R(-0.5) * nut * (o[q] + MIr[r][q]);
+          s0[c] = o[0];
+          shu[c] = o[1];
+          shv[c] = o[2];
         }
       }
     }
@@ -1642,7 +1595,7 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
       for (int f = 0; f < 3; ++f) {
         R fl;
         if constexpr (BOTH) fl = X[r][f] + W[(Lo::NWP + f) * NEDGE + k];
-        else fl = DS ? Y[DS ? r : 0][f] : X[r][f];
+        else fl = DS ? Y[DS ? r : 0][f] : X[PRIM ? r : 0][f];
         const R* fa = Ftr + 3 * (j * (M + 1) + i);
         const R* ga = Gtr + 3 * (i * (M + 1) + j);
         const R tf = trv ? nux * (fa[3 + f] - fa[f]) + nuy * (ga[3 + f] - ga[f]) : R(0);
