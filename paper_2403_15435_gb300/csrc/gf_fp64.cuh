@@ -11,9 +11,10 @@
 // needs 468; the division and square-root sequences (some eight to ten
 // FP64 operations each, about 50 of them per cell) were most of the rest.
 //
-// The header also compiles for the host, where the reciprocal seeds are
-// perturbed by up to GF_SEED_ERR so that a test can cover the whole range of
-// errors the device's approximations may have.
+// The header also compiles for the host, where a program provides the seeds:
+// a test draws their relative errors from the whole range that the device's
+// approximations may have (reciprocals and roots up to 2^-22, about twice the
+// documented bounds; cube roots 2^-20).
 #pragma once
 
 #include <cmath>
@@ -87,8 +88,9 @@ constexpr long long D_INF = 0x7ffll << 52;
 // a / b.  Digit recurrence on the 53-bit significands ma, mb: three quotient
 // digits of 20, 20 and 15 bits, each the remainder's leading bits times an
 // FP32 reciprocal of mb rounded to an integer, with the remainder updated
-// exactly modulo 2^64.  The reciprocal is within 2^-21.5 (23-bit truncation
-// of mb plus the approximation), so a digit is off by less than 2 units, the
+// exactly modulo 2^64.  The reciprocal is within 2^-21.4 of 1 / mb (2^-23
+// from the truncation of mb to 23 bits, 2^-22 allowed to the approximation),
+// so a digit is off by less than 2 units, the
 // remainder stays below 2^55 and the last digit (15 bits) is within 0.6 of
 // the exact one: the sign of the last remainder says whether the 56-bit
 // quotient is one too large, and whether it is zero is the sticky bit.
