@@ -145,9 +145,14 @@ struct GfView {
   // Launch order of the patch step (or null: patch order).  sched[0] counts
   // the launches modulo 6; its parity selects which of ord0/ord1 a launch
   // reads; the launch writes the other one with the patches that took the
-  // step first (sched[1], sched[2] count those and the others), and its last
-  // CTA advances sched[0] and stores the number of the others in
-  // inactive[parity ^ 1].  (Without run flags: the patches whose tile held
+  // step first (sched[1] or, writing ord0, sched[3] counts them) and the
+  // others from the end (sched[2] or sched[4]), and its last CTA advances
+  // sched[0], stores the number of the others in inactive[parity ^ 1] and
+  // clears the two counters of the next launch.  It does not clear its own: a
+  // CTA that changed nothing counts itself done without a fence, so that
+  // nothing orders its entry before the last CTA's writes; were the counter
+  // cleared first, the next launch would start it at one and write before the
+  // order's first place.  (Without run flags: the patches whose tile held
   // water first.)  Only with a controller (done != null).
   //
   // A launch reads inactive[parity]; the host alternates parity from launch

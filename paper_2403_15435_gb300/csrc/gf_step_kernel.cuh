@@ -101,6 +101,12 @@ struct TileHdr {
   int* order;     // the next launch order (or null: another CTA enters the patch)
 };
 
+// Counters of a launch order that is being written (GfView::sched): [0] its
+// head, [1] its tail.
+__device__ __forceinline__ unsigned* order_ends(const GfView& V, const int* order) {
+  return V.sched + (order == V.ord0 ? 3 : 1);
+}
+
 template <typename R>
 __device__ __forceinline__ R warp_max(R v) {
 #pragma unroll
@@ -926,7 +932,7 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
     // the patch in the next launch order meanwhile (at the tile's end the
     // round trip would be waited for)
     if (dir == 1 && tid == NT - 1 && H.order != nullptr)
-      H.order[atomicAdd(V.sched + 1, 1u)] = p;
+      H.order[atomicAdd(order_ends(V, H.order), 1u)] = p;
     constexpr int PTP = M * (M + 4);          // one plane
     constexpr int PT = dir == 0 ? M : M + 4;  // its rows
     R* Tr = Ftr;
@@ -1945,13 +1951,23 @@ __device__ void step_finish(const GfGeom& G, const GfView& V, int cells_per_patc
   // has ended, which orders these writes before it (a thread without a
   // scenario, if there is one: its loads go beside the controller's)
   if (threadIdx.x == NT - 1 && V.sched) {
-    V.sched[0] = (V.sched[0] + 1u) % 6u;
+    const unsigned count = V.sched[0], par = count & 1u;
     // patches that took no step, at the tail of the next order
     // (in the word this launch does not read: CTAs beyond the working ones
-    // may start after this and must still find themselves beyond)
-    if (V.inactive) V.inactive[V.parity ^ 1u] = V.sched[2];
-    V.sched[1] = 0u;
-    V.sched[2] = 0u;
+    // may start after this and must still find themselves beyond).  CTAs that
+    // did not fence may have entries on their way that this does not count;
+    // those patches get CTAs of their own next time.
+    unsigned tail;
+    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];"
+                 : "=r"(tail)
+                 : "l"(V.sched + 2 + 2 * par)
+                 : "memory");
+    V.sched[0] = (count + 1u) % 6u;
+    if (V.inactive) V.inactive[V.parity ^ 1u] = tail;
+    // the next launch's counters, which no CTA of this one touches: its own
+    // may still be counted up
+    V.sched[3 - 2 * par] = 0u;
+    V.sched[4 - 2 * par] = 0u;
   }
   if (threadIdx.x == 0) *V.done = 0u;
 }
@@ -2042,7 +2058,7 @@ __global__ void __launch_bounds__(NT, MINB)
       flags(2u)[pl] = 0;
       if (skip) {
         int* nxt = par ? V.ord0 : V.ord1;
-        nxt[V.npatch - 1 - (int)atomicAdd(V.sched + 2, 1u)] = pl;
+        nxt[V.npatch - 1 - (int)atomicAdd(order_ends(V, nxt) + 1, 1u)] = pl;
       }
     }
   }
@@ -2092,8 +2108,9 @@ __global__ void __launch_bounds__(NT, MINB)
       }
     }
     if (nxt != nullptr && threadIdx.x == 0 && !(Lo::FAST && wet > 0)) {
-      if (use_flags || wet) nxt[atomicAdd(V.sched + 1, 1u)] = p;
-      else nxt[V.npatch - 1 - (int)atomicAdd(V.sched + 2, 1u)] = p;
+      unsigned* ends = order_ends(V, nxt);
+      if (use_flags || wet) nxt[atomicAdd(ends, 1u)] = p;
+      else nxt[V.npatch - 1 - (int)atomicAdd(ends + 1, 1u)] = p;
     }
     return wet;
   };
