@@ -159,8 +159,9 @@ struct GfView {
   // to launch, so that no launch writes the word it reads: every CTA of it,
   // however late it starts, counts the same working CTAs.  The value decides
   // only how the order is shared out, never which patches run: above npatch
-  // (nothing known yet) every patch gets its own CTAs, and an older launch's
-  // number is right too.  A chunk's last launch writes inactive[1], which the
+  // (nothing known yet) every patch gets its own CTAs and keeps its place in
+  // the order (npatch + 1: for one more launch), and an older launch's number
+  // is right too.  A chunk's last launch writes inactive[1], which the
   // next chunk reads first if its launches are even in number; otherwise it
   // reads inactive[0], where ctl_begin has put the same.
   unsigned* sched;
