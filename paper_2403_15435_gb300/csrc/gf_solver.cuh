@@ -654,9 +654,10 @@ __device__ __forceinline__ float jump_bound(float dh, float s1, float s3, float 
 // for both halves at once.  (One after the other through a general solver of
 // their own such edges doubled the phase's time in a front's tile: 64 patches
 // of 16 x 16 with a front 16.7 us a step, 15.4 so.)
-// DRY = false: both cells of every edge that counts are wet.
+// DRY = false: both cells of every edge that counts are wet.  Returns whether
+// both edges took the straight line alone, which no edge with a dry cell does.
 template <bool DRY>
-__device__ __forceinline__ void riemann32x2(Prim32x2 l, Prim32x2 r, float g, float sg, f2 nz,
+__device__ __forceinline__ bool riemann32x2(Prim32x2 l, Prim32x2 r, float g, float sg, f2 nz,
                                             f2 (&z)[8], f2& s1, f2& s3) {
   f2 hl = sub2(l.w, l.b), hr = sub2(r.w, r.b);
   float ql0, ql1, qr0, qr1;
@@ -722,7 +723,8 @@ __device__ __forceinline__ void riemann32x2(Prim32x2 l, Prim32x2 r, float g, flo
   float ok0, ok1;
   upk(ok, ok0, ok1);
   f2 d1 = deta;
-  if (!(ok0 > 0.0f && ok1 > 0.0f)) {
+  const bool usual = ok0 > 0.0f && ok1 > 0.0f;
+  if (!usual) {
     // the stationary wave's depth jump, bounded for non-negative depths
     const f2 hh = mulr2(mulr2(x, rden, nz), den, nz);
     const f2 b1 = mul2(hh, rcp2(s1)), b3 = mul2(hh, rcp2(s3));
@@ -761,6 +763,7 @@ __device__ __forceinline__ void riemann32x2(Prim32x2 l, Prim32x2 r, float g, flo
     s1 = sel2(e0, e1, 0ull, s1);
     s3 = sel2(e0, e1, 0ull, s3);
   }
+  return usual;
 }
 
 // riemann32x2 of one edge with a wet and a dry cell (fields w, b, n, u, v, q).

@@ -327,7 +327,10 @@ __device__ __forceinline__ void cell_item(int k, int dir, int& a, int& line) {
 // neighbours; the copies of the edge cells follow the update side by side.
 // 4 km x 2 km valley, 10496 patches, 5012 of them with water: 269 M -> 191 M
 // warp instructions, 393 -> 312 us per launch; 17 km x 9 km canyon of 19350 16
-// x 16 patches, 1837 with water: 182 -> 75 us.  Results keep every bit.
+// x 16 patches, 1837 with water: 182 -> 75 us.  Results are those of one edge to
+// a thread bit for bit, but for waves below 1e-19, which no longer switch their
+// limiter off: equal on uniform grids, a rounding apart (1e-8 relative) in
+// refined forests.
 //
 // Scheme variants (Sec. 3.2): G.first_order drops the limited corrections,
 // G.no_transverse the transverse terms; DS (dimensional splitting) takes the
@@ -771,25 +774,53 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
         return gfk::ld2(p + c + CS);
       }
     };
-    auto solve = [&](int k, unsigned both, auto dryc) {
+    // Edges between a wet and a dry cell: the blocks they add to a pair cost a
+    // warp the same for one lane as for all.  With one pair to a thread they
+    // are taken on the way; with several (whole 32 x 32 tiles, where a front
+    // touches nearly every warp in every round) they are set aside and taken
+    // together, one edge to a thread.  256 patches with a front: 22.2 us a
+    // step on the way, 21.5 so.  What such a pair needs is found behind the
+    // solver's own test for unusual edges, so that pairs of wet cells pay
+    // nothing for it (valley of 6827 patches: 178.4 us a step with the
+    // wetness of every pair found first, 175.8 so).
+    constexpr bool LATER = Lo::ASIDE > 0 && N1 > NT;
+#pragma unroll 1
+    for (int k = tid; k < N1; k += NT) {
       const int m = k % (PW / 2), row = k / (PW / 2);
-      const int c = cell_of(k);
-      auto pair_l = [&](const R* p) { return gfk::ld2(p + c); };
-      const gfk::Prim32x2 L{pair_l(s0), pair_l(sb), pair_l(sn),
-                            pair_l(un), pair_l(ut), pair_l(sq)};
-      const gfk::Prim32x2 Rt{pair_r(s0, c, L.w), pair_r(sb, c, L.b), pair_r(sn, c, L.n),
-                             pair_r(un, c, L.u), pair_r(ut, c, L.v), pair_r(sq, c, L.q)};
-      f2 z[8], s1, s3;
-      constexpr bool DRY = decltype(dryc)::value;
-      gfk::riemann32x2<DRY>(L, Rt, g, sg, nz, z, s1, s3);
-      if (!DRY && both != 3u) {  // nothing (yet) where a cell is dry
-        const bool b0 = both & 1u, b1 = both & 2u;
+      const int c = cell_of(k), e = row * PW + 2 * m;
+      R* w = W + e;
+      const f2 ql = gfk::ld2(sq + c), qr = pair_r(sq, c, ql);
+      if ((ql | qr) == 0ull) {  // dry cells
 #pragma unroll
-        for (int q = 0; q < 8; ++q) z[q] = gfk::sel2(b0, b1, z[q], 0ull);
-        s1 = gfk::sel2(b0, b1, s1, 0ull);
-        s3 = gfk::sel2(b0, b1, s3, 0ull);
+        for (int q = 0; q < 10; ++q) gfk::st2(w + q * NEDGE, 0ull);
+        continue;
       }
-      R* w = W + row * PW + 2 * m;
+      auto pair_l = [&](const R* p) { return gfk::ld2(p + c); };
+      const gfk::Prim32x2 L{pair_l(s0), pair_l(sb), pair_l(sn), pair_l(un), pair_l(ut), ql};
+      const gfk::Prim32x2 Rt{pair_r(s0, c, L.w), pair_r(sb, c, L.b), pair_r(sn, c, L.n),
+                             pair_r(un, c, L.u), pair_r(ut, c, L.v), qr};
+      f2 z[8], s1, s3;
+      const bool usual = gfk::riemann32x2<!LATER>(L, Rt, g, sg, nz, z, s1, s3);
+      if constexpr (LATER) {
+        if (!usual) {
+          // nothing (yet) where a cell is dry
+          float a0, a1, b0, b1;
+          gfk::upk(ql, a0, a1);
+          gfk::upk(qr, b0, b1);
+          const bool x0 = a0 > 0.0f, x1 = a1 > 0.0f, y0 = b0 > 0.0f, y1 = b1 > 0.0f;
+#pragma unroll
+          for (int q = 0; q < 8; ++q) z[q] = gfk::sel2(x0 && y0, x1 && y1, z[q], 0ull);
+          s1 = gfk::sel2(x0 && y0, x1 && y1, s1, 0ull);
+          s3 = gfk::sel2(x0 && y0, x1 && y1, s3, 0ull);
+          const bool mix0 = x0 != y0, mix1 = x1 != y1;
+          if (mix0 || mix1) {
+            const unsigned at = atomicAdd(naside, (mix0 ? 1u : 0u) + (mix1 ? 1u : 0u));
+            const unsigned at1 = at + (mix0 ? 1u : 0u);
+            if (mix0 && at < (unsigned)Lo::ASIDE) aside[at] = (unsigned short)e;
+            if (mix1 && at1 < (unsigned)Lo::ASIDE) aside[at1] = (unsigned short)(e + 1);
+          }
+        }
+      }
 #pragma unroll
       for (int q = 0; q < 8; ++q) gfk::st2(w + q * NEDGE, z[q]);
       gfk::st2(w + 8 * NEDGE, s1);
@@ -807,50 +838,6 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
       } else {
         if ((unsigned)(row - 1) <= (unsigned)M && m > 0 && m <= M2)
           smax = fmaxf(smax, fmaxf(ma, mb));
-      }
-    };
-    // Edges between a wet and a dry cell: the blocks they add to a pair cost a
-    // warp the same for one lane as for all.  With one pair to a thread they
-    // are taken on the way; with several (whole 32 x 32 tiles, where a front
-    // touches nearly every warp in every round) they are set aside and taken
-    // together, one edge to a thread.  256 patches with a front: 22.2 us a
-    // step on the way, 21.5 so.
-    constexpr bool LATER = Lo::ASIDE > 0 && N1 > NT;
-    // the wet sides of pair k: bits 0, 1 left (below), 2, 3 right
-    auto wetness = [&](int k) {
-      const int c = cell_of(k);
-      const f2 ql = gfk::ld2(sq + c), qr = pair_r(sq, c, ql);
-      float a0, a1, b0, b1;
-      gfk::upk(ql, a0, a1);
-      gfk::upk(qr, b0, b1);
-      return (a0 > 0.0f ? 1u : 0u) | (a1 > 0.0f ? 2u : 0u) | (b0 > 0.0f ? 4u : 0u) |
-             (b1 > 0.0f ? 8u : 0u);
-    };
-#pragma unroll 1
-    for (int k = tid; k < N1; k += NT) {
-      const unsigned wn = wetness(k), both = wn & (wn >> 2);
-      if (LATER ? both == 0u : wn == 0u) {
-        R* w = W + (k / (PW / 2)) * PW + 2 * (k % (PW / 2));
-#pragma unroll
-        for (int q = 0; q < 10; ++q) gfk::st2(w + q * NEDGE, 0ull);
-      } else {
-        solve(k, both, std::bool_constant<!LATER>{});
-      }
-      if constexpr (LATER) {
-        const unsigned mixed = (wn ^ (wn >> 2)) & 3u, now = __activemask();
-        if (__any_sync(now, mixed != 0u)) {
-          const unsigned m0 = __ballot_sync(now, mixed & 1u), m1 = __ballot_sync(now, mixed & 2u);
-          const int lane = tid & 31, lead = __ffs(now) - 1;
-          unsigned at = 0u;
-          if (lane == lead) at = atomicAdd(naside, (unsigned)(__popc(m0) + __popc(m1)));
-          at = __shfl_sync(now, at, lead);
-          const unsigned below = (1u << lane) - 1u;
-          const unsigned at0 = at + __popc(m0 & below);
-          const unsigned at1 = at + __popc(m0) + __popc(m1 & below);
-          const int e = (k / (PW / 2)) * PW + 2 * (k % (PW / 2));
-          if ((mixed & 1u) && at0 < (unsigned)Lo::ASIDE) aside[at0] = (unsigned short)e;
-          if ((mixed & 2u) && at1 < (unsigned)Lo::ASIDE) aside[at1] = (unsigned short)(e + 1);
-        }
       }
     }
     if constexpr (LATER) {
@@ -1494,6 +1481,7 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
         // corners.  In the domain it is a cell of the neighbour there; beyond
         // its boundary a mirror cell of this patch or, at a corner beyond one
         // side only, of the neighbour along the other.
+        const bool inland = Pt.px > 0 && Pt.px < nxp - 1 && Pt.py > 0 && Pt.py < nyp - 1;
         for (int k = tid; k < 8 * M + 16; k += NT) {
           int r, i, j;  // region, source cell
           if (k < 4 * M) {
@@ -1514,6 +1502,16 @@ __device__ __forceinline__ int patch_body(const GfGeom& G, const GfView& V,
           // its direction
           const int sx = r == 0 || r == 4 || r == 6 ? -1 : (r == 1 || r == 5 || r == 7 ? 1 : 0);
           const int sy = r == 2 || r == 4 || r == 5 ? -1 : (r == 3 || r == 6 || r == 7 ? 1 : 0);
+          if (inland) {  // (most patches: no mirrors)
+            const int pn = push ? snb[r] : -1;
+            if (pn < 0) continue;
+            const R* v = nv + j * M + i;
+            R* d = qnext + (size_t)pn * 3 * TG + tix<M>(i - sx * M, j - sy * M);
+            d[0] = v[0];
+            d[TG] = v[M * M];
+            d[2 * TG] = v[2 * M * M];
+            continue;
+          }
           const bool bx = sx != 0 && (unsigned)(Pt.px + sx) >= (unsigned)nxp;
           const bool by = sy != 0 && (unsigned)(Pt.py + sy) >= (unsigned)nyp;
           // the patch that holds it
@@ -1925,10 +1923,9 @@ static __device__ void ctl_finish(const GfGeom& G, GfCtl* Cp, unsigned long long
 // scenario, one thread per scenario (the scenarios' rules are independent).
 // The volume of the state is not part of the step; geoflood_mass computes it
 // on demand.
-// idle: the number of idle patches that the launch started from.
 template <int NT>
 __device__ void step_finish(const GfGeom& G, const GfView& V, int cells_per_patch, bool wrote,
-                            unsigned nctas, unsigned idle) {
+                            unsigned nctas) {
   __shared__ int last;
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -1965,9 +1962,10 @@ __device__ void step_finish(const GfGeom& G, const GfView& V, int cells_per_patc
                  : "memory");
     V.sched[0] = (count + 1u) % 6u;
     // After a write of the state nothing is known for two launches.
-    const unsigned none = (unsigned)V.npatch + 1u;
-    if (V.inactive)
+    if (V.inactive) {
+      const unsigned none = (unsigned)V.npatch + 1u, idle = V.inactive[V.parity];
       V.inactive[V.parity ^ 1u] = idle < none ? tail : (idle == none ? 0u : none);
+    }
     // the next launch's counters, which no CTA of this one touches: its own
     // may still be counted up
     V.sched[3 - 2 * par] = 0u;
@@ -2149,7 +2147,7 @@ __global__ void __launch_bounds__(NT, MINB)
   }
   }
   if (V.done)
-    step_finish<NT>(G, V, MP * MP, wrote, working, idle);
+    step_finish<NT>(G, V, MP * MP, wrote, working);
 }
 
 // Launch the patch step on every patch: MP x MP patches, M x M sub-tiles
