@@ -81,13 +81,14 @@ FP64_LANES_PER_SM = 2  # measured: DFMA throughput 1.20 TFLOP/s on 152 SMs
 N_SM = 152
 # DRAM bytes (read + write) of one patch-step launch, from the ncu captures
 # summarised in profiles/ (cold caches); None when the kernel has changed
-# since (the uniform workloads).  Valley: the launch at t = 30 s (6815
-# patches) of variant 0, which the autotuner picks there, 82 736 640 B read
-# and 31 502 336 B written over 6 978 560 cells, scaled to the cells of an
-# average timed launch.
-TRAFFIC_PER_LAUNCH_FP32 = None
+# since (the uniform workload in FP64).  Valley: the launch at t = 30 s (6815
+# patches) of variant 0, which the autotuner picks there, 83 906 304 B read
+# and 28 998 400 B written over 6 978 560 cells, scaled to the cells of an
+# average timed launch.  Uniform workload: launch 151 (t = 29.5 s), 5 615 360 B
+# read and 8192 B written.
+TRAFFIC_PER_LAUNCH_FP32 = 5615360 + 8192
 TRAFFIC_PER_LAUNCH_FP64 = None
-TRAFFIC_PER_CELL_VALLEY_FP32 = (82736640 + 31502336) / 6978560
+TRAFFIC_PER_CELL_VALLEY_FP32 = (83906304 + 28998400) / 6978560
 
 
 def parse():

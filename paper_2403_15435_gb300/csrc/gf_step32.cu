@@ -18,10 +18,13 @@ namespace gf {
 // KB of shared memory each), except where the sub-tiles of all patches are
 // resident at once (152 SMs x 4 CTAs): a tile's chain of barriers, not the
 // arithmetic, is then the launch's time, and smaller tiles have shorter ones.
-// Measured, us per step of a third-wet grid, whole / 16 x 16 / 8 x 8: 16
-// patches 23.8 / 17.7 / 16.4, 36 patches 25.1 / 17.8 / 17.0, 64 patches 23.9 /
-// 17.9 / 17.7, 144 patches 24.8 / 20.8 / 23.8, 256 patches 26.0 / 25.0 / 34.0
-// (every cell wet: 24.7 / 31.7 / 48.5), 1024 patches 45.9 / 54.6 / 87.2.
+// Measured, us per step with a front (a third wet) and with every cell wet,
+// whole tiles / 16 x 16 / 8 x 8 (whole tiles of up to 152 patches in shape 3,
+// one CTA per SM): 16 patches 20.5 / 14.7 / 13.7 and 18.0 / 13.3 / 13.4; 36
+// patches 19.6 / 14.9 / 14.2 and 18.0 / 14.1 / 14.2; 64 patches 19.7 / 15.0 /
+// 14.9 and 17.4 / 14.2 / 15.1; 144 patches 20.0 / 17.2 / 19.0 and 17.9 / 18.0 /
+// 28.4; 256 patches 21.1 / 20.9 / 28.7 and 22.7 / 29.5 / 45.7; 1024 patches
+// 39.3 / 45.3 / 71.7 and 68.0 / 89.6 / 146.
 int launch_patch_step_f32(const GfGeom& g, const GfView& v, int variant,
                           void* stream) {
   if (v.npatch <= 0) return 0;
